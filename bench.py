@@ -344,11 +344,10 @@ def run_workload(w, args, steps, warmup, ctx, want_e2e, want_cpu, sketches, fact
     dom_launches_per_step = prof_dom["launches"] / steps
     if dominant == "eig_shrink":
         achieved = eig_flops / (dom_ms_per_step * 1e-3) / 1e12
-        roof = {"kernel": "k_eig_shrink_fast" if 2 * ell <= 64 else "k_eig_shrink_dsm", "bound": "alu", "achieved": achieved,
+        roof = {"kernel": "k_tridiag + k_tridiag_vectors", "bound": "alu", "achieved": achieved,
                 "peak": FP32_ALU_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP32_ALU_PEAK_TFLOPS, "traffic": None,
                 "peak_source": "derived: 148 SMs x 128 fp32 FMA lanes x 2 flop x 1.965 GHz",
-                "algorithmic": "9*n^3 flop per n x n symmetric eigen-solve (textbook count)",
-                "frac_of_the_sms_it_runs_on": achieved / (FP32_ALU_PEAK_TFLOPS * (1 if 2 * ell <= 64 else 8) / 148.0)}
+                "algorithmic": "9*n^3 flop per n x n symmetric eigen-solve (textbook count)"}
     else:
         gbs = per_step_bytes.get(dominant, 0) / (dom_ms_per_step * 1e-3) / 1e9
         kname = {"gram": "k_tc_gemm_nt_x3 (Gram)", "rebuild": "k_tc_rebuild", "append": "k_append",

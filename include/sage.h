@@ -247,7 +247,7 @@ typedef struct {
     int64_t rows_seen;      /* rows given to sage_fd_update since create/reset */
     int64_t shrinks;        /* shrinks applied (including the one in finalize, if any) */
     double sum_delta;       /* sum of delta over shrinks: an upper bound on ||G^T G - S^T S||_2 */
-    int32_t last_sweeps;    /* Jacobi sweeps of the most recent eigen-solve */
+    int32_t last_sweeps;    /* Jacobi sweeps of the most recent eigen-solve (0: the direct solve, option 5) */
     int32_t max_sweeps;     /* largest sweep count seen */
     int32_t last_rank;      /* numerical rank found by the most recent factorisation */
     uint32_t device_flags;  /* bit 0: eigen-solver not converged, bit 1: non-finite input seen,
@@ -266,9 +266,9 @@ sage_status_t sage_fd_stats(sage_fd_t* h, sage_stats_t* out);
  * kernel classes to time with CUDA events on the launching stream (see sage_fd_profile; default 0); key 4 =
  * 1 (default) to use the tensor-core kernels wherever the operands meet their alignment rules (16-byte
  * aligned base, row pitch a multiple of 16 bytes), 0 to use the CUDA-core kernels everywhere; key 5 = which
- * kernels run the eigen-solve: 0 (default) a cluster of 8 thread blocks with the Jacobi columns in distributed
- * shared memory, 1 the single-block kernel (buffers of up to 192 rows) or the cluster kernel that keeps the
- * matrix in L2. Same algorithm either way; results agree up to rounding order.
+ * kernels run the eigen-solve: 0 (default) the direct one (tridiagonalisation in fp32, eigenvalues and eigenvectors of
+ * the tridiagonal matrix in fp64), 1 the iterative one (one-sided Jacobi on a Cholesky factor; the sweep limit of
+ * option 2 and the sweep counts of sage_stats_t are its own). Results agree up to rounding.
  * Before the first update: key 6 = P, the number of sketches of the merged form of pass 1 (1 .. 64, default 1 = the
  * paper's single sequential sketch); key 7 = rows per dealt block (default ell + 1). With P > 1 the row stream is cut into
  * blocks of that many consecutive rows, block b (counted from the first row ever given, across calls) goes to sketch

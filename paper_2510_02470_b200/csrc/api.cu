@@ -142,9 +142,10 @@ struct sage_fd {
     size_t gram_part_floats = 0;   // at least kGramPartFloats; 16 slices of m x m for buffers of more than 256 rows
     float* Wsplit = nullptr;       // rebuild factors split for the tensor cores: wsplit_ld rows x wsplit_ld floats
     int wsplit_ld = 256;           // 256 (buffers of up to 256 rows) or 512
-    float* Kmat = nullptr;         // m x m
+    float* Kmat = nullptr;         // m x m, pitch ldk
+    int ldk = 0;                   // m rounded up to 4: the eigen-solve reads rows as float4
     float* Ur = nullptr;           // m x m
-    float* eig_work = nullptr;     // m x m
+    float* eig_work = nullptr;     // eig_work_floats(m) floats
     float* sigma = nullptr;        // ell
     EigInfo* info = nullptr;       // device
     // scoring
@@ -176,7 +177,7 @@ struct sage_fd {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int* tc_err = nullptr;         // set by a tensor-core kernel whose bounded wait ran out
     bool use_tc = true;            // option 4: tensor-core kernels where their alignment rules hold
-    int eig_variant = 0;           // option 5: 0 cluster eigen-solve in distributed shared memory, 1 the one-CTA / L2 kernels
+    int eig_variant = 0;           // option 5: 0 the direct eigen-solve, 1 the iterative one
     int64_t launches = 0;
     int64_t tc_launches = 0;       // how many of them were tensor-core (tcgen05) kernels
     int64_t rows_in_place = 0;     // rows that shrink cycles read where the caller held them (never appended)
@@ -268,7 +269,7 @@ sage_status_t enqueue_freeze_aux(sage_fd* h, cudaStream_t st) {
     return SAGE_OK;
 }
 
-// Gram of the first r buffer rows -> Kmat (r x r, pitch m).
+// Gram of the first r buffer rows -> Kmat (r x r, pitch ldk).
 sage_status_t enqueue_gram(sage_fd* h, int r, cudaStream_t st) {
     float* Bc = h->B[h->cur];
     if (h->use_tc) {
@@ -286,9 +287,9 @@ sage_status_t enqueue_gram(sage_fd* h, int r, cudaStream_t st) {
         if (e == cudaSuccess) {
             h->tc_launches += 1;
             if (sym)
-                CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_gram_sym_reduce(h->gram_parts, splits, stride, r, ldc, h->Kmat, h->m, st); }));
+                CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_gram_sym_reduce(h->gram_parts, splits, stride, r, ldc, h->Kmat, h->ldk, st); }));
             else   // sums the K slices and fills the tiles below the diagonal from their mirror images
-                CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_split_reduce(h->gram_parts, splits, stride, r, r, ldc, h->Kmat, h->m, st, 1); }));
+                CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_split_reduce(h->gram_parts, splits, stride, r, r, ldc, h->Kmat, h->ldk, st, 1); }));
             return SAGE_OK;
         }
         if (e != cudaErrorNotSupported) CU_TRY(e);
@@ -300,12 +301,12 @@ sage_status_t enqueue_gram(sage_fd* h, int r, cudaStream_t st) {
     const int r_pad = ((r + 63) / 64) * 64;
     const int64_t stride = (int64_t)r_pad * r_pad;
     if (splits == 1) {
-        CU_TRY(timed(h, K_GRAM, 1, st, [&] { return launch_gemm_nt(Bc, SAGE_F32, h->pitch, Bc, h->pitch, r, r, h->D, 1, h->Kmat, h->m, 0, st); }));
+        CU_TRY(timed(h, K_GRAM, 1, st, [&] { return launch_gemm_nt(Bc, SAGE_F32, h->pitch, Bc, h->pitch, r, r, h->D, 1, h->Kmat, h->ldk, 0, st); }));
     } else {
         CU_TRY(timed(h, K_GRAM, 1, st, [&] {
             return launch_gemm_nt(Bc, SAGE_F32, h->pitch, Bc, h->pitch, r, r, h->D, splits, h->gram_parts, r_pad, stride, st);
         }));
-        CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_split_reduce(h->gram_parts, splits, stride, r, r, r_pad, h->Kmat, h->m, st); }));
+        CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_split_reduce(h->gram_parts, splits, stride, r, r, r_pad, h->Kmat, h->ldk, st); }));
     }
     return SAGE_OK;
 }
@@ -316,8 +317,8 @@ sage_status_t enqueue_factor(sage_fd* h, int r, int do_shrink, int keep, int zer
     CU_TRY(cudaEventRecord(h->ev_fork, st));       // from here on HBM is idle until the rebuild: see sage_fd_update
     const int j_pad = ((keep + 15) / 16) * 16;
     const bool tc_rebuild = h->use_tc && h->Wsplit && keep > 0 && j_pad <= h->wsplit_ld / 2 && r <= h->wsplit_ld;
-    CU_TRY(timed(h, K_EIG, 1, st, [&] {
-        return launch_eig_shrink(h->Kmat, h->m, r, do_shrink, h->delta_rank, keep, h->Ur, h->m, h->sigma, h->ell, h->eig_work,
+    CU_TRY(timed(h, K_EIG, eig_launches(r, h->eig_variant), st, [&] {
+        return launch_eig_shrink(h->Kmat, h->ldk, r, do_shrink, h->delta_rank, keep, h->Ur, h->m, h->sigma, h->ell, h->eig_work,
                                  h->max_sweeps, h->info, tc_rebuild ? h->Wsplit : nullptr, h->wsplit_ld, j_pad, h->eig_variant, st);
     }));
     const int m_total = zero_to > keep ? zero_to : keep;
@@ -426,7 +427,8 @@ static sage_status_t create_handle(sage_fd_t** out, int64_t D, int32_t ell, sage
     h->block = ell + 1;
     h->pitch = ((D + 31) / 32) * 32;
     const size_t bbytes = (size_t)h->m * h->pitch * sizeof(float);
-    const size_t mm = (size_t)h->m * h->m * sizeof(float);
+    h->ldk = (h->m + 3) & ~3;
+    const size_t mm = (size_t)h->m * h->ldk * sizeof(float);
     auto fail = [&](cudaError_t e, const char* what) {
         set_err("sage_fd_create: %s failed: %s", what, cudaGetErrorString(e));
         sage_fd_destroy(h);
@@ -446,9 +448,7 @@ static sage_status_t create_handle(sage_fd_t** out, int64_t D, int32_t ell, sage
     if ((e = cudaMemset(h->Wsplit, 0, (size_t)h->wsplit_ld * h->wsplit_ld * sizeof(float))) != cudaSuccess) return fail(e, "cudaMemset");
     if ((e = cudaMalloc((void**)&h->Kmat, mm)) != cudaSuccess) return fail(e, "cudaMalloc(K)");
     if ((e = cudaMalloc((void**)&h->Ur, mm)) != cudaSuccess) return fail(e, "cudaMalloc(U)");
-    // eigen workspace: the matrix padded to 256 or 512 rows/columns plus a few flag words
-    const size_t ew = h->m > 256 ? (size_t)512 * 512 : (size_t)256 * 256;
-    if ((e = cudaMalloc((void**)&h->eig_work, (ew + 64) * sizeof(float))) != cudaSuccess)
+    if ((e = cudaMalloc((void**)&h->eig_work, eig_work_floats(h->m) * sizeof(float))) != cudaSuccess)
         return fail(e, "cudaMalloc(eig)");
     if ((e = cudaMalloc((void**)&h->sigma, ell * sizeof(float))) != cudaSuccess) return fail(e, "cudaMalloc(sigma)");
     if ((e = cudaMalloc((void**)&h->info, sizeof(EigInfo))) != cudaSuccess) return fail(e, "cudaMalloc(info)");
@@ -671,10 +671,10 @@ static sage_status_t sketch_factor_direct(sage_fd* s, const void* rows, int64_t 
     }
     CU_TRY(e);
     s->tc_launches += 1;
-    CU_TRY(timed(s, K_GRAM_REDUCE, 1, chain, [&] { return launch_gram_sym_reduce(s->gram_parts, splits, stride, r, ldc, s->Kmat, s->m, chain); }));
+    CU_TRY(timed(s, K_GRAM_REDUCE, 1, chain, [&] { return launch_gram_sym_reduce(s->gram_parts, splits, stride, r, ldc, s->Kmat, s->ldk, chain); }));
     CU_TRY(cudaEventRecord(s->ev_fork, chain));
-    CU_TRY(timed(s, K_EIG, 1, chain, [&] {
-        return launch_eig_shrink(s->Kmat, s->m, r, 1, s->delta_rank, keep, s->Ur, s->m, s->sigma, s->ell, s->eig_work, s->max_sweeps, s->info,
+    CU_TRY(timed(s, K_EIG, eig_launches(r, s->eig_variant), chain, [&] {
+        return launch_eig_shrink(s->Kmat, s->ldk, r, 1, s->delta_rank, keep, s->Ur, s->m, s->sigma, s->ell, s->eig_work, s->max_sweeps, s->info,
                                  s->Wsplit, s->wsplit_ld, j_pad, s->eig_variant, chain);
     }));
     e = timed(s, K_REBUILD, 1, chain, [&] {

@@ -118,14 +118,18 @@ cudaError_t launch_rebuild(const float* Ur, int ldu, const float* Bsrc, float* B
 // matrix has fewer eigenvalues), keep = delta_rank-1 columns. do_shrink == 0: delta = 0, keep columns.
 // Writes Ur[i*ldu + j] = U[i][j] * sqrt(max(1 - delta/lambda_j, 0)) for j < keep (eigenvalues descending),
 // sigma_out[j] = sqrt(max(lambda_j - delta, 0)) for j < n_sigma, and updates *info.
-// `work` is scratch of at least 256*256 + 64 floats (512*512 + 64 when n > 256), used when the matrix does not fit in
-// shared memory.
+// `work` is scratch of at least eig_work_floats(n) floats. variant 0: the direct solve (eig_tridiag.cu; ldk a multiple of 4),
+// 1: the iterative one (eig.cu; max_sweeps bounds its sweeps).
 // Wsplit != nullptr: also writes the factors transposed and split for launch_tc_rebuild, rows [0, j_pad) =
 // W rounded to 11 significant bits and rows [j_pad, 2 j_pad) = the remainders, W[j][i] = Ur[i][j], pitch ldw >= n,
 // zero outside j < keep, i < n.
 cudaError_t launch_eig_shrink(const float* K, int ldk, int n, int do_shrink, int delta_rank, int keep, float* Ur,
                               int ldu, float* sigma_out, int n_sigma, float* work, int max_sweeps, EigInfo* info,
                               float* Wsplit, int ldw, int j_pad, int variant, cudaStream_t st);
+cudaError_t launch_eig_direct(const float* K, int ldk, int n, int do_shrink, int delta_rank, int keep, float* Ur, int ldu, float* sigma_out,
+                              int n_sigma, float* work, EigInfo* info, float* Wsplit, int ldw, int j_pad, cudaStream_t st);
+size_t eig_work_floats(int n);             // scratch of either variant
+int eig_launches(int n, int variant);      // kernels of one solve
 
 // Z (n x ell, pitch ldz; planes > 1: that many partial planes plane_stride floats apart, summed in plane order with fp64
 // accumulation) -> zhat rows, ||z|| and per-block partial sums of zhat. zsum (ell doubles, may be null) += the partial sums in
