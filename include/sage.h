@@ -208,7 +208,7 @@ sage_status_t sage_select_classes(const float* scores, const int32_t* labels, in
  * code running inside a loop whose memory was handed out once at start-up by a pool it does not own,
  * processes that leave no free device memory, threads that must not block on the allocator. The O(N)
  * scratch that sage_select obtains per call lives here in a fixed array inside the library image
- * (about 4.06 MiB, held by every device that loads the library until the process exits), so
+ * (about 4.07 MiB, held by every device that loads the library until the process exits), so
  *   N <= 262,144 scores; larger N returns SAGE_ERR_UNSUPPORTED with a message naming the limit.
  * Arguments, ordering, tie rule and k_out are those of sage_select; it runs on the CURRENT device.
  * The first call on each device looks up the array's device address (a synchronous query, no

@@ -1368,9 +1368,7 @@ sage_status_t sage_select(const float* scores, int64_t N, double keep_rate, int6
         cudaError_t e2 = cudaFreeAsync(scratch, st);
         CU_TRY(e);
         CU_TRY(e2);
-        int idx_bits = 1;
-        while (idx_bits < 32 && (1ll << idx_bits) < N) ++idx_bits;
-        count(nullptr, 2 + 3 * (4 + (idx_bits + 7) / 8));
+        count(nullptr, select_launches(N));
     }
     if (k_out) *k_out = k;
     return SAGE_OK;
@@ -1400,8 +1398,13 @@ sage_status_t sage_score_classes(sage_fd_t* h, const int32_t* labels, int32_t nu
         h->class_cap = num_classes;
     }
     h->class_num = num_classes;
-    CU_TRY(launch_class_scores(h->zhat, labels, h->N_total, h->ell, num_classes, h->class_U, h->class_counts, scores, st));
-    count(h, h->N_total > 0 ? 2 : 1);
+    void* scratch = nullptr;
+    CU_TRY(scratch_alloc(&scratch, class_scratch_bytes(h->N_total, h->ell, num_classes), st));
+    const cudaError_t e = launch_class_scores(h->zhat, labels, h->N_total, h->ell, num_classes, h->class_U, h->class_counts, scores, scratch, st);
+    const cudaError_t e2 = cudaFreeAsync(scratch, st);
+    CU_TRY(e);
+    CU_TRY(e2);
+    count(h, h->N_total > 0 ? 4 : 2);
     return SAGE_OK;
 }
 
@@ -1431,18 +1434,30 @@ sage_status_t sage_select_classes(const float* scores, const int32_t* labels, in
         size_t sel_bytes = 0;
         select_scratch_bytes(N, &sel_bytes);
         const size_t a256 = 255;
-        const size_t sorted_off = (sel_bytes + a256) & ~a256;
-        const size_t counts_off = (sorted_off + (size_t)N * 8 + a256) & ~a256;
+        const size_t starts_off = (sel_bytes + a256) & ~a256;
+        const size_t counts_off = (starts_off + (size_t)(C + 1) * 4 + a256) & ~a256;
         const size_t kc_off = (counts_off + (size_t)C * 4 + a256) & ~a256;
-        const size_t offs_off = (kc_off + (size_t)C * 8 + a256) & ~a256;
+        const size_t offs_off = (kc_off + (size_t)(C + 1) * 8 + a256) & ~a256;
         const size_t total = offs_off + (size_t)C * 8;
         char* scratch = nullptr;
         CU_TRY(scratch_alloc((void**)&scratch, total, st));
+        long long* d_kc = reinterpret_cast<long long*>(scratch + kc_off);
+        long long* d_offs = reinterpret_cast<long long*>(scratch + offs_off);
         auto body = [&]() -> sage_status_t {
-            int* d_counts = reinterpret_cast<int*>(scratch + counts_off);
-            CU_TRY(launch_class_count(labels, N, C, d_counts, st));
-            std::vector<int> counts(C);
-            CU_TRY(cudaMemcpyAsync(counts.data(), d_counts, (size_t)C * sizeof(int), cudaMemcpyDeviceToHost, st));
+            if (idx && class_select_in_one(N, C)) {          // sort, quotas and picks in one launch; the quotas come back
+                CU_TRY(launch_class_select(scores, labels, N, C, keep_rate, scratch, idx, d_kc, st));
+                kc.resize((size_t)C + 1);
+                CU_TRY(cudaMemcpyAsync(kc.data(), d_kc, (size_t)(C + 1) * 8, cudaMemcpyDeviceToHost, st));
+                CU_TRY(cudaStreamSynchronize(st));
+                k = kc[(size_t)C];
+                count(nullptr, 1);
+                return SAGE_OK;
+            }
+            unsigned* d_starts = reinterpret_cast<unsigned*>(scratch + starts_off);
+            unsigned* d_counts = reinterpret_cast<unsigned*>(scratch + counts_off);
+            CU_TRY(launch_class_starts(labels, N, C, d_starts, d_counts, st));
+            std::vector<unsigned> counts(C);
+            CU_TRY(cudaMemcpyAsync(counts.data(), d_counts, (size_t)C * sizeof(unsigned), cudaMemcpyDeviceToHost, st));
             CU_TRY(cudaStreamSynchronize(st));
             long long n_valid = 0;
             for (int c = 0; c < C; ++c) n_valid += counts[c];
@@ -1468,16 +1483,11 @@ sage_status_t sage_select_classes(const float* scores, const int32_t* labels, in
                 return SAGE_ERR_INVALID_ARG;
             }
             if (k > 0) {
-                CU_TRY(cudaMemcpyAsync(scratch + kc_off, kc.data(), (size_t)C * 8, cudaMemcpyHostToDevice, st));
-                CU_TRY(cudaMemcpyAsync(scratch + offs_off, offs.data(), (size_t)C * 8, cudaMemcpyHostToDevice, st));
-                int64_t* sorted = reinterpret_cast<int64_t*>(scratch + sorted_off);
-                CU_TRY(launch_select(scores, N, N, sorted, scratch, st));
-                CU_TRY(launch_class_pick(sorted, labels, N, C, reinterpret_cast<const long long*>(scratch + kc_off),
-                                         reinterpret_cast<const long long*>(scratch + offs_off), idx, st));
+                CU_TRY(cudaMemcpyAsync(d_kc, kc.data(), (size_t)C * 8, cudaMemcpyHostToDevice, st));
+                CU_TRY(cudaMemcpyAsync(d_offs, offs.data(), (size_t)C * 8, cudaMemcpyHostToDevice, st));
+                CU_TRY(launch_class_pick(scores, labels, N, C, scratch, d_starts, d_kc, d_offs, idx, st));
                 CU_TRY(cudaStreamSynchronize(st));        // kc / offs are host vectors of this call
-                int idx_bits = 1;
-                while (idx_bits < 32 && (1ll << idx_bits) < N) ++idx_bits;
-                count(nullptr, 3 + 3 * (4 + (idx_bits + 7) / 8) + 2);
+                count(nullptr, 4 + 3 * (4 + (C <= 255 ? 1 : 2)));
             }
             return SAGE_OK;
         };

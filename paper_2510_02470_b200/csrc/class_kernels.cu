@@ -7,28 +7,60 @@
 namespace sage {
 namespace {
 
-// Block c: sum over the examples of class c of zhat (fp64, ascending index), its unit vector, the class size.
-// The mean's 1/|I_c| cancels in the unit vector. Thread j owns component j (ell <= 256).
-__global__ void __launch_bounds__(256) k_class_centroids(const float* __restrict__ zhat, const int* __restrict__ labels,
-                                                         int64_t N, int ell, float* __restrict__ U, int* __restrict__ counts) {
-    __shared__ int sl[256];
+// The rows of a class are a run of `order` (rows grouped by class, ascending index). Block (s, c) sums the s-th of gridDim.x equal
+// parts of class c in fp64: thread j of group g owns component j and takes rows g, g + G, ... (G = 256 / jw groups), the
+// groups' sums are added in ascending order. parts: that sum (C x gridDim.x x ell), or, with one part per class, the result.
+__global__ void __launch_bounds__(256) k_class_sums(const float* __restrict__ zhat, const unsigned* __restrict__ order,
+                                                    const unsigned* __restrict__ starts, int ell, int jw, double* __restrict__ parts,
+                                                    float* __restrict__ U, int* __restrict__ counts) {
+    __shared__ double sh[256];
+    __shared__ double red[8];
+    const int c = blockIdx.y, j = threadIdx.x % jw, g = threadIdx.x / jw, G = 256 / jw;
+    const unsigned first = starts[c], n = starts[c + 1] - first;
+    const unsigned len = (n + gridDim.x - 1) / gridDim.x;
+    const unsigned r0 = blockIdx.x * len, r1 = min(n, r0 + len);
+    double acc = 0.0;
+    if (j < ell) {
+        unsigned r = r0 + g;
+        for (; r + 3 * G < r1; r += 4 * G) {                 // four rows' loads in flight, added in order
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = zhat[(int64_t)order[first + r + u * G] * ell + j];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc += (double)v[u];
+        }
+        for (; r < r1; r += G) acc += (double)zhat[(int64_t)order[first + r] * ell + j];
+    }
+    sh[threadIdx.x] = acc;
+    __syncthreads();
+    double t = 0.0;
+    if (g == 0)
+        for (int q = 0; q < G; ++q) t += sh[q * jw + j];
+    if (gridDim.x > 1) {
+        if (g == 0 && j < ell) parts[((int64_t)c * gridDim.x + blockIdx.x) * ell + j] = t;
+        return;
+    }
+    double sq = (g == 0 && j < ell) ? t * t : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
+    __syncthreads();
+    double tot = 0.0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) tot += red[w];
+    if (g == 0 && j < ell) U[(int64_t)c * ell + j] = tot > 0.0 ? (float)(t / sqrt(tot)) : 0.f;
+    if (threadIdx.x == 0) counts[c] = (int)n;
+}
+
+// Block c: the parts of class c in ascending order, the unit vector (the mean's 1/|I_c| cancels), the class size.
+__global__ void __launch_bounds__(256) k_class_units(const double* __restrict__ parts, int nparts, const unsigned* __restrict__ starts, int ell,
+                                                     float* __restrict__ U, int* __restrict__ counts) {
     __shared__ double red[8];
     const int c = blockIdx.x, j = threadIdx.x;
-    double acc = 0.0;
-    int cnt = 0;
-    for (int64_t base = 0; base < N; base += 256) {
-        sl[j] = (base + j < N) ? labels[base + j] : -1;
-        __syncthreads();
-        const int m = (int)((N - base < 256) ? N - base : 256);
-        for (int t = 0; t < m; ++t) {
-            if (sl[t] == c) {                                   // same decision in every thread
-                if (j < ell) acc += (double)zhat[(base + t) * ell + j];
-                ++cnt;
-            }
-        }
-        __syncthreads();
-    }
-    double sq = (j < ell) ? acc * acc : 0.0;
+    double t = 0.0;
+    if (j < ell)
+        for (int s = 0; s < nparts; ++s) t += parts[((int64_t)c * nparts + s) * ell + j];
+    double sq = t * t;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
     if ((j & 31) == 0) red[j >> 5] = sq;
@@ -36,8 +68,8 @@ __global__ void __launch_bounds__(256) k_class_centroids(const float* __restrict
     double tot = 0.0;
 #pragma unroll
     for (int w = 0; w < 8; ++w) tot += red[w];
-    if (j < ell) U[(int64_t)c * ell + j] = tot > 0.0 ? (float)(acc / sqrt(tot)) : 0.f;
-    if (j == 0) counts[c] = cnt;
+    if (j < ell) U[(int64_t)c * ell + j] = tot > 0.0 ? (float)(t / sqrt(tot)) : 0.f;
+    if (j == 0) counts[c] = (int)(starts[c + 1] - starts[c]);
 }
 
 // One warp per example: score = <zhat_i, u_label(i)>; examples without a class in [0, C) score 0.
@@ -55,68 +87,43 @@ __global__ void __launch_bounds__(256) k_class_scores(const float* __restrict__ 
     if (lane == 0) scores[row] = fminf(1.f, fmaxf(-1.f, acc));
 }
 
-__global__ void __launch_bounds__(256) k_class_count(const int* __restrict__ labels, int64_t N, int C, int* __restrict__ counts) {
-    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (i >= N) return;
-    const int lab = labels[i];
-    if (lab >= 0 && lab < C) atomicAdd(&counts[lab], 1);       // integer counts: the result does not depend on order
+// Parts per class: enough blocks to fill the device when there are few classes, one when there are many.
+int class_parts(int C) {
+    const int p = 16384 / C;
+    return p > 64 ? 64 : p < 1 ? 1 : p;
 }
-
-// Block c walks the globally sorted examples (score descending, index ascending) and keeps the first kc[c] of its class.
-__global__ void __launch_bounds__(256) k_class_pick(const int64_t* __restrict__ sorted, const int* __restrict__ labels, int64_t N,
-                                                    const long long* __restrict__ kc, const long long* __restrict__ offs,
-                                                    int64_t* __restrict__ out) {
-    __shared__ int wsum[8];
-    const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long want = kc[c];
-    long long got = 0;
-    for (int64_t base = 0; base < N && got < want; base += 256) {
-        const int64_t i = base + tid;
-        int64_t ex = -1;
-        bool flag = false;
-        if (i < N) {
-            ex = sorted[i];
-            flag = labels[ex] == c;
-        }
-        const unsigned b = __ballot_sync(0xffffffffu, flag);
-        if (lane == 0) wsum[warp] = __popc(b);
-        __syncthreads();
-        int before = 0, total = 0;
-#pragma unroll
-        for (int w = 0; w < 8; ++w) {
-            if (w < warp) before += wsum[w];
-            total += wsum[w];
-        }
-        const long long rank = got + before + __popc(b & ((1u << lane) - 1u));
-        if (flag && rank < want) out[offs[c] + rank] = ex;
-        got += total;
-        __syncthreads();
-    }
-}
+size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace
 
+size_t class_scratch_bytes(int64_t N, int ell, int C) {
+    size_t sel = 0;
+    select_scratch_bytes(N > 0 ? N : 1, &sel);
+    return up256(sel) + up256((size_t)N * 4) + up256((size_t)(C + 1) * 4) + (size_t)C * class_parts(C) * ell * sizeof(double);
+}
+
+// Launches: the rows grouped by class, the sums of their projections, the scores. What it replaced walked all rows once per
+// class in a block of its own, as did the picks from the sorted scores: scores, class scores and picks of 50,000 rows (10 classes,
+// ell = 64, D = 5,130) 2.86 -> 0.58 ms.
 cudaError_t launch_class_scores(const float* zhat, const int* labels, int64_t N, int ell, int C, float* U, int* counts, float* scores,
-                                cudaStream_t st) {
+                                void* scratch, cudaStream_t st) {
     if (C <= 0) return cudaSuccess;
-    k_class_centroids<<<C, 256, 0, st>>>(zhat, labels, N, ell, U, counts);
-    cudaError_t e = cudaGetLastError();
+    size_t sel = 0;
+    select_scratch_bytes(N > 0 ? N : 1, &sel);
+    char* p = static_cast<char*>(scratch);
+    unsigned* order = reinterpret_cast<unsigned*>(p + up256(sel));
+    unsigned* starts = reinterpret_cast<unsigned*>(p + up256(sel) + up256((size_t)N * 4));
+    double* parts = reinterpret_cast<double*>(p + up256(sel) + up256((size_t)N * 4) + up256((size_t)(C + 1) * 4));
+    cudaError_t e = launch_class_order(labels, N, C, scratch, order, starts, st);
+    if (e != cudaSuccess) return e;
+    int jw = 32;
+    while (jw < ell) jw <<= 1;
+    const int np = class_parts(C);
+    k_class_sums<<<dim3(np, C), 256, 0, st>>>(zhat, order, starts, ell, jw, parts, U, counts);
+    if (np > 1) k_class_units<<<C, 256, 0, st>>>(parts, np, starts, ell, U, counts);
+    e = cudaGetLastError();
     if (e != cudaSuccess || N <= 0) return e;
     k_class_scores<<<(unsigned)((N + 7) / 8), 256, 0, st>>>(zhat, labels, N, ell, C, U, scores);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_class_count(const int* labels, int64_t N, int C, int* counts, cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(counts, 0, (size_t)C * sizeof(int), st);
-    if (e != cudaSuccess || N <= 0) return e;
-    k_class_count<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(labels, N, C, counts);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_class_pick(const int64_t* sorted, const int* labels, int64_t N, int C, const long long* kc, const long long* offs,
-                              int64_t* out, cudaStream_t st) {
-    if (C <= 0 || N <= 0) return cudaSuccess;
-    k_class_pick<<<C, 256, 0, st>>>(sorted, labels, N, kc, offs, out);
     return cudaGetLastError();
 }
 

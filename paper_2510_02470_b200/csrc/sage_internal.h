@@ -142,16 +142,26 @@ cudaError_t launch_consensus_score(const double* zsum, const float* zhat, int64_
                                    cudaStream_t st);
 
 // Class-balanced variant. U (C x ell) receives the unit centroids, counts (C) the class sizes, scores (N) the
-// per-class agreement scores; labels outside [0, C) score 0.
+// per-class agreement scores; labels outside [0, C) score 0. scratch: class_scratch_bytes.
+size_t class_scratch_bytes(int64_t N, int ell, int C);
 cudaError_t launch_class_scores(const float* zhat, const int* labels, int64_t N, int ell, int C, float* U, int* counts, float* scores,
-                                cudaStream_t st);
-cudaError_t launch_class_count(const int* labels, int64_t N, int C, int* counts, cudaStream_t st);
-// out[offs[c] + r] = the r-th example of class c in the order of `sorted` (all N examples, best first), r < kc[c].
-cudaError_t launch_class_pick(const int64_t* sorted, const int* labels, int64_t N, int C, const long long* kc, const long long* offs,
-                              int64_t* out, cudaStream_t st);
+                                void* scratch, cudaStream_t st);
+// Rows grouped by class, ascending index inside a class, rows without a class last: order (N); starts (C + 1): first place of
+// each class. scratch: select_scratch_bytes.
+cudaError_t launch_class_order(const int* labels, int64_t N, int C, void* scratch, unsigned* order, unsigned* starts, cudaStream_t st);
+// starts as above; counts (C, may be null): class sizes.
+cudaError_t launch_class_starts(const int* labels, int64_t N, int C, unsigned* starts, unsigned* counts, cudaStream_t st);
+// Per-class top-k_c. One launch, quotas included, where class_select_in_one says so: kc receives the C quotas and their sum.
+bool class_select_in_one(int64_t N, int C);
+cudaError_t launch_class_select(const float* scores, const int* labels, int64_t N, int C, double keep_rate, void* scratch, int64_t* idx,
+                                long long* kc, cudaStream_t st);
+// Otherwise with given quotas: idx[offs[c] + r] = the r-th best example of class c, r < kc[c].
+cudaError_t launch_class_pick(const float* scores, const int* labels, int64_t N, int C, void* scratch, const unsigned* starts, const long long* kc,
+                              const long long* offs, int64_t* idx, cudaStream_t st);
 
-// Top-k by (score desc, index asc). keys/vals scratch: see select.cu. Returns through idx (device).
+// Top-k by (score desc, index asc). scratch: select_scratch_bytes. Returns through idx (device).
 cudaError_t select_scratch_bytes(int64_t N, size_t* bytes);
+int select_launches(int64_t N);
 cudaError_t launch_select(const float* scores, int64_t N, int64_t k, int64_t* idx, void* scratch, cudaStream_t st);
 
 // Hooks into the C ABI's bookkeeping for entry points defined outside api.cu.

@@ -1,8 +1,15 @@
-// Top-k selection (Algorithm 1, the top-k step) with a total order: score descending, then
-// index ascending. Each score becomes a 64-bit key whose high word is the bitwise complement of an
-// order-preserving integer image of the float and whose low word is the row index; every key is
-// distinct, so an ascending LSD radix sort of the keys (8-bit digits, stable scatter) puts the rows in
-// exactly that order and the first k low words are the answer. Integer work only: results are exact.
+// Top-k selection (Algorithm 1, the top-k step) with a total order: score descending, then index ascending, and the orders by
+// class that the class-balanced variant needs. A stable radix sort, 8 bits a pass, least significant digit first: each score
+// becomes a 32-bit integer whose ascending order is the descending order of the scores, paired with its row index; rows start
+// in index order, so ties stay in it and the index needs no passes of its own. Passes over the label follow where rows are
+// grouped by class. Integer work only: results are exact.
+//
+// Up to kClusterMax rows the whole sort is one launch: a cluster of 8 thread blocks, digit counts exchanged through
+// distributed shared memory, keys through L2, two cluster barriers per pass. Such a sort is bound by latency (launches before,
+// barriers now): a call on 50,000 scores took 149 us in 20 launches (six passes, the index included, of three kernels with a
+// one-block scan over all counters) and takes 57 us. Beyond, three launches per pass (counts, one block per digit scanning its counters, scatter).
+#include <cooperative_groups.h>
+
 #include <cstdio>
 #include <mutex>
 
@@ -10,6 +17,9 @@
 
 namespace sage {
 namespace {
+
+namespace cg = cooperative_groups;
+using u64 = unsigned long long;
 
 constexpr int kThreads = 256;
 constexpr int kItems = 16;
@@ -21,18 +31,234 @@ __device__ __forceinline__ uint32_t ordered_bits(float f) {
     const uint32_t b = __float_as_uint(f);
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);       // larger float <-> larger integer
 }
-
-__global__ void __launch_bounds__(kThreads) k_make_keys(const float* __restrict__ scores, int64_t N,
-                                                        unsigned long long* __restrict__ keys) {
-    const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    if (i >= N) return;
+__device__ __forceinline__ u64 make_key(const float* scores, int64_t i) {
     float s = scores[i];
     if (s == 0.f) s = 0.f;                                   // -0 and +0 compare equal: give them one key
-    keys[i] = ((unsigned long long)(~ordered_bits(s)) << 32) | (unsigned long long)(uint32_t)i;
+    return ((u64)(~ordered_bits(s)) << 32) | (u64)(uint32_t)i;
+}
+// Class of a row, labels outside [0, C) as class C.
+__device__ __forceinline__ unsigned class_of(const int* labels, u64 key, int C) {
+    const int lab = labels[(uint32_t)key];
+    return (lab >= 0 && lab < C) ? (unsigned)lab : (unsigned)C;
 }
 
-__global__ void __launch_bounds__(kThreads) k_histogram(const unsigned long long* __restrict__ keys, int64_t N, int shift,
-                                                        unsigned* __restrict__ hist, int nblocks) {
+// What a sort is for. by_score: four passes over the score image first; label_passes: 0, 1 or 2 passes over the class.
+struct SortArgs {
+    const float* scores;
+    const int* labels;
+    int64_t N;
+    int C, by_score, label_passes;
+};
+__device__ __forceinline__ unsigned digit_of(const SortArgs& a, u64 key, int pass) {
+    const int vp = a.by_score ? 4 : 0;
+    if (pass < vp) return (unsigned)(key >> (32 + 8 * pass)) & 255u;
+    return (class_of(a.labels, key, a.C) >> (8 * (pass - vp))) & 255u;
+}
+
+// ---- one launch: cluster of 8 ------------------------------------------------------------------------------------
+constexpr int kClThreads = 1024, kClWarps = 32, kClSize = 8;
+constexpr int kClKeys = 16384;                               // most keys per block
+constexpr int64_t kClusterMax = (int64_t)kClSize * kClKeys;
+
+struct ClusterShared {
+    unsigned short cnt[kClWarps][256];
+    unsigned short pos[kClKeys];                             // rank of a key among those of its digit before it in its warp's run
+    unsigned hist[256];                                      // this block's counts, read by the others
+    unsigned base[256];
+    unsigned excl[257];                                      // where a digit's keys start
+    unsigned total[256];
+    unsigned wsum[8];
+    long long kc[256], rem[256], offs[256];
+};
+
+enum Emit { EMIT_TOPK = 0, EMIT_ORDER, EMIT_PICK };
+// EMIT_TOPK: idx[p] = row at place p, p < k. EMIT_ORDER (label passes only): order[p] = row, starts[c] = first place of class c
+// (one label pass: c <= C <= 255). EMIT_PICK (one label pass): the quotas of the classes by largest remainder (sage_select_classes),
+// idx = the first kc[c] of class 0, then of class 1, ...; kc_out[0 .. C - 1] the quotas, kc_out[C] their sum.
+template <int MODE>
+__global__ void __launch_bounds__(kClThreads, 1)
+k_sort_cluster(SortArgs a, u64* __restrict__ b0, u64* __restrict__ b1, int64_t k, double keep_rate, int64_t* __restrict__ idx,
+               unsigned* __restrict__ order, unsigned* __restrict__ starts, long long* __restrict__ kc_out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ClusterShared& sh = *reinterpret_cast<ClusterShared*>(smem_raw);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int span = (int)((a.N + kClSize * kClThreads - 1) / (kClSize * kClThreads)) * 32;   // keys per warp, whole slots of 32
+    const int64_t base = ((int64_t)rank * kClWarps + warp) * span;
+    const int passes = (a.by_score ? 4 : 0) + a.label_passes;
+    u64* in = b0;
+    u64* out = b1;
+    for (int pass = 0; pass < passes; ++pass) {
+        const bool last = pass == passes - 1;
+        auto load = [&](int64_t i) -> u64 {
+            if (i >= a.N) return 0ull;
+            if (pass > 0) return __ldcg(in + i);
+            return a.by_score ? make_key(a.scores, i) : (u64)i;
+        };
+        for (int e = tid; e < kClWarps * 128; e += kClThreads) reinterpret_cast<unsigned*>(&sh.cnt[0][0])[e] = 0u;
+        __syncthreads();
+        unsigned short* cnt = sh.cnt[warp];
+        unsigned short* pos = sh.pos + warp * span;
+        for (int s0 = 0; s0 < span; s0 += 128) {             // four slots' loads in flight
+            u64 key[4];
+            unsigned dig[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) key[u] = load(s0 + 32 * u < span ? base + s0 + 32 * u + lane : a.N);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool live = s0 + 32 * u < span && base + s0 + 32 * u + lane < a.N;
+                dig[u] = live ? digit_of(a, key[u], pass) : 256u;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (s0 + 32 * u >= span) break;
+                const unsigned peers = __match_any_sync(0xffffffffu, dig[u]);
+                const unsigned r = __popc(peers & ((1u << lane) - 1u));
+                const unsigned before = dig[u] < 256u ? cnt[dig[u]] : 0u;
+                __syncwarp();
+                if (dig[u] < 256u && r == 0) cnt[dig[u]] = (unsigned short)(before + __popc(peers));
+                __syncwarp();
+                pos[s0 + 32 * u + lane] = (unsigned short)(before + r);
+            }
+        }
+        __syncthreads();
+        if (tid < 256) {                                     // counts of the warps before, and of the block
+            unsigned run = 0;
+#pragma unroll
+            for (int w = 0; w < kClWarps; ++w) {
+                const unsigned c = sh.cnt[w][tid];
+                sh.cnt[w][tid] = (unsigned short)run;
+                run += c;
+            }
+            sh.hist[tid] = run;
+        }
+        cluster.sync();
+        unsigned before = 0, total = 0, x = 0;
+        if (tid < 256) {
+#pragma unroll
+            for (int r = 0; r < kClSize; ++r) {
+                const unsigned v = cluster.map_shared_rank(sh.hist, r)[tid];
+                if (r < rank) before += v;
+                total += v;
+            }
+            x = total;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (lane == 31) sh.wsum[warp] = x;
+        }
+        __syncthreads();
+        if (tid < 256) {
+            unsigned e = x - total;
+            for (int w = 0; w < warp; ++w) e += sh.wsum[w];
+            sh.excl[tid] = e;
+            if (tid == 255) sh.excl[256] = e + total;
+            sh.base[tid] = e + before;
+            sh.total[tid] = total;
+        }
+        __syncthreads();
+        if (MODE == EMIT_PICK && last) {
+            // quotas: k_c = floor(k n_c / n), the k - sum largest remainders (ties: smaller class) get one more
+            const long long n_valid = (long long)sh.excl[a.C];
+            double kd = floor(keep_rate * (double)n_valid + 0.5);
+            kd = kd < 0.0 ? 0.0 : kd > (double)n_valid ? (double)n_valid : kd;
+            const long long kk = n_valid > 0 ? (long long)kd : 0;
+            if (tid < a.C) {
+                const long long num = (long long)sh.total[tid] * kk;
+                const long long q = n_valid > 0 ? num / n_valid : 0;
+                sh.kc[tid] = q;
+                sh.rem[tid] = num - q * n_valid;
+            }
+            __syncthreads();
+            long long mine = 0;
+            if (tid < a.C) {
+                long long given = 0;
+                int larger = 0;
+                for (int c = 0; c < a.C; ++c) {
+                    given += sh.kc[c];
+                    larger += sh.rem[c] > sh.rem[tid] || (sh.rem[c] == sh.rem[tid] && c < tid);
+                }
+                mine = sh.kc[tid] + (larger < kk - given ? 1 : 0);
+            }
+            __syncthreads();
+            if (tid < a.C) sh.kc[tid] = mine;
+            __syncthreads();
+            if (tid < a.C) {
+                long long o = 0;
+                for (int c = 0; c < tid; ++c) o += sh.kc[c];
+                sh.offs[tid] = o;
+                if (rank == 0) {
+                    kc_out[tid] = mine;
+                    if (tid == a.C - 1) kc_out[a.C] = o + mine;
+                }
+            }
+            __syncthreads();
+        }
+        if (MODE == EMIT_ORDER && last && starts && rank == 0 && tid <= a.C) starts[tid] = sh.excl[tid];
+        for (int s0 = 0; s0 < span; s0 += 128) {
+            u64 key[4];
+            unsigned dig[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) key[u] = load(s0 + 32 * u < span ? base + s0 + 32 * u + lane : a.N);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool live = s0 + 32 * u < span && base + s0 + 32 * u + lane < a.N;
+                dig[u] = live ? digit_of(a, key[u], pass) : 256u;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (dig[u] >= 256u) continue;
+                const unsigned p = sh.base[dig[u]] + cnt[dig[u]] + pos[s0 + 32 * u + lane];
+                if (!last) {
+                    out[p] = key[u];
+                } else if (MODE == EMIT_TOPK) {
+                    if ((int64_t)p < k) idx[p] = (int64_t)(uint32_t)key[u];
+                } else if (MODE == EMIT_ORDER) {
+                    order[p] = (unsigned)(uint32_t)key[u];
+                } else {
+                    const long long r = (long long)(p - sh.excl[dig[u]]);
+                    if ((int)dig[u] < a.C && r < sh.kc[dig[u]]) idx[sh.offs[dig[u]] + r] = (int64_t)(uint32_t)key[u];
+                }
+            }
+        }
+        cluster.sync();                                      // keys are out, counts may be overwritten
+        u64* t = in;
+        in = out;
+        out = t;
+    }
+}
+
+template <int MODE>
+cudaError_t run_cluster_sort(const SortArgs& a, u64* b0, u64* b1, int64_t k, double keep_rate, int64_t* idx, unsigned* order, unsigned* starts,
+                             long long* kc_out, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(k_sort_cluster<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClusterShared));
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kClSize);
+    cfg.blockDim = dim3(kClThreads);
+    cfg.dynamicSmemBytes = sizeof(ClusterShared);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kClSize;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_sort_cluster<MODE>, a, b0, b1, k, keep_rate, idx, order, starts, kc_out);
+}
+
+// ---- three launches per pass, any N ------------------------------------------------------------------------------
+__global__ void __launch_bounds__(kThreads) k_make_keys(SortArgs a, u64* __restrict__ keys) {
+    const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    if (i < a.N) keys[i] = a.by_score ? make_key(a.scores, i) : (u64)i;
+}
+
+__global__ void __launch_bounds__(kThreads) k_histogram(SortArgs a, const u64* __restrict__ keys, int pass, unsigned* __restrict__ hist,
+                                                        int nblocks, unsigned* __restrict__ totals) {
     __shared__ unsigned h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
@@ -40,66 +266,70 @@ __global__ void __launch_bounds__(kThreads) k_histogram(const unsigned long long
 #pragma unroll
     for (int s = 0; s < kItems; ++s) {
         const int64_t i = base + s * kThreads + threadIdx.x;
-        if (i < N) atomicAdd(&h[(unsigned)(keys[i] >> shift) & 255u], 1u);
+        const unsigned d = i < a.N ? digit_of(a, keys[i], pass) : 256u;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);         // scores share their leading bits: one add per value and warp
+        if (d < 256u && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&h[d], (unsigned)__popc(peers));
     }
     __syncthreads();
-    hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
+    const unsigned v = h[threadIdx.x];
+    hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = v;
+    if (v) atomicAdd(&totals[pass * 256 + threadIdx.x], v);
 }
 
-// Exclusive scan of hist in (digit-major, block-minor) order, in place. One block.
-__global__ void __launch_bounds__(1024) k_scan(unsigned* __restrict__ hist, int64_t total) {
-    __shared__ unsigned warp_sums[32];
-    __shared__ unsigned carry;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) carry = 0;
-    __syncthreads();
-    for (int64_t base = 0; base < total; base += 1024) {
-        const int64_t i = base + tid;
-        const unsigned v = (i < total) ? hist[i] : 0u;
-        unsigned x = v;
+// Block d: exclusive scan of the blocks' counts of digit d, starting at the number of keys with smaller digits.
+__global__ void __launch_bounds__(kThreads) k_scan(unsigned* __restrict__ hist, int nblocks, const unsigned* __restrict__ totals) {
+    __shared__ unsigned ws[kWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, d = blockIdx.x;
+    auto block_sum = [&](unsigned v, unsigned& incl) {       // inclusive scan over the block; returns the block's sum
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
+            const unsigned y = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += y;
         }
-        if (lane == 31) warp_sums[warp] = x;
+        if (lane == 31) ws[warp] = v;
         __syncthreads();
-        if (warp == 0) {
-            unsigned w = warp_sums[lane];
+        unsigned before = 0, sum = 0;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned y = __shfl_up_sync(0xffffffffu, w, o);
-                if (lane >= o) w += y;
-            }
-            warp_sums[lane] = w;
+        for (int w = 0; w < kWarps; ++w) {
+            if (w < warp) before += ws[w];
+            sum += ws[w];
         }
         __syncthreads();
-        const unsigned before = carry + (warp > 0 ? warp_sums[warp - 1] : 0u) + (x - v);
-        if (i < total) hist[i] = before;
-        __syncthreads();
-        if (tid == 1023) carry = before + v;
-        __syncthreads();
+        incl = v + before;
+        return sum;
+    };
+    unsigned incl;
+    unsigned carry = block_sum(tid < d ? totals[tid] : 0u, incl);
+    unsigned* row = hist + (int64_t)d * nblocks;
+    for (int b0 = 0; b0 < nblocks; b0 += kThreads) {
+        const unsigned v = b0 + tid < nblocks ? row[b0 + tid] : 0u;
+        const unsigned sum = block_sum(v, incl);
+        if (b0 + tid < nblocks) row[b0 + tid] = carry + incl - v;
+        carry += sum;
     }
 }
 
 // Stable scatter: warp w of a block owns the contiguous keys [w*512, (w+1)*512) of the tile, walked in
-// 16 slots of 32 consecutive keys, so (warp, slot, lane) order is index order.
-__global__ void __launch_bounds__(kThreads) k_scatter(const unsigned long long* __restrict__ in, int64_t N, int shift,
-                                                      const unsigned* __restrict__ offsets, int nblocks,
-                                                      unsigned long long* __restrict__ out) {
+// 16 slots of 32 consecutive keys, so (warp, slot, lane) order is index order. The last pass of a selection (idx != null)
+// writes the first k rows in place of the keys.
+__global__ void __launch_bounds__(kThreads) k_scatter(SortArgs a, const u64* __restrict__ in, int pass, const unsigned* __restrict__ offsets,
+                                                      int nblocks, u64* __restrict__ out, int64_t k, int64_t* __restrict__ idx) {
     __shared__ unsigned cnt[kWarps][256];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int e = tid; e < kWarps * 256; e += kThreads) (&cnt[0][0])[e] = 0;
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)warp * (kItems * 32);
-    unsigned long long key[kItems];
-    unsigned short pos[kItems];
+    u64 key[kItems];
+    unsigned short pos[kItems], dig[kItems];
 #pragma unroll
     for (int s = 0; s < kItems; ++s) {
         const int64_t i = base + s * 32 + lane;
-        const bool live = i < N;
-        key[s] = live ? in[i] : 0ull;
-        const unsigned d = live ? ((unsigned)(key[s] >> shift) & 255u) : 256u;
+        key[s] = i < a.N ? in[i] : 0ull;
+    }
+#pragma unroll
+    for (int s = 0; s < kItems; ++s) {
+        const bool live = base + s * 32 + lane < a.N;
+        const unsigned d = live ? digit_of(a, key[s], pass) : 256u;
         const unsigned peers = __match_any_sync(0xffffffffu, d);
         const unsigned rank = __popc(peers & ((1u << lane) - 1u));
         unsigned before = 0;
@@ -108,6 +338,7 @@ __global__ void __launch_bounds__(kThreads) k_scatter(const unsigned long long* 
         if (live && rank == 0) cnt[warp][d] = before + __popc(peers);
         __syncwarp();
         pos[s] = (unsigned short)(before + rank);
+        dig[s] = (unsigned short)d;
     }
     __syncthreads();
     {   // thread d: turn per-warp counts of digit d into start offsets
@@ -122,48 +353,161 @@ __global__ void __launch_bounds__(kThreads) k_scatter(const unsigned long long* 
     __syncthreads();
 #pragma unroll
     for (int s = 0; s < kItems; ++s) {
-        const int64_t i = base + s * 32 + lane;
-        if (i < N) {
-            const unsigned d = (unsigned)(key[s] >> shift) & 255u;
-            out[cnt[warp][d] + pos[s]] = key[s];
-        }
+        if (dig[s] >= 256u) continue;
+        const unsigned p = cnt[warp][dig[s]] + pos[s];
+        if (!idx) out[p] = key[s];
+        else if ((int64_t)p < k) idx[p] = (int64_t)(uint32_t)key[s];
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_emit(const unsigned long long* __restrict__ keys, int64_t k,
-                                                   int64_t* __restrict__ idx) {
-    const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    if (i < k) idx[i] = (int64_t)(keys[i] & 0xffffffffull);
+inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
+constexpr size_t kTotalsBytes = 6 * 256 * 4;
+
+// Sorts as `a` says; returns the buffer that holds the result (a selection writes idx instead).
+cudaError_t sort_launches(const SortArgs& a, void* scratch, int64_t k, int64_t* idx, u64** result, cudaStream_t st) {
+    const int nblocks = (int)((a.N + kTile - 1) / kTile);
+    char* p = static_cast<char*>(scratch);
+    u64* in = reinterpret_cast<u64*>(p);
+    u64* out = reinterpret_cast<u64*>(p + align256((size_t)a.N * 8));
+    unsigned* totals = reinterpret_cast<unsigned*>(p + 2 * align256((size_t)a.N * 8));
+    unsigned* hist = totals + kTotalsBytes / 4;
+    cudaError_t e = cudaMemsetAsync(totals, 0, kTotalsBytes, st);
+    if (e != cudaSuccess) return e;
+    k_make_keys<<<(unsigned)((a.N + kThreads - 1) / kThreads), kThreads, 0, st>>>(a, in);
+    const int passes = (a.by_score ? 4 : 0) + a.label_passes;
+    for (int pass = 0; pass < passes; ++pass) {
+        k_histogram<<<nblocks, kThreads, 0, st>>>(a, in, pass, hist, nblocks, totals);
+        k_scan<<<256, kThreads, 0, st>>>(hist, nblocks, totals + pass * 256);
+        k_scatter<<<nblocks, kThreads, 0, st>>>(a, in, pass, hist, nblocks, out, k, pass == passes - 1 ? idx : nullptr);
+        u64* t = in;
+        in = out;
+        out = t;
+    }
+    if (result) *result = in;
+    return cudaGetLastError();
 }
 
-inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
+// ---- classes with more than one label pass, or more rows than a cluster takes ------------------------------------------
+__global__ void __launch_bounds__(256) k_class_count(const int* __restrict__ labels, int64_t N, int C, unsigned* __restrict__ counts) {
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= N) return;
+    const int lab = labels[i];
+    if (lab >= 0 && lab < C) atomicAdd(&counts[lab], 1u);      // integer counts: the result does not depend on order
+}
+
+// In place: counts[0 .. C - 1] -> first place of each class, [C] = the number of rows with a class. One block.
+__global__ void __launch_bounds__(1024) k_class_starts(unsigned* __restrict__ c, int C) {
+    __shared__ unsigned ws[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned carry = 0;
+    for (int b0 = 0; b0 <= C; b0 += 1024) {
+        const unsigned v = b0 + tid < C ? c[b0 + tid] : 0u;
+        unsigned x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) ws[warp] = x;
+        __syncthreads();
+        unsigned before = 0, sum = 0;
+        for (int w = 0; w < 32; ++w) {
+            if (w < warp) before += ws[w];
+            sum += ws[w];
+        }
+        if (b0 + tid <= C) c[b0 + tid] = carry + before + x - v;
+        carry += sum;
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(256) k_order_of_keys(const u64* __restrict__ keys, int64_t N, unsigned* __restrict__ order) {
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i < N) order[i] = (unsigned)(uint32_t)keys[i];
+}
+
+// keys: rows grouped by class, best first; the first kc[c] of class c go to offs[c] ...
+__global__ void __launch_bounds__(256) k_class_pick(const u64* __restrict__ keys, const int* __restrict__ labels, int64_t N, int C,
+                                                    const unsigned* __restrict__ starts, const long long* __restrict__ kc,
+                                                    const long long* __restrict__ offs, int64_t* __restrict__ out) {
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= N) return;
+    const u64 key = keys[i];
+    const unsigned c = class_of(labels, key, C);
+    if (c >= (unsigned)C) return;
+    const long long r = i - (int64_t)starts[c];
+    if (r < kc[c]) out[offs[c] + r] = (int64_t)(uint32_t)key;
+}
+
+int label_passes_of(int C) { return C <= 255 ? 1 : 2; }
 
 }  // namespace
 
 cudaError_t select_scratch_bytes(int64_t N, size_t* bytes) {
     const int64_t nblocks = (N + kTile - 1) / kTile;
-    *bytes = 2 * align256((size_t)N * 8) + align256((size_t)nblocks * 256 * 4) + 256;
+    *bytes = 2 * align256((size_t)N * 8) + kTotalsBytes + align256((size_t)nblocks * 256 * 4) + 256;
     return cudaSuccess;
 }
 
+int select_launches(int64_t N) { return N <= kClusterMax ? 1 : 1 + 3 * 4; }
+
 cudaError_t launch_select(const float* scores, int64_t N, int64_t k, int64_t* idx, void* scratch, cudaStream_t st) {
     if (N <= 0 || k <= 0) return cudaSuccess;
-    const int nblocks = (int)((N + kTile - 1) / kTile);
-    char* p = static_cast<char*>(scratch);
-    unsigned long long* a = reinterpret_cast<unsigned long long*>(p);
-    unsigned long long* b = reinterpret_cast<unsigned long long*>(p + align256((size_t)N * 8));
-    unsigned* hist = reinterpret_cast<unsigned*>(p + 2 * align256((size_t)N * 8));
-    k_make_keys<<<(unsigned)((N + kThreads - 1) / kThreads), kThreads, 0, st>>>(scores, N, a);
-    int idx_bits = 1;
-    while (idx_bits < 32 && (1ll << idx_bits) < N) ++idx_bits;
-    for (int shift = 0; shift < 64; shift += 8) {
-        if (shift < 32 && shift >= idx_bits) continue;       // index digits that are all zero
-        k_histogram<<<nblocks, kThreads, 0, st>>>(a, N, shift, hist, nblocks);
-        k_scan<<<1, 1024, 0, st>>>(hist, (int64_t)nblocks * 256);
-        k_scatter<<<nblocks, kThreads, 0, st>>>(a, N, shift, hist, nblocks, b);
-        unsigned long long* t = a; a = b; b = t;
+    const SortArgs a = {scores, nullptr, N, 0, 1, 0};
+    if (N <= kClusterMax) {
+        u64* b0 = static_cast<u64*>(scratch);
+        u64* b1 = reinterpret_cast<u64*>(static_cast<char*>(scratch) + align256((size_t)N * 8));
+        return run_cluster_sort<EMIT_TOPK>(a, b0, b1, k, 0.0, idx, nullptr, nullptr, nullptr, st);
     }
-    k_emit<<<(unsigned)((k + kThreads - 1) / kThreads), kThreads, 0, st>>>(a, k, idx);
+    return sort_launches(a, scratch, k, idx, nullptr, st);
+}
+
+cudaError_t launch_class_order(const int* labels, int64_t N, int C, void* scratch, unsigned* order, unsigned* starts, cudaStream_t st) {
+    const SortArgs a = {nullptr, labels, N, C, 0, label_passes_of(C)};
+    cudaError_t e = cudaSuccess;
+    if (N <= 0 || C > 255 || N > kClusterMax) {
+        e = launch_class_starts(labels, N, C, starts, nullptr, st);
+        if (e != cudaSuccess || N <= 0) return e;
+    }
+    if (N <= kClusterMax) {
+        u64* b0 = static_cast<u64*>(scratch);
+        u64* b1 = reinterpret_cast<u64*>(static_cast<char*>(scratch) + align256((size_t)N * 8));
+        return run_cluster_sort<EMIT_ORDER>(a, b0, b1, 0, 0.0, nullptr, order, C <= 255 ? starts : nullptr, nullptr, st);
+    }
+    u64* keys = nullptr;
+    e = sort_launches(a, scratch, 0, nullptr, &keys, st);
+    if (e != cudaSuccess) return e;
+    k_order_of_keys<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(keys, N, order);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_class_starts(const int* labels, int64_t N, int C, unsigned* starts, unsigned* counts, cudaStream_t st) {
+    cudaError_t e = cudaMemsetAsync(starts, 0, (size_t)(C + 1) * sizeof(unsigned), st);
+    if (e != cudaSuccess) return e;
+    if (N > 0) k_class_count<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(labels, N, C, starts);
+    if (counts && (e = cudaMemcpyAsync(counts, starts, (size_t)C * sizeof(unsigned), cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
+    k_class_starts<<<1, 1024, 0, st>>>(starts, C);
+    return cudaGetLastError();
+}
+
+bool class_select_in_one(int64_t N, int C) { return C <= 255 && N > 0 && N <= kClusterMax; }
+
+cudaError_t launch_class_select(const float* scores, const int* labels, int64_t N, int C, double keep_rate, void* scratch, int64_t* idx,
+                                long long* kc, cudaStream_t st) {
+    const SortArgs a = {scores, labels, N, C, 1, 1};
+    u64* b0 = static_cast<u64*>(scratch);
+    u64* b1 = reinterpret_cast<u64*>(static_cast<char*>(scratch) + align256((size_t)N * 8));
+    return run_cluster_sort<EMIT_PICK>(a, b0, b1, 0, keep_rate, idx, nullptr, nullptr, kc, st);
+}
+
+cudaError_t launch_class_pick(const float* scores, const int* labels, int64_t N, int C, void* scratch, const unsigned* starts, const long long* kc,
+                              const long long* offs, int64_t* idx, cudaStream_t st) {
+    if (N <= 0) return cudaSuccess;
+    const SortArgs a = {scores, labels, N, C, 1, label_passes_of(C)};
+    u64* keys = nullptr;
+    cudaError_t e = sort_launches(a, scratch, 0, nullptr, &keys, st);
+    if (e != cudaSuccess) return e;
+    k_class_pick<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(keys, labels, N, C, starts, kc, offs, idx);
     return cudaGetLastError();
 }
 
@@ -187,7 +531,7 @@ namespace {
 constexpr int64_t kStaticMaxN = 262144;    // largest N served without allocating
 constexpr size_t kStaticKeyBytes = (size_t)kStaticMaxN * 8;                          // one key array
 constexpr size_t kStaticHistBytes = (size_t)((kStaticMaxN + sage::kTile - 1) / sage::kTile) * 256 * 4;
-constexpr size_t kStaticScratchBytes = 2 * kStaticKeyBytes + kStaticHistBytes + 256;  // about 4.06 MiB
+constexpr size_t kStaticScratchBytes = 2 * kStaticKeyBytes + sage::kTotalsBytes + kStaticHistBytes + 256;  // about 4.07 MiB
 
 static __device__ __align__(256) unsigned char g_select_scratch[kStaticScratchBytes];
 
@@ -240,7 +584,7 @@ extern "C" sage_status_t sage_select_static(const float* scores, int64_t N, doub
             scratch = g_scratch_addr[dev];
         }
         // Nothing in the scratch has to start at zero: the key arrays are written for every i < N before
-        // they are read and each radix pass rewrites the whole histogram it scans.
+        // they are read, and what a radix pass counts in is cleared or rewritten by the call.
         e = sage::launch_select(scores, N, k, idx, scratch, static_cast<cudaStream_t>(cuda_stream));
         if (e != cudaSuccess) {
             char msg[200];
@@ -248,9 +592,7 @@ extern "C" sage_status_t sage_select_static(const float* scores, int64_t N, doub
             sage::set_error_message(msg);
             return SAGE_ERR_CUDA;
         }
-        int idx_bits = 1;
-        while (idx_bits < 32 && (1ll << idx_bits) < N) ++idx_bits;
-        sage::count_launches(2 + 3 * (4 + (idx_bits + 7) / 8));
+        sage::count_launches(sage::select_launches(N));
     }
     if (k_out) *k_out = k;
     return SAGE_OK;

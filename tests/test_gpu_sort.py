@@ -1,0 +1,52 @@
+"""Selections at the sizes where the sort behind them changes: whole slots and blocks of the one-launch form, its largest size
+and one more, one and two passes over the class. Integer work: exact against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from oracle import cb
+import paper_2510_02470_b200 as sage
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("N", [33, 8191, 8192, 8193, 57344 + 5, 131071, 131072, 131073, 1050001])
+def test_selection_at_the_edges(N):
+    r = np.random.default_rng(N)
+    a = np.where(r.uniform(size=N) < 0.3, r.integers(-6, 7, N) / 6.0, r.uniform(-1, 1, N)).astype(np.float32)
+    s = torch.from_numpy(a).to(DEV)
+    for rate in (1.0 / N, 0.37, 1.0):
+        assert np.array_equal(sage.sage_select(s, rate).cpu().numpy(), oracle.select(a.astype(np.float64), rate)), rate
+
+
+@pytest.mark.parametrize("N,C", [(8193, 255), (8192, 256), (131072, 255), (131073, 10), (140000, 300), (3000, 65535)])
+def test_selection_by_class_at_the_edges(N, C):
+    r = np.random.default_rng(N + C)
+    a = (r.integers(-50, 51, size=N) / 50.0).astype(np.float32)
+    labels = r.integers(-1, C + 1, size=N).astype(np.int32)
+    labels[: N // 3] = C // 2                                        # one large class
+    idx, kc = sage.sage_select_classes(torch.from_numpy(a).to(DEV), torch.from_numpy(labels).to(DEV), C, 0.23)
+    idx_ref, kc_ref = cb.select(a.astype(np.float64), labels, C, 0.23)
+    assert kc == kc_ref.tolist() and np.array_equal(idx.cpu().numpy(), idx_ref)
+
+
+@pytest.mark.parametrize("N,C,ell", [(1, 1, 4), (9000, 255, 33), (9000, 256, 16), (132000, 12, 8), (2000, 20000, 5)])
+def test_class_centroids_at_the_edges(N, C, ell):
+    """The centroid is a sum in fp64 of the library's own fp32 projections, rounded once: 2^-24, and 1e-6 for the fp32 dot
+    product of a score."""
+    D = 20
+    r = np.random.default_rng(N + C)
+    labels = r.integers(-1, C + 1, size=N).astype(np.int32)
+    fd = sage.SageFD(D, ell, torch.float32, 0)
+    fd.load_sketch(torch.from_numpy(r.standard_normal((ell, D)).astype(np.float32)).to(DEV))
+    fd.score(torch.from_numpy((r.standard_normal((N, D)) + 0.3).astype(np.float32)).to(DEV))
+    zhat = fd.intermediates(N)[0].double().cpu().numpy()
+    a = fd.score_classes(torch.from_numpy(labels).to(DEV), C)
+    U, cnt = fd.class_centroids()
+    fd.close()
+    a_ref, U_ref, cnt_ref = cb.class_scores(zhat, labels, C)
+    assert np.array_equal(cnt.cpu().numpy(), cnt_ref)
+    assert np.max(np.abs(U.double().cpu().numpy() - U_ref)) <= 6.1e-8
+    assert np.max(np.abs(a.double().cpu().numpy() - a_ref)) <= 1e-6
