@@ -19,8 +19,8 @@
 //
 // Why: the solve is a chain of dependent steps, and this one is shorter than the iterative solve's (sweeps x (n - 1) rounds):
 // n - 2 steps of about 1,050 cycles for the reduction, then 30 to 75 thousand cycles, all eigenvectors side by side. Measured, one
-// solve in a row of solves, iterative -> direct: 64 rows 156 -> 44 us, 128 rows 389 -> 90 us (random matrices; 254 -> 95 us
-// in a run on last-layer rows), 256 rows 1,422 -> 228 us, 512 rows 7,093 -> 734 us. Error of the shrunk sketch, relative to the
+// solve in a row of solves, iterative -> direct: 64 rows 156 -> 44 us, 128 rows 389 -> 89 us (random matrices; 254 -> 95 us
+// in a run on last-layer rows), 256 rows 1,422 -> 213 us, 512 rows 7,093 -> 705 us. Error of the shrunk sketch, relative to the
 // largest eigenvalue: 3 to 5e-7 at every size (iterative: 1e-6 at 64 rows to 6e-6 at 512).
 #include "sage_internal.h"
 
@@ -60,8 +60,10 @@ __device__ __forceinline__ void send_pair(uint32_t addr, float x, float y, uint3
 }
 constexpr long long kWaitCycles = 400000000ll;   // about 0.2 s
 // A warp waits for a phase of a barrier of its block; gives up after kWaitCycles, or as soon as another block has (*abort).
+// The same answer in every lane.
 __device__ __forceinline__ bool wait_bytes(uint32_t bar, uint32_t parity, const int* abort) {
-    const long long t0 = clock64();
+    long long t0 = 0;
+    bool fine = true;
     for (int it = 0;; ++it) {
         uint32_t ok;
         asm volatile(
@@ -73,10 +75,16 @@ __device__ __forceinline__ bool wait_bytes(uint32_t bar, uint32_t parity, const 
             : "=r"(ok)
             : "r"(bar), "r"(parity)
             : "memory");
-        const bool up = !ok && (it & 63) == 63 && (clock64() - t0 > kWaitCycles || __ldcg(abort) != 0);
-        if (__any_sync(0xffffffffu, up)) return false;     // the same answer in every lane
-        if (__all_sync(0xffffffffu, ok != 0)) return true;
+        if (ok) break;
+        if ((it & 63) == 63) {
+            if (t0 == 0) t0 = clock64();
+            if (clock64() - t0 > kWaitCycles || __ldcg(abort) != 0) {
+                fine = false;
+                break;
+            }
+        }
     }
+    return __all_sync(0xffffffffu, fine);
 }
 
 // ---- scratch of one solve (floats): reflectors, tridiagonal, what the cluster leaves, a header ---------------------
@@ -159,7 +167,6 @@ struct TriState {
     float vr[S::RI];     // a at this thread's rows
     float y[S::RI];      // A a: this thread's part (its columns) of its rows
     float ak, b, tau;    // a at position kk; the reflector is v = a + b e_kk, H = I - tau v v^T
-    int it;
 };
 
 __device__ __forceinline__ float rsqrt_fast(float x) {
@@ -179,7 +186,8 @@ __device__ __forceinline__ float pick(const float (&t)[4], int s) { return (s & 
 // w = tau y - (tau^2 v^T y / 2) v the update is A -= v w^T + w v^T, and column kk after it follows from the same vectors.
 // One exchange of (y, A e_kk) between warps (blocks) per column; everything else is computed by every thread for its own rows and
 // columns. The norm of the new column, its square root and the reciprocal only enter through b and tau: they overlap with the update
-// of the tile and the product with the new column. What bounds it: n - 2 dependent steps, each the exchange, a few dozen
+// of the tile and the product with the new column. Positions that are done keep being transformed like the others (their part
+// of A is not used again, and a is zero there); only a is masked. What bounds it: n - 2 dependent steps, each the exchange, a few dozen
 // dependent operations, 3 multiply-adds per element of the tile and log2(LC) shuffles.
 template <typename S, int Q0>
 __device__ __forceinline__ bool tri_phase(TriState<S>& T, TriShared<S>& sh, int o, const TriWork& wk, int base, int pitch, int cta, int w, int lr, int lc) {
@@ -193,9 +201,9 @@ __device__ __forceinline__ bool tri_phase(TriState<S>& T, TriShared<S>& sh, int 
     const int rglob = irow * RB + rowbase;
     const int kbeg = o > Q0 * CB ? o : Q0 * CB;
     const int kend = S::LAST < Q0 * CB + CB - 1 ? S::LAST : Q0 * CB + CB - 1;
-    for (int kk = kbeg; kk <= kend; ++kk, ++T.it) {
-        const int b = T.it & 1;
-        const int lk = (kk >> 2) & (LC - 1), sk = kk & 3;   // lane column and element of position kk
+    auto step = [&](int kk, int sk) -> bool {               // sk = kk % 4: element of position kk in its lane's four columns
+        const int b = sk & 1;
+        const int lk = (kk >> 2) & (LC - 1);                // lane column of position kk
         const int d0 = kk - (CB * Q0 + 4 * lc);             // position kk is this thread's element d0 of slot Q0
         float2* xb = sh.x[b];
         float* yb = reinterpret_cast<float*>(xb);           // one block: y, then column kk
@@ -249,7 +257,7 @@ __device__ __forceinline__ bool tri_phase(TriState<S>& T, TriShared<S>& sh, int 
                 const uint32_t la = s_addr(&xb[rglob]), lb = s_addr(&sh.bar[b]);
                 for (int t = lc & (REP - 1); t < CL; t += REP) send_pair(map_to_cta(la, t), ysum, cval, map_to_cta(lb, t));
             }
-            if (!wait_bytes(s_addr(&sh.bar[b]), (T.it >> 1) & 1, wk.abort)) return false;
+            if (!wait_bytes(s_addr(&sh.bar[b]), (sk >> 1) & 1, wk.abort)) return false;
         }
         // both vectors at this thread's columns (pairs) and rows
         const float2 xk = CL == 1 ? make_float2(yb[kk], cb[kk]) : xb[kk];
@@ -319,14 +327,8 @@ __device__ __forceinline__ bool tri_phase(TriState<S>& T, TriShared<S>& sh, int 
         const u64 nt2 = pk(-T.tau, -T.tau), c2 = pk(c, c), v12 = pk(v1, v1), nw12 = pk(nw1, nw1);
 #pragma unroll
         for (int p = P0; p < 8; ++p) {
-            u64 ww = fma2(T.vc[p], c2, mul2(yc[p], nt2));   // -w
-            if (p < P0 + 2) {
-                float a0, a1;
-                upk(ww, a0, a1);
-                ww = pk(d0 <= 2 * (p - P0) ? a0 : 0.f, d0 <= 2 * (p - P0) + 1 ? a1 : 0.f);
-            }
-            nw[p] = ww;
-            a2[p] = fma2(T.vc[p], nw12, fma2(ww, v12, a2[p]));
+            nw[p] = fma2(T.vc[p], c2, mul2(yc[p], nt2));    // -w
+            a2[p] = fma2(T.vc[p], nw12, fma2(nw[p], v12, a2[p]));
         }
         float ak[4];                                        // column kk (after the update) at slot Q0, then masked
         upk(a2[P0], ak[0], ak[1]);
@@ -382,9 +384,8 @@ __device__ __forceinline__ bool tri_phase(TriState<S>& T, TriShared<S>& sh, int 
         }
 #pragma unroll
         for (int i = I0; i < RI; ++i) {
-            float nwr = fmaf(T.vr[i], c, __fmul_rn(xy[i], -T.tau));
+            const float nwr = fmaf(T.vr[i], c, __fmul_rn(xy[i], -T.tau));
             const int r = i * RB + rowbase;
-            if (i < I0 + NB && r < kk) nwr = 0.f;
             float ar = fmaf(T.vr[i], nw1, fmaf(nwr, v1, xc[i]));
             if (i < I0 + NB && r <= kk) ar = 0.f;
             const u64 v2 = pk(T.vr[i], T.vr[i]), n2 = pk(nwr, nwr);
@@ -422,6 +423,13 @@ __device__ __forceinline__ bool tri_phase(TriState<S>& T, TriShared<S>& sh, int 
         T.ak = an;
         T.b = some ? copysignf(beta, an) : 0.f;
         T.tau = some ? 2.f * q : 0.f;
+        return true;
+    };
+#pragma unroll 1
+    for (int kk = kbeg; kk <= kend; kk += 2) {              // kbeg is a multiple of 4; two steps, by four the code outgrows the instruction cache
+        if (!step(kk, kk & 2)) return false;
+        if (kk == kend) break;
+        if (!step(kk + 1, (kk & 2) | 1)) return false;
     }
     return true;
 }
@@ -500,7 +508,6 @@ k_tridiag(const float* __restrict__ K, int ldk, int n, int scaled, TriWork wk, i
 #pragma unroll
     for (int p = 0; p < 8; ++p) T.vc[p] = 0ull;
     T.ak = T.b = T.tau = 0.f;
-    T.it = 0;
     if constexpr (S::CL > 1) {
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
