@@ -194,9 +194,9 @@ struct sage_fd {
     bool app_pending = false;      // appends on `side` that the chain stream has not been made to wait for yet
     int64_t in_epoch = -1;         // the update call whose entry event `side` already waits for
     cudaEvent_t ev_in = nullptr;   // the caller's stream at the entry of an update call (sketch 0 only)
-    cudaEvent_t ev_rows = nullptr; // after the last append of the current update call
+    cudaEvent_t ev_rows = nullptr; // end of the current update call on the stream that reads its rows
     cudaEvent_t ev_done = nullptr; // end of the chain stream (joins)
-    bool used = false;             // fed during the current update call
+    cudaStream_t used = nullptr;   // the stream that reads rows of the current update call
 };
 
 namespace {
@@ -311,10 +311,18 @@ sage_status_t enqueue_gram(sage_fd* h, int r, cudaStream_t st) {
     return SAGE_OK;
 }
 
+// The appends of the next cycle may run beside the Gram kernel (they write the other buffer copy) and, unless the buffer is large,
+// they do: an event recorded inside the chain would end the overlap of its kernels. A buffer beyond the L2 cache keeps them
+// behind the Gram kernel, where they do not take its bandwidth (11 M columns: 3.10 s a pass behind it, 3.33 s beside it).
+bool appends_early(const sage_fd* h) { return (size_t)h->m * h->pitch * sizeof(float) <= ((size_t)64 << 20); }
+
 // Factor the first r rows and rebuild `keep` rows into the other buffer; rows keep..zero_to-1 are zeroed.
 sage_status_t enqueue_factor(sage_fd* h, int r, int do_shrink, int keep, int zero_to, cudaStream_t st) {
+    // where the appends of the next cycle may start: see sketch_feed
+    const bool fork = !(h->chain && st == h->chain), early = fork && appends_early(h);
+    if (early) CU_TRY(cudaEventRecord(h->ev_fork, st));
     ST_TRY(enqueue_gram(h, r, st));
-    CU_TRY(cudaEventRecord(h->ev_fork, st));       // from here on HBM is idle until the rebuild: see sage_fd_update
+    if (fork && !early) CU_TRY(cudaEventRecord(h->ev_fork, st));       // from here on HBM is idle until the rebuild
     const int j_pad = ((keep + 15) / 16) * 16;
     const bool tc_rebuild = h->use_tc && h->Wsplit && keep > 0 && j_pad <= h->wsplit_ld / 2 && r <= h->wsplit_ld;
     CU_TRY(timed(h, K_EIG, eig_launches(r, h->eig_variant), st, [&] {
@@ -369,6 +377,21 @@ sage_status_t check_handle(const sage_fd* h) {
 }  // namespace
 
 namespace sage {
+cudaError_t allow_smem(const void* kernel, int bytes) {
+    // set once per kernel and device: which is remembered in a small list (a handful of kernels)
+    struct Seen { const void* kernel; int dev, bytes; };
+    static std::mutex mu;
+    static std::vector<Seen> seen;
+    int dev = 0;
+    const cudaError_t e0 = cudaGetDevice(&dev);
+    if (e0 != cudaSuccess) return e0;
+    std::lock_guard<std::mutex> lock(mu);
+    for (Seen& x : seen)
+        if (x.kernel == kernel && x.dev == dev && x.bytes >= bytes) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) seen.push_back({kernel, dev, bytes});
+    return e;
+}
 void set_error_message(const char* msg) { set_err("%s", msg); }
 void count_launches(int k) { count(nullptr, k); }
 }  // namespace sage
@@ -624,9 +647,9 @@ sage_status_t sage_fd_set_option(sage_fd_t* h, int key, double value) {
 // caller's stream for a single sketch, the sketch's own stream in the merged form). An append writes rows
 // [fill, fill + take) of the current buffer copy and touches nothing the eigen-solve or the rebuild of the previous
 // shrink reads or writes (the rebuild fills rows [0, keep) of the same copy), so appends run beside the eigen-solve,
-// which leaves HBM idle. The side stream starts after the Gram kernel of the previous shrink (running beside it only
-// takes bandwidth from it; that also puts it after the rebuild before, which read the copy now being filled) and
-// the chain waits for the appends before the next Gram kernel.
+// which leaves HBM idle. The side stream starts before the Gram kernel of the previous shrink, or for large buffers
+// after it (appends_early): either way after the rebuild before, which read the copy now being filled. The chain waits
+// for the appends before the next Gram kernel. In the merged form the appends run on the chain stream itself.
 
 static sage_status_t sketch_join_appends(sage_fd* s, cudaStream_t chain) {
     if (s->app_pending) {
@@ -640,7 +663,7 @@ static sage_status_t sketch_join_appends(sage_fd* s, cudaStream_t chain) {
 static sage_status_t sketch_factor(sage_fd* s, int r, int do_shrink, int keep, int zero_to, cudaStream_t chain) {
     ST_TRY(sketch_join_appends(s, chain));
     ST_TRY(enqueue_factor(s, r, do_shrink, keep, zero_to, chain));
-    CU_TRY(cudaStreamWaitEvent(s->side, s->ev_fork, 0));
+    if (!(s->chain && chain == s->chain)) CU_TRY(cudaStreamWaitEvent(s->side, s->ev_fork, 0));
     return SAGE_OK;
 }
 
@@ -726,7 +749,7 @@ struct RowSrc {
 
 // Appends n rows of type dt and shrinks whenever the buffer fills. e_in (may be null): the event after which `rows`
 // are valid; epoch identifies the update call it belongs to. on_chain: appends run on the chain stream itself (used
-// where the rows to append are produced by that stream). Leaves s->ev_rows recorded after the last append.
+// where the rows to append are produced by that stream). Leaves the stream that reads the rows in s->used.
 static sage_status_t sketch_feed(sage_fd* s, RowSrc src, int64_t n, cudaStream_t chain, cudaEvent_t e_in, int64_t epoch, bool on_chain) {
     // merged form: the appends run on the chain stream too (the chains of the other sketches fill the device while this
     // one waits, and half as many streams keep every chain on a hardware queue of its own)
@@ -767,11 +790,7 @@ static sage_status_t sketch_feed(sage_fd* s, RowSrc src, int64_t n, cudaStream_t
         return SAGE_OK;
     };
     const sage_status_t rc = body();
-    if (appended && from_caller) {   // also on the error path: the caller's stream must not run ahead of appends that read `rows`
-        const cudaError_t e = cudaEventRecord(s->ev_rows, as);
-        if (rc == SAGE_OK) CU_TRY(e);
-        s->used = true;
-    }
+    if (appended && from_caller) s->used = as;   // also on the error path: the caller's stream must not run ahead of appends that read `rows`
     return rc;
 }
 
@@ -842,9 +861,10 @@ static sage_status_t update_from(sage_fd* h, RowSrc src, int64_t n, cudaStream_t
     for (int p = 0; p < h->P && p <= (int)h->kids.size(); ++p) {
         sage_fd* s = sketch_at(h, p);
         if (s->used) {
-            const cudaError_t e = cudaStreamWaitEvent(st, s->ev_rows, 0);
+            cudaError_t e = cudaEventRecord(s->ev_rows, s->used);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, s->ev_rows, 0);
+            s->used = nullptr;
             if (rc == SAGE_OK) CU_TRY(e);
-            s->used = false;
         }
     }
     return rc;

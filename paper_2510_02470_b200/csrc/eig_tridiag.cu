@@ -442,6 +442,7 @@ k_tridiag(const float* __restrict__ K, int ldk, int n, int scaled, TriWork wk, i
     const int cta = S::CL == 1 ? 0 : (int)blockIdx.x;
     const int o = (S::G - n) & ~3;
     float kscale = 1.f;
+    chain_wait();
     TriState<S> T;                                          // the loads of the tile first, all in flight together
 #pragma unroll
     for (int i = 0; i < S::RI; ++i) {
@@ -515,6 +516,7 @@ k_tridiag(const float* __restrict__ K, int ldk, int n, int scaled, TriWork wk, i
     bool ok = tri_phase<S, 0>(T, sh, o, wk, base, pitch, cta, w, lr, lc);
     ok = ok && tri_phase<S, 1>(T, sh, o, wk, base, pitch, cta, w, lr, lc);
     ok = ok && tri_phase<S, 2>(T, sh, o, wk, base, pitch, cta, w, lr, lc);
+    if (S::CL > 1 || S::G == 128) chain_release();
     if constexpr (S::G != 256) ok = ok && tri_phase<S, 3>(T, sh, o, wk, base, pitch, cta, w, lr, lc);
     if constexpr (S::CL == 1) {
         if (tid == S::NT - 1) {                             // the last diagonal element; two positions have no reflector
@@ -710,6 +712,7 @@ k_tridiag_vectors(TriWork wk, int G, int n, int do_shrink, int delta_rank, int k
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
+    chain_wait();
     for (int c = 0; c < RING; ++c) fetch(c);       // on their way while the eigenvalues are found
 
     const float dmax = *wk.dmax;
@@ -933,6 +936,7 @@ k_tridiag_vectors(TriWork wk, int G, int n, int do_shrink, int delta_rank, int k
         for (int t = 0; t < 4 * NQ; ++t) x[t] = (float)(v[t] * inv);
     }
 
+    chain_release();
     // ---- U = H_0 H_1 ... applied to the vectors, the last reflector first, four at a time: with c_i = v_i . x and the inner
     // products of the four among each other the four coefficients follow without another pass over x
     const bool resident = nch <= RING;
@@ -1043,13 +1047,15 @@ cudaError_t run_cluster(const float* K, int ldk, int n, TriWork wk, EigInfo* inf
     cfg.gridDim = dim3(S::CL);
     cfg.blockDim = dim3(S::NT);
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = S::CL;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, k_tridiag<S>, K, ldk, n, 0, wk, 0, (int)S::G, info);
 }
 
@@ -1058,11 +1064,10 @@ cudaError_t run_vectors(TriWork wk, int G, int n, int do_shrink, int delta_rank,
                         EigInfo* info, float* Wsplit, int ldw, int j_pad, cudaStream_t st) {
     const int rows = Wsplit && j_pad > keep ? j_pad : keep;
     const int blocks = rows > 0 ? (rows + kVecWarps - 1) / kVecWarps : 1;
-    cudaError_t e = cudaFuncSetAttribute(k_tridiag_vectors<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(VecShared<NQ>));
+    cudaError_t e = allow_smem((const void*)k_tridiag_vectors<NQ>, (int)sizeof(VecShared<NQ>));
     if (e != cudaSuccess) return e;
-    k_tridiag_vectors<NQ><<<blocks, kVecThreads, sizeof(VecShared<NQ>), st>>>(wk, G, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out, n_sigma, info,
-                                                                             Wsplit, ldw, j_pad);
-    return cudaGetLastError();
+    return launch_chained(k_tridiag_vectors<NQ>, dim3(blocks), dim3(kVecThreads), sizeof(VecShared<NQ>), st, wk, G, n, do_shrink, delta_rank, keep, Ur, ldu,
+                          sigma_out, n_sigma, info, Wsplit, ldw, j_pad);
 }
 
 }  // namespace
@@ -1082,13 +1087,11 @@ cudaError_t launch_eig_direct(const float* K, int ldk, int n, int do_shrink, int
     const TriWork wk = tri_work(work, G);
     cudaError_t e = cudaSuccess;
     if (G == 128) {
-        k_tridiag<Tri128><<<1, Tri128::NT, 0, st>>>(K, ldk, n, 0, wk, 0, G, info);
-        e = cudaGetLastError();
+        e = launch_chained(k_tridiag<Tri128>, dim3(1), dim3(Tri128::NT), 0, st, K, ldk, n, 0, wk, 0, G, info);
     } else {
         e = G == 256 ? run_cluster<Tri256>(K, ldk, n, wk, info, st) : run_cluster<Tri512>(K, ldk, n, wk, info, st);
         if (e != cudaSuccess) return e;
-        k_tridiag<Tri128><<<1, Tri128::NT, 0, st>>>(wk.trail, 128, 128, 1, wk, G - 128, G, info);
-        e = cudaGetLastError();
+        e = launch_chained(k_tridiag<Tri128>, dim3(1), dim3(Tri128::NT), 0, st, wk.trail, 128, 128, 1, wk, G - 128, G, info);
     }
     if (e != cudaSuccess) return e;
     if (G == 128) return run_vectors<1>(wk, G, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out, n_sigma, info, Wsplit, ldw, j_pad, st);

@@ -9,6 +9,34 @@
 
 namespace sage {
 
+// ---- launches of the shrink cycle ------------------------------------------------------------------------------------
+// The kernels of a cycle follow one another on a stream and each is short, so the gaps between them count. They are launched
+// with programmatic stream serialisation: a kernel may start, set up its barriers and allocate while its predecessor ends;
+// chain_wait() in it returns when every kernel before it on the stream has finished and its results are visible (each kernel
+// of the chain waits, so this holds for all of them), and nothing of theirs is touched before. chain_release() lets the next
+// one start; kernels that run long call it near their end, so that the next does not sit on an SM for nothing.
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
+// Lets a kernel use up to `bytes` of dynamic shared memory; the driver is asked once per kernel and device.
+cudaError_t allow_smem(const void* kernel, int bytes);
+
 // Device-side flags accumulated in the handle's status word.
 constexpr uint32_t kFlagNotConverged = 1u;
 constexpr uint32_t kFlagNonFinite = 2u;

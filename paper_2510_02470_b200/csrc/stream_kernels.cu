@@ -17,6 +17,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_append(const T* __restrict__ rows, int64_t n, int64_t ld, int64_t D,
                                                 float* __restrict__ B, int64_t pitch, int dst_row0) {
     constexpr int V = 16 / sizeof(T);   // elements per 16-byte load
+    chain_wait();
+    chain_release();
     const int64_t row = blockIdx.y;
     const T* src = rows + row * ld;
     float* dst = B + (int64_t)(dst_row0 + row) * pitch;
@@ -52,6 +54,8 @@ __global__ void __launch_bounds__(256) k_append(const T* __restrict__ rows, int6
 template <typename T>
 __global__ void __launch_bounds__(256) k_append_outer(const T* __restrict__ q, int64_t ldq, const T* __restrict__ feat, int64_t ldf, int C,
                                                       int F, float* __restrict__ B, int64_t pitch, int dst_row0) {
+    chain_wait();
+    chain_release();
     const int64_t row = blockIdx.y;
     const T* qr = q + row * ldq;
     const T* hr = feat + row * ldf;
@@ -207,6 +211,8 @@ __global__ void __launch_bounds__(256) k_split_tf32(const float* __restrict__ sr
 // the tiles below the diagonal are read from their mirror image.
 __global__ void __launch_bounds__(256) k_split_reduce(const float* __restrict__ parts, int splits, int64_t split_stride,
                                                       int M, int N, int64_t ldp, float* __restrict__ out, int64_t ldo, int mirror) {
+    chain_release();                        // the next kernel of a shrink is one small block
+    chain_wait();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)M * N) return;
     const int i = (int)(e / N), j = (int)(e % N);
@@ -226,6 +232,8 @@ __global__ void __launch_bounds__(1024) k_gram_sym_reduce(const float* __restric
     // 16 x 16 outputs per block; the four z-layers of the block each sum a quarter of the partial matrices
     // (several loads in flight per thread: the kernel is bound by load latency, not by bytes).
     __shared__ double sa[4][16][17], sb[4][16][17];
+    chain_release();                        // the next kernel of a shrink is one small block
+    chain_wait();
     const int tx = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;
     const int i = blockIdx.y * 16 + ty, j = blockIdx.x * 16 + tx;          // direct element (i, j)
     const int ti = blockIdx.x * 16 + ty, tj = blockIdx.y * 16 + tx;        // element (ti, tj) of the mirrored tile
@@ -319,9 +327,9 @@ cudaError_t launch_append(const void* rows, sage_dtype_t dt, int64_t n, int64_t 
     if (bx < 1) bx = 1;
     dim3 grid((unsigned)bx, (unsigned)n);
     if (dt == SAGE_F32)
-        k_append<float><<<grid, 256, 0, st>>>(static_cast<const float*>(rows), n, ld, D, B, pitch, dst_row0);
+        return launch_chained(k_append<float>, grid, dim3(256), 0, st, static_cast<const float*>(rows), n, ld, D, B, pitch, dst_row0);
     else
-        k_append<__nv_bfloat16><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(rows), n, ld, D, B, pitch, dst_row0);
+        return launch_chained(k_append<__nv_bfloat16>, grid, dim3(256), 0, st, static_cast<const __nv_bfloat16*>(rows), n, ld, D, B, pitch, dst_row0);
     return cudaGetLastError();
 }
 
@@ -334,10 +342,10 @@ cudaError_t launch_append_outer(const void* q, int64_t ldq, const void* feat, in
     if (bx < 1) bx = 1;
     dim3 grid((unsigned)bx, (unsigned)n);
     if (dt == SAGE_F32)
-        k_append_outer<float><<<grid, 256, 0, st>>>(static_cast<const float*>(q), ldq, static_cast<const float*>(feat), ldf, C, F, B, pitch,
+        return launch_chained(k_append_outer<float>, grid, dim3(256), 0, st, static_cast<const float*>(q), ldq, static_cast<const float*>(feat), ldf, C, F, B, pitch,
                                                     dst_row0);
     else
-        k_append_outer<__nv_bfloat16><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(q), ldq, static_cast<const __nv_bfloat16*>(feat),
+        return launch_chained(k_append_outer<__nv_bfloat16>, grid, dim3(256), 0, st, static_cast<const __nv_bfloat16*>(q), ldq, static_cast<const __nv_bfloat16*>(feat),
                                                             ldf, C, F, B, pitch, dst_row0);
     return cudaGetLastError();
 }
@@ -381,16 +389,14 @@ cudaError_t launch_split_reduce(const float* parts, int splits, int64_t split_st
                                 int64_t ldo, cudaStream_t st, int mirror) {
     const int64_t total = (int64_t)M * N;
     if (total <= 0) return cudaSuccess;
-    k_split_reduce<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(parts, splits, split_stride, M, N, ldp, out, ldo, mirror);
-    return cudaGetLastError();
+    return launch_chained(k_split_reduce, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, parts, splits, split_stride, M, N, ldp, out, ldo, mirror);
 }
 
 cudaError_t launch_gram_sym_reduce(const float* parts, int splits, int64_t stride, int r, int64_t ldp, float* out, int64_t ldo,
                                    cudaStream_t st) {
     if (r <= 0) return cudaSuccess;
     const unsigned t = (unsigned)((r + 15) / 16);
-    k_gram_sym_reduce<<<dim3(t, t), dim3(16, 16, 4), 0, st>>>(parts, splits, stride, r, ldp, out, ldo);
-    return cudaGetLastError();
+    return launch_chained(k_gram_sym_reduce, dim3(t, t), dim3(16, 16, 4), 0, st, parts, splits, stride, r, ldp, out, ldo);
 }
 
 cudaError_t launch_rebuild(const float* Ur, int ldu, const float* Bsrc, float* Bdst, int64_t pitch, int64_t D, int r, int keep,

@@ -130,6 +130,7 @@ k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    chain_wait();
 
     if (warp == 0) {
         if (lane == 0) {
@@ -302,6 +303,7 @@ k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             while (ok && drained < nchunks && (drained + 1 + ring / 2) * kChunk - kstep <= kt) drain(drained++);
         }
         while (ok && drained < nchunks) drain(drained++);
+        chain_release();
         const int row = m0 + quarter * 32 + lane;
         if (proj) {
             // lane = sketch row (0-63: hi part, 64-127: lo part), register c = data row chalf * 64 + c of the tile:
@@ -359,7 +361,8 @@ cudaError_t launch_tc_gemm_nt_x3(const float* A, int64_t lda, const float* Bm, i
     CUtensorMap tmA, tmB;
     if (!tc::make_tmap_2d(&tmA, A, 4, (uint64_t)M, (uint64_t)(class_F > 0 ? class_F : K), (uint64_t)lda, tc::kTileM)) return cudaErrorNotSupported;
     const int b_box_rows = proj ? tc::kTileN : (N >= tc::kTileN ? tc::kTileN : ((N + 15) / 16) * 16);
-    if (!tc::make_tmap_2d(&tmB, Bm, 4, (uint64_t)(proj ? 128 : N), (uint64_t)K, (uint64_t)ldb, (uint32_t)b_box_rows)) return cudaErrorNotSupported;
+    if (gram && M <= tc::kTileM) tmB = tmA;           // not used: diagonal tile only
+    else if (!tc::make_tmap_2d(&tmB, Bm, 4, (uint64_t)(proj ? 128 : N), (uint64_t)K, (uint64_t)ldb, (uint32_t)b_box_rows)) return cudaErrorNotSupported;
     int64_t kps = (K + splits - 1) / splits;
     kps = ((kps + tc::BK - 1) / tc::BK) * tc::BK;
     if (class_F > 0) kps = class_F;
@@ -378,11 +381,10 @@ cudaError_t launch_tc_gemm_nt_x3(const float* A, int64_t lda, const float* Bm, i
     const int G = deep ? stages : ((stages & 1) ? 1 : 2);
     const size_t smem = (size_t)stages * stage_bytes + 1024 + (3 * stages + 2 * tc::kAccs) * 8 + 16;
     dim3 grid((unsigned)((M + tc::kTileM - 1) / tc::kTileM), proj ? 1u : (unsigned)((N + tc::kTileN - 1) / tc::kTileN), (unsigned)splits);
-    cudaError_t e = cudaFuncSetAttribute(tc::k_tc_gemm_nt_x3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void*)tc::k_tc_gemm_nt_x3, 227 * 1024);
     if (e != cudaSuccess) return e;
-    tc::k_tc_gemm_nt_x3<<<grid, tc::kThreads, smem, st>>>(tmA, tmB, M, N, gram, b_box_rows, sym, K, kps, class_F > 0 ? 1 : 0, C, ldc, split_stride, stages,
-                                                                 stage_bytes, G, 0, 0, err);
-    return cudaGetLastError();
+    return launch_chained(tc::k_tc_gemm_nt_x3, grid, dim3(tc::kThreads), smem, st, tmA, tmB, M, N, gram, b_box_rows, sym, K, kps, class_F > 0 ? 1 : 0, C,
+                          ldc, split_stride, stages, stage_bytes, G, 0, 0, err);
 }
 
 // See sage_internal.h.
@@ -406,11 +408,10 @@ cudaError_t launch_tc_gram_direct(const float* Bold, int64_t pitch, int old_rows
     const int G = deep ? stages : ((stages & 1) ? 1 : 2);
     const size_t smem = (size_t)stages * stage_bytes + 1024 + (3 * stages + 2 * tc::kAccs) * 8 + 16;
     dim3 grid(1u, 1u, (unsigned)splits);
-    cudaError_t e = cudaFuncSetAttribute(tc::k_tc_gemm_nt_x3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void*)tc::k_tc_gemm_nt_x3, 227 * 1024);
     if (e != cudaSuccess) return e;
-    tc::k_tc_gemm_nt_x3<<<grid, tc::kThreads, smem, st>>>(tmA, tmB, M, M, 1, 0, 1, D, kps, 0, C, ldc, split_stride, stages, stage_bytes, G, n_new,
-                                                         src_box, err);
-    return cudaGetLastError();
+    return launch_chained(tc::k_tc_gemm_nt_x3, grid, dim3(tc::kThreads), smem, st, tmA, tmB, M, M, 1, 0, 1, D, kps, 0, C, ldc, split_stride, stages,
+                          stage_bytes, G, n_new, src_box, err);
 }
 
 }  // namespace sage

@@ -90,6 +90,7 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    chain_wait();
 
     if (warp == 0) {
         if (lane == 0) {
@@ -219,6 +220,7 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
+            if (lt == my_tiles - 1) chain_release();
             const long long d = (blockIdx.x + lt * gridDim.x) * kTileD + quarter * 32 + lane;
             const uint32_t acc = lane_base + (uint32_t)(b * n_mma);
             for (int j0 = 0; j0 < j_pad; j0 += 32) {
@@ -324,11 +326,10 @@ static cudaError_t launch_tc_rebuild_part(const float* Wsplit, int ldw, int j_pa
     const size_t smem = (size_t)stages * stage_bytes + (w_res ? w_all : 0) + 1024 + (3 * stages + 5) * 8 + 16;
     const long long num_tiles = (pitch + tc::kTileD - 1) / tc::kTileD;
     const int grid = (int)(num_tiles < 148 ? num_tiles : 148);
-    cudaError_t e = cudaFuncSetAttribute(tc::k_tc_rebuild, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void*)tc::k_tc_rebuild, 227 * 1024);
     if (e != cudaSuccess) return e;
-    tc::k_tc_rebuild<<<grid, tc::kThreads, smem, st>>>(tmBuf, tmW, tmSrc, tmSrc1, src ? n_new : 0, r, keep, j_pad, pitch, num_tiles, Bdst, stages,
-                                                       w_res, err);
-    return cudaGetLastError();
+    return launch_chained(tc::k_tc_rebuild, dim3(grid), dim3(tc::kThreads), smem, st, tmBuf, tmW, tmSrc, tmSrc1, src ? n_new : 0, r, keep, j_pad, pitch,
+                          num_tiles, Bdst, stages, w_res, err);
 }
 
 // See sage_internal.h. One launch takes at most 128 output rows (accumulator width) of up to 512 buffer rows; 129 to 256
