@@ -123,6 +123,34 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
     return cudaMallocFromPoolAsync(p, bytes, pools[dev], st);
 }
 
+// Where the rows of an update come from: a dense matrix (rows, pitch ld), or the two factors of structured last-layer
+// rows (q: pitch ldq, C values per row; feat: pitch ldf, F values per row), expanded on the fly.
+struct RowSrc {
+    const void* rows = nullptr;
+    int64_t ld = 0;
+    const void* q = nullptr;
+    const void* feat = nullptr;
+    int64_t ldq = 0, ldf = 0;
+    int C = 0, F = 0;
+    sage_dtype_t dt = SAGE_F32;
+    bool outer() const { return q != nullptr; }
+    RowSrc advanced(int64_t k) const {       // the same source, k rows further on
+        RowSrc r = *this;
+        const size_t es = elem_size(dt);
+        if (rows) r.rows = static_cast<const char*>(rows) + (size_t)k * ld * es;
+        if (q) r.q = static_cast<const char*>(q) + (size_t)k * ldq * es;
+        if (feat) r.feat = static_cast<const char*>(feat) + (size_t)k * ldf * es;
+        return r;
+    }
+    // `take` rows, followed by the first `take2` rows of `more` (same type, pitches and shape)
+    cudaError_t append(int64_t take, int64_t D, float* B, int64_t pitch, int dst_row0, cudaStream_t st, const RowSrc* more = nullptr,
+                       int64_t take2 = 0) const {
+        if (outer())
+            return launch_append_outer(q, ldq, feat, ldf, dt, take, C, F, B, pitch, dst_row0, st, more ? more->q : nullptr, more ? more->feat : nullptr, take2);
+        return launch_append(rows, dt, take, ld, D, B, pitch, dst_row0, st, more ? more->rows : nullptr, take2);
+    }
+};
+
 }  // namespace
 
 struct sage_fd {
@@ -196,6 +224,15 @@ struct sage_fd {
     cudaEvent_t ev_in = nullptr;   // the caller's stream at the entry of an update call (sketch 0 only)
     cudaEvent_t ev_rows = nullptr; // end of the current update call on the stream that reads its rows
     cudaEvent_t ev_done = nullptr; // end of the chain stream (joins)
+    RowSrc pend;                   // rows of the current update call that still have to be appended, pend_n of them, to row pend_row
+    int64_t pend_n = 0;            // (merged form: the dealt blocks cut a cycle's rows in two; one launch appends both parts)
+    int pend_row = 0;
+    struct Cycle {                 // merged form: a whole cycle's launches as a graph, one per buffer copy (see run_cycle)
+        cudaGraphExec_t exec = nullptr;
+        int launches = 0, tc_launches = 0;
+    } cycle[2];
+    int cycles_run = 0;
+    bool cycle_graphs = true;
     cudaStream_t used = nullptr;   // the stream that reads rows of the current update call
 };
 
@@ -424,6 +461,17 @@ int64_t sage_select_count(int64_t N, double keep_rate) {
     return (int64_t)k;
 }
 
+// Forgets the captured cycles (their launches hold what the options said); waits for the device if there are any.
+static void drop_cycles(sage_fd* s) {
+    if (s->cycle[0].exec || s->cycle[1].exec) cudaDeviceSynchronize();
+    for (sage_fd::Cycle& c : s->cycle) {
+        if (c.exec) cudaGraphExecDestroy(c.exec);
+        c = sage_fd::Cycle();
+    }
+    s->cycles_run = 0;
+    for (sage_fd* k : s->kids) drop_cycles(k);
+}
+
 static sage_status_t create_handle(sage_fd_t** out, int64_t D, int32_t ell, sage_dtype_t row_dtype, int device, bool sketch_only) {
     if (!out || D < 1 || (row_dtype != SAGE_F32 && row_dtype != SAGE_BF16) || device < 0) {
         set_err("sage_fd_create: bad argument (out=%p D=%lld dtype=%d device=%d)", (void*)out, (long long)D, (int)row_dtype, device);
@@ -515,6 +563,7 @@ void sage_fd_destroy(sage_fd_t* h) {
     cudaDeviceSynchronize();
     for (sage_fd* k : h->kids) sage_fd_destroy(k);
     h->kids.clear();
+    drop_cycles(h);
     if (h->chain) cudaStreamDestroy(h->chain);
     for (cudaEvent_t ev : {h->ev_in, h->ev_rows, h->ev_done})
         if (ev) cudaEventDestroy(ev);
@@ -580,6 +629,10 @@ sage_status_t sage_fd_set_option(sage_fd_t* h, int key, double value) {
         h->prof.mask = (unsigned)value & ((1u << K_NCLASS) - 1u);
         for (sage_fd* k : h->kids) k->prof.mask = h->prof.mask;
         return SAGE_OK;
+    }
+    {
+        DeviceGuard g(h->device);
+        drop_cycles(h);
     }
     if (key == 4) {                          // 0: CUDA-core kernels only, 1: tensor-core kernels where possible
         h->use_tc = value != 0.0;
@@ -660,8 +713,54 @@ static sage_status_t sketch_join_appends(sage_fd* s, cudaStream_t chain) {
     return SAGE_OK;
 }
 
+// A full buffer's cycle in the merged form. Sixteen chains share the device and one host thread enqueues for all of them, so the
+// host bounds a pass over short rows: the launches of a cycle (the same every time but for the buffer copy) are captured
+// once the sketch has run a few and replayed as a graph, one host call instead of five.
+static sage_status_t run_cycle(sage_fd* s, cudaStream_t chain) {
+    const int keep = s->delta_rank - 1;
+    constexpr int kDirect = 8;                 // cycles before a capture pays
+    sage_fd::Cycle& c = s->cycle[s->cur];
+    if (c.exec) {
+        CU_TRY(cudaGraphLaunch(c.exec, chain));
+        count(s, c.launches);
+        s->tc_launches += c.tc_launches;
+        s->cur = 1 - s->cur;
+        s->fill = keep;
+        return SAGE_OK;
+    }
+    if (!s->cycle_graphs || s->cycles_run < kDirect) {
+        ++s->cycles_run;
+        return enqueue_factor(s, s->m, 1, keep, 0, chain);
+    }
+    const int cur = s->cur, fill = s->fill;
+    const int64_t l0 = s->launches, t0 = s->tc_launches;
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(chain, cudaStreamCaptureModeThreadLocal);
+    sage_status_t rc = SAGE_ERR_CUDA;
+    if (e == cudaSuccess) {
+        rc = enqueue_factor(s, s->m, 1, keep, 0, chain);
+        e = cudaStreamEndCapture(chain, &g);
+        if (e == cudaSuccess && rc == SAGE_OK) e = cudaGraphInstantiate(&c.exec, g, 0);
+        if (g) cudaGraphDestroy(g);
+    }
+    if (e != cudaSuccess || rc != SAGE_OK) {   // not captured: nothing has run yet
+        (void)cudaGetLastError();
+        c = sage_fd::Cycle();
+        s->cycle_graphs = false;
+        s->cur = cur;
+        s->fill = fill;
+        return enqueue_factor(s, s->m, 1, keep, 0, chain);
+    }
+    c.launches = (int)(s->launches - l0);
+    c.tc_launches = (int)(s->tc_launches - t0);
+    CU_TRY(cudaGraphLaunch(c.exec, chain));
+    return SAGE_OK;
+}
+
 static sage_status_t sketch_factor(sage_fd* s, int r, int do_shrink, int keep, int zero_to, cudaStream_t chain) {
     ST_TRY(sketch_join_appends(s, chain));
+    if (s->chain && chain == s->chain && r == s->m && do_shrink && zero_to == 0 && keep == s->delta_rank - 1 && s->prof.mask == 0)
+        return run_cycle(s, chain);
     ST_TRY(enqueue_factor(s, r, do_shrink, keep, zero_to, chain));
     if (!(s->chain && chain == s->chain)) CU_TRY(cudaStreamWaitEvent(s->side, s->ev_fork, 0));
     return SAGE_OK;
@@ -722,30 +821,13 @@ static sage_status_t sketch_factor_direct(sage_fd* s, const void* rows, int64_t 
     return SAGE_OK;
 }
 
-// Where the rows of an update come from: a dense matrix (rows, pitch ld), or the two factors of structured last-layer
-// rows (q: pitch ldq, C values per row; feat: pitch ldf, F values per row), expanded on the fly.
-struct RowSrc {
-    const void* rows = nullptr;
-    int64_t ld = 0;
-    const void* q = nullptr;
-    const void* feat = nullptr;
-    int64_t ldq = 0, ldf = 0;
-    int C = 0, F = 0;
-    sage_dtype_t dt = SAGE_F32;
-    bool outer() const { return q != nullptr; }
-    RowSrc advanced(int64_t k) const {       // the same source, k rows further on
-        RowSrc r = *this;
-        const size_t es = elem_size(dt);
-        if (rows) r.rows = static_cast<const char*>(rows) + (size_t)k * ld * es;
-        if (q) r.q = static_cast<const char*>(q) + (size_t)k * ldq * es;
-        if (feat) r.feat = static_cast<const char*>(feat) + (size_t)k * ldf * es;
-        return r;
-    }
-    cudaError_t append(int64_t take, int64_t D, float* B, int64_t pitch, int dst_row0, cudaStream_t st) const {
-        if (outer()) return launch_append_outer(q, ldq, feat, ldf, dt, take, C, F, B, pitch, dst_row0, st);
-        return launch_append(rows, dt, take, ld, D, B, pitch, dst_row0, st);
-    }
-};
+static sage_status_t flush_pending(sage_fd* s, cudaStream_t as) {
+    if (s->pend_n == 0) return SAGE_OK;
+    const int64_t n = s->pend_n;
+    s->pend_n = 0;
+    CU_TRY(timed(s, K_APPEND, 1, as, [&] { return s->pend.append(n, s->D, s->B[s->cur], s->pitch, s->pend_row, as); }));
+    return SAGE_OK;
+}
 
 // Appends n rows of type dt and shrinks whenever the buffer fills. e_in (may be null): the event after which `rows`
 // are valid; epoch identifies the update call it belongs to. on_chain: appends run on the chain stream itself (used
@@ -778,13 +860,24 @@ static sage_status_t sketch_feed(sage_fd* s, RowSrc src, int64_t n, cudaStream_t
                     continue;
                 }
             }
-            CU_TRY(timed(s, K_APPEND, 1, as, [&] { return src.append(take, s->D, s->B[s->cur], s->pitch, s->fill, as); }));
+            if (on_chain && from_caller && s->pend_n == 0) {     // appended together with the next part, or by flush_pending
+                s->pend = src;
+                s->pend_n = take;
+                s->pend_row = s->fill;
+            } else if (s->pend_n > 0) {
+                const int64_t first = s->pend_n;
+                s->pend_n = 0;
+                CU_TRY(timed(s, K_APPEND, 1, as, [&] { return s->pend.append(first, s->D, s->B[s->cur], s->pitch, s->pend_row, as, &src, take); }));
+            } else {
+                CU_TRY(timed(s, K_APPEND, 1, as, [&] { return src.append(take, s->D, s->B[s->cur], s->pitch, s->fill, as); }));
+            }
             appended = true;
             if (!on_chain) s->app_pending = true;
             s->fill += (int)take;
             s->rows_seen += take;
             src = src.advanced(take);
             n -= take;
+            if (s->fill == s->m) ST_TRY(flush_pending(s, as));
             if (s->fill == s->m) ST_TRY(sketch_factor(s, s->m, 1, s->delta_rank - 1, 0, chain));
         }
         return SAGE_OK;
@@ -861,6 +954,8 @@ static sage_status_t update_from(sage_fd* h, RowSrc src, int64_t n, cudaStream_t
     for (int p = 0; p < h->P && p <= (int)h->kids.size(); ++p) {
         sage_fd* s = sketch_at(h, p);
         if (s->used) {
+            const sage_status_t fl = flush_pending(s, s->used);
+            if (rc == SAGE_OK) rc = fl;
             cudaError_t e = cudaEventRecord(s->ev_rows, s->used);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(st, s->ev_rows, 0);
             s->used = nullptr;
@@ -1650,7 +1745,7 @@ sage_status_t sage_fd_import(sage_fd_t* h, const void* src_host, size_t bytes, v
     ST_TRY(sage_fd_reset(h));
     ST_TRY(sage_fd_set_option(h, 6, (double)hd.P));
     h->block = hd.block;
-    h->delta_rank = hd.delta_rank;
+    h->delta_rank = hd.delta_rank;                           // (the call above dropped the captured cycles)
     for (sage_fd* k : h->kids) k->delta_rank = hd.delta_rank;
     if (hd.nsk > 1) ST_TRY(ensure_sketches(h));
     const char* q = static_cast<const char*>(src_host) + sizeof hd;

@@ -56,14 +56,16 @@ struct EigInfo {
 // ---- launchers (each enqueues on `st` and returns cudaGetLastError()) -----------------------------
 
 // B[dst_row0 + i, 0:D] = float(rows[i, 0:D]) for i < n; columns D..pitch-1 of those rows are zeroed.
+// n2 > 0: the n2 rows after them come from rows2 (same type and pitch).
 cudaError_t launch_append(const void* rows, sage_dtype_t dt, int64_t n, int64_t ld, int64_t D, float* B,
-                          int64_t pitch, int dst_row0, cudaStream_t st);
+                          int64_t pitch, int dst_row0, cudaStream_t st, const void* rows2 = nullptr, int64_t n2 = 0);
 
 // Structured last-layer rows: B[dst_row0 + i, :] = [vec_rowmajor(q_i feat_i^T) ; q_i] for i < n, with q n x C (pitch ldq) and feat
 // n x F (pitch ldf) of element type dt; products in fp32 (exact for bf16 factors); columns C F + C .. pitch-1 zeroed. pitch
 // must be a multiple of 4.
 cudaError_t launch_append_outer(const void* q, int64_t ldq, const void* feat, int64_t ldf, sage_dtype_t dt, int64_t n, int C, int F,
-                                float* B, int64_t pitch, int dst_row0, cudaStream_t st);
+                                float* B, int64_t pitch, int dst_row0, cudaStream_t st, const void* q2 = nullptr, const void* feat2 = nullptr,
+                                int64_t n2 = 0);
 
 // Projection of structured rows from per-class planes: with T[c] = feat * S_c^T (n x ell, the sum of pp consecutive planes of
 // `planes`, plane_stride floats apart, n x ell each with pitch ell) and S_c the columns [c F, c F + F) of the sketch,

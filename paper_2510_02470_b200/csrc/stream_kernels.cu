@@ -14,13 +14,13 @@ __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162flo
 // One block row of threads walks a row with 16-byte accesses where the addresses allow it.
 // ------------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(256) k_append(const T* __restrict__ rows, int64_t n, int64_t ld, int64_t D,
+__global__ void __launch_bounds__(256) k_append(const T* __restrict__ rows, int64_t n, const T* __restrict__ rows2, int64_t ld, int64_t D,
                                                 float* __restrict__ B, int64_t pitch, int dst_row0) {
     constexpr int V = 16 / sizeof(T);   // elements per 16-byte load
     chain_wait();
     chain_release();
     const int64_t row = blockIdx.y;
-    const T* src = rows + row * ld;
+    const T* src = row < n ? rows + row * ld : rows2 + (row - n) * ld;      // n rows from `rows`, the others from `rows2`
     float* dst = B + (int64_t)(dst_row0 + row) * pitch;
     const bool vec_ok = ((reinterpret_cast<uintptr_t>(src) & 15) == 0);
     const int64_t chunk0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
@@ -52,13 +52,13 @@ __global__ void __launch_bounds__(256) k_append(const T* __restrict__ rows, int6
 // from the two factors and written straight into the destination rows, so the C F + C values never exist in the caller's
 // memory. Products are taken in fp32 (exact for bf16 factors). Columns from C F + C up to the pitch are zeroed.
 template <typename T>
-__global__ void __launch_bounds__(256) k_append_outer(const T* __restrict__ q, int64_t ldq, const T* __restrict__ feat, int64_t ldf, int C,
-                                                      int F, float* __restrict__ B, int64_t pitch, int dst_row0) {
+__global__ void __launch_bounds__(256) k_append_outer(const T* __restrict__ q, const T* __restrict__ feat, int64_t n, const T* __restrict__ q2,
+                                                      const T* __restrict__ feat2, int64_t ldq, int64_t ldf, int C, int F, float* __restrict__ B, int64_t pitch, int dst_row0) {
     chain_wait();
     chain_release();
     const int64_t row = blockIdx.y;
-    const T* qr = q + row * ldq;
-    const T* hr = feat + row * ldf;
+    const T* qr = row < n ? q + row * ldq : q2 + (row - n) * ldq;            // n rows from the first pair, the others from the second
+    const T* hr = row < n ? feat + row * ldf : feat2 + (row - n) * ldf;
     float* dst = B + (int64_t)(dst_row0 + row) * pitch;
     const int64_t CF = (int64_t)C * F, D = CF + C;
     const int64_t c0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
@@ -319,35 +319,34 @@ __global__ void __launch_bounds__(256) k_rebuild(const float* __restrict__ Ur, i
 }  // namespace
 
 cudaError_t launch_append(const void* rows, sage_dtype_t dt, int64_t n, int64_t ld, int64_t D, float* B, int64_t pitch,
-                          int dst_row0, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
+                          int dst_row0, cudaStream_t st, const void* rows2, int64_t n2) {
+    if (n + n2 <= 0) return cudaSuccess;
     const int V = dt == SAGE_F32 ? 4 : 8;
     int64_t bx = (pitch / V + 255) / 256;
     if (bx > 592) bx = 592;
     if (bx < 1) bx = 1;
-    dim3 grid((unsigned)bx, (unsigned)n);
+    dim3 grid((unsigned)bx, (unsigned)(n + n2));
     if (dt == SAGE_F32)
-        return launch_chained(k_append<float>, grid, dim3(256), 0, st, static_cast<const float*>(rows), n, ld, D, B, pitch, dst_row0);
-    else
-        return launch_chained(k_append<__nv_bfloat16>, grid, dim3(256), 0, st, static_cast<const __nv_bfloat16*>(rows), n, ld, D, B, pitch, dst_row0);
-    return cudaGetLastError();
+        return launch_chained(k_append<float>, grid, dim3(256), 0, st, static_cast<const float*>(rows), n, static_cast<const float*>(rows2), ld, D, B,
+                              pitch, dst_row0);
+    using bf = __nv_bfloat16;
+    return launch_chained(k_append<bf>, grid, dim3(256), 0, st, static_cast<const bf*>(rows), n, static_cast<const bf*>(rows2), ld, D, B, pitch, dst_row0);
 }
 
 cudaError_t launch_append_outer(const void* q, int64_t ldq, const void* feat, int64_t ldf, sage_dtype_t dt, int64_t n, int C, int F,
-                                float* B, int64_t pitch, int dst_row0, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
+                                float* B, int64_t pitch, int dst_row0, cudaStream_t st, const void* q2, const void* feat2, int64_t n2) {
+    if (n + n2 <= 0) return cudaSuccess;
     if (pitch & 3) return cudaErrorInvalidValue;
     int64_t bx = (pitch / 4 + 255) / 256;
     if (bx > 592) bx = 592;
     if (bx < 1) bx = 1;
-    dim3 grid((unsigned)bx, (unsigned)n);
+    dim3 grid((unsigned)bx, (unsigned)(n + n2));
     if (dt == SAGE_F32)
-        return launch_chained(k_append_outer<float>, grid, dim3(256), 0, st, static_cast<const float*>(q), ldq, static_cast<const float*>(feat), ldf, C, F, B, pitch,
-                                                    dst_row0);
-    else
-        return launch_chained(k_append_outer<__nv_bfloat16>, grid, dim3(256), 0, st, static_cast<const __nv_bfloat16*>(q), ldq, static_cast<const __nv_bfloat16*>(feat),
-                                                            ldf, C, F, B, pitch, dst_row0);
-    return cudaGetLastError();
+        return launch_chained(k_append_outer<float>, grid, dim3(256), 0, st, static_cast<const float*>(q), static_cast<const float*>(feat), n,
+                              static_cast<const float*>(q2), static_cast<const float*>(feat2), ldq, ldf, C, F, B, pitch, dst_row0);
+    using bf = __nv_bfloat16;
+    return launch_chained(k_append_outer<bf>, grid, dim3(256), 0, st, static_cast<const bf*>(q), static_cast<const bf*>(feat), n,
+                          static_cast<const bf*>(q2), static_cast<const bf*>(feat2), ldq, ldf, C, F, B, pitch, dst_row0);
 }
 
 cudaError_t launch_gemm_nt(const void* A, sage_dtype_t dt, int64_t lda, const float* Bm, int64_t ldb, int M, int N,
