@@ -1483,7 +1483,7 @@ sage_status_t sage_select(const float* scores, int64_t N, double keep_rate, int6
         cudaError_t e2 = cudaFreeAsync(scratch, st);
         CU_TRY(e);
         CU_TRY(e2);
-        count(nullptr, select_launches(N));
+        count(nullptr, select_launches(N, k));
     }
     if (k_out) *k_out = k;
     return SAGE_OK;

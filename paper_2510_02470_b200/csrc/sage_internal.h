@@ -191,7 +191,7 @@ cudaError_t launch_class_pick(const float* scores, const int* labels, int64_t N,
 
 // Top-k by (score desc, index asc). scratch: select_scratch_bytes. Returns through idx (device).
 cudaError_t select_scratch_bytes(int64_t N, size_t* bytes);
-int select_launches(int64_t N);
+int select_launches(int64_t N, int64_t k);
 cudaError_t launch_select(const float* scores, int64_t N, int64_t k, int64_t* idx, void* scratch, cudaStream_t st);
 
 // Hooks into the C ABI's bookkeeping for entry points defined outside api.cu.

@@ -6,8 +6,9 @@
 //
 // Up to kClusterMax rows the whole sort is one launch: a cluster of 8 thread blocks, digit counts exchanged through
 // distributed shared memory, keys through L2, two cluster barriers per pass. Such a sort is bound by latency (launches before,
-// barriers now): a call on 50,000 scores took 149 us in 20 launches (six passes, the index included, of three kernels with a
-// one-block scan over all counters) and takes 57 us. Beyond, three launches per pass (counts, one block per digit scanning its counters, scatter).
+// barriers and shared-memory conflicts now). Beyond, three launches per pass (counts, one block per digit scanning its
+// counters, scatter). A selection sorts as little as it can (select_filters). Measured, a call on 50,000 scores, a tenth wanted:
+// 149 us (20 launches, all scores sorted, index included) -> 57 us (one cluster sort) -> 32 us (the 5,000 picks ranked).
 #include <cooperative_groups.h>
 
 #include <cstdio>
@@ -48,11 +49,25 @@ struct SortArgs {
     const int* labels;
     int64_t N;
     int C, by_score, label_passes;
+    bool given = false;                                      // the keys are in the first buffer already (one-launch form)
 };
 __device__ __forceinline__ unsigned digit_of(const SortArgs& a, u64 key, int pass) {
     const int vp = a.by_score ? 4 : 0;
     if (pass < vp) return (unsigned)(key >> (32 + 8 * pass)) & 255u;
     return (class_of(a.labels, key, a.C) >> (8 * (pass - vp))) & 255u;
+}
+
+// Lanes that hold the same digit (256: a lane without a key), by a vote per bit: a match instruction takes longer the more values
+// there are (2,000 cycles per 32 keys and warp on random digits).
+__device__ __forceinline__ unsigned same_digit(unsigned d) {
+    const unsigned none = __ballot_sync(0xffffffffu, d == 256u);
+    unsigned m = d == 256u ? none : ~none;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const unsigned v = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+        m &= (d >> b) & 1u ? v : ~v;
+    }
+    return m;
 }
 
 // ---- one launch: cluster of 8 ------------------------------------------------------------------------------------
@@ -63,11 +78,13 @@ constexpr int64_t kClusterMax = (int64_t)kClSize * kClKeys;
 struct ClusterShared {
     unsigned short cnt[kClWarps][256];
     unsigned short pos[kClKeys];                             // rank of a key among those of its digit before it in its warp's run
+    u64 local[kClKeys];                                      // the block's keys by digit, so that they leave in runs
     unsigned hist[256];                                      // this block's counts, read by the others
-    unsigned base[256];
+    unsigned base[256];                                      // where this block's keys of a digit go, minus lexcl
+    unsigned lexcl[256];                                     // where they start in `local`
     unsigned excl[257];                                      // where a digit's keys start
     unsigned total[256];
-    unsigned wsum[8];
+    unsigned wsum[16];
     long long kc[256], rem[256], offs[256];
 };
 
@@ -89,11 +106,12 @@ k_sort_cluster(SortArgs a, u64* __restrict__ b0, u64* __restrict__ b1, int64_t k
     const int passes = (a.by_score ? 4 : 0) + a.label_passes;
     u64* in = b0;
     u64* out = b1;
+    chain_wait();
     for (int pass = 0; pass < passes; ++pass) {
         const bool last = pass == passes - 1;
         auto load = [&](int64_t i) -> u64 {
             if (i >= a.N) return 0ull;
-            if (pass > 0) return __ldcg(in + i);
+            if (pass > 0 || a.given) return __ldcg(in + i);
             return a.by_score ? make_key(a.scores, i) : (u64)i;
         };
         for (int e = tid; e < kClWarps * 128; e += kClThreads) reinterpret_cast<unsigned*>(&sh.cnt[0][0])[e] = 0u;
@@ -113,7 +131,7 @@ k_sort_cluster(SortArgs a, u64* __restrict__ b0, u64* __restrict__ b1, int64_t k
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (s0 + 32 * u >= span) break;
-                const unsigned peers = __match_any_sync(0xffffffffu, dig[u]);
+                const unsigned peers = same_digit(dig[u]);
                 const unsigned r = __popc(peers & ((1u << lane) - 1u));
                 const unsigned before = dig[u] < 256u ? cnt[dig[u]] : 0u;
                 __syncwarp();
@@ -134,7 +152,7 @@ k_sort_cluster(SortArgs a, u64* __restrict__ b0, u64* __restrict__ b1, int64_t k
             sh.hist[tid] = run;
         }
         cluster.sync();
-        unsigned before = 0, total = 0, x = 0;
+        unsigned before = 0, total = 0, x = 0, xl = 0;
         if (tid < 256) {
 #pragma unroll
             for (int r = 0; r < kClSize; ++r) {
@@ -143,20 +161,31 @@ k_sort_cluster(SortArgs a, u64* __restrict__ b0, u64* __restrict__ b1, int64_t k
                 total += v;
             }
             x = total;
+            xl = sh.hist[tid];
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
+                const unsigned y = __shfl_up_sync(0xffffffffu, x, o), yl = __shfl_up_sync(0xffffffffu, xl, o);
+                if (lane >= o) {
+                    x += y;
+                    xl += yl;
+                }
             }
-            if (lane == 31) sh.wsum[warp] = x;
+            if (lane == 31) {
+                sh.wsum[warp] = x;
+                sh.wsum[8 + warp] = xl;
+            }
         }
         __syncthreads();
         if (tid < 256) {
-            unsigned e = x - total;
-            for (int w = 0; w < warp; ++w) e += sh.wsum[w];
+            unsigned e = x - total, el = xl - sh.hist[tid];
+            for (int w = 0; w < warp; ++w) {
+                e += sh.wsum[w];
+                el += sh.wsum[8 + w];
+            }
             sh.excl[tid] = e;
             if (tid == 255) sh.excl[256] = e + total;
-            sh.base[tid] = e + before;
+            sh.base[tid] = e + before - el;
+            sh.lexcl[tid] = el;
             sh.total[tid] = total;
         }
         __syncthreads();
@@ -209,19 +238,23 @@ k_sort_cluster(SortArgs a, u64* __restrict__ b0, u64* __restrict__ b1, int64_t k
                 dig[u] = live ? digit_of(a, key[u], pass) : 256u;
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (dig[u] >= 256u) continue;
-                const unsigned p = sh.base[dig[u]] + cnt[dig[u]] + pos[s0 + 32 * u + lane];
-                if (!last) {
-                    out[p] = key[u];
-                } else if (MODE == EMIT_TOPK) {
-                    if ((int64_t)p < k) idx[p] = (int64_t)(uint32_t)key[u];
-                } else if (MODE == EMIT_ORDER) {
-                    order[p] = (unsigned)(uint32_t)key[u];
-                } else {
-                    const long long r = (long long)(p - sh.excl[dig[u]]);
-                    if ((int)dig[u] < a.C && r < sh.kc[dig[u]]) idx[sh.offs[dig[u]] + r] = (int64_t)(uint32_t)key[u];
-                }
+            for (int u = 0; u < 4; ++u)
+                if (dig[u] < 256u) sh.local[sh.lexcl[dig[u]] + cnt[dig[u]] + pos[s0 + 32 * u + lane]] = key[u];
+        }
+        __syncthreads();
+        const int mine = max((long long)0, min((long long)span * kClWarps, (long long)(a.N - (int64_t)rank * kClWarps * span)));
+        for (int i = tid; i < mine; i += kClThreads) {
+            const u64 key = sh.local[i];
+            const unsigned d = digit_of(a, key, pass), p = sh.base[d] + (unsigned)i;
+            if (!last) {
+                out[p] = key;
+            } else if (MODE == EMIT_TOPK) {
+                if ((int64_t)p < k) idx[p] = (int64_t)(uint32_t)key;
+            } else if (MODE == EMIT_ORDER) {
+                order[p] = (unsigned)(uint32_t)key;
+            } else {
+                const long long r = (long long)(p - sh.excl[d]);
+                if ((int)d < a.C && r < sh.kc[d]) idx[sh.offs[d] + r] = (int64_t)(uint32_t)key;
             }
         }
         cluster.sync();                                      // keys are out, counts may be overwritten
@@ -234,21 +267,213 @@ k_sort_cluster(SortArgs a, u64* __restrict__ b0, u64* __restrict__ b1, int64_t k
 template <int MODE>
 cudaError_t run_cluster_sort(const SortArgs& a, u64* b0, u64* b1, int64_t k, double keep_rate, int64_t* idx, unsigned* order, unsigned* starts,
                              long long* kc_out, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(k_sort_cluster<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClusterShared));
+    cudaError_t e = allow_smem((const void*)k_sort_cluster<MODE>, (int)sizeof(ClusterShared));
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kClSize);
     cfg.blockDim = dim3(kClThreads);
     cfg.dynamicSmemBytes = sizeof(ClusterShared);
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = kClSize;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, k_sort_cluster<MODE>, a, b0, b1, k, keep_rate, idx, order, starts, kc_out);
+}
+
+// ---- few picks: the k-th key first, then only the k best are put in order --------------------------------------------
+// k_top_keys: one cluster of 8. The k-th smallest score image is found by its digits (11, 11, 10 bits, counts exchanged through
+// distributed shared memory), ties at it go to the smaller indices, and the k keys are written in index order. Up to
+// kClusterMax rows each block keeps its scores in shared memory; beyond it reads them again (from L2) at every step.
+constexpr int64_t kFilterMax = 1 << 18;                     // 500,000 scores, a tenth wanted: 146 us this way, 105 us by sorting on all SMs
+constexpr int kBins = 2048;
+struct FilterShared {
+    unsigned hist[kBins];
+    unsigned sum[kBins];
+    unsigned wsum[kClWarps];
+    unsigned nless[kClWarps], neq[kClWarps];
+    unsigned cta_less, cta_eq;                               // read by the other blocks
+    unsigned digit, below;
+    unsigned val[kClKeys];
+};
+__global__ void __launch_bounds__(kClThreads, 1) k_top_keys(const float* __restrict__ scores, int64_t N, int64_t k, u64* __restrict__ out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    FilterShared& sh = *reinterpret_cast<FilterShared*>(smem_raw);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int span = (int)((N + kClSize * kClThreads - 1) / (kClSize * kClThreads)) * 32;     // scores per warp, whole slots of 32
+    const int64_t base = ((int64_t)rank * kClWarps + warp) * span;
+    const int live = (int)max((int64_t)0, min((int64_t)span, N - base));
+    const bool resident = N <= kClusterMax;
+    unsigned* vals = sh.val + (resident ? warp * span : 0);
+    auto image = [&](int i) -> unsigned { return (unsigned)(make_key(scores, base + i) >> 32); };
+    chain_wait();
+    chain_release();
+    if (resident) {
+#pragma unroll 4
+        for (int i = lane; i < live; i += 32) vals[i] = image(i);
+        __syncwarp();
+    }
+    auto value = [&](int i) -> unsigned { return resident ? vals[i] : image(i); };
+    unsigned prefix = 0, mask = 0, want = (unsigned)k;       // looking for the want-th smallest among values with v & mask == prefix
+#pragma unroll 1
+    for (int step = 0; step < 3; ++step) {
+        const int shift = step == 0 ? 21 : step == 1 ? 10 : 0, bits = step == 2 ? 10 : 11;
+        for (int e = tid; e < kBins; e += kClThreads) sh.hist[e] = 0u;
+        __syncthreads();
+#pragma unroll 4
+        for (int s0 = 0; s0 < span; s0 += 32) {
+            const int i = s0 + lane;
+            const unsigned v = i < live ? value(i) : 0u;
+            const bool on = i < live && (v & mask) == prefix;
+            const unsigned d = (v >> shift) & ((1u << bits) - 1u);
+            const unsigned act = __ballot_sync(0xffffffffu, on);
+            if (act == 0u) continue;
+            const unsigned d0 = __shfl_sync(0xffffffffu, d, __ffs(act) - 1);
+            if (__ballot_sync(0xffffffffu, on && d != d0) == 0u) {         // all alike: one add
+                if (lane == 0) atomicAdd(&sh.hist[d0], (unsigned)__popc(act));
+            } else if (on) {
+                atomicAdd(&sh.hist[d], 1u);
+            }
+        }
+        cluster.sync();
+        unsigned h[2] = {0u, 0u};                            // bins 2 tid, 2 tid + 1 over the whole cluster
+#pragma unroll
+        for (int r = 0; r < kClSize; ++r) {
+            const uint2 v = *reinterpret_cast<const uint2*>(cluster.map_shared_rank(sh.hist, r) + 2 * tid);
+            h[0] += v.x;
+            h[1] += v.y;
+        }
+        const unsigned mine = h[0] + h[1];
+        unsigned x = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) sh.wsum[warp] = x;
+        __syncthreads();
+        unsigned e = x - mine;
+        for (int w = 0; w < warp; ++w) e += sh.wsum[w];
+        if (e < want && want <= e + h[0]) { sh.digit = 2 * tid; sh.below = e; }
+        if (e + h[0] < want && want <= e + mine) { sh.digit = 2 * tid + 1; sh.below = e + h[0]; }
+        cluster.sync();                                      // the counts have been read by everybody
+        prefix |= sh.digit << shift;
+        mask |= ((1u << bits) - 1u) << shift;
+        want -= sh.below;
+    }
+    // prefix is the k-th value; all smaller ones and the first `want` equal ones are picked
+    unsigned nl = 0, ne = 0;
+#pragma unroll 4
+    for (int i = lane; i < live; i += 32) {
+        const unsigned v = value(i);
+        nl += v < prefix;
+        ne += v == prefix;
+    }
+    nl = __reduce_add_sync(0xffffffffu, nl);
+    ne = __reduce_add_sync(0xffffffffu, ne);
+    if (lane == 0) {
+        sh.nless[warp] = nl;
+        sh.neq[warp] = ne;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned a = __reduce_add_sync(0xffffffffu, sh.nless[lane]), b = __reduce_add_sync(0xffffffffu, sh.neq[lane]);
+        if (lane == 0) {
+            sh.cta_less = a;
+            sh.cta_eq = b;
+        }
+    }
+    cluster.sync();
+    unsigned less = 0, eq = 0;                               // before this warp's run
+    for (int r = 0; r < rank; ++r) {
+        less += *cluster.map_shared_rank(&sh.cta_less, r);
+        eq += *cluster.map_shared_rank(&sh.cta_eq, r);
+    }
+    for (int w = 0; w < warp; ++w) {
+        less += sh.nless[w];
+        eq += sh.neq[w];
+    }
+#pragma unroll 2
+    for (int s0 = 0; s0 < span; s0 += 32) {
+        const int i = s0 + lane;
+        const unsigned v = i < live ? value(i) : 0xffffffffu;
+        const bool lt = i < live && v < prefix, same = i < live && v == prefix;
+        const unsigned bl = __ballot_sync(0xffffffffu, lt), be = __ballot_sync(0xffffffffu, same), mine = (1u << lane) - 1u;
+        const unsigned e = eq + __popc(be & mine);
+        if (lt || (same && e < want)) out[less + __popc(bl & mine) + min(e, want)] = ((u64)v << 32) | (u64)(uint32_t)(base + i);
+        less += __popc(bl);
+        eq += __popc(be);
+    }
+    cluster.sync();                                          // no block leaves while another reads its counts
+}
+
+// Few keys: a key's place is the number of smaller ones. Block: 32 keys (one per lane), each of its 16 warps compares them with a
+// sixteenth of all. keys == nullptr: made from the scores. n <= kRankMax: 8,192 keys take 5 us on all SMs, about what the sort
+// takes on eight; the work grows with the square.
+constexpr int kRankMax = 8192;
+constexpr int kRankThreads = 512;
+__global__ void __launch_bounds__(kRankThreads) k_rank(const u64* __restrict__ keys, const float* __restrict__ scores, int n, int64_t k,
+                                                       int64_t* __restrict__ idx) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    u64* all = reinterpret_cast<u64*>(smem_raw);             // n, rounded up to 32 with keys that no other is larger than
+    __shared__ unsigned place[kRankThreads / 32][32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int np = (n + 31) & ~31;
+    chain_wait();
+#pragma unroll 4
+    for (int i = tid; i < np; i += kRankThreads) all[i] = i < n ? (keys ? __ldcg(keys + i) : make_key(scores, i)) : ~0ull;
+    __syncthreads();
+    const int me = blockIdx.x * 32 + lane;
+    const u64 mine = me < np ? all[me] : ~0ull;
+    unsigned less = 0;
+    const ulonglong2* two = reinterpret_cast<const ulonglong2*>(all);
+#pragma unroll 4
+    for (int i = warp; i < np / 2; i += kRankThreads / 32) {
+        const ulonglong2 o = two[i];
+        less += (o.x < mine) + (o.y < mine);
+    }
+    place[warp][lane] = less;
+    __syncthreads();
+    if (warp == 0 && me < n) {
+        unsigned p = 0;
+#pragma unroll
+        for (int w = 0; w < kRankThreads / 32; ++w) p += place[w][lane];
+        if ((int64_t)p < k) idx[p] = (int64_t)(uint32_t)mine;
+    }
+}
+
+cudaError_t run_rank(const u64* keys, const float* scores, int n, int64_t k, int64_t* idx, cudaStream_t st) {
+    const int np = (n + 31) & ~31;
+    cudaError_t e = allow_smem((const void*)k_rank, kRankMax * 8);
+    if (e != cudaSuccess) return e;
+    return launch_chained(k_rank, dim3((unsigned)(np / 32)), dim3(kRankThreads), (size_t)np * 8, st, keys, scores, n, k, idx);
+}
+
+cudaError_t run_top_keys(const float* scores, int64_t N, int64_t k, u64* out, cudaStream_t st) {
+    cudaError_t e = allow_smem((const void*)k_top_keys, (int)sizeof(FilterShared));
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kClSize);
+    cfg.blockDim = dim3(kClThreads);
+    cfg.dynamicSmemBytes = sizeof(FilterShared);
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kClSize;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, k_top_keys, scores, N, k, out);
 }
 
 // ---- three launches per pass, any N ------------------------------------------------------------------------------
@@ -267,7 +492,7 @@ __global__ void __launch_bounds__(kThreads) k_histogram(SortArgs a, const u64* _
     for (int s = 0; s < kItems; ++s) {
         const int64_t i = base + s * kThreads + threadIdx.x;
         const unsigned d = i < a.N ? digit_of(a, keys[i], pass) : 256u;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);         // scores share their leading bits: one add per value and warp
+        const unsigned peers = same_digit(d);         // scores share their leading bits: one add per value and warp
         if (d < 256u && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&h[d], (unsigned)__popc(peers));
     }
     __syncthreads();
@@ -330,7 +555,7 @@ __global__ void __launch_bounds__(kThreads) k_scatter(SortArgs a, const u64* __r
     for (int s = 0; s < kItems; ++s) {
         const bool live = base + s * 32 + lane < a.N;
         const unsigned d = live ? digit_of(a, key[s], pass) : 256u;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const unsigned peers = same_digit(d);
         const unsigned rank = __popc(peers & ((1u << lane) - 1u));
         unsigned before = 0;
         if (live) before = cnt[warp][d];
@@ -449,16 +674,26 @@ cudaError_t select_scratch_bytes(int64_t N, size_t* bytes) {
     return cudaSuccess;
 }
 
-int select_launches(int64_t N) { return N <= kClusterMax ? 1 : 1 + 3 * 4; }
+// Few rows: ranked. At most half of them wanted: the k-th key first, then the picks ranked or sorted. Otherwise all are sorted.
+static bool select_filters(int64_t N, int64_t k) { return N > kRankMax && N <= kFilterMax && k <= N / 2 && k <= kClusterMax; }
+
+int select_launches(int64_t N, int64_t k) { return N <= kRankMax ? 1 : select_filters(N, k) ? 2 : N <= kClusterMax ? 1 : 1 + 3 * 4; }
 
 cudaError_t launch_select(const float* scores, int64_t N, int64_t k, int64_t* idx, void* scratch, cudaStream_t st) {
     if (N <= 0 || k <= 0) return cudaSuccess;
-    const SortArgs a = {scores, nullptr, N, 0, 1, 0};
-    if (N <= kClusterMax) {
-        u64* b0 = static_cast<u64*>(scratch);
-        u64* b1 = reinterpret_cast<u64*>(static_cast<char*>(scratch) + align256((size_t)N * 8));
+    if (N <= kRankMax) return run_rank(nullptr, scores, (int)N, k, idx, st);
+    SortArgs a = {scores, nullptr, N, 0, 1, 0};
+    u64* b0 = static_cast<u64*>(scratch);
+    u64* b1 = reinterpret_cast<u64*>(static_cast<char*>(scratch) + align256((size_t)N * 8));
+    if (select_filters(N, k)) {
+        const cudaError_t e = run_top_keys(scores, N, k, b0, st);
+        if (e != cudaSuccess) return e;
+        if (k <= kRankMax) return run_rank(b0, nullptr, (int)k, k, idx, st);
+        a.N = k;
+        a.given = true;
         return run_cluster_sort<EMIT_TOPK>(a, b0, b1, k, 0.0, idx, nullptr, nullptr, nullptr, st);
     }
+    if (N <= kClusterMax) return run_cluster_sort<EMIT_TOPK>(a, b0, b1, k, 0.0, idx, nullptr, nullptr, nullptr, st);
     return sort_launches(a, scratch, k, idx, nullptr, st);
 }
 
@@ -592,7 +827,7 @@ extern "C" sage_status_t sage_select_static(const float* scores, int64_t N, doub
             sage::set_error_message(msg);
             return SAGE_ERR_CUDA;
         }
-        sage::count_launches(sage::select_launches(N));
+        sage::count_launches(sage::select_launches(N, k));
     }
     if (k_out) *k_out = k;
     return SAGE_OK;

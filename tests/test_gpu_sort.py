@@ -12,12 +12,12 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-@pytest.mark.parametrize("N", [33, 8191, 8192, 8193, 57344 + 5, 131071, 131072, 131073, 1050001])
+@pytest.mark.parametrize("N", [1, 33, 8191, 8192, 8193, 57344 + 5, 131071, 131072, 131073, 262144, 262145, 1050001])
 def test_selection_at_the_edges(N):
     r = np.random.default_rng(N)
-    a = np.where(r.uniform(size=N) < 0.3, r.integers(-6, 7, N) / 6.0, r.uniform(-1, 1, N)).astype(np.float32)
+    a = np.where(r.uniform(size=N) < 0.3, r.integers(-6, 7, N) / 6.0, r.uniform(-1, 1, N)).astype(np.float32)   # ties at many places
     s = torch.from_numpy(a).to(DEV)
-    for rate in (1.0 / N, 0.37, 1.0):
+    for rate in (1.0 / N, min(8192, N) / N, min(8193, N) / N, 0.37, 0.5, 0.51, 1.0):
         assert np.array_equal(sage.sage_select(s, rate).cpu().numpy(), oracle.select(a.astype(np.float64), rate)), rate
 
 
