@@ -16,6 +16,8 @@ __global__ void __launch_bounds__(256) k_class_sums(const float* __restrict__ zh
     __shared__ double sh[256];
     __shared__ double red[8];
     const int c = blockIdx.y, j = threadIdx.x % jw, g = threadIdx.x / jw, G = 256 / jw;
+    chain_wait();
+    chain_release();
     const unsigned first = starts[c], n = starts[c + 1] - first;
     const unsigned len = (n + gridDim.x - 1) / gridDim.x;
     const unsigned r0 = blockIdx.x * len, r1 = min(n, r0 + len);
@@ -58,8 +60,19 @@ __global__ void __launch_bounds__(256) k_class_units(const double* __restrict__ 
     __shared__ double red[8];
     const int c = blockIdx.x, j = threadIdx.x;
     double t = 0.0;
-    if (j < ell)
-        for (int s = 0; s < nparts; ++s) t += parts[((int64_t)c * nparts + s) * ell + j];
+    chain_wait();
+    chain_release();
+    if (j < ell) {
+        int s = 0;
+        for (; s + 8 <= nparts; s += 8) {                    // eight loads in flight, added in order
+            double v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = parts[((int64_t)c * nparts + s + u) * ell + j];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) t += v[u];
+        }
+        for (; s < nparts; ++s) t += parts[((int64_t)c * nparts + s) * ell + j];
+    }
     double sq = t * t;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
@@ -72,19 +85,39 @@ __global__ void __launch_bounds__(256) k_class_units(const double* __restrict__ 
     if (j == 0) counts[c] = (int)(starts[c + 1] - starts[c]);
 }
 
-// One warp per example: score = <zhat_i, u_label(i)>; examples without a class in [0, C) score 0.
+// One warp per example, four of a warp's in flight: score = <zhat_i, u_label(i)>; examples without a class in [0, C) score 0.
+template <int T>
 __global__ void __launch_bounds__(256) k_class_scores(const float* __restrict__ zhat, const int* __restrict__ labels, int64_t N,
                                                       int ell, int C, const float* __restrict__ U, float* __restrict__ scores) {
+    constexpr int RB = T > 4 ? 2 : 4;
     const int lane = threadIdx.x & 31;
-    const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (row >= N) return;
-    const int lab = labels[row];
-    float acc = 0.f;
-    if (lab >= 0 && lab < C)
-        for (int j = lane; j < ell; j += 32) acc = fmaf(zhat[row * ell + j], U[(int64_t)lab * ell + j], acc);
+    const int64_t stride = (int64_t)gridDim.x * 8;
+    chain_wait();
+    chain_release();
+    for (int64_t r0 = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r0 < N; r0 += RB * stride) {
+        float acc[RB];
+        int lab[RB];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) scores[row] = fminf(1.f, fmaxf(-1.f, acc));
+        for (int r = 0; r < RB; ++r) {
+            lab[r] = r0 + r * stride < N ? labels[r0 + r * stride] : -1;
+            if (lab[r] >= C) lab[r] = -1;
+        }
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            acc[r] = 0.f;
+#pragma unroll
+            for (int t = 0; t < T; ++t)
+                if (lab[r] >= 0 && lane + 32 * t < ell)
+                    acc[r] = fmaf(zhat[(r0 + r * stride) * ell + lane + 32 * t], U[(int64_t)lab[r] * ell + lane + 32 * t], acc[r]);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int r = 0; r < RB; ++r) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
+#pragma unroll
+        for (int r = 0; r < RB; ++r)
+            if (lane == 0 && r0 + r * stride < N) scores[r0 + r * stride] = fminf(1.f, fmaxf(-1.f, acc[r]));
+    }
 }
 
 // Parts per class: enough blocks to fill the device when there are few classes, one when there are many.
@@ -119,12 +152,13 @@ cudaError_t launch_class_scores(const float* zhat, const int* labels, int64_t N,
     int jw = 32;
     while (jw < ell) jw <<= 1;
     const int np = class_parts(C);
-    k_class_sums<<<dim3(np, C), 256, 0, st>>>(zhat, order, starts, ell, jw, parts, U, counts);
-    if (np > 1) k_class_units<<<C, 256, 0, st>>>(parts, np, starts, ell, U, counts);
-    e = cudaGetLastError();
+    e = launch_chained(k_class_sums, dim3(np, C), dim3(256), 0, st, zhat, order, starts, ell, jw, parts, U, counts);
+    if (e == cudaSuccess && np > 1) e = launch_chained(k_class_units, dim3(C), dim3(256), 0, st, parts, np, starts, ell, U, counts);
     if (e != cudaSuccess || N <= 0) return e;
-    k_class_scores<<<(unsigned)((N + 7) / 8), 256, 0, st>>>(zhat, labels, N, ell, C, U, scores);
-    return cudaGetLastError();
+    int64_t blocks = (N + 7) / 8;
+    if (blocks > 148 * 8) blocks = 148 * 8;
+    auto run = [&](auto kernel) { return launch_chained(kernel, dim3((unsigned)blocks), dim3(256), 0, st, zhat, labels, N, ell, C, U, scores); };
+    return ell <= 32 ? run(k_class_scores<1>) : ell <= 64 ? run(k_class_scores<2>) : ell <= 128 ? run(k_class_scores<4>) : run(k_class_scores<8>);
 }
 
 }  // namespace sage

@@ -8,82 +8,104 @@ namespace sage {
 namespace {
 
 constexpr int kRowsPerBlock = 64;   // rows whose zhat are summed into one partial
-constexpr int kMaxPerLane = 8;      // ell <= 256
 
-// One warp per row, 8 warps per block, each warp walks rows w, w+8, ... of the block's 64 rows.
+// One warp per row, 8 warps per block, each warp walks rows w, w+8, ... of the block's 64 rows, 8 / T of them at a time (T: 32-wide
+// pieces of a row): the kernel is bound by the latency of its loads and reductions, so several rows' are in flight (50,000 rows
+// of 64 values in two planes, 38 MB: 52 us with one row at a time).
 // planes > 1: the projections arrive as that many partial planes (K slices of the projection, `plane_stride` floats apart),
 // which are summed here in ascending plane order with fp64 accumulation before the row is normalised.
+template <int T>
 __global__ void __launch_bounds__(256) k_normalise(const float* __restrict__ Z, int planes, int64_t plane_stride, int64_t ldz, int64_t n,
                                                    int ell, float* __restrict__ zhat, float* __restrict__ znorm,
                                                    float* __restrict__ partials, unsigned* __restrict__ flags) {
-    __shared__ float part[8][256];
+    constexpr int RB = 8 / T;
+    __shared__ float part[8][32 * T];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t row0 = (int64_t)blockIdx.x * kRowsPerBlock;
-    float sum[kMaxPerLane];
+    const int64_t row0 = (int64_t)blockIdx.x * kRowsPerBlock + warp;
+    float sum[T];
 #pragma unroll
-    for (int t = 0; t < kMaxPerLane; ++t) sum[t] = 0.f;
+    for (int t = 0; t < T; ++t) sum[t] = 0.f;
     bool bad = false;
-    for (int rr = warp; rr < kRowsPerBlock; rr += 8) {
-        const int64_t row = row0 + rr;
-        if (row >= n) break;
-        float z[kMaxPerLane];
-        float amax = 0.f;
-        bool finite = true;
+    chain_wait();
+    chain_release();
+#pragma unroll 1
+    for (int q0 = 0; q0 < kRowsPerBlock / 8; q0 += RB) {
+        float z[RB][T];
+        if (planes == 1) {
 #pragma unroll
-        for (int t = 0; t < kMaxPerLane; ++t) {
-            const int j = lane + 32 * t;
-            if (j >= ell) {
-                z[t] = 0.f;
-            } else if (planes == 1) {
-                z[t] = Z[row * ldz + j];
-            } else {
-                const float* src = Z + row * ldz + j;
-                double acc = 0.0;
-                int pz = 0;
-                for (; pz + 4 <= planes; pz += 4) {      // four loads in flight, added in plane order
-                    const float a0 = src[(int64_t)pz * plane_stride], a1 = src[(int64_t)(pz + 1) * plane_stride];
-                    const float a2 = src[(int64_t)(pz + 2) * plane_stride], a3 = src[(int64_t)(pz + 3) * plane_stride];
-                    acc += (double)a0;
-                    acc += (double)a1;
-                    acc += (double)a2;
-                    acc += (double)a3;
+            for (int r = 0; r < RB; ++r)
+#pragma unroll
+                for (int t = 0; t < T; ++t) {
+                    const int64_t row = row0 + 8 * (q0 + r);
+                    z[r][t] = row < n && lane + 32 * t < ell ? Z[row * ldz + lane + 32 * t] : 0.f;
                 }
-                for (; pz < planes; ++pz) acc += (double)src[(int64_t)pz * plane_stride];
-                z[t] = (float)acc;
+        } else {
+            double acc[RB][T];
+#pragma unroll
+            for (int r = 0; r < RB; ++r)
+#pragma unroll
+                for (int t = 0; t < T; ++t) acc[r][t] = 0.0;
+#pragma unroll 2
+            for (int pz = 0; pz < planes; ++pz)
+#pragma unroll
+                for (int r = 0; r < RB; ++r)
+#pragma unroll
+                    for (int t = 0; t < T; ++t) {
+                        const int64_t row = row0 + 8 * (q0 + r);
+                        if (row < n && lane + 32 * t < ell) acc[r][t] += (double)Z[pz * plane_stride + row * ldz + lane + 32 * t];
+                    }
+#pragma unroll
+            for (int r = 0; r < RB; ++r)
+#pragma unroll
+                for (int t = 0; t < T; ++t) z[r][t] = (float)acc[r][t];
+        }
+        float amax[RB], s[RB];
+        bool finite[RB];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            amax[r] = 0.f;
+            finite[r] = true;
+#pragma unroll
+            for (int t = 0; t < T; ++t) {
+                finite[r] = finite[r] && (fabsf(z[r][t]) <= 3.0e38f);   // false for NaN and Inf
+                amax[r] = fmaxf(amax[r], fabsf(z[r][t]));
             }
-            finite = finite && (fabsf(z[t]) <= 3.0e38f);   // false for NaN and Inf
-            amax = fmaxf(amax, fabsf(z[t]));
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-        finite = __all_sync(0xffffffffu, finite);
-        float nrm = 0.f, scale = 0.f;
-        if (finite && amax > 0.f) {
-            const float inv = 1.f / amax;
-            float s = 0.f;
+        for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-            for (int t = 0; t < kMaxPerLane; ++t) {
-                z[t] *= inv;
-                s = fmaf(z[t], z[t], s);
+            for (int r = 0; r < RB; ++r) amax[r] = fmaxf(amax[r], __shfl_xor_sync(0xffffffffu, amax[r], o));
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            finite[r] = __all_sync(0xffffffffu, finite[r]);
+            const float inv = finite[r] && amax[r] > 0.f ? 1.f / amax[r] : 0.f;
+            s[r] = 0.f;
+#pragma unroll
+            for (int t = 0; t < T; ++t) {
+                z[r][t] = inv > 0.f ? z[r][t] * inv : 0.f;
+                s[r] = fmaf(z[r][t], z[r][t], s[r]);
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            const float rs = sqrtf(s);
-            nrm = amax * rs;
-            scale = 1.f / rs;
         }
-        if (!finite) bad = true;
 #pragma unroll
-        for (int t = 0; t < kMaxPerLane; ++t) {
-            const int j = lane + 32 * t;
-            const float v = z[t] * scale;       // scale = 0 for zero / non-finite rows
-            if (j < ell) zhat[row * ell + j] = (scale > 0.f) ? v : 0.f;
-            sum[t] += (scale > 0.f) ? v : 0.f;
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int r = 0; r < RB; ++r) s[r] += __shfl_xor_sync(0xffffffffu, s[r], o);
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            const int64_t row = row0 + 8 * (q0 + r);
+            const float rs = sqrtf(s[r]), scale = s[r] > 0.f ? 1.f / rs : 0.f;       // 0 for zero and non-finite rows
+            if (!finite[r] && row < n) bad = true;
+#pragma unroll
+            for (int t = 0; t < T; ++t) {
+                const float v = scale > 0.f ? z[r][t] * scale : 0.f;
+                if (row < n && lane + 32 * t < ell) zhat[row * ell + lane + 32 * t] = v;
+                sum[t] += v;
+            }
+            if (row < n && lane == 0) znorm[row] = s[r] > 0.f ? amax[r] * rs : 0.f;
         }
-        if (lane == 0) znorm[row] = nrm;
     }
 #pragma unroll
-    for (int t = 0; t < kMaxPerLane; ++t) part[warp][lane + 32 * t] = sum[t];
+    for (int t = 0; t < T; ++t) part[warp][lane + 32 * t] = sum[t];
     __syncthreads();
     if (threadIdx.x < ell) {
         float s = 0.f;
@@ -103,8 +125,19 @@ __global__ void __launch_bounds__(1024) k_accumulate(const float* __restrict__ p
     const int G = 1024 / jw;
     const int j = threadIdx.x % jw, g = threadIdx.x / jw;
     double s = 0.0;
-    if (j < ell)
-        for (int b = g; b < nblocks; b += G) s += (double)partials[(int64_t)b * ell + j];
+    chain_wait();
+    chain_release();
+    if (j < ell) {
+        int b = g;
+        for (; b + 7 * G < nblocks; b += 8 * G) {           // eight loads in flight, added in order
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = partials[(int64_t)(b + u * G) * ell + j];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) s += (double)v[u];
+        }
+        for (; b < nblocks; b += G) s += (double)partials[(int64_t)b * ell + j];
+    }
     sh[threadIdx.x] = s;
     __syncthreads();
     if (g == 0 && j < ell) {
@@ -114,13 +147,17 @@ __global__ void __launch_bounds__(1024) k_accumulate(const float* __restrict__ p
     }
 }
 
-// u = zsum/||zsum|| (the 1/N of the mean cancels); alpha_i = <zhat_i, u>. One warp per row.
+// u = zsum/||zsum|| (the 1/N of the mean cancels); alpha_i = <zhat_i, u>. One warp per row, four rows of a warp in flight; a warp
+// takes more rows when there are many (every block forms u for itself).
+template <int T>
 __global__ void __launch_bounds__(256) k_consensus_score(const double* __restrict__ zsum, const float* __restrict__ zhat,
                                                          int64_t N, int ell, float* __restrict__ u_out,
                                                          float* __restrict__ scores) {
     __shared__ float u[256];
     __shared__ double red[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    chain_wait();
+    chain_release();
     double v = (tid < ell) ? zsum[tid] : 0.0;
     double sq = v * v;
 #pragma unroll
@@ -134,13 +171,29 @@ __global__ void __launch_bounds__(256) k_consensus_score(const double* __restric
     u[tid] = (nrm > 0.0 && tid < ell) ? (float)(v / nrm) : 0.f;
     if (blockIdx.x == 0 && tid < ell) u_out[tid] = u[tid];
     __syncthreads();
-    const int64_t row = (int64_t)blockIdx.x * 8 + warp;
-    if (row >= N) return;
-    float acc = 0.f;
-    for (int j = lane; j < ell; j += 32) acc = fmaf(zhat[row * ell + j], u[j], acc);
+    float uu[T];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) scores[row] = fminf(1.f, fmaxf(-1.f, acc));
+    for (int t = 0; t < T; ++t) uu[t] = u[lane + 32 * t];
+    constexpr int RB = T > 4 ? 2 : 4;
+    const int64_t stride = (int64_t)gridDim.x * 8;
+    for (int64_t r0 = (int64_t)blockIdx.x * 8 + warp; r0 < N; r0 += RB * stride) {
+        float acc[RB];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            const int64_t row = r0 + r * stride;
+            acc[r] = 0.f;
+#pragma unroll
+            for (int t = 0; t < T; ++t)
+                if (row < N && lane + 32 * t < ell) acc[r] = fmaf(zhat[row * ell + lane + 32 * t], uu[t], acc[r]);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int r = 0; r < RB; ++r) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
+#pragma unroll
+        for (int r = 0; r < RB; ++r)
+            if (lane == 0 && r0 + r * stride < N) scores[r0 + r * stride] = fminf(1.f, fmaxf(-1.f, acc[r]));
+    }
 }
 
 
@@ -223,13 +276,12 @@ cudaError_t launch_normalise(const float* Z, int planes, int64_t plane_stride, i
                              float* znorm, float* partials, double* zsum, unsigned* flags, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     const int nblocks = (int)((n + kRowsPerBlock - 1) / kRowsPerBlock);
-    k_normalise<<<nblocks, 256, 0, st>>>(Z, planes, plane_stride, ldz, n, ell, zhat, znorm, partials, flags);
-    cudaError_t e = cudaGetLastError();
+    auto run = [&](auto kernel) { return launch_chained(kernel, dim3(nblocks), dim3(256), 0, st, Z, planes, plane_stride, ldz, n, ell, zhat, znorm, partials, flags); };
+    const cudaError_t e = ell <= 32 ? run(k_normalise<1>) : ell <= 64 ? run(k_normalise<2>) : ell <= 128 ? run(k_normalise<4>) : run(k_normalise<8>);
     if (e != cudaSuccess || !zsum) return e;
     int jw = 32;
     while (jw < ell) jw <<= 1;
-    k_accumulate<<<1, 1024, 0, st>>>(partials, nblocks, ell, jw, zsum);
-    return cudaGetLastError();
+    return launch_chained(k_accumulate, dim3(1), dim3(1024), 0, st, partials, nblocks, ell, jw, zsum);
 }
 
 cudaError_t launch_outer_combine(const void* q, int64_t ldq, sage_dtype_t dt, int C, const float* planes, int pp, int64_t plane_stride,
@@ -262,9 +314,10 @@ cudaError_t launch_outer_combine(const void* q, int64_t ldq, sage_dtype_t dt, in
 
 cudaError_t launch_consensus_score(const double* zsum, const float* zhat, int64_t N, int ell, float* u, float* scores,
                                    cudaStream_t st) {
-    const int64_t blocks = N > 0 ? (N + 7) / 8 : 1;
-    k_consensus_score<<<(unsigned)blocks, 256, 0, st>>>(zsum, zhat, N, ell, u, scores);
-    return cudaGetLastError();
+    int64_t blocks = N > 0 ? (N + 7) / 8 : 1;
+    if (blocks > 148 * 8) blocks = 148 * 8;                 // one wave: 8 blocks of 256 threads per SM
+    auto run = [&](auto kernel) { return launch_chained(kernel, dim3((unsigned)blocks), dim3(256), 0, st, zsum, zhat, N, ell, u, scores); };
+    return ell <= 32 ? run(k_consensus_score<1>) : ell <= 64 ? run(k_consensus_score<2>) : ell <= 128 ? run(k_consensus_score<4>) : run(k_consensus_score<8>);
 }
 
 }  // namespace sage

@@ -207,20 +207,57 @@ __global__ void __launch_bounds__(256) k_split_tf32(const float* __restrict__ sr
     }
 }
 
-// mirror != 0 (a symmetric matrix of which only the 128 x 128 tiles on and above the diagonal were computed): elements of
-// the tiles below the diagonal are read from their mirror image.
 __global__ void __launch_bounds__(256) k_split_reduce(const float* __restrict__ parts, int splits, int64_t split_stride,
-                                                      int M, int N, int64_t ldp, float* __restrict__ out, int64_t ldo, int mirror) {
-    chain_release();                        // the next kernel of a shrink is one small block
+                                                      int M, int N, int64_t ldp, float* __restrict__ out, int64_t ldo) {
+    chain_release();
     chain_wait();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)M * N) return;
     const int i = (int)(e / N), j = (int)(e % N);
-    const bool below = mirror && (i >> 7) > (j >> 7);
-    const float* src = parts + (below ? (int64_t)j * ldp + i : (int64_t)i * ldp + j);
+    const float* src = parts + (int64_t)i * ldp + j;
     double s = 0.0;
-    for (int z = 0; z < splits; ++z) s += (double)src[(int64_t)z * split_stride];
+    int z = 0;
+    for (; z + 8 <= splits; z += 8) {                       // eight loads in flight, added in order
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = src[(int64_t)(z + u) * split_stride];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s += (double)v[u];
+    }
+    for (; z < splits; ++z) s += (double)src[(int64_t)z * split_stride];
     out[(int64_t)i * ldo + j] = (float)s;
+}
+
+// The same for a symmetric r x r matrix of which only the 128 x 128 tiles on and above the diagonal were computed. Block: 32 x 32
+// outputs of the upper part, the slices dealt to four layers of threads (the kernel is bound by load latency), written twice, the mirror
+// image through shared memory.
+__global__ void __launch_bounds__(1024) k_split_reduce_sym(const float* __restrict__ parts, int splits, int64_t split_stride, int r, int64_t ldp,
+                                                           float* __restrict__ out, int64_t ldo) {
+    __shared__ double sh[4][32][33];
+    if (blockIdx.y > blockIdx.x) return;
+    chain_release();                        // the next kernel of a shrink is one small block
+    chain_wait();
+    const int tx = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;       // 32 x 8 x 4
+    const int j = blockIdx.x * 32 + tx;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    const int64_t o = (int64_t)(blockIdx.y * 32 + ty) * ldp + j;
+#pragma unroll 2
+    for (int z = tz; z < splits; z += 4)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (blockIdx.y * 32 + ty + 8 * u < r && j < r) a[u] += (double)parts[(int64_t)z * split_stride + o + (int64_t)(8 * u) * ldp];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) sh[tz][ty + 8 * u][tx] = a[u];
+    __syncthreads();
+    const int row = tz * 8 + ty;                                          // 32 rows x 32 columns, one output per thread
+    const int i = blockIdx.y * 32 + row;
+    const double s = (sh[0][row][tx] + sh[1][row][tx]) + (sh[2][row][tx] + sh[3][row][tx]);
+    if (i < r && j < r) out[(int64_t)i * ldo + j] = (float)s;
+    if (blockIdx.x != blockIdx.y) {
+        const double m = (sh[0][tx][row] + sh[1][tx][row]) + (sh[2][tx][row] + sh[3][tx][row]);
+        const int mi = blockIdx.x * 32 + row, mj = blockIdx.y * 32 + tx;
+        if (mi < r && mj < r) out[(int64_t)mi * ldo + mj] = (float)m;
+    }
 }
 
 // Split reduction of a Gram matrix computed in the symmetric form: slice z left T_z = hi*hi^T + 2*hi*lo^T at
@@ -388,7 +425,8 @@ cudaError_t launch_split_reduce(const float* parts, int splits, int64_t split_st
                                 int64_t ldo, cudaStream_t st, int mirror) {
     const int64_t total = (int64_t)M * N;
     if (total <= 0) return cudaSuccess;
-    return launch_chained(k_split_reduce, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, parts, splits, split_stride, M, N, ldp, out, ldo, mirror);
+    if (mirror) return launch_chained(k_split_reduce_sym, dim3((N + 31) / 32, (N + 31) / 32), dim3(32, 8, 4), 0, st, parts, splits, split_stride, N, ldp, out, ldo);
+    return launch_chained(k_split_reduce, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, parts, splits, split_stride, M, N, ldp, out, ldo);
 }
 
 cudaError_t launch_gram_sym_reduce(const float* parts, int splits, int64_t stride, int r, int64_t ldp, float* out, int64_t ldo,
