@@ -222,6 +222,8 @@ sage_status_t sage_select_static(const float* scores, int64_t N, double keep_rat
 /* The whole path for rows that live in HOST memory (pinned memory gives overlap of copies and
  * kernels): streams the rows to the device in chunks for pass 1, freezes, streams them again for
  * pass 2, selects, and copies scores (N floats, may be NULL) and indices back to the host.
+ * Rows that fit the staging memory (chunk_rows of them, by default 512 MB) stay on the device and cross the bus once.
+ * Device memory comes from a pool of the library's own that keeps up to 1 GiB for the next call.
  * Synchronous. chunk_rows <= 0 picks a default. */
 sage_status_t sage_select_from_host(const void* rows_host, int64_t N, int64_t D, int64_t ld, int32_t ell,
                                     sage_dtype_t row_dtype, double keep_rate, int64_t chunk_rows, int device,

@@ -93,9 +93,11 @@ struct Prof {
 
 size_t elem_size(sage_dtype_t dt) { return dt == SAGE_F32 ? 4 : 2; }
 
-// Stream-ordered scratch of the selection entry points comes from a pool of the library's own whose memory stays
-// cached across synchronisations (the device's default pool gives its memory back at every synchronisation, and
-// getting it again costs milliseconds). One pool per device, created on first use, kept until the process exits.
+// Stream-ordered scratch of the selection entry points, and all memory of a sage_select_from_host call, comes from a pool of
+// the library's own that keeps up to kPoolKeep bytes across synchronisations and gives the rest back (the device's default pool
+// gives everything back at every synchronisation, and getting it again costs milliseconds). One pool per device, created on first
+// use, kept until the process exits.
+constexpr unsigned long long kPoolKeep = 1ull << 30;
 cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
     static cudaMemPool_t pools[64] = {};
     static std::mutex mu;
@@ -114,7 +116,7 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
             cudaMemPool_t pool = nullptr;
             e = cudaMemPoolCreate(&pool, &props);
             if (e != cudaSuccess) return e;
-            unsigned long long keep = ~0ull;
+            unsigned long long keep = kPoolKeep;
             e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
             if (e != cudaSuccess) return e;
             pools[dev] = pool;
@@ -154,6 +156,8 @@ struct RowSrc {
 }  // namespace
 
 struct sage_fd {
+    bool pooled = false;           // a handle that lives for one call: its memory comes from the library's pool, ordered on pool_stream
+    cudaStream_t pool_stream = nullptr;
     int64_t D = 0;
     int ell = 0, m = 0;
     sage_dtype_t dtype = SAGE_F32;
@@ -393,12 +397,20 @@ sage_status_t enqueue_factor(sage_fd* h, int r, int do_shrink, int keep, int zer
     return SAGE_OK;
 }
 
-sage_status_t ensure(float** p, size_t* have, size_t need) {
+cudaError_t dev_malloc(const sage_fd* h, void** p, size_t bytes) {
+    return h->pooled ? scratch_alloc(p, bytes, h->pool_stream) : cudaMalloc(p, bytes);
+}
+cudaError_t dev_free(const sage_fd* h, void* p) {
+    if (!p) return cudaSuccess;
+    return h->pooled ? cudaFreeAsync(p, h->pool_stream) : cudaFree(p);
+}
+
+sage_status_t ensure(const sage_fd* h, float** p, size_t* have, size_t need) {
     if (*have >= need) return SAGE_OK;
-    if (*p) CU_TRY(cudaFree(*p));
+    if (*p) CU_TRY(dev_free(h, *p));
     *p = nullptr;
     *have = 0;
-    CU_TRY(cudaMalloc(reinterpret_cast<void**>(p), need));
+    CU_TRY(dev_malloc(h, reinterpret_cast<void**>(p), need));
     *have = need;
     return SAGE_OK;
 }
@@ -472,7 +484,8 @@ static void drop_cycles(sage_fd* s) {
     for (sage_fd* k : s->kids) drop_cycles(k);
 }
 
-static sage_status_t create_handle(sage_fd_t** out, int64_t D, int32_t ell, sage_dtype_t row_dtype, int device, bool sketch_only) {
+static sage_status_t create_handle(sage_fd_t** out, int64_t D, int32_t ell, sage_dtype_t row_dtype, int device, bool sketch_only,
+                                   bool pooled = false, cudaStream_t pool_stream = nullptr) {
     if (!out || D < 1 || (row_dtype != SAGE_F32 && row_dtype != SAGE_BF16) || device < 0) {
         set_err("sage_fd_create: bad argument (out=%p D=%lld dtype=%d device=%d)", (void*)out, (long long)D, (int)row_dtype, device);
         return SAGE_ERR_INVALID_ARG;
@@ -488,6 +501,8 @@ static sage_status_t create_handle(sage_fd_t** out, int64_t D, int32_t ell, sage
     }
     sage_fd* h = new (std::nothrow) sage_fd();
     if (!h) return SAGE_ERR_ALLOC;
+    h->pooled = pooled;
+    h->pool_stream = pool_stream;
     h->D = D;
     h->ell = ell;
     h->m = 2 * ell;
@@ -507,48 +522,48 @@ static sage_status_t create_handle(sage_fd_t** out, int64_t D, int32_t ell, sage
     };
     cudaError_t e;
     for (int i = 0; i < 2; ++i)
-        if ((e = cudaMalloc((void**)&h->B[i], bbytes)) != cudaSuccess) return fail(e, "cudaMalloc(buffer)");
+        if ((e = dev_malloc(h, (void**)&h->B[i], bbytes)) != cudaSuccess) return fail(e, "cudaMalloc(buffer)");
     h->gram_part_floats = kGramPartFloats;
     if ((size_t)16 * h->m * h->m > h->gram_part_floats) h->gram_part_floats = (size_t)16 * h->m * h->m;
-    if ((e = cudaMalloc((void**)&h->gram_parts, h->gram_part_floats * sizeof(float))) != cudaSuccess) return fail(e, "cudaMalloc(gram)");
+    if ((e = dev_malloc(h, (void**)&h->gram_parts, h->gram_part_floats * sizeof(float))) != cudaSuccess) return fail(e, "cudaMalloc(gram)");
     h->wsplit_ld = h->m <= 256 ? 256 : 512;
-    if ((e = cudaMalloc((void**)&h->Wsplit, (size_t)h->wsplit_ld * h->wsplit_ld * sizeof(float))) != cudaSuccess)
+    if ((e = dev_malloc(h, (void**)&h->Wsplit, (size_t)h->wsplit_ld * h->wsplit_ld * sizeof(float))) != cudaSuccess)
         return fail(e, "cudaMalloc(W)");
     // rows of the split factors beyond the ones an eigen-solve writes are read by the rebuild's MMA (and ignored by its
     // epilogue): they must hold finite values
-    if ((e = cudaMemset(h->Wsplit, 0, (size_t)h->wsplit_ld * h->wsplit_ld * sizeof(float))) != cudaSuccess) return fail(e, "cudaMemset");
-    if ((e = cudaMalloc((void**)&h->Kmat, mm)) != cudaSuccess) return fail(e, "cudaMalloc(K)");
-    if ((e = cudaMalloc((void**)&h->Ur, mm)) != cudaSuccess) return fail(e, "cudaMalloc(U)");
-    if ((e = cudaMalloc((void**)&h->eig_work, eig_work_floats(h->m) * sizeof(float))) != cudaSuccess)
+    if ((e = cudaMemsetAsync(h->Wsplit, 0, (size_t)h->wsplit_ld * h->wsplit_ld * sizeof(float), pool_stream)) != cudaSuccess) return fail(e, "cudaMemset");
+    if ((e = dev_malloc(h, (void**)&h->Kmat, mm)) != cudaSuccess) return fail(e, "cudaMalloc(K)");
+    if ((e = dev_malloc(h, (void**)&h->Ur, mm)) != cudaSuccess) return fail(e, "cudaMalloc(U)");
+    if ((e = dev_malloc(h, (void**)&h->eig_work, eig_work_floats(h->m) * sizeof(float))) != cudaSuccess)
         return fail(e, "cudaMalloc(eig)");
-    if ((e = cudaMalloc((void**)&h->sigma, ell * sizeof(float))) != cudaSuccess) return fail(e, "cudaMalloc(sigma)");
-    if ((e = cudaMalloc((void**)&h->info, sizeof(EigInfo))) != cudaSuccess) return fail(e, "cudaMalloc(info)");
+    if ((e = dev_malloc(h, (void**)&h->sigma, ell * sizeof(float))) != cudaSuccess) return fail(e, "cudaMalloc(sigma)");
+    if ((e = dev_malloc(h, (void**)&h->info, sizeof(EigInfo))) != cudaSuccess) return fail(e, "cudaMalloc(info)");
     if (!sketch_only) {
-        if ((e = cudaMalloc((void**)&h->zsum, 256 * sizeof(double))) != cudaSuccess) return fail(e, "cudaMalloc(zsum)");
-        if ((e = cudaMalloc((void**)&h->u, 256 * sizeof(float))) != cudaSuccess) return fail(e, "cudaMalloc(u)");
+        if ((e = dev_malloc(h, (void**)&h->zsum, 256 * sizeof(double))) != cudaSuccess) return fail(e, "cudaMalloc(zsum)");
+        if ((e = dev_malloc(h, (void**)&h->u, 256 * sizeof(float))) != cudaSuccess) return fail(e, "cudaMalloc(u)");
     }
-    if ((e = cudaMalloc((void**)&h->tc_err, sizeof(int))) != cudaSuccess) return fail(e, "cudaMalloc(err)");
+    if ((e = dev_malloc(h, (void**)&h->tc_err, sizeof(int))) != cudaSuccess) return fail(e, "cudaMalloc(err)");
     if ((e = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking)) != cudaSuccess) return fail(e, "cudaStreamCreate");
     for (cudaEvent_t* ev : {&h->ev_fork, &h->ev_join, &h->ev_in, &h->ev_rows, &h->ev_done})
         if ((e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming)) != cudaSuccess) return fail(e, "cudaEventCreate");
-    if ((e = cudaMemset(h->tc_err, 0, sizeof(int))) != cudaSuccess) return fail(e, "cudaMemset");
+    if ((e = cudaMemsetAsync(h->tc_err, 0, sizeof(int), pool_stream)) != cudaSuccess) return fail(e, "cudaMemset");
     if (row_dtype == SAGE_BF16 && !sketch_only) {
         // Two-term bf16 sketch (16 significant bits) for short rows, where the rounding errors of a one-term
         // sketch would average over too few terms; long rows take the one-term sketch (half the operand traffic).
         h->p16_npad = ((ell + 15) / 16) * 16;
         h->p16_fold = (2 * h->p16_npad <= 256 && D < 16384) ? 1 : 0;
         const size_t prow = h->p16_fold ? 2 * (size_t)h->p16_npad : (size_t)ell;
-        if ((e = cudaMalloc((void**)&h->P16, prow * h->pitch * sizeof(__nv_bfloat16))) != cudaSuccess) return fail(e, "cudaMalloc(P16)");
-        if ((e = cudaMemset(h->P16, 0, prow * h->pitch * sizeof(__nv_bfloat16))) != cudaSuccess) return fail(e, "cudaMemset");
+        if ((e = dev_malloc(h, (void**)&h->P16, prow * h->pitch * sizeof(__nv_bfloat16))) != cudaSuccess) return fail(e, "cudaMalloc(P16)");
+        if ((e = cudaMemsetAsync(h->P16, 0, prow * h->pitch * sizeof(__nv_bfloat16), pool_stream)) != cudaSuccess) return fail(e, "cudaMemset");
     }
     if (row_dtype == SAGE_F32 && ell <= 64 && !sketch_only) {
         // fp32 rows, small sketch: the projection multiplies the rows against the sketch pre-split into tf32 hi / lo rows
-        if ((e = cudaMalloc((void**)&h->S32split, (size_t)128 * h->pitch * sizeof(float))) != cudaSuccess) return fail(e, "cudaMalloc(S split)");
-        if ((e = cudaMemset(h->S32split, 0, (size_t)128 * h->pitch * sizeof(float))) != cudaSuccess) return fail(e, "cudaMemset");
+        if ((e = dev_malloc(h, (void**)&h->S32split, (size_t)128 * h->pitch * sizeof(float))) != cudaSuccess) return fail(e, "cudaMalloc(S split)");
+        if ((e = cudaMemsetAsync(h->S32split, 0, (size_t)128 * h->pitch * sizeof(float), pool_stream)) != cudaSuccess) return fail(e, "cudaMemset");
     }
-    if ((e = cudaMemset(h->info, 0, sizeof(EigInfo))) != cudaSuccess) return fail(e, "cudaMemset");
-    if ((e = cudaMemset(h->sigma, 0, ell * sizeof(float))) != cudaSuccess) return fail(e, "cudaMemset");
-    if ((e = cudaDeviceSynchronize()) != cudaSuccess) return fail(e, "cudaDeviceSynchronize");
+    if ((e = cudaMemsetAsync(h->info, 0, sizeof(EigInfo), pool_stream)) != cudaSuccess) return fail(e, "cudaMemset");
+    if ((e = cudaMemsetAsync(h->sigma, 0, ell * sizeof(float), pool_stream)) != cudaSuccess) return fail(e, "cudaMemset");
+    if (!pooled && (e = cudaDeviceSynchronize()) != cudaSuccess) return fail(e, "cudaDeviceSynchronize");
     *out = h;
     return SAGE_OK;
 }
@@ -567,28 +582,9 @@ void sage_fd_destroy(sage_fd_t* h) {
     if (h->chain) cudaStreamDestroy(h->chain);
     for (cudaEvent_t ev : {h->ev_in, h->ev_rows, h->ev_done})
         if (ev) cudaEventDestroy(ev);
-    cudaFree(h->B[0]);
-    cudaFree(h->B[1]);
-    cudaFree(h->gram_parts);
-    cudaFree(h->Wsplit);
-    cudaFree(h->Kmat);
-    cudaFree(h->Ur);
-    cudaFree(h->eig_work);
-    cudaFree(h->sigma);
-    cudaFree(h->info);
-    cudaFree(h->zhat);
-    cudaFree(h->znorm);
-    cudaFree(h->zwork);
-    cudaFree(h->partials);
-    cudaFree(h->zred);
-    cudaFree(h->bias_t);
-    cudaFree(h->zsum);
-    cudaFree(h->u);
-    cudaFree(h->class_U);
-    cudaFree(h->class_counts);
-    cudaFree(h->P16);
-    cudaFree(h->S32split);
-    cudaFree(h->tc_err);
+    void* memory[] = {h->B[0], h->B[1], h->gram_parts, h->Wsplit, h->Kmat, h->Ur, h->eig_work, h->sigma, h->info, h->zhat, h->znorm, h->zwork,
+                      h->partials, h->zred, h->bias_t, h->zsum, h->u, h->class_U, h->class_counts, h->P16, h->S32split, h->tc_err};
+    for (void* p : memory) dev_free(h, p);
     if (h->side) cudaStreamDestroy(h->side);
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
@@ -1152,12 +1148,12 @@ sage_status_t sage_score_begin(sage_fd_t* h, int64_t N_total, void* cuda_stream)
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if (!h->strict && N_total > h->zcap) {
         CU_TRY(cudaStreamSynchronize(st));
-        if (h->zhat) CU_TRY(cudaFree(h->zhat));
-        if (h->znorm) CU_TRY(cudaFree(h->znorm));
+        if (h->zhat) CU_TRY(dev_free(h, h->zhat));
+        if (h->znorm) CU_TRY(dev_free(h, h->znorm));
         h->zhat = h->znorm = nullptr;
         h->zcap = 0;
-        CU_TRY(cudaMalloc((void**)&h->zhat, (size_t)N_total * h->ell * sizeof(float)));
-        CU_TRY(cudaMalloc((void**)&h->znorm, (size_t)N_total * sizeof(float)));
+        CU_TRY(dev_malloc(h, (void**)&h->zhat, (size_t)N_total * h->ell * sizeof(float)));
+        CU_TRY(dev_malloc(h, (void**)&h->znorm, (size_t)N_total * sizeof(float)));
         h->zcap = N_total;
     }
     CU_TRY(cudaMemsetAsync(h->zsum, 0, 256 * sizeof(double), st));
@@ -1217,15 +1213,15 @@ static sage_status_t score_rows(sage_fd* h, const void* rows, sage_dtype_t dt, i
     for (int64_t r0 = 0; r0 < n; r0 += sub_max) {
         const int64_t sub = (n - r0 < sub_max) ? n - r0 : sub_max;
         const size_t nb = (size_t)((sub + 63) / 64);
-        ST_TRY(ensure(&h->partials, &h->partials_bytes, nb * ell * sizeof(float)));
+        ST_TRY(ensure(h, &h->partials, &h->partials_bytes, nb * ell * sizeof(float)));
         if (store_at < 0 && sub > h->zcap) {         // strict-memory mode: normalised projections of one sub-chunk only
             CU_TRY(cudaStreamSynchronize(st));
-            if (h->zhat) CU_TRY(cudaFree(h->zhat));
-            if (h->znorm) CU_TRY(cudaFree(h->znorm));
+            if (h->zhat) CU_TRY(dev_free(h, h->zhat));
+            if (h->znorm) CU_TRY(dev_free(h, h->znorm));
             h->zhat = h->znorm = nullptr;
             h->zcap = 0;
-            CU_TRY(cudaMalloc((void**)&h->zhat, (size_t)sub * ell * sizeof(float)));
-            CU_TRY(cudaMalloc((void**)&h->znorm, (size_t)sub * sizeof(float)));
+            CU_TRY(dev_malloc(h, (void**)&h->zhat, (size_t)sub * ell * sizeof(float)));
+            CU_TRY(dev_malloc(h, (void**)&h->znorm, (size_t)sub * sizeof(float)));
             h->zcap = sub;
         }
         const size_t zred = (size_t)sub * ell * sizeof(float);
@@ -1237,7 +1233,7 @@ static sage_status_t score_rows(sage_fd* h, const void* rows, sage_dtype_t dt, i
             // sketches of at most 64 rows: one wide MMA per K step against the pre-split sketch, two partial planes per K slice
             const bool wide = h->S32split != nullptr;
             const int planes = wide ? 2 * splits : splits;
-            ST_TRY(ensure(&h->zwork, &h->zwork_bytes, zred * planes));
+            ST_TRY(ensure(h, &h->zwork, &h->zwork_bytes, zred * planes));
             float* out = h->zwork;
             cudaError_t e = timed(h, K_PROJECT, 1, st, [&] {
                 return launch_tc_gemm_nt_x3(reinterpret_cast<const float*>(p + r0 * row_bytes), ld, wide ? h->S32split : S, h->pitch, (int)sub,
@@ -1265,7 +1261,7 @@ static sage_status_t score_rows(sage_fd* h, const void* rows, sage_dtype_t dt, i
             const int64_t slices_at_least = structured ? oC : (K / 4096 > 0 ? K / 4096 : 1);
             while (mt > 1 && (int64_t)((tiles + mt - 1) / mt) * slices_at_least < 148) mt >>= 1;
             const int splits = structured ? oC : pick_splits_waves((tiles + mt - 1) / mt, K, 4096, 148);
-            ST_TRY(ensure(&h->zwork, &h->zwork_bytes, zred * splits));
+            ST_TRY(ensure(h, &h->zwork, &h->zwork_bytes, zred * splits));
             float* out = h->zwork;
             cudaError_t e = timed(h, K_PROJECT, 1, st, [&] {
                 return launch_tc_gemm_nt(p + r0 * row_bytes, SAGE_BF16, ld, h->P16, h->pitch, (int)sub, ell, h->p16_fold, mt, K, splits,
@@ -1285,7 +1281,7 @@ static sage_status_t score_rows(sage_fd* h, const void* rows, sage_dtype_t dt, i
         if (!done) {
             const int tiles = (int)((sub + 63) / 64) * ((ell + 63) / 64);
             const int splits = structured ? oC : pick_splits(tiles, K, 1024);
-            ST_TRY(ensure(&h->zwork, &h->zwork_bytes, zred * splits));
+            ST_TRY(ensure(h, &h->zwork, &h->zwork_bytes, zred * splits));
             CU_TRY(timed(h, K_PROJECT, 1, st, [&] {
                 return launch_gemm_nt(p + r0 * row_bytes, dt, ld, S, h->pitch, (int)sub, ell, K, splits, h->zwork, ell,
                                       (int64_t)sub * ell, st, class_F);
@@ -1295,11 +1291,11 @@ static sage_status_t score_rows(sage_fd* h, const void* rows, sage_dtype_t dt, i
         }
         if (structured) {
             // z = sum_c q_c (T_c + bias column c), classes in ascending order
-            ST_TRY(ensure(&h->zred, &h->zred_bytes, zred));
+            ST_TRY(ensure(h, &h->zred, &h->zred_bytes, zred));
             const float* parts = Zparts;
             const int pp = nplanes / oC;
             const char* qsub = static_cast<const char*>(oq) + (size_t)r0 * oldq * elem_size(dt);
-            ST_TRY(ensure(&h->bias_t, &h->bias_t_bytes, (size_t)oC * ell * sizeof(float)));
+            ST_TRY(ensure(h, &h->bias_t, &h->bias_t_bytes, (size_t)oC * ell * sizeof(float)));
             CU_TRY(timed(h, K_PROJECT_REDUCE, 2, st, [&] {
                 return launch_outer_combine(qsub, oldq, dt, oC, parts, pp, (int64_t)sub * ell, S + K, h->pitch, h->bias_t, sub, ell, h->zred, st);
             }));
@@ -1309,7 +1305,7 @@ static sage_status_t score_rows(sage_fd* h, const void* rows, sage_dtype_t dt, i
         // Many K slices (few rows per launch, as in the 512-row chunks of very long rows): summed first by a kernel with a
         // thread per element; the normalise kernel has a warp per row and would walk the slices one after the other.
         if (nplanes > 4) {
-            ST_TRY(ensure(&h->zred, &h->zred_bytes, zred));
+            ST_TRY(ensure(h, &h->zred, &h->zred_bytes, zred));
             const float* parts = Zparts;
             const int np = nplanes;
             CU_TRY(timed(h, K_PROJECT_REDUCE, 1, st,
@@ -1503,13 +1499,13 @@ sage_status_t sage_score_classes(sage_fd_t* h, const int32_t* labels, int32_t nu
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if (num_classes > h->class_cap) {
         CU_TRY(cudaStreamSynchronize(st));
-        if (h->class_U) CU_TRY(cudaFree(h->class_U));
-        if (h->class_counts) CU_TRY(cudaFree(h->class_counts));
+        if (h->class_U) CU_TRY(dev_free(h, h->class_U));
+        if (h->class_counts) CU_TRY(dev_free(h, h->class_counts));
         h->class_U = nullptr;
         h->class_counts = nullptr;
         h->class_cap = 0;
-        CU_TRY(cudaMalloc((void**)&h->class_U, (size_t)num_classes * h->ell * sizeof(float)));
-        CU_TRY(cudaMalloc((void**)&h->class_counts, (size_t)num_classes * sizeof(int)));
+        CU_TRY(dev_malloc(h, (void**)&h->class_U, (size_t)num_classes * h->ell * sizeof(float)));
+        CU_TRY(dev_malloc(h, (void**)&h->class_counts, (size_t)num_classes * sizeof(int)));
         h->class_cap = num_classes;
     }
     h->class_num = num_classes;
@@ -1864,32 +1860,45 @@ sage_status_t sage_select_from_host(const void* rows_host, int64_t N, int64_t D,
         set_err("sage_select_from_host: null idx_host");
         return SAGE_ERR_INVALID_ARG;
     }
-    sage_fd_t* h = nullptr;
-    ST_TRY(sage_fd_create(&h, D, ell, row_dtype, device));
     DeviceGuard g(device);
-    const size_t es = elem_size(row_dtype);
+    if (!g.ok) {
+        set_err("sage_select_from_host: cannot select CUDA device %d: %s", device, cudaGetErrorString(cudaGetLastError()));
+        return SAGE_ERR_CUDA;
+    }
+    const size_t es = elem_size(row_dtype), row_bytes = (size_t)ld * es;
+    constexpr size_t kStage = (size_t)256 << 20;                         // bytes of a staging buffer by default
+    // Rows that fit the two staging buffers stay on the device: they cross the bus once, in pieces so that the sketch starts
+    // with the first one, and pass 2 takes them as they are. (The caller's chunk_rows sets the memory where it asks for less.)
+    const bool resident = chunk_rows >= N || (chunk_rows <= 0 && (size_t)N * row_bytes <= 2 * kStage);
     if (chunk_rows <= 0) {
-        chunk_rows = (int64_t)((256ull << 20) / ((size_t)ld * es));     // about 256 MB per staging buffer
+        chunk_rows = (int64_t)(kStage / row_bytes);
+        if (resident) chunk_rows = (N + 7) / 8;
         if (chunk_rows < 2 * ell) chunk_rows = 2 * ell;
     }
     if (chunk_rows > N) chunk_rows = N;
-    const size_t chunk_bytes = (size_t)chunk_rows * ld * es;
+    const int nstage = resident ? 1 : 2;
+    const size_t stage_bytes = (size_t)(resident ? N : chunk_rows) * row_bytes;
+    sage_fd_t* h = nullptr;
     void* stage[2] = {nullptr, nullptr};
     float* d_scores = nullptr;
     int64_t* d_idx = nullptr;
     cudaStream_t s_copy = nullptr, s_comp = nullptr;
-    cudaEvent_t copied[2] = {nullptr, nullptr}, consumed[2] = {nullptr, nullptr};
+    cudaEvent_t copied[2] = {nullptr, nullptr}, consumed[2] = {nullptr, nullptr}, ready = nullptr;
     sage_status_t rc = SAGE_OK;
     auto body = [&]() -> sage_status_t {
         CU_TRY(cudaStreamCreateWithFlags(&s_copy, cudaStreamNonBlocking));
         CU_TRY(cudaStreamCreateWithFlags(&s_comp, cudaStreamNonBlocking));
+        CU_TRY(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
         for (int i = 0; i < 2; ++i) {
-            CU_TRY(cudaMalloc(&stage[i], chunk_bytes));
+            if (i < nstage) CU_TRY(scratch_alloc(&stage[i], stage_bytes, s_comp));
             CU_TRY(cudaEventCreateWithFlags(&copied[i], cudaEventDisableTiming));
             CU_TRY(cudaEventCreateWithFlags(&consumed[i], cudaEventDisableTiming));
         }
-        CU_TRY(cudaMalloc((void**)&d_scores, (size_t)N * sizeof(float)));
-        if (k > 0) CU_TRY(cudaMalloc((void**)&d_idx, (size_t)k * sizeof(int64_t)));
+        CU_TRY(cudaEventRecord(ready, s_comp));                          // the staging memory is this call's from here on
+        CU_TRY(cudaStreamWaitEvent(s_copy, ready, 0));
+        ST_TRY(create_handle(&h, D, ell, row_dtype, device, false, true, s_comp));
+        CU_TRY(scratch_alloc((void**)&d_scores, (size_t)N * sizeof(float), s_comp));
+        if (k > 0) CU_TRY(scratch_alloc((void**)&d_idx, (size_t)k * sizeof(int64_t), s_comp));
         const char* src = static_cast<const char*>(rows_host);
         for (int pass = 0; pass < 2; ++pass) {
             if (pass == 1) {
@@ -1897,20 +1906,25 @@ sage_status_t sage_select_from_host(const void* rows_host, int64_t N, int64_t D,
                 if (f != SAGE_OK && f != SAGE_ERR_NOT_CONVERGED && f != SAGE_ERR_NONFINITE) return f;
                 if (f != SAGE_OK) rc = f;
                 ST_TRY(sage_score_begin(h, N, s_comp));
+                if (resident) {
+                    ST_TRY(sage_score_chunk(h, stage[0], N, ld, 0, s_comp));
+                    break;
+                }
             }
             int64_t c = 0;
             for (int64_t r0 = 0; r0 < N; r0 += chunk_rows, ++c) {
                 const int b = (int)(c & 1);
                 const int64_t n = (N - r0 < chunk_rows) ? N - r0 : chunk_rows;
-                if (c >= 2 || pass == 1) CU_TRY(cudaStreamWaitEvent(s_copy, consumed[b], 0));
-                CU_TRY(cudaMemcpyAsync(stage[b], src + (size_t)r0 * ld * es, (size_t)n * ld * es, cudaMemcpyHostToDevice, s_copy));
+                char* at = static_cast<char*>(resident ? stage[0] : stage[b]) + (resident ? (size_t)r0 * row_bytes : 0);
+                if (!resident && (c >= 2 || pass == 1)) CU_TRY(cudaStreamWaitEvent(s_copy, consumed[b], 0));
+                CU_TRY(cudaMemcpyAsync(at, src + (size_t)r0 * row_bytes, (size_t)n * row_bytes, cudaMemcpyHostToDevice, s_copy));
                 CU_TRY(cudaEventRecord(copied[b], s_copy));
                 CU_TRY(cudaStreamWaitEvent(s_comp, copied[b], 0));
                 if (pass == 0)
-                    ST_TRY(sage_fd_update(h, stage[b], n, ld, s_comp));
+                    ST_TRY(sage_fd_update(h, at, n, ld, s_comp));
                 else
-                    ST_TRY(sage_score_chunk(h, stage[b], n, ld, r0, s_comp));
-                CU_TRY(cudaEventRecord(consumed[b], s_comp));
+                    ST_TRY(sage_score_chunk(h, at, n, ld, r0, s_comp));
+                if (!resident) CU_TRY(cudaEventRecord(consumed[b], s_comp));
             }
         }
         ST_TRY(sage_score_end(h, d_scores, s_comp));
@@ -1938,15 +1952,16 @@ sage_status_t sage_select_from_host(const void* rows_host, int64_t N, int64_t D,
     sage_status_t s = body();
     cudaDeviceSynchronize();
     for (int i = 0; i < 2; ++i) {
-        cudaFree(stage[i]);
+        if (stage[i]) cudaFreeAsync(stage[i], s_comp);
         if (copied[i]) cudaEventDestroy(copied[i]);
         if (consumed[i]) cudaEventDestroy(consumed[i]);
     }
-    cudaFree(d_scores);
-    cudaFree(d_idx);
+    if (ready) cudaEventDestroy(ready);
+    if (d_scores) cudaFreeAsync(d_scores, s_comp);
+    if (d_idx) cudaFreeAsync(d_idx, s_comp);
+    sage_fd_destroy(h);
     if (s_copy) cudaStreamDestroy(s_copy);
     if (s_comp) cudaStreamDestroy(s_comp);
-    sage_fd_destroy(h);
     if (s != SAGE_OK) return s;
     if (k_out) *k_out = k;
     return rc;
