@@ -321,7 +321,11 @@ sage_status_t enqueue_gram(sage_fd* h, int r, cudaStream_t st) {
         const int sym = r <= 128 ? 1 : 0;    // one diagonal tile: one wide MMA per K step, transpose added in the reduction
         int cap = (int)(h->gram_part_floats / (size_t)stride);
         if (cap > 148) cap = 148;
-        const int splits = pick_splits_waves(t * (t + 1) / 2, h->D, 256, cap);   // only the tiles on and above the diagonal run
+        // Slices of 256 columns; short rows in up to 16 slices of 64 and more: the kernel is a chain of K tiles there, while many
+        // slices cost the reduction what they save (a cycle on rows of 257, 1,024, 3,001 values: 34.9 -> 32.8, 58.7 -> 56.6, 82.3 -> 81.3 us;
+        // slices of 64 throughout: 5,130 values 107.9 -> 108.8, 20,000 values 113.7 -> 118.2 us)
+        const int64_t min_k = t > 1 || h->D >= 4096 ? 256 : h->D >= 1024 ? (h->D + 15) / 16 : 64;
+        const int splits = pick_splits_waves(t * (t + 1) / 2, h->D, min_k, cap);   // only the tiles on and above the diagonal run
         cudaError_t e = timed(h, K_GRAM, 1, st, [&] {
             return launch_tc_gemm_nt_x3(Bc, h->pitch, Bc, h->pitch, r, r, h->D, splits, h->gram_parts, ldc, stride, sym, h->tc_err, st);
         });

@@ -8,7 +8,7 @@
 //      matrix in registers (k_tridiag). n <= 128: one thread block of 4 warps; larger: a cluster of 8 blocks works until
 //      128 rows are left, the one-block kernel does the rest.
 //   2. Every wanted eigenvalue of T (the kept ones and delta) is found by multisection on the sign changes of the
-//      leading principal minors, in fp64, one warp per eigenvalue, 33 sub-intervals per pass over T.
+//      leading principal minors, in fp64, one warp per eigenvalue, 32 places per pass over T, with secants at the end.
 //   3. Its eigenvector is read off the forward and the backward three-term recurrence, joined where their product (the
 //      diagonal of the resolvent) is largest, in fp64.
 //   4. The reflections are applied to it in reverse (fp32, groups of four), it is scaled and written.
@@ -637,35 +637,44 @@ __device__ __forceinline__ double eigenvalue(const double2* up, const double2* d
     double h = 1.0 / (kPoints + 1);
     if (k < kPoints) hi = fma(h, (double)(k + 1), lo);
     if (k > 0) lo = fma(h, (double)k, lo);
-    // 129 * 33^6 * 31 = 5.2e12, then the secant through the determinants at the two places around the eigenvalue: exact to
-    // rounding, if it is alone there; if not, two passes more.
-    double lam = 0.5 * (lo + hi);
-    for (int pass = 0; pass < 9; ++pass) {
-        const bool ends = pass >= 6;                       // the places include lo and hi themselves
-        h = (hi - lo) * (ends ? 1.0 / 31.0 : 1.0 / 33.0);
-        const double x = ends ? (lane == 31 ? hi : fma(h, (double)lane, lo)) : fma(h, (double)(lane + 1), lo);
+    // The secant through the determinants at the two places around an eigenvalue is off by no more than their distance squared over
+    // four times the distance to the next eigenvalue, and that is at least the distance to the ends of an interval in which the
+    // eigenvalue is known to be alone. Even cuts until the places are near by that measure, then cuts whose places close in on the
+    // secant from both sides, each four times nearer than the one before; the last secant is exact to rounding. Four cuts where
+    // eigenvalues are apart (even cuts alone: seven). In a cluster even cuts go on for longer.
+    double lam = 0.5 * (lo + hi), ilo = lo, ihi = hi;
+    bool alone = false;
+    bool isolated = (k < kPoints ? first[k] : below + 1) == below + 1 && (k > 0 ? first[k - 1] : below) == below;
+    for (int pass = 0; pass < 20; ++pass) {
+        const double wid = hi - lo;
+        double x;
+        if (alone && 8.0 * wid < fmin(lam - ilo, ihi - lam)) {   // lanes 0 .. 15: lam - wid 4^-lane, lanes 16 .. 31: lam + wid 4^(lane - 31)
+            const int e = lane < 16 ? lane : 31 - lane;
+            const double off = wid * __hiloint2double((1023 - 2 * e) << 20, 0);
+            x = lane < 16 ? fmax(lam - off, lo) : fmin(lam + off, hi);
+        } else {
+            x = lane == 31 ? hi : fma(wid * (1.0 / 31.0), (double)lane, lo);
+        }
         double det;
         int ex;
         const int c = count_below(up, down, mid, M, x, det, ex);
         k = __popc(__ballot_sync(0xffffffffu, c <= below));
-        const double l0 = lo;
-        if (!ends) {
-            if (k > 0) lo = fma(h, (double)k, l0);
-            if (k < 32) hi = fma(h, (double)(k + 1), l0);
-            continue;
-        }
-        const int a = min(max(k - 1, 0), 30), b = a + 1;
+        const int a = min(max(k - 1, 0), 30), b = a + 1;   // lanes 0 and 31 are at lo and hi
         lo = __shfl_sync(0xffffffffu, x, a);
         hi = __shfl_sync(0xffffffffu, x, b);
-        lam = 0.5 * (lo + hi);
         const double da = __shfl_sync(0xffffffffu, det, a), db = __shfl_sync(0xffffffffu, det, b);
         const int ea = __shfl_sync(0xffffffffu, ex, a), eb = __shfl_sync(0xffffffffu, ex, b);
         const int ca = __shfl_sync(0xffffffffu, c, a), cb = __shfl_sync(0xffffffffu, c, b);
         const double r = db / da * pow2(min(eb - ea, 1000));               // f(hi) / f(lo), negative with one eigenvalue between
-        if (cb == ca + 1 && r <= 0.0) {
-            lam = fma(hi - lo, 1.0 / (1.0 - r), lo);
-            break;
+        alone = cb == ca + 1 && r <= 0.0;
+        lam = alone ? fma(hi - lo, 1.0 / (1.0 - r), lo) : 0.5 * (lo + hi);
+        if (alone && !isolated) {
+            ilo = lo;
+            ihi = hi;
+            isolated = true;
         }
+        const double d = hi - lo;
+        if ((alone && (d <= 2e-13 || 0.25 * d * d <= 5e-17 * fmin(lam - ilo, ihi - lam))) || d <= 1e-16) break;
     }
     return lam;
 }
@@ -686,7 +695,7 @@ struct VecShared {
 };
 
 // One warp per eigenvector, three per block, whatever n: no communication between blocks (each finds delta for itself). Bound by
-// dependent latency: 8 passes of n / 2 fp64 steps over T, n steps of the recurrences, n / 4 groups of reflections.
+// dependent latency: five or so passes of n / 2 fp64 steps over T, n steps of the recurrences, n / 4 groups of reflections.
 template <int NQ>                                  // quads of positions per lane: N <= 128 NQ
 __global__ void __launch_bounds__(kVecThreads, 1)
 k_tridiag_vectors(TriWork wk, int G, int n, int do_shrink, int delta_rank, int keep, float* __restrict__ Ur, int ldu,
