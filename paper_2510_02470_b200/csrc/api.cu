@@ -298,6 +298,13 @@ int pick_splits_waves(int tiles, int64_t K, int64_t min_k, int max_splits) {
     return best;
 }
 
+// K slices of the Gram matrix, 256 columns and more; with one tile and short rows up to 16 slices of 64 and more: the kernel is a
+// chain of K tiles there, while many slices cost the reduction what they save (a cycle on rows of 257, 1,024, 3,001 values:
+// 34.9 -> 32.7, 58.7 -> 56.3, 82.3 -> 80.8 us; slices of 64 throughout: 5,130 values 107.9 -> 108.8, 20,000 values 113.7 -> 118.2 us).
+int gram_splits(int tiles, int64_t D, int cap) {
+    return pick_splits_waves(tiles, D, tiles > 1 || D >= 4096 ? 256 : D >= 1024 ? (D + 15) / 16 : 64, cap);
+}
+
 // After the sketch is frozen: the bf16 copy the tensor-core projection reads (bf16 handles only).
 sage_status_t enqueue_freeze_aux(sage_fd* h, cudaStream_t st) {
     if (h->dtype == SAGE_F32 && h->S32split)
@@ -321,11 +328,7 @@ sage_status_t enqueue_gram(sage_fd* h, int r, cudaStream_t st) {
         const int sym = r <= 128 ? 1 : 0;    // one diagonal tile: one wide MMA per K step, transpose added in the reduction
         int cap = (int)(h->gram_part_floats / (size_t)stride);
         if (cap > 148) cap = 148;
-        // Slices of 256 columns; short rows in up to 16 slices of 64 and more: the kernel is a chain of K tiles there, while many
-        // slices cost the reduction what they save (a cycle on rows of 257, 1,024, 3,001 values: 34.9 -> 32.8, 58.7 -> 56.6, 82.3 -> 81.3 us;
-        // slices of 64 throughout: 5,130 values 107.9 -> 108.8, 20,000 values 113.7 -> 118.2 us)
-        const int64_t min_k = t > 1 || h->D >= 4096 ? 256 : h->D >= 1024 ? (h->D + 15) / 16 : 64;
-        const int splits = pick_splits_waves(t * (t + 1) / 2, h->D, min_k, cap);   // only the tiles on and above the diagonal run
+        const int splits = gram_splits(t * (t + 1) / 2, h->D, cap);   // only the tiles on and above the diagonal run
         cudaError_t e = timed(h, K_GRAM, 1, st, [&] {
             return launch_tc_gemm_nt_x3(Bc, h->pitch, Bc, h->pitch, r, r, h->D, splits, h->gram_parts, ldc, stride, sym, h->tc_err, st);
         });
@@ -782,7 +785,7 @@ static sage_status_t sketch_factor_direct(sage_fd* s, const void* rows, int64_t 
     const int64_t stride = (int64_t)r * ldc;
     int cap = (int)(s->gram_part_floats / (size_t)stride);
     if (cap > 148) cap = 148;
-    const int splits = pick_splits_waves(1, s->D, 256, cap);
+    const int splits = gram_splits(1, s->D, cap);
     float* Bc = s->B[s->cur];
     cudaError_t e = timed(s, K_GRAM, 1, chain, [&] {
         return launch_tc_gram_direct(Bc, s->pitch, old_rows, rows, ld, n_new, s->D, splits, s->gram_parts, ldc, stride, s->tc_err, chain);
