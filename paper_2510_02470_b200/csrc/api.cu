@@ -380,19 +380,18 @@ sage_status_t enqueue_factor(sage_fd* h, int r, int do_shrink, int keep, int zer
     const int m_total = zero_to > keep ? zero_to : keep;
     bool done = false;
     if (tc_rebuild) {
-        const int parts = j_pad > 128 ? 2 : 1;                            // launches: 128 output rows each
-        cudaError_t e = timed(h, K_REBUILD, parts, st, [&] {
+        cudaError_t e = timed(h, K_REBUILD, 1, st, [&] {
             return launch_tc_rebuild(h->Wsplit, h->wsplit_ld, j_pad, h->B[h->cur], h->B[1 - h->cur], h->pitch, h->D, r, keep, h->tc_err, st);
         });
         if (e == cudaSuccess) {
             done = true;
-            h->tc_launches += parts;
+            h->tc_launches += 1;
             if (m_total > keep)
                 CU_TRY(cudaMemsetAsync(h->B[1 - h->cur] + (size_t)keep * h->pitch, 0, (size_t)(m_total - keep) * h->pitch * sizeof(float), st));
         } else if (e != cudaErrorNotSupported) {
             CU_TRY(e);
         } else {
-            count(h, -parts);
+            count(h, -1);
         }
     }
     if (!done)

@@ -8,9 +8,8 @@
 // fp32 fidelity as in the Gram kernel: the tensor cores read a buffer value as hi (its low 13 bits ignored),
 // the split warps write lo = x - hi into a second buffer; W arrives already split from global memory as two stacked operands [W_hi; W_lo],
 // so one MMA of width 2*j_pad gives hi*W_hi and hi*W_lo side by side and a second one adds lo*W_hi; the
-// epilogue adds the two halves. One TMEM accumulator takes at most 8 chunks (256 buffer rows); with more buffer rows
-// (up to 512) a tile uses both accumulators, one per half of the rows, and the epilogue adds them in registers (the
-// tiles then no longer alternate between the accumulators, so a tile's MMAs start after the previous tile's epilogue).
+// epilogue adds the two halves. One TMEM accumulator takes at most 8 chunks (256 buffer rows) this way; more than 256 buffer rows
+// or more than 128 output rows go to k_tc_rebuild_wide.
 //
 //   warp 0    TMA producer: per chunk 4 boxes of [32 rows][32 columns] of the buffer (128-byte swizzle with
 //             32-byte atoms, the only layout the tensor cores take for 32-bit MN-major operands) and one box of W; where
@@ -32,6 +31,24 @@ constexpr int kTileD = 128;                 // buffer columns per tile (MMA M)
 constexpr int kChunkRows = 32;              // buffer rows per stage (MMA K = 4 x 8)
 constexpr int kBufBytes = kChunkRows * kTileD * 4;   // 16 KB: 4 spans of [32 rows][128 bytes]
 constexpr int kSpanBytes = kChunkRows * 128;         // 4 KB
+
+// The remainders of a landed chunk, by kSplitThreads threads. The tensor cores ignore the low 13 bits of an fp32 word, so the raw
+// tile is the hi operand as it stands; lo = x - hi (exact), rounded to 11 significant bits so that the same truncation cuts
+// nothing from it. Row zero_row gets remainders of zero.
+__device__ __forceinline__ void split_chunk(const uint4* hi, uint4* lo, int t, int zero_row = -1) {
+#pragma unroll
+    for (int cc = 0; cc < kBufBytes / 16 / kSplitThreads; ++cc) {
+        const int idx = t + cc * kSplitThreads;
+        const uint4 v = hi[idx];
+        uint4 l;
+        l.x = (__float_as_uint(__uint_as_float(v.x) - __uint_as_float(v.x & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
+        l.y = (__float_as_uint(__uint_as_float(v.y) - __uint_as_float(v.y & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
+        l.z = (__float_as_uint(__uint_as_float(v.z) - __uint_as_float(v.z & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
+        l.w = (__float_as_uint(__uint_as_float(v.w) - __uint_as_float(v.w & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
+        if (((idx >> 3) & 31) == zero_row) l = make_uint4(0u, 0u, 0u, 0u);
+        lo[idx] = l;
+    }
+}
 
 __global__ void __launch_bounds__(kThreads, 1)
 k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmSrc,
@@ -63,7 +80,6 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_mma = 2 * j_pad;                           // <= 256
-    const bool two = nchunk > 8;                           // both accumulators serve one tile
     uint32_t tmem_cols = 32;
     while (tmem_cols < (uint32_t)(2 * n_mma)) tmem_cols <<= 1;
     // tiles of this CTA: blockIdx.x, blockIdx.x + gridDim.x, ...
@@ -142,20 +158,19 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
             const uint32_t wres0 = smem_u32(wres);
             if (w_res) alive = mbar_wait(w_full, 0, abort);
             for (long long lt = 0; lt < my_tiles && alive; ++lt) {
-                const int b = two ? 0 : (int)(lt & 1);
-                const uint32_t par = two ? (uint32_t)lt : (uint32_t)(lt >> 1);
+                const int b = (int)(lt & 1);
+                const uint32_t par = (uint32_t)(lt >> 1);
                 alive = mbar_wait(&acc_empty[b], (par & 1u) ^ 1u, abort);
                 if (!alive) break;
                 for (int c = 0; c < nchunk; ++c) {
-                    const uint32_t acc = tmem_base + (uint32_t)((two ? (c >> 3) : b) * n_mma);
-                    const int c_in = two ? (c & 7) : c;       // position within this accumulator's run
+                    const uint32_t acc = tmem_base + (uint32_t)(b * n_mma);
                     if (!mbar_wait(&split_done[s], ph, abort)) { alive = false; break; }
                     tc_fence_after();
                     const uint64_t d_w = desc_w | ((w_res ? wres0 + (uint32_t)(c * w_bytes) : st + 2 * kBufBytes) >> 4);
                     const uint64_t d_hi = desc_buf | (st >> 4), d_lo = desc_buf | ((st + kBufBytes) >> 4);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {          // 8 buffer rows per MMA: one 1024-byte row group (64 descriptor units)
-                        mma_tf32(acc, d_hi + 64 * k, d_w + 2 * k, idesc_fold, (c_in | k) != 0);   // hi*W_hi | hi*W_lo
+                        mma_tf32(acc, d_hi + 64 * k, d_w + 2 * k, idesc_fold, (c | k) != 0);   // hi*W_hi | hi*W_lo
                         if (c <= cb) mma_tf32(acc, d_lo + 64 * k, d_w + 2 * k, idesc_half, 1);     // + lo*W_hi (zero for bfloat16 rows)
                     }
                     mma_commit(&empty[s]);
@@ -174,21 +189,8 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
             uint4* hi = reinterpret_cast<uint4*>(smem + (size_t)s * stage_bytes);
             uint4* lo = reinterpret_cast<uint4*>(smem + (size_t)s * stage_bytes + kBufBytes);
             if (c <= cb) {
-#pragma unroll
-                for (int cc = 0; cc < kBufBytes / 16 / kSplitThreads; ++cc) {
-                    const int idx = t + cc * kSplitThreads;
-                    // the tensor cores ignore the low 13 bits of an fp32 word, so the raw tile is the hi operand as it stands;
-                    // lo = x - hi (exact), rounded to 11 significant bits so that the same truncation cuts nothing from it
-                    const uint4 v = hi[idx];
-                    uint4 l;
-                    l.x = (__float_as_uint(__uint_as_float(v.x) - __uint_as_float(v.x & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
-                    l.y = (__float_as_uint(__uint_as_float(v.y) - __uint_as_float(v.y & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
-                    l.z = (__float_as_uint(__uint_as_float(v.z) - __uint_as_float(v.z & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
-                    l.w = (__float_as_uint(__uint_as_float(v.w) - __uint_as_float(v.w & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
-                    // the last row of chunk cb is a placeholder for the caller's first row (a bfloat16 row: remainder zero)
-                    if (c == cb && ((idx >> 3) & 31) == kChunkRows - 1) l = make_uint4(0u, 0u, 0u, 0u);
-                    lo[idx] = l;
-                }
+                // the last row of chunk cb is a placeholder for the caller's first row (a bfloat16 row: remainder zero)
+                split_chunk(hi, lo, t, c == cb ? kChunkRows - 1 : -1);
             }
             if (c >= cb) {
                 // bfloat16 rows from the staging area (256 bytes = 128 columns per row): 8 values -> two chunks of 4 floats
@@ -214,8 +216,8 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
         const int quarter = warp & 3;
         const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
         for (long long lt = 0; lt < my_tiles; ++lt) {
-            const int b = two ? 0 : (int)(lt & 1);
-            const uint32_t par = two ? (uint32_t)lt : (uint32_t)(lt >> 1);
+            const int b = (int)(lt & 1);
+            const uint32_t par = (uint32_t)(lt >> 1);
             bool ok = mbar_wait(&acc_full[b], par & 1u, abort);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -245,25 +247,6 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
 #pragma unroll
                     for (int j = 0; j < 16; ++j) a1[j] = __uint_as_float(v1[j]) + __uint_as_float(w1[j]);
                 }
-                if (two) {                                  // the second half of the buffer rows, from the other accumulator
-                    tmem_ld16_issue(acc + (uint32_t)(n_mma + j0), v0);
-                    tmem_ld16_issue(acc + (uint32_t)(n_mma + j_pad + j0), w0);
-                    if (second) {
-                        tmem_ld16_issue(acc + (uint32_t)(n_mma + j0 + 16), v1);
-                        tmem_ld16_issue(acc + (uint32_t)(n_mma + j_pad + j0 + 16), w1);
-                    }
-                    tmem_ld_wait();
-                    tmem_ld_use(v0);
-                    tmem_ld_use(w0);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) a0[j] += __uint_as_float(v0[j]) + __uint_as_float(w0[j]);
-                    if (second) {
-                        tmem_ld_use(v1);
-                        tmem_ld_use(w1);
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) a1[j] += __uint_as_float(v1[j]) + __uint_as_float(w1[j]);
-                    }
-                }
                 if (d < pitch) {
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
@@ -283,9 +266,239 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
     __syncthreads();
     if (warp == 1) {
         if (my_tiles > 0 && !*abort)
-            mbar_wait_quiet(&acc_full[two ? 0 : (my_tiles - 1) & 1], (uint32_t)(two ? my_tiles - 1 : (my_tiles - 1) >> 1) & 1u, kWaitLimitCycles);
+            mbar_wait_quiet(&acc_full[(my_tiles - 1) & 1], (uint32_t)((my_tiles - 1) >> 1) & 1u, kWaitLimitCycles);
         tc_fence_after();
         tmem_dealloc(tmem_base, tmem_cols);
+    }
+    if (threadIdx.x == 0 && *abort) atomicExch(err, 1);
+}
+
+// More than 256 buffer rows or more than 128 output rows (up to 512 onto 256): a tile's buffer data is loaded once for all output
+// rows. A chunk costs 12 MMAs of width j_pad (hi*W_hi, lo*W_hi and hi*W_lo for its 4 steps of 8 rows) that add into ONE accumulator
+// of j_pad columns, so that two of them fit TMEM and one is drained while the other fills. A run of kRunChunks chunks makes 60
+// additions to an accumulator, where the narrow kernel makes 64; the epilogue keeps the sums of a tile's runs in registers
+// (128 a thread, hence the register split below).
+// A chunk's factors are four times its buffer data, and come out of the L2 cache: they have a ring of their own, whose slots (hi
+// and lo apart) are shorter-lived than the buffer's, and whose loads do not wait for buffer data.
+//   warp 0 loads buffer chunks, warp 1 issues MMAs, warp 2 loads factors, warps 4-7 write the lo parts, warps 8-15 are the
+//   epilogue (8-11: output rows 0-127, 12-15: the others).
+// 512 rows onto 255, 262,144 columns: 422 -> 282 us (two launches of the narrow kernel, each over the whole buffer, before: their
+// loads and hand-offs alone took 344 us). What bounds it is shared memory: a chunk writes 80 KB, its split moves 32 KB and its MMAs
+// read 144 KB, 2,050 cycles at 128 bytes each of the 2,400 that it takes; the MMAs themselves are 1,540.
+constexpr int kWideThreads = 512;
+constexpr int kWideRegs = 128;              // what every thread is launched with: the sum of the shares below is 4 x 128 x 128
+constexpr int kBufStages = 3, kWSlots = 4;
+constexpr int kWSlotBytes = 256 * 128;      // [256 output rows][32 buffer rows] of W_hi or W_lo
+constexpr int kRunChunks = 5;
+constexpr size_t kWideSmem = 1024 + (size_t)kBufStages * 2 * kBufBytes + (size_t)kWSlots * kWSlotBytes + (3 * kBufStages + 2 * kWSlots + 4) * 8 + 16;
+
+__global__ void __launch_bounds__(kWideThreads, 1)
+k_tc_rebuild_wide(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ CUtensorMap tmW, int r, int keep, int j_pad, int lo_row,
+                  long long pitch, long long num_tiles, float* __restrict__ out, int* __restrict__ err) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    uint8_t* wring = smem + kBufStages * 2 * kBufBytes;
+    uint64_t* full = reinterpret_cast<uint64_t*>(wring + kWSlots * kWSlotBytes);
+    uint64_t* split_done = full + kBufStages;
+    uint64_t* empty = split_done + kBufStages;
+    uint64_t* w_full = empty + kBufStages;
+    uint64_t* w_empty = w_full + kWSlots;
+    uint64_t* acc_full = w_empty + kWSlots;                // [2]
+    uint64_t* acc_empty = acc_full + 2;                    // [2]
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+    volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int halves = j_pad > 128 ? 2 : 1;
+    const int nchunk = (r + kChunkRows - 1) / kChunkRows;
+    const int nruns = (nchunk + kRunChunks - 1) / kRunChunks, run_len = (nchunk + nruns - 1) / nruns;
+    // every run has at least one chunk: nchunk <= 16 gives runs of 1 to 5, ceil(nchunk / run_len) == nruns for all of them
+    const long long my_tiles = num_tiles > blockIdx.x ? (num_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kBufStages; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&split_done[s], kSplitThreads);
+            mbar_init(&empty[s], 1);
+        }
+        for (int s = 0; s < kWSlots; ++s) {
+            mbar_init(&w_full[s], 1);
+            mbar_init(&w_empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], 128 * halves);
+        }
+        *abort = 0;
+        mbar_fence_init();
+        tma_prefetch_desc(&tmBuf);
+        tma_prefetch_desc(&tmW);
+    }
+    if (warp == 1) tmem_alloc(tmem_slot, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    chain_wait();
+
+    if (warp < 8) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        if (warp == 0) {
+            if (lane == 0) {
+                long long issued = 0;
+                bool alive = true;
+                int s = 0;
+                uint32_t ph = 1;
+                for (long long lt = 0; lt < my_tiles && alive; ++lt) {
+                    const int d0 = (int)((blockIdx.x + lt * gridDim.x) * kTileD);
+                    for (int c = 0; c < nchunk; ++c) {
+                        if (!mbar_wait(&empty[s], ph, abort)) { alive = false; break; }
+                        uint8_t* st = smem + (size_t)s * 2 * kBufBytes;
+                        mbar_expect_tx(&full[s], (uint32_t)kBufBytes);
+#pragma unroll
+                        for (int sp = 0; sp < 4; ++sp) tma_load_2d(st + sp * kSpanBytes, &tmBuf, &full[s], d0 + 32 * sp, c * kChunkRows);
+                        ++issued;
+                        if (++s == kBufStages) { s = 0; ph ^= 1u; }
+                    }
+                }
+                if (*abort)
+                    for (long long k = issued > kBufStages ? issued - kBufStages : 0; k < issued; ++k)
+                        mbar_wait_quiet(&full[k % kBufStages], (uint32_t)(k / kBufStages) & 1u, 20000000ll);
+            }
+        } else if (warp == 2) {
+            if (lane == 0) {
+                long long issued = 0;
+                bool alive = true;
+                int s = 0;
+                uint32_t ph = 1;
+                for (long long lt = 0; lt < my_tiles && alive; ++lt)
+                    for (int c = 0; c < nchunk && alive; ++c)
+                        for (int part = 0; part < 2; ++part) {
+                            if (!mbar_wait(&w_empty[s], ph, abort)) { alive = false; break; }
+                            uint8_t* dst = wring + (size_t)s * kWSlotBytes;
+                            mbar_expect_tx(&w_full[s], (uint32_t)(halves * 128 * 128));
+                            for (int q = 0; q < halves; ++q)
+                                tma_load_2d(dst + q * 128 * 128, &tmW, &w_full[s], c * kChunkRows, q * 256 + part * lo_row);
+                            ++issued;
+                            if (++s == kWSlots) { s = 0; ph ^= 1u; }
+                        }
+                if (*abort)
+                    for (long long k = issued > kWSlots ? issued - kWSlots : 0; k < issued; ++k)
+                        mbar_wait_quiet(&w_full[k % kWSlots], (uint32_t)(k / kWSlots) & 1u, 20000000ll);
+            }
+        } else if (warp == 1) {
+            if (lane == 0) {
+                const uint32_t idesc = instr_desc(2, kTileD, j_pad, 1, 0);                // A (buffer) MN-major, B (W) K-major
+                const uint64_t desc_w = smem_desc_k_sw128(0), desc_buf = smem_desc_mn_sw128_atom32(0, kSpanBytes);
+                const uint32_t st0 = smem_u32(smem), w0 = smem_u32(wring);
+                bool alive = true;
+                int s = 0, ws = 0;
+                uint32_t ph = 0, wph = 0, run = 0;
+                for (long long lt = 0; lt < my_tiles && alive; ++lt) {
+                    for (int c0 = 0; c0 < nchunk && alive; c0 += run_len, ++run) {
+                        const int c1 = c0 + run_len < nchunk ? c0 + run_len : nchunk;
+                        const uint32_t b = run & 1u, acc = tmem_base + b * 256u;
+                        alive = mbar_wait(&acc_empty[b], ((run >> 1) & 1u) ^ 1u, abort);
+                        for (int c = c0; c < c1 && alive; ++c) {
+                            alive = mbar_wait(&w_full[ws], wph, abort) && mbar_wait(&split_done[s], ph, abort);
+                            if (!alive) break;
+                            tc_fence_after();
+                            const uint32_t st = st0 + (uint32_t)(s * 2 * kBufBytes);
+                            const uint64_t d_hi = desc_buf | (st >> 4), d_lo = desc_buf | ((st + kBufBytes) >> 4);
+                            uint64_t d_w = desc_w | ((w0 + (uint32_t)(ws * kWSlotBytes)) >> 4);
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                mma_tf32(acc, d_hi + 64 * k, d_w + 2 * k, idesc, c != c0 || k != 0);
+                                mma_tf32(acc, d_lo + 64 * k, d_w + 2 * k, idesc, 1);
+                            }
+                            mma_commit(&w_empty[ws]);
+                            if (++ws == kWSlots) { ws = 0; wph ^= 1u; }
+                            alive = mbar_wait(&w_full[ws], wph, abort);
+                            if (!alive) break;
+                            tc_fence_after();
+                            d_w = desc_w | ((w0 + (uint32_t)(ws * kWSlotBytes)) >> 4);
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) mma_tf32(acc, d_hi + 64 * k, d_w + 2 * k, idesc, 1);
+                            mma_commit(&w_empty[ws]);
+                            mma_commit(&empty[s]);
+                            if (++ws == kWSlots) { ws = 0; wph ^= 1u; }
+                            if (++s == kBufStages) { s = 0; ph ^= 1u; }
+                        }
+                        if (alive) mma_commit(&acc_full[b]);
+                    }
+                }
+            }
+        } else if (warp >= 4) {
+            const int t = threadIdx.x - 128;
+            const long long total = my_tiles * nchunk;
+            int s = 0;
+            uint32_t ph = 0;
+            for (long long q = 0; q < total; ++q) {
+                if (!mbar_wait(&full[s], ph, abort)) break;
+                uint4* hi = reinterpret_cast<uint4*>(smem + (size_t)s * 2 * kBufBytes);
+                split_chunk(hi, hi + kBufBytes / 16, t);
+                fence_proxy_async_smem();
+                mbar_arrive(&split_done[s]);
+                if (++s == kBufStages) { s = 0; ph ^= 1u; }
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 184;");
+        const int quarter = warp & 3, half = (warp - 8) >> 2;
+        if (half < halves) {
+            const int j_n = j_pad - half * 128 < 128 ? j_pad - half * 128 : 128;         // output rows of this half, a multiple of 16
+            const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + (uint32_t)(half * 128);
+            uint32_t run = 0;
+            bool ok = true;
+            for (long long lt = 0; lt < my_tiles && ok; ++lt) {
+                float sum[128];
+#pragma unroll
+                for (int j = 0; j < 128; ++j) sum[j] = 0.f;
+                for (int g = 0; g < nruns; ++g, ++run) {
+                    const uint32_t b = run & 1u;
+                    ok = mbar_wait(&acc_full[b], (run >> 1) & 1u, abort);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (lt == my_tiles - 1 && g == nruns - 1) chain_release();
+#pragma unroll
+                    for (int j0 = 0; j0 < 128; j0 += 32) {
+                        if (j0 < j_n) {                     // the upper 16 columns of the last group may lie beyond j_n: added, never stored
+                            uint32_t v0[16], v1[16];
+                            tmem_ld16_issue(lane_base + b * 256u + (uint32_t)j0, v0);
+                            tmem_ld16_issue(lane_base + b * 256u + (uint32_t)(j0 + 16), v1);
+                            tmem_ld_wait();
+                            tmem_ld_use(v0);
+                            tmem_ld_use(v1);
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) {
+                                sum[j0 + j] += __uint_as_float(v0[j]);
+                                sum[j0 + 16 + j] += __uint_as_float(v1[j]);
+                            }
+                        }
+                    }
+                    tc_fence_before();
+                    mbar_arrive(&acc_empty[b]);
+                }
+                const long long d = (blockIdx.x + lt * gridDim.x) * kTileD + quarter * 32 + lane;
+                if (ok && d < pitch) {
+                    float* o = out + (long long)(half * 128) * pitch + d;
+#pragma unroll
+                    for (int j = 0; j < 128; ++j, o += pitch)
+                        if (half * 128 + j < keep) *o = sum[j];
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        if (my_tiles > 0 && !*abort) {
+            const long long last = my_tiles * nruns - 1;
+            mbar_wait_quiet(&acc_full[last & 1], (uint32_t)(last >> 1) & 1u, kWaitLimitCycles);
+        }
+        tc_fence_after();
+        tmem_dealloc(tmem_base, 512);
     }
     if (threadIdx.x == 0 && *abort) atomicExch(err, 1);
 }
@@ -298,7 +511,7 @@ static cudaError_t launch_tc_rebuild_part(const float* Wsplit, int ldw, int j_pa
                                           int keep, int* err, cudaStream_t st, const void* src = nullptr, int64_t ld_src = 0, int n_new = 0,
                                           int64_t D = 0) {
     if (keep <= 0 || r <= 0) return cudaSuccess;
-    if (j_pad < 16 || j_pad > 128 || (j_pad & 15) || keep > j_pad || r > 512) return cudaErrorNotSupported;
+    if (j_pad < 16 || j_pad > 128 || (j_pad & 15) || keep > j_pad || r > 256) return cudaErrorNotSupported;
     CUtensorMap tmBuf, tmW;
     // buffer: columns beyond D up to the pitch are zero and are rebuilt as zero, so the map spans the pitch
     // direct form (src != nullptr): only the rows that are in the buffer, plus the placeholder row, are addressable
@@ -332,23 +545,34 @@ static cudaError_t launch_tc_rebuild_part(const float* Wsplit, int ldw, int j_pa
                           num_tiles, Bdst, stages, w_res, err);
 }
 
-// See sage_internal.h. One launch takes at most 128 output rows (accumulator width) of up to 512 buffer rows; 129 to 256
-// output rows (ell = 256: 255 rows out of 512) run as two launches over the same buffer rows.
+static cudaError_t launch_tc_rebuild_wide(const float* Wsplit, int ldw, int j_pad, const float* Bsrc, float* Bdst, int64_t pitch, int r, int keep,
+                                          int* err, cudaStream_t st) {
+    const int kcols = ((r + tc::kChunkRows - 1) / tc::kChunkRows) * tc::kChunkRows;
+    const int rows = j_pad > 128 ? 512 : 256;              // W rows: [hi ; lo] of 128 output rows, twice, or of j_pad <= 128
+    if (kcols > ldw || rows > ldw) return cudaErrorNotSupported;
+    CUtensorMap tmBuf, tmW;
+    if (!tc::make_tmap_2d(&tmBuf, Bsrc, 4, (uint64_t)r, (uint64_t)pitch, (uint64_t)pitch, tc::kChunkRows, 1) ||
+        !tc::make_tmap_2d(&tmW, Wsplit, 4, (uint64_t)rows, (uint64_t)kcols, (uint64_t)ldw, 128))
+        return cudaErrorNotSupported;
+    // the kernel hands registers from one half of its warps to the other: only as many as the launch holds
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, tc::k_tc_rebuild_wide);
+    if (e != cudaSuccess) return e;
+    if (fa.numRegs != tc::kWideRegs) return cudaErrorNotSupported;
+    if ((e = allow_smem((const void*)tc::k_tc_rebuild_wide, 227 * 1024)) != cudaSuccess) return e;
+    const long long num_tiles = (pitch + tc::kTileD - 1) / tc::kTileD;
+    return launch_chained(tc::k_tc_rebuild_wide, dim3((int)(num_tiles < 148 ? num_tiles : 148)), dim3(tc::kWideThreads), tc::kWideSmem, st, tmBuf, tmW,
+                          r, keep, j_pad, j_pad > 128 ? 128 : j_pad, pitch, num_tiles, Bdst, err);
+}
+
+// See sage_internal.h.
 cudaError_t launch_tc_rebuild(const float* Wsplit, int ldw, int j_pad, const float* Bsrc, float* Bdst, int64_t pitch, int64_t D, int r,
                               int keep, int* err, cudaStream_t st) {
     (void)D;
     if (keep <= 0 || r <= 0) return cudaSuccess;
     if (j_pad < 16 || j_pad > 256 || (j_pad & 15) || keep > j_pad || r > 512) return cudaErrorNotSupported;
-    const int jparts = j_pad > 128 ? 2 : 1;
-    for (int jh = 0; jh < jparts; ++jh) {
-        const int jp = jparts == 2 ? 128 : j_pad;
-        const int keep_h = keep - jh * 128 < jp ? keep - jh * 128 : jp;
-        if (keep_h <= 0) continue;
-        const float* Wb = Wsplit + (size_t)(jparts == 2 ? jh * 256 : 0) * ldw;
-        cudaError_t e = launch_tc_rebuild_part(Wb, ldw, jp, Bsrc, Bdst + (size_t)jh * 128 * pitch, pitch, r, keep_h, err, st);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    if (r > 256 || j_pad > 128) return launch_tc_rebuild_wide(Wsplit, ldw, j_pad, Bsrc, Bdst, pitch, r, keep, err, st);
+    return launch_tc_rebuild_part(Wsplit, ldw, j_pad, Bsrc, Bdst, pitch, r, keep, err, st);
 }
 
 // See sage_internal.h.
