@@ -171,7 +171,7 @@ struct sage_fd {
     int delta_rank = 0, max_sweeps = 30;
     // Gram / eigen workspaces
     float* gram_parts = nullptr;   // split-K partials of the Gram matrix (gram_part_floats floats)
-    size_t gram_part_floats = 0;   // at least kGramPartFloats; 16 slices of m x m for buffers of more than 256 rows
+    size_t gram_part_floats = 0;   // at least kGramPartFloats; 74 or 30 slices of m x m for buffers of more than 128 or 256 rows
     float* Wsplit = nullptr;       // rebuild factors split for the tensor cores: wsplit_ld rows x wsplit_ld floats
     int wsplit_ld = 256;           // 256 (buffers of up to 256 rows) or 512
     float* Kmat = nullptr;         // m x m, pitch ldk
@@ -298,11 +298,21 @@ int pick_splits_waves(int tiles, int64_t K, int64_t min_k, int max_splits) {
     return best;
 }
 
-// K slices of the Gram matrix, 256 columns and more; with one tile and short rows up to 16 slices of 64 and more: the kernel is a
-// chain of K tiles there, while many slices cost the reduction what they save (a cycle on rows of 257, 1,024, 3,001 values:
+// K slices of the Gram matrix of up to 128 rows, 256 columns and more; with short rows up to 16 slices of 64 and more: the kernel is
+// a chain of K tiles there, while many slices cost the reduction what they save (a cycle on rows of 257, 1,024, 3,001 values:
 // 34.9 -> 32.7, 58.7 -> 56.3, 82.3 -> 80.8 us; slices of 64 throughout: 5,130 values 107.9 -> 108.8, 20,000 values 113.7 -> 118.2 us).
-int gram_splits(int tiles, int64_t D, int cap) {
-    return pick_splits_waves(tiles, D, tiles > 1 || D >= 4096 ? 256 : D >= 1024 ? (D + 15) / 16 : 64, cap);
+int gram_splits(int64_t D, int cap) {
+    return pick_splits_waves(1, D, D >= 4096 ? 256 : D >= 1024 ? (D + 15) / 16 : 64, cap);
+}
+
+// The same for the 74 pairs of SMs that a buffer of more than 128 rows takes (tc_gram_pair.cu). More than 256 rows: 22 slices of each
+// tile on the diagonal (8 MMAs a K tile), 30 of the one above it (12 MMAs): 512 rows of 262,144 columns take 304, 293, 295 us with 21, 22,
+// 23 slices of the former. At least 64 columns a slice (256 columns: a Gram matrix of 256 rows of 2,052 columns 29.9 instead of 27.4 us).
+constexpr int kDiagSlices = 22, kOffSlices = 74 - 2 * kDiagSlices;
+void pair_splits(int r, int64_t D, int cap, int* n_diag, int* n_off) {
+    const int64_t most = std::max<int64_t>(1, std::min<int64_t>((D + 63) / 64, cap));
+    *n_diag = (int)std::min<int64_t>(r > 256 ? kDiagSlices : 74, most);
+    *n_off = r > 256 ? (int)std::min<int64_t>(kOffSlices, most) : 0;
 }
 
 // After the sketch is frozen: the bf16 copy the tensor-core projection reads (bf16 handles only).
@@ -321,23 +331,21 @@ sage_status_t enqueue_freeze_aux(sage_fd* h, cudaStream_t st) {
 sage_status_t enqueue_gram(sage_fd* h, int r, cudaStream_t st) {
     float* Bc = h->B[h->cur];
     if (h->use_tc) {
-        // tensor cores: 128 x 128 output tiles, as many K slices as fill the SMs (each at least 256 columns)
-        const int t = (r + 127) / 128;
+        // tensor cores: one tile, or 256 x 256 tiles on pairs of SMs, in as many K slices as fill the SMs
         const int ldc = ((r + 3) / 4) * 4;
         const int64_t stride = (int64_t)r * ldc;
-        const int sym = r <= 128 ? 1 : 0;    // one diagonal tile: one wide MMA per K step, transpose added in the reduction
         int cap = (int)(h->gram_part_floats / (size_t)stride);
         if (cap > 148) cap = 148;
-        const int splits = gram_splits(t * (t + 1) / 2, h->D, cap);   // only the tiles on and above the diagonal run
+        int splits, n_off = 0;
+        if (r > 128) pair_splits(r, h->D, cap, &splits, &n_off);
+        else splits = gram_splits(h->D, cap);
         cudaError_t e = timed(h, K_GRAM, 1, st, [&] {
-            return launch_tc_gemm_nt_x3(Bc, h->pitch, Bc, h->pitch, r, r, h->D, splits, h->gram_parts, ldc, stride, sym, h->tc_err, st);
+            if (r > 128) return launch_tc_gram_pair(Bc, h->pitch, r, h->D, splits, n_off, h->gram_parts, ldc, stride, h->tc_err, st);
+            return launch_tc_gemm_nt_x3(Bc, h->pitch, Bc, h->pitch, r, r, h->D, splits, h->gram_parts, ldc, stride, 1, h->tc_err, st);
         });
         if (e == cudaSuccess) {
             h->tc_launches += 1;
-            if (sym)
-                CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_gram_sym_reduce(h->gram_parts, splits, stride, r, ldc, h->Kmat, h->ldk, st); }));
-            else   // sums the K slices and fills the tiles below the diagonal from their mirror images
-                CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_split_reduce(h->gram_parts, splits, stride, r, r, ldc, h->Kmat, h->ldk, st, 1); }));
+            CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_gram_sym_reduce(h->gram_parts, splits, stride, r, ldc, h->Kmat, h->ldk, st, n_off); }));
             return SAGE_OK;
         }
         if (e != cudaErrorNotSupported) CU_TRY(e);
@@ -530,7 +538,8 @@ static sage_status_t create_handle(sage_fd_t** out, int64_t D, int32_t ell, sage
     for (int i = 0; i < 2; ++i)
         if ((e = dev_malloc(h, (void**)&h->B[i], bbytes)) != cudaSuccess) return fail(e, "cudaMalloc(buffer)");
     h->gram_part_floats = kGramPartFloats;
-    if ((size_t)16 * h->m * h->m > h->gram_part_floats) h->gram_part_floats = (size_t)16 * h->m * h->m;
+    const size_t slices = h->m > 256 ? kOffSlices : h->m > 128 ? 74 : 0;
+    if (slices * h->m * ((h->m + 3) / 4 * 4) > h->gram_part_floats) h->gram_part_floats = slices * h->m * ((h->m + 3) / 4 * 4);
     if ((e = dev_malloc(h, (void**)&h->gram_parts, h->gram_part_floats * sizeof(float))) != cudaSuccess) return fail(e, "cudaMalloc(gram)");
     h->wsplit_ld = h->m <= 256 ? 256 : 512;
     if ((e = dev_malloc(h, (void**)&h->Wsplit, (size_t)h->wsplit_ld * h->wsplit_ld * sizeof(float))) != cudaSuccess)
@@ -784,7 +793,7 @@ static sage_status_t sketch_factor_direct(sage_fd* s, const void* rows, int64_t 
     const int64_t stride = (int64_t)r * ldc;
     int cap = (int)(s->gram_part_floats / (size_t)stride);
     if (cap > 148) cap = 148;
-    const int splits = gram_splits(1, s->D, cap);
+    const int splits = gram_splits(s->D, cap);
     float* Bc = s->B[s->cur];
     cudaError_t e = timed(s, K_GRAM, 1, chain, [&] {
         return launch_tc_gram_direct(Bc, s->pitch, old_rows, rows, ld, n_new, s->D, splits, s->gram_parts, ldc, stride, s->tc_err, chain);

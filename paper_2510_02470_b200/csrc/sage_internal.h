@@ -95,9 +95,8 @@ cudaError_t launch_tc_gemm_nt(const void* A, sage_dtype_t dt, int64_t lda, const
 
 // fp32-faithful tensor-core C[z] = A_z * Bm_z^T for fp32 operands (three tf32 MMAs on hi/lo halves split in shared
 // memory, accumulator drained into registers every few K tiles). Same alignment rules and return convention as
-// launch_tc_gemm_nt; any N. When A == Bm (a Gram matrix) the diagonal tiles load one operand only and the 128 x 128
-// tiles below the diagonal are NOT computed (their part of C is left untouched): reduce with mirror = 1.
-// sym != 0 (only for a Gram matrix of at most 128 rows): two MMAs per K step instead of three; slice z then stores
+// launch_tc_gemm_nt; any N.
+// sym == 1 (a Gram matrix of at most 128 rows, A == Bm): two MMAs per K step instead of three; slice z then stores
 // T_z = hi*hi^T + 2*hi*lo^T and the Gram matrix is sum_z (T_z + T_z^T)/2: see launch_gram_sym_reduce.
 // sym == 2 (projection onto at most 64 sketch rows): Bm is the sketch already split by launch_split_tf32 (128 rows);
 // one MMA per K step; C receives 2 * splits partial planes (split_stride apart) whose sum is A * S^T (M x N).
@@ -109,8 +108,15 @@ cudaError_t launch_tc_gemm_nt_x3(const float* A, int64_t lda, const float* Bm, i
 // bfloat16 rows at src (pitch ld_src). old_rows + n_new <= 128, old_rows + 1 a multiple of 8. Same output as the appended form.
 cudaError_t launch_tc_gram_direct(const float* Bold, int64_t pitch, int old_rows, const void* src, int64_t ld_src, int n_new, int64_t D,
                                   int splits, float* C, int64_t ldc, int64_t split_stride, int* err, cudaStream_t st);
+// Sums the slices of a Gram matrix in the symmetric form; n_off: slices of the 256 x 256 tile above the diagonal (more than 256 rows).
 cudaError_t launch_gram_sym_reduce(const float* parts, int splits, int64_t stride, int r, int64_t ldp, float* out, int64_t ldo,
-                                   cudaStream_t st);
+                                   cudaStream_t st, int n_off = 0);
+
+// Gram matrix of 129 to 512 rows (tc_gram_pair.cu): partials of K slice z at C + z * split_stride, n_diag slices of the 256 x 256 tiles on
+// the diagonal in the symmetric form (launch_gram_sym_reduce), n_off of the one above it (0 without one). ldc a multiple of 4, C
+// 16-byte aligned; cudaErrorNotSupported otherwise.
+cudaError_t launch_tc_gram_pair(const float* B, int64_t ldb, int r, int64_t K, int n_diag, int n_off, float* C, int64_t ldc, int64_t split_stride, int* err,
+                                cudaStream_t st);
 
 // Tensor-core rebuild: Bdst[j][d] = sum_{i<r} W[j][i] * Bsrc[i][d] for j < keep, d < pitch (fp32-faithful, see
 // tc_rebuild.cu). Wsplit holds W already split for tf32: rows [0, j_pad) = W rounded to 11 significant bits, rows
@@ -137,7 +143,7 @@ cudaError_t launch_to_bf16(const float* src, int64_t lds, int rows, int64_t cols
 cudaError_t launch_split_tf32(const float* src, int64_t lds, int rows, int64_t cols, float* out, int64_t ldo, cudaStream_t st);
 
 cudaError_t launch_split_reduce(const float* parts, int splits, int64_t split_stride, int M, int N, int64_t ldp,
-                                float* out, int64_t ldo, cudaStream_t st, int mirror = 0);
+                                float* out, int64_t ldo, cudaStream_t st);
 
 // out[j][d] = sum_{i<r} Ur[i*ldu + j] * Bsrc[i*pitch + d] for j < keep; rows keep..m_total-1 of out are zeroed.
 cudaError_t launch_rebuild(const float* Ur, int ldu, const float* Bsrc, float* Bdst, int64_t pitch, int64_t D, int r,

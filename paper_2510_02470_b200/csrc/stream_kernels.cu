@@ -228,69 +228,49 @@ __global__ void __launch_bounds__(256) k_split_reduce(const float* __restrict__ 
     out[(int64_t)i * ldo + j] = (float)s;
 }
 
-// The same for a symmetric r x r matrix of which only the 128 x 128 tiles on and above the diagonal were computed. Block: 32 x 32
-// outputs of the upper part, the slices dealt to four layers of threads (the kernel is bound by load latency), written twice, the mirror
-// image through shared memory.
-__global__ void __launch_bounds__(1024) k_split_reduce_sym(const float* __restrict__ parts, int splits, int64_t split_stride, int r, int64_t ldp,
-                                                           float* __restrict__ out, int64_t ldo) {
-    __shared__ double sh[4][32][33];
+// Split reduction of a Gram matrix computed in the symmetric form: slice z left T_z = hi*hi^T + 2*hi*lo^T at parts + z*stride;
+// K = sum_z (T_z + T_z^T) / 2 in fp64. One block of 16 x 16 x 4 threads per 16 x 16 tile (I, J) on or above the diagonal: thread
+// (ty, tx) of layer tz sums T[I+ty][J+tx] and T[J+ty][I+tx] (both read along rows) over the slices z = tz, tz+4, ... (several
+// loads in flight: the kernel is bound by load latency, not by bytes); the four layers are added in a fixed order, layer 0 writes
+// K[I+ty][J+tx] and layer 1 its mirror image, the other operand of each transposed through shared memory.
+// More than 256 rows: the 256 x 256 tile above the diagonal has n_off slices and is K itself.
+__global__ void __launch_bounds__(1024) k_gram_sym_reduce(const float* __restrict__ parts, int splits, int n_off, int64_t stride, int r,
+                                                          int64_t ldp, float* __restrict__ out, int64_t ldo) {
+    __shared__ double sa[4][16][17], sb[4][16][17];
     if (blockIdx.y > blockIdx.x) return;
     chain_release();                        // the next kernel of a shrink is one small block
     chain_wait();
-    const int tx = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;       // 32 x 8 x 4
-    const int j = blockIdx.x * 32 + tx;
-    double a[4] = {0.0, 0.0, 0.0, 0.0};
-    const int64_t o = (int64_t)(blockIdx.y * 32 + ty) * ldp + j;
-#pragma unroll 2
-    for (int z = tz; z < splits; z += 4)
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (blockIdx.y * 32 + ty + 8 * u < r && j < r) a[u] += (double)parts[(int64_t)z * split_stride + o + (int64_t)(8 * u) * ldp];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) sh[tz][ty + 8 * u][tx] = a[u];
-    __syncthreads();
-    const int row = tz * 8 + ty;                                          // 32 rows x 32 columns, one output per thread
-    const int i = blockIdx.y * 32 + row;
-    const double s = (sh[0][row][tx] + sh[1][row][tx]) + (sh[2][row][tx] + sh[3][row][tx]);
-    if (i < r && j < r) out[(int64_t)i * ldo + j] = (float)s;
-    if (blockIdx.x != blockIdx.y) {
-        const double m = (sh[0][tx][row] + sh[1][tx][row]) + (sh[2][tx][row] + sh[3][tx][row]);
-        const int mi = blockIdx.x * 32 + row, mj = blockIdx.y * 32 + tx;
-        if (mi < r && mj < r) out[(int64_t)mi * ldo + mj] = (float)m;
-    }
-}
-
-// Split reduction of a Gram matrix computed in the symmetric form: slice z left T_z = hi*hi^T + 2*hi*lo^T at
-// parts + z*stride; K = sum_z (T_z + T_z^T) / 2 in fp64. One block of 16 x 16 x 4 threads per 16 x 16 tile (I, J): thread
-// (ty, tx) of layer tz sums T[I+ty][J+tx] and T[J+ty][I+tx] (both read along rows) over the slices z = tz, tz+4, ...;
-// the four layers are added in a fixed order and the second sum is transposed through shared memory.
-__global__ void __launch_bounds__(1024) k_gram_sym_reduce(const float* __restrict__ parts, int splits, int64_t stride, int r,
-                                                          int64_t ldp, float* __restrict__ out, int64_t ldo) {
-    // 16 x 16 outputs per block; the four z-layers of the block each sum a quarter of the partial matrices
-    // (several loads in flight per thread: the kernel is bound by load latency, not by bytes).
-    __shared__ double sa[4][16][17], sb[4][16][17];
-    chain_release();                        // the next kernel of a shrink is one small block
-    chain_wait();
     const int tx = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;
-    const int i = blockIdx.y * 16 + ty, j = blockIdx.x * 16 + tx;          // direct element (i, j)
+    const int i = blockIdx.y * 16 + ty, j = blockIdx.x * 16 + tx;          // element (i, j)
     const int ti = blockIdx.x * 16 + ty, tj = blockIdx.y * 16 + tx;        // element (ti, tj) of the mirrored tile
+    const bool whole = (blockIdx.x >> 4) != (blockIdx.y >> 4);
     double a = 0.0, b = 0.0;
     const bool in_a = i < r && j < r, in_b = ti < r && tj < r;
     const float* pa = parts + (in_a ? (int64_t)i * ldp + j : 0);
     const float* pb = parts + (in_b ? (int64_t)ti * ldp + tj : 0);
+    if (whole) {
+#pragma unroll 8
+        for (int z = tz; z < n_off; z += 4) a += (double)pa[(int64_t)z * stride];
+    } else {
 #pragma unroll 4
-    for (int z = tz; z < splits; z += 4) {
-        const float va = pa[(int64_t)z * stride], vb = pb[(int64_t)z * stride];
-        a += (double)va;
-        b += (double)vb;
+        for (int z = tz; z < splits; z += 4) {
+            const float va = pa[(int64_t)z * stride], vb = pb[(int64_t)z * stride];
+            a += (double)va;
+            b += (double)vb;
+        }
     }
     sa[tz][ty][tx] = a;
     sb[tz][ty][tx] = b;                                                    // belongs to out[I + tx'][J + ty'] after the transpose
     __syncthreads();
+    const double f = whole ? 1.0 : 0.5;
     if (tz == 0 && in_a) {
         const double sum_a = (sa[0][ty][tx] + sa[1][ty][tx]) + (sa[2][ty][tx] + sa[3][ty][tx]);
         const double sum_b = (sb[0][tx][ty] + sb[1][tx][ty]) + (sb[2][tx][ty] + sb[3][tx][ty]);
-        out[(int64_t)i * ldo + j] = (float)(0.5 * (sum_a + sum_b));
+        out[(int64_t)i * ldo + j] = (float)(f * (sum_a + sum_b));
+    } else if (tz == 1 && in_b && blockIdx.x != blockIdx.y) {
+        const double sum_a = (sa[0][tx][ty] + sa[1][tx][ty]) + (sa[2][tx][ty] + sa[3][tx][ty]);
+        const double sum_b = (sb[0][ty][tx] + sb[1][ty][tx]) + (sb[2][ty][tx] + sb[3][ty][tx]);
+        out[(int64_t)ti * ldo + tj] = (float)(f * (sum_a + sum_b));
     }
 }
 
@@ -422,18 +402,17 @@ cudaError_t launch_split_tf32(const float* src, int64_t lds, int rows, int64_t c
 }
 
 cudaError_t launch_split_reduce(const float* parts, int splits, int64_t split_stride, int M, int N, int64_t ldp, float* out,
-                                int64_t ldo, cudaStream_t st, int mirror) {
+                                int64_t ldo, cudaStream_t st) {
     const int64_t total = (int64_t)M * N;
     if (total <= 0) return cudaSuccess;
-    if (mirror) return launch_chained(k_split_reduce_sym, dim3((N + 31) / 32, (N + 31) / 32), dim3(32, 8, 4), 0, st, parts, splits, split_stride, N, ldp, out, ldo);
     return launch_chained(k_split_reduce, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, parts, splits, split_stride, M, N, ldp, out, ldo);
 }
 
 cudaError_t launch_gram_sym_reduce(const float* parts, int splits, int64_t stride, int r, int64_t ldp, float* out, int64_t ldo,
-                                   cudaStream_t st) {
+                                   cudaStream_t st, int n_off) {
     if (r <= 0) return cudaSuccess;
     const unsigned t = (unsigned)((r + 15) / 16);
-    return launch_chained(k_gram_sym_reduce, dim3(t, t), dim3(16, 16, 4), 0, st, parts, splits, stride, r, ldp, out, ldo);
+    return launch_chained(k_gram_sym_reduce, dim3(t, t), dim3(16, 16, 4), 0, st, parts, splits, n_off, stride, r, ldp, out, ldo);
 }
 
 cudaError_t launch_rebuild(const float* Ur, int ldu, const float* Bsrc, float* Bdst, int64_t pitch, int64_t D, int r, int keep,

@@ -64,6 +64,23 @@ __device__ __forceinline__ void mbar_wait_quiet(uint64_t* bar, uint32_t parity, 
     while (!mbar_try_wait(bar, parity) && clock64() - t0 < limit_cycles) {}
 }
 
+// Arrival on the barrier at the same place in CTA `cta` of the cluster. What it orders is read by the
+// tensor cores, to which the arriving warp's proxy fence (or its fence behind a finished TMEM load) has shown it before; a release
+// at cluster scope, which waits for everything that its thread has in flight, made a Gram kernel's chain of hand-offs 40 % longer.
+__device__ __forceinline__ void mbar_arrive_cta(uint64_t* bar, uint32_t cta) {
+    asm volatile(
+        "{\n"
+        ".reg .b32 a;\n"
+        "mapa.shared::cluster.u32 a, %0, %1;\n"
+        "mbarrier.arrive.shared::cluster.b64 _, [a];\n"
+        "}\n" ::"r"(smem_u32(bar)), "r"(cta)
+        : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {                                    // all threads of all CTAs
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // ---- TMA -----------------------------------------------------------------------------------------
 // 2-D tile load; x is the innermost (contiguous) coordinate in elements and must make x * element size a
 // multiple of 16 bytes; y is the row. Completion is signalled on the mbarrier as transferred bytes.
@@ -85,6 +102,19 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* tmap) {
 }
 // Makes shared-memory writes of ordinary threads visible to the async proxy (tensor cores, TMA).
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// True in one lane of a converged warp, the same one each time.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "elect.sync _|p, 0xffffffff;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(p));
+    return p != 0;
+}
 
 // ---- tcgen05 -------------------------------------------------------------------------------------
 __device__ __forceinline__ void tmem_alloc(uint32_t* smem_result, uint32_t ncols) {   // whole warp, ncols power of two >= 32
@@ -122,6 +152,32 @@ __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t adesc, uint64
 // The mbarrier gets one arrival when every MMA issued so far by this thread has finished.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// The same on a pair of CTAs (a cluster of two): each holds half of the rows of A and of B at the same places of its shared memory
+// and gets its rows of D; one thread of CTA 0 issues. Allocation and release take a warp of each CTA.
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* smem_result, uint32_t ncols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_result)), "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+__device__ __forceinline__ void mma_tf32_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "setp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n"
+        "}\n" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// The barriers at this place in both CTAs get one arrival each when every MMA issued so far by this thread has finished.
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
+                 "h"((unsigned short)3)
+                 : "memory");
 }
 // 16 consecutive fp32 columns of this thread's TMEM lane (lane = 32 * (warp % 4) + lane id).
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {

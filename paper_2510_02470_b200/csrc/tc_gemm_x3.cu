@@ -1,6 +1,6 @@
 // fp32-faithful tensor-core contraction C[z] = A_z * B_z^T for fp32 operands (both contiguous along the
-// contraction index): the Gram matrix K = B B^T of the sketch buffer (Method, first paragraph: the SVD of
-// the buffer is taken through the eigen-decomposition of B B^T) and the pass-2 projection of fp32 rows.
+// contraction index): the Gram matrix K = B B^T of a sketch buffer of at most 128 rows (Method, first paragraph: the SVD of
+// the buffer is taken through the eigen-decomposition of B B^T; larger buffers: tc_gram_pair.cu) and the pass-2 projection of fp32 rows.
 //
 // Two things keep fp32 fidelity on tensor cores:
 //   * tcgen05 kind::tf32 reads an fp32 word by ignoring its low 13 bits (11 significant bits), so every value x
@@ -25,8 +25,7 @@
 // The producer and the MMA thread keep running stage / phase / chunk counters and advance the operand descriptors by a
 // constant per stage: with integer divisions and freshly built descriptors in its loop the single MMA-issuing thread took
 // 1,500 cycles per K tile and was what bounded the kernel (now about 600).
-// On the diagonal tiles of a Gram matrix only one operand tile is loaded and used on both sides. A Gram matrix
-// of at most 128 rows (sym mode) needs ONE 256-wide MMA per K step: the hi tile and the lo tile lie back to back
+// Of a Gram matrix (sym mode) only one operand tile is loaded and used on both sides, and it needs ONE 256-wide MMA per K step: the hi tile and the lo tile lie back to back
 // in the stage and serve as one 256-row B operand, so the accumulator holds hi*hi^T | hi*lo^T side by side; the drain
 // forms T = hi*hi^T + 2*hi*lo^T (the doubling is exact), which satisfies (T + T^T)/2 = hi*hi^T + hi*lo^T + lo*hi^T,
 // formed by the split reduction. (A 128 x 128 x 8 tf32 MMA executes in about 70 cycles, less than issuing it costs
@@ -64,17 +63,16 @@ __device__ __forceinline__ uint32_t lo_of(uint32_t x) {
 __device__ __forceinline__ uint4 lo4(const uint4 v) { return make_uint4(lo_of(v.x), lo_of(v.y), lo_of(v.z), lo_of(v.w)); }
 
 __global__ void __launch_bounds__(kThreads, 1)
-k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M, int N, int gram,
+k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M, int N,
                 int b_box_rows, int sym, long long K, long long k_per_split, int a_shared, float* __restrict__ C, long long ldc,
                 long long split_stride, int stages, int stage_bytes, int G, int direct_new, int direct_box, int* __restrict__ err) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int m0 = blockIdx.x * kTileM, n0 = blockIdx.y * kTileN;
-    if (gram && m0 > n0) return;                          // a Gram matrix is symmetric: the reduction mirrors the upper tiles
     const bool proj = sym == 2;
     const bool wide = sym != 0;                           // one 256-wide MMA per K step
-    const bool diag = gram && m0 == n0;                   // A tile == B tile: load once
-    // stage layout: [hi: A | B][lo: A | B]; on diagonal tiles there is no separate B; proj: [hi: rows][lo: rows][sketch]
+    const bool diag = sym == 1;                           // A tile == B tile: load once
+    // stage layout: [hi: A | B][lo: A | B]; sym: no separate B; proj: [hi: rows][lo: rows][sketch]
     const int half_bytes = (diag || proj) ? kTileBytes : kTileBytes + b_box_rows * 128;
     // direct_new > 0 (a symmetric Gram matrix of at most 128 rows whose last direct_new rows are still bfloat16 rows in the
     // caller's memory): tmA covers the first M - direct_new + 1 buffer rows (the last of them is a placeholder), tmB the
@@ -201,7 +199,6 @@ k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         }
     } else {
         // ---- workers: write the lo part of landed stages; drain finished accumulators ----
-        const int t = threadIdx.x - 64;                 // 0..255
         const int chunks16 = direct_new ? old_rows * 8 : half_bytes / 16;     // direct: remainders of the buffer rows only
         const float lo_scale = sym == 1 ? 2.f : 1.f;          // sym: the lo half of the accumulator counts twice (folded into the drain)
         const int quarter = warp & 3, chalf = (warp - 2) >> 2;
@@ -352,23 +349,23 @@ cudaError_t launch_tc_gemm_nt_x3(const float* A, int64_t lda, const float* Bm, i
                                  float* C, int64_t ldc, int64_t split_stride, int sym, int* err, cudaStream_t st, int64_t class_F) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
     if (splits < 1 || splits > 65535) return cudaErrorNotSupported;
-    const int gram = (A == Bm && lda == ldb && M == N) ? 1 : 0;
+    const bool gram = sym == 1;       // Bm is A
     const bool proj = sym == 2;       // Bm: the sketch split into [hi (64 rows) ; lo (64 rows)], 128 rows of pitch ldb; N <= 64
-    if (sym == 1 && !(gram && M <= tc::kTileM)) return cudaErrorInvalidValue;
-    if (proj && (N > 64 || gram)) return cudaErrorInvalidValue;
+    if (gram && (A != Bm || lda != ldb || M != N || M > tc::kTileM)) return cudaErrorInvalidValue;
+    if (proj && N > 64) return cudaErrorInvalidValue;
     // class slices: see launch_tc_gemm_nt
     if (class_F > 0 && (gram || class_F % 4 != 0 || (int64_t)splits * class_F != K)) return cudaErrorNotSupported;
     CUtensorMap tmA, tmB;
     if (!tc::make_tmap_2d(&tmA, A, 4, (uint64_t)M, (uint64_t)(class_F > 0 ? class_F : K), (uint64_t)lda, tc::kTileM)) return cudaErrorNotSupported;
     const int b_box_rows = proj ? tc::kTileN : (N >= tc::kTileN ? tc::kTileN : ((N + 15) / 16) * 16);
-    if (gram && M <= tc::kTileM) tmB = tmA;           // not used: diagonal tile only
+    if (gram) tmB = tmA;                              // not used
     else if (!tc::make_tmap_2d(&tmB, Bm, 4, (uint64_t)(proj ? 128 : N), (uint64_t)K, (uint64_t)ldb, (uint32_t)b_box_rows)) return cudaErrorNotSupported;
     int64_t kps = (K + splits - 1) / splits;
     kps = ((kps + tc::BK - 1) / tc::BK) * tc::BK;
     if (class_F > 0) kps = class_F;
     // a trailing slice may be empty after rounding to whole K tiles: its CTAs store zeros
-    // a Gram matrix of at most 128 rows has diagonal tiles only: one operand per stage
-    const int stage_bytes = proj ? 3 * tc::kTileBytes : 2 * ((gram && M <= tc::kTileM) ? tc::kTileBytes : tc::kTileBytes + b_box_rows * 128);
+    // a Gram matrix is one tile: one operand per stage
+    const int stage_bytes = proj ? 3 * tc::kTileBytes : 2 * (gram ? tc::kTileBytes : tc::kTileBytes + b_box_rows * 128);
     // Long K slices of the one-MMA-per-step forms (16 KB of remainders per stage): as many stages as fit the 227 KB a block
     // may have (7 of 32 KB, 4 of 48 KB), each slot with a worker group of its own (8 / stages warps), so that many
     // remainder chains overlap. Short slices, and the three-MMA form (32 KB of remainders per stage, 3 stages): the
@@ -383,7 +380,7 @@ cudaError_t launch_tc_gemm_nt_x3(const float* A, int64_t lda, const float* Bm, i
     dim3 grid((unsigned)((M + tc::kTileM - 1) / tc::kTileM), proj ? 1u : (unsigned)((N + tc::kTileN - 1) / tc::kTileN), (unsigned)splits);
     cudaError_t e = allow_smem((const void*)tc::k_tc_gemm_nt_x3, 227 * 1024);
     if (e != cudaSuccess) return e;
-    return launch_chained(tc::k_tc_gemm_nt_x3, grid, dim3(tc::kThreads), smem, st, tmA, tmB, M, N, gram, b_box_rows, sym, K, kps, class_F > 0 ? 1 : 0, C,
+    return launch_chained(tc::k_tc_gemm_nt_x3, grid, dim3(tc::kThreads), smem, st, tmA, tmB, M, N, b_box_rows, sym, K, kps, class_F > 0 ? 1 : 0, C,
                           ldc, split_stride, stages, stage_bytes, G, 0, 0, err);
 }
 
@@ -410,7 +407,7 @@ cudaError_t launch_tc_gram_direct(const float* Bold, int64_t pitch, int old_rows
     dim3 grid(1u, 1u, (unsigned)splits);
     cudaError_t e = allow_smem((const void*)tc::k_tc_gemm_nt_x3, 227 * 1024);
     if (e != cudaSuccess) return e;
-    return launch_chained(tc::k_tc_gemm_nt_x3, grid, dim3(tc::kThreads), smem, st, tmA, tmB, M, M, 1, 0, 1, D, kps, 0, C, ldc, split_stride, stages,
+    return launch_chained(tc::k_tc_gemm_nt_x3, grid, dim3(tc::kThreads), smem, st, tmA, tmB, M, M, 0, 1, D, kps, 0, C, ldc, split_stride, stages,
                           stage_bytes, G, n_new, src_box, err);
 }
 
