@@ -1219,8 +1219,8 @@ static sage_status_t score_rows(sage_fd* h, const void* rows, sage_dtype_t dt, i
     // up to 8 waves go into one launch (fewer launch-scale overheads per pass)
     if (tc32_ok && h->S32split) sub_max *= 8;
     if (structured) {
-        // one plane per class (two with the pre-split sketch): keep the planes of a sub-chunk within 1 GiB
-        const int64_t per_row = (int64_t)oC * ((tc32_ok && h->S32split) ? 2 : 1) * ell * (int64_t)sizeof(float);
+        // one plane per class: keep the planes of a sub-chunk within 1 GiB
+        const int64_t per_row = (int64_t)oC * ell * (int64_t)sizeof(float);
         int64_t fit = ((int64_t)1 << 30) / per_row / 128 * 128;
         if (fit < 128) fit = 128;
         if (sub_max > fit) sub_max = fit;
@@ -1244,15 +1244,16 @@ static sage_status_t score_rows(sage_fd* h, const void* rows, sage_dtype_t dt, i
         const float* Zparts = nullptr;       // the projections of this sub-chunk as nplanes partial planes of sub x ell floats
         int nplanes = 1;
         if (tc32_ok) {
+            // sketches of at most 64 rows: a kernel of their own, against the pre-split sketch
+            const bool narrow = h->S32split != nullptr;
             const int splits = structured ? oC : pick_splits_waves((int)((sub + 127) / 128), K, 2048, 64);
-            // sketches of at most 64 rows: one wide MMA per K step against the pre-split sketch, two partial planes per K slice
-            const bool wide = h->S32split != nullptr;
-            const int planes = wide ? 2 * splits : splits;
+            const int planes = narrow ? project_planes(sub, K, class_F) : splits;
             ST_TRY(ensure(h, &h->zwork, &h->zwork_bytes, zred * planes));
             float* out = h->zwork;
             cudaError_t e = timed(h, K_PROJECT, 1, st, [&] {
-                return launch_tc_gemm_nt_x3(reinterpret_cast<const float*>(p + r0 * row_bytes), ld, wide ? h->S32split : S, h->pitch, (int)sub,
-                                            ell, K, splits, out, ell, (int64_t)sub * ell, wide ? 2 : 0, h->tc_err, st, class_F);
+                const float* g = reinterpret_cast<const float*>(p + r0 * row_bytes);
+                if (narrow) return launch_tc_project(g, ld, h->S32split, h->pitch, sub, ell, K, class_F, out, (int64_t)sub * ell, h->tc_err, st);
+                return launch_tc_gemm_nt_x3(g, ld, S, h->pitch, (int)sub, ell, K, splits, out, ell, (int64_t)sub * ell, 0, h->tc_err, st, class_F);
             });
             if (e == cudaSuccess) {
                 done = true;

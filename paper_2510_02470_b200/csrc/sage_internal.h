@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <algorithm>
 
 #include "sage.h"
 
@@ -98,8 +99,6 @@ cudaError_t launch_tc_gemm_nt(const void* A, sage_dtype_t dt, int64_t lda, const
 // launch_tc_gemm_nt; any N.
 // sym == 1 (a Gram matrix of at most 128 rows, A == Bm): two MMAs per K step instead of three; slice z then stores
 // T_z = hi*hi^T + 2*hi*lo^T and the Gram matrix is sum_z (T_z + T_z^T)/2: see launch_gram_sym_reduce.
-// sym == 2 (projection onto at most 64 sketch rows): Bm is the sketch already split by launch_split_tf32 (128 rows);
-// one MMA per K step; C receives 2 * splits partial planes (split_stride apart) whose sum is A * S^T (M x N).
 cudaError_t launch_tc_gemm_nt_x3(const float* A, int64_t lda, const float* Bm, int64_t ldb, int M, int N, int64_t K, int splits,
                                  float* C, int64_t ldc, int64_t split_stride, int sym, int* err, cudaStream_t st,
                                  int64_t class_F = 0);   // class slices as in launch_gemm_nt; needs class_F a multiple of 4
@@ -111,6 +110,16 @@ cudaError_t launch_tc_gram_direct(const float* Bold, int64_t pitch, int old_rows
 // Sums the slices of a Gram matrix in the symmetric form; n_off: slices of the 256 x 256 tile above the diagonal (more than 256 rows).
 cudaError_t launch_gram_sym_reduce(const float* parts, int splits, int64_t stride, int r, int64_t ldp, float* out, int64_t ldo,
                                    cudaStream_t st, int n_off = 0);
+
+// Projection of M fp32 rows onto a sketch of ell <= 64 rows (tc_project.cu), given as launch_split_tf32 leaves it: Z as partial planes
+// of M x ell floats at out, plane_stride apart, project_planes(M, K, class_F) of them. class_F as in launch_gemm_nt (a multiple of 4).
+// cudaErrorNotSupported where launch_tc_gemm_nt_x3 returns it.
+inline int64_t project_pairs(int64_t tiles, int64_t nkt) {      // of SMs: one for every 16 K tiles of 256 rows or for every row tile
+    return std::min<int64_t>(74, std::max(tiles, tiles * nkt / 16));
+}
+int project_planes(int64_t M, int64_t K, int64_t class_F);
+cudaError_t launch_tc_project(const float* rows, int64_t ld, const float* sk_split, int64_t lds, int64_t M, int ell, int64_t K, int64_t class_F,
+                              float* out, int64_t plane_stride, int* err, cudaStream_t st);
 
 // Gram matrix of 129 to 512 rows (tc_gram_pair.cu): partials of K slice z at C + z * split_stride, n_diag slices of the 256 x 256 tiles on
 // the diagonal in the symmetric form (launch_gram_sym_reduce), n_off of the one above it (0 without one). ldc a multiple of 4, C

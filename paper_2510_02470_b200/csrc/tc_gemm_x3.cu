@@ -1,6 +1,7 @@
 // fp32-faithful tensor-core contraction C[z] = A_z * B_z^T for fp32 operands (both contiguous along the
 // contraction index): the Gram matrix K = B B^T of a sketch buffer of at most 128 rows (Method, first paragraph: the SVD of
-// the buffer is taken through the eigen-decomposition of B B^T; larger buffers: tc_gram_pair.cu) and the pass-2 projection of fp32 rows.
+// the buffer is taken through the eigen-decomposition of B B^T; larger buffers: tc_gram_pair.cu) and the pass-2 projection of fp32 rows onto
+// more than 64 sketch rows (fewer: tc_project.cu).
 //
 // Two things keep fp32 fidelity on tensor cores:
 //   * tcgen05 kind::tf32 reads an fp32 word by ignoring its low 13 bits (11 significant bits), so every value x
@@ -25,17 +26,10 @@
 // The producer and the MMA thread keep running stage / phase / chunk counters and advance the operand descriptors by a
 // constant per stage: with integer divisions and freshly built descriptors in its loop the single MMA-issuing thread took
 // 1,500 cycles per K tile and was what bounded the kernel (now about 600).
-// Of a Gram matrix (sym mode) only one operand tile is loaded and used on both sides, and it needs ONE 256-wide MMA per K step: the hi tile and the lo tile lie back to back
-// in the stage and serve as one 256-row B operand, so the accumulator holds hi*hi^T | hi*lo^T side by side; the drain
-// forms T = hi*hi^T + 2*hi*lo^T (the doubling is exact), which satisfies (T + T^T)/2 = hi*hi^T + hi*lo^T + lo*hi^T,
-// formed by the split reduction. (A 128 x 128 x 8 tf32 MMA executes in about 70 cycles, less than issuing it costs
-// the issuing thread: narrow MMAs leave the tensor pipe idle, wide ones do not.)
-// The projection of fp32 rows onto a sketch of at most 64 rows (proj mode, sym = 2) uses the same wide form with the
-// operands' roles exchanged: the sketch, split once into [hi (64 rows) ; lo (64 rows)] when it was frozen, is the
-// 128-row A operand and needs no work per stage; the tile of 128 data rows is split by the workers into hi | lo and
-// serves as one 256-row B operand. One MMA per K step leaves S_hi (G_hi | G_lo) on TMEM lanes 0-63 and
-// S_lo (G_hi | G_lo) on lanes 64-127; the drain adds the two column halves, and the lane halves are stored as two
-// partial planes of the (transposed) output, which the split reduction sums with the K slices.
+// Of a Gram matrix (sym mode) only one operand tile is loaded and used on both sides, and it needs ONE 256-wide MMA per K step: the hi
+// tile and the lo tile lie back to back in the stage and serve as one 256-row B operand, so the accumulator holds hi*hi^T | hi*lo^T
+// side by side; the drain forms T = hi*hi^T + 2*hi*lo^T (the doubling is exact), which satisfies
+// (T + T^T)/2 = hi*hi^T + hi*lo^T + lo*hi^T, formed by the split reduction.
 #include "sage_internal.h"
 #include "tc05.cuh"
 
@@ -69,11 +63,9 @@ k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int m0 = blockIdx.x * kTileM, n0 = blockIdx.y * kTileN;
-    const bool proj = sym == 2;
-    const bool wide = sym != 0;                           // one 256-wide MMA per K step
-    const bool diag = sym == 1;                           // A tile == B tile: load once
-    // stage layout: [hi: A | B][lo: A | B]; sym: no separate B; proj: [hi: rows][lo: rows][sketch]
-    const int half_bytes = (diag || proj) ? kTileBytes : kTileBytes + b_box_rows * 128;
+    const bool diag = sym != 0;                           // A tile == B tile: load once, one 256-wide MMA per K step
+    // stage layout: [hi: A | B][lo: A | B]; sym: no separate B
+    const int half_bytes = diag ? kTileBytes : kTileBytes + b_box_rows * 128;
     // direct_new > 0 (a symmetric Gram matrix of at most 128 rows whose last direct_new rows are still bfloat16 rows in the
     // caller's memory): tmA covers the first M - direct_new + 1 buffer rows (the last of them is a placeholder), tmB the
     // caller's rows (boxes of direct_box rows x 64 bytes, no swizzle) which land behind the two tiles of the stage; the
@@ -95,11 +87,10 @@ k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const int nkt = k_end > k_begin ? (int)((k_end - k_begin + BK - 1) / BK) : 0;
     const int kChunk = kChunkTiles;
     const int nchunks = (nkt + kChunk - 1) / kChunk;
-    const int acc_cols = wide ? 2 * kTileN : kTileN;      // sym: P and 2Q side by side; proj: hi and lo columns of the rows
+    const int acc_cols = diag ? 2 * kTileN : kTileN;      // sym: P and 2Q side by side
     const int ring = (kAccs * kTileN) / acc_cols;         // accumulators in flight: 4, or 2 in sym mode
     int n_pad = N - n0 < kTileN ? N - n0 : kTileN;        // MMA width of this tile, a multiple of 16
     n_pad = ((n_pad + 15) / 16) * 16;
-    if (proj) n_pad = kTileN;                             // accumulator columns are the 128 data rows of the tile
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) {
@@ -137,12 +128,12 @@ k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             uint32_t ph = 1;                                    // parity of the empty-barrier phase to wait for
             int x = (int)k_begin, xa = a_shared ? 0 : (int)k_begin;   // class slices: the same columns of A for every slice
             uint8_t* st = smem;
-            const uint32_t tx_bytes = direct_new ? (uint32_t)((old_rows + 1) * 128 + direct_box * 64) : (uint32_t)(proj ? 2 * kTileBytes : half_bytes);
+            const uint32_t tx_bytes = direct_new ? (uint32_t)((old_rows + 1) * 128 + direct_box * 64) : (uint32_t)half_bytes;
             for (int kt = 0; kt < nkt; ++kt) {
                 if (!mbar_wait(&empty[s], ph, abort)) break;
                 mbar_expect_tx(&full[s], tx_bytes);
                 tma_load_2d(st, &tmA, &full[s], xa, m0);
-                if (proj || direct_new) tma_load_2d(st + 2 * kTileBytes, &tmB, &full[s], x, 0);
+                if (direct_new) tma_load_2d(st + 2 * kTileBytes, &tmB, &full[s], x, 0);
                 else if (!diag) tma_load_2d(st + kTileBytes, &tmB, &full[s], x, n0);
                 issued = kt + 1;
                 x += BK;
@@ -156,13 +147,13 @@ k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t idesc = instr_desc(2, kTileM, wide ? 2 * kTileN : n_pad, 0, 0);
+            const uint32_t idesc = instr_desc(2, kTileM, diag ? 2 * kTileN : n_pad, 0, 0);
             // everything but the start address of an operand descriptor (see smem_desc_k_sw128); the addresses advance by
             // stage_bytes per stage
             const uint64_t desc_hi = smem_desc_k_sw128(0);
             const uint32_t st0 = smem_u32(smem);
-            const uint32_t a_hi_off = proj ? 2 * kTileBytes : 0, a_lo_off = half_bytes;   // proj: A = the split sketch
-            const uint32_t b_hi_off = (diag || proj) ? 0 : kTileBytes, b_lo_off = b_hi_off + half_bytes;
+            const uint32_t a_lo_off = half_bytes;
+            const uint32_t b_hi_off = diag ? 0 : kTileBytes, b_lo_off = b_hi_off + half_bytes;
             int s = 0, in_chunk = 0, b = 0;
             uint32_t ph = 0, acc_par = 1;
             uint32_t st = st0;
@@ -170,9 +161,9 @@ k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 if (in_chunk == 0 && !mbar_wait(&acc_empty[b], acc_par, abort)) break;
                 if (!mbar_wait(&split_done[s], ph, abort)) break;
                 tc_fence_after();
-                const uint64_t d_ahi = desc_hi | ((st + a_hi_off) >> 4), d_bhi = desc_hi | ((st + b_hi_off) >> 4);
+                const uint64_t d_ahi = desc_hi | (st >> 4), d_bhi = desc_hi | ((st + b_hi_off) >> 4);
                 const uint32_t acc = tmem_base + (uint32_t)(b * acc_cols);
-                if (wide) {                                 // sym: B = [hi ; lo] (the drain doubles the lo half), proj: [hi ; lo]
+                if (diag) {                                 // sym: B = [hi ; lo] (the drain doubles the lo half)
                     mma_tf32(acc, d_ahi, d_bhi, idesc, in_chunk != 0);
                     mma_tf32(acc, d_ahi + 2, d_bhi + 2, idesc, 1);       // 4 x 8 tf32 elements per 128-byte row
                     mma_tf32(acc, d_ahi + 4, d_bhi + 4, idesc, 1);
@@ -200,7 +191,6 @@ k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     } else {
         // ---- workers: write the lo part of landed stages; drain finished accumulators ----
         const int chunks16 = direct_new ? old_rows * 8 : half_bytes / 16;     // direct: remainders of the buffer rows only
-        const float lo_scale = sym == 1 ? 2.f : 1.f;          // sym: the lo half of the accumulator counts twice (folded into the drain)
         const int quarter = warp & 3, chalf = (warp - 2) >> 2;
         const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + (uint32_t)(chalf * 64);
         float acc[64];
@@ -214,7 +204,7 @@ k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             if (!w) { ok = false; return; }
             tc_fence_after();
             // two TMEM loads in flight per wait (a wait after every load made the drain a third of the workers' time)
-            if (wide) {                                      // columns c and kTileN + c belong together
+            if (diag) {                                      // columns c and kTileN + c belong together, the latter count twice
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     if (chalf * 64 + 16 * q < n_pad) {
@@ -225,7 +215,7 @@ k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         tmem_ld_use(v0);
                         tmem_ld_use(v1);
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) acc[16 * q + j] += fmaf(lo_scale, __uint_as_float(v1[j]), __uint_as_float(v0[j]));
+                        for (int j = 0; j < 16; ++j) acc[16 * q + j] += fmaf(2.f, __uint_as_float(v1[j]), __uint_as_float(v0[j]));
                     }
                 }
             } else {
@@ -302,19 +292,7 @@ k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         while (ok && drained < nchunks) drain(drained++);
         chain_release();
         const int row = m0 + quarter * 32 + lane;
-        if (proj) {
-            // lane = sketch row (0-63: hi part, 64-127: lo part), register c = data row chalf * 64 + c of the tile:
-            // the output is stored transposed, 32 consecutive sketch rows of one data row per warp instruction
-            const int mrow = quarter * 32 + lane, plane = mrow >> 6, j = mrow & 63;
-            float* cbase = C + (2ll * blockIdx.z + plane) * split_stride + j;
-            if (j < N) {
-#pragma unroll
-                for (int c = 0; c < 64; ++c) {
-                    const int r = m0 + chalf * 64 + c;
-                    if (r < M) cbase[(long long)r * ldc] = acc[c];
-                }
-            }
-        } else if (row < M) {
+        if (row < M) {
             float* crow = C + (long long)blockIdx.z * split_stride + (long long)row * ldc + n0 + chalf * 64;
             const bool vec = (ldc % 4 == 0) && ((reinterpret_cast<uintptr_t>(C) & 15u) == 0) && (split_stride % 4 == 0);
 #pragma unroll
@@ -350,24 +328,22 @@ cudaError_t launch_tc_gemm_nt_x3(const float* A, int64_t lda, const float* Bm, i
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
     if (splits < 1 || splits > 65535) return cudaErrorNotSupported;
     const bool gram = sym == 1;       // Bm is A
-    const bool proj = sym == 2;       // Bm: the sketch split into [hi (64 rows) ; lo (64 rows)], 128 rows of pitch ldb; N <= 64
     if (gram && (A != Bm || lda != ldb || M != N || M > tc::kTileM)) return cudaErrorInvalidValue;
-    if (proj && N > 64) return cudaErrorInvalidValue;
     // class slices: see launch_tc_gemm_nt
     if (class_F > 0 && (gram || class_F % 4 != 0 || (int64_t)splits * class_F != K)) return cudaErrorNotSupported;
     CUtensorMap tmA, tmB;
     if (!tc::make_tmap_2d(&tmA, A, 4, (uint64_t)M, (uint64_t)(class_F > 0 ? class_F : K), (uint64_t)lda, tc::kTileM)) return cudaErrorNotSupported;
-    const int b_box_rows = proj ? tc::kTileN : (N >= tc::kTileN ? tc::kTileN : ((N + 15) / 16) * 16);
+    const int b_box_rows = N >= tc::kTileN ? tc::kTileN : ((N + 15) / 16) * 16;
     if (gram) tmB = tmA;                              // not used
-    else if (!tc::make_tmap_2d(&tmB, Bm, 4, (uint64_t)(proj ? 128 : N), (uint64_t)K, (uint64_t)ldb, (uint32_t)b_box_rows)) return cudaErrorNotSupported;
+    else if (!tc::make_tmap_2d(&tmB, Bm, 4, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, (uint32_t)b_box_rows)) return cudaErrorNotSupported;
     int64_t kps = (K + splits - 1) / splits;
     kps = ((kps + tc::BK - 1) / tc::BK) * tc::BK;
     if (class_F > 0) kps = class_F;
     // a trailing slice may be empty after rounding to whole K tiles: its CTAs store zeros
     // a Gram matrix is one tile: one operand per stage
-    const int stage_bytes = proj ? 3 * tc::kTileBytes : 2 * (gram ? tc::kTileBytes : tc::kTileBytes + b_box_rows * 128);
-    // Long K slices of the one-MMA-per-step forms (16 KB of remainders per stage): as many stages as fit the 227 KB a block
-    // may have (7 of 32 KB, 4 of 48 KB), each slot with a worker group of its own (8 / stages warps), so that many
+    const int stage_bytes = 2 * (gram ? tc::kTileBytes : tc::kTileBytes + b_box_rows * 128);
+    // Long K slices of the one-MMA-per-step form (16 KB of remainders per stage): as many stages as fit the 227 KB a block
+    // may have (7 of 32 KB), each slot with a worker group of its own (8 / stages warps), so that many
     // remainder chains overlap. Short slices, and the three-MMA form (32 KB of remainders per stage, 3 stages): the
     // eight warps work on a stage together (odd number of stages) or as two groups of four on alternate stages, which
     // finishes a single stage sooner.
@@ -377,7 +353,7 @@ cudaError_t launch_tc_gemm_nt_x3(const float* A, int64_t lda, const float* Bm, i
     if (stages < 2) return cudaErrorNotSupported;
     const int G = deep ? stages : ((stages & 1) ? 1 : 2);
     const size_t smem = (size_t)stages * stage_bytes + 1024 + (3 * stages + 2 * tc::kAccs) * 8 + 16;
-    dim3 grid((unsigned)((M + tc::kTileM - 1) / tc::kTileM), proj ? 1u : (unsigned)((N + tc::kTileN - 1) / tc::kTileN), (unsigned)splits);
+    dim3 grid((unsigned)((M + tc::kTileM - 1) / tc::kTileM), (unsigned)((N + tc::kTileN - 1) / tc::kTileN), (unsigned)splits);
     cudaError_t e = allow_smem((const void*)tc::k_tc_gemm_nt_x3, 227 * 1024);
     if (e != cudaSuccess) return e;
     return launch_chained(tc::k_tc_gemm_nt_x3, grid, dim3(tc::kThreads), smem, st, tmA, tmB, M, N, b_box_rows, sym, K, kps, class_F > 0 ? 1 : 0, C,

@@ -35,11 +35,6 @@ constexpr int kRunTiles = 8;                // as tc_gemm_x3.cu: 96 additions be
 constexpr int kHiTiles = 8, kLoTiles = 6;
 constexpr size_t kPairSmem = 1024 + (size_t)(kHiTiles + kLoTiles) * kOpBytes + (2 * kHiTiles + kLoTiles + 4) * 8 + 16;
 
-__device__ __forceinline__ uint32_t remainder_of(uint32_t x, float scale) {
-    const float l = scale * (__uint_as_float(x) - __uint_as_float(x & 0xffffe000u));
-    return (__float_as_uint(l) + 0x1000u) & 0xffffe000u;
-}
-
 __global__ void __launch_bounds__(kPairThreads, 1)
 k_tc_gram_pair(const __grid_constant__ CUtensorMap tm, int r, long long K, int n_diag, int n_off, float* __restrict__ C, long long ldc,
                long long split_stride, int* __restrict__ err) {
@@ -193,7 +188,7 @@ k_tc_gram_pair(const __grid_constant__ CUtensorMap tm, int r, long long K, int n
                 for (int u = 0; u < 4; ++u) v[u] = hi[u * nt];
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
-                    lo[u * nt] = make_uint4(remainder_of(v[u].x, scale), remainder_of(v[u].y, scale), remainder_of(v[u].z, scale), remainder_of(v[u].w, scale));
+                    lo[u * nt] = make_uint4(remainder_tf32(v[u].x, scale), remainder_tf32(v[u].y, scale), remainder_tf32(v[u].z, scale), remainder_tf32(v[u].w, scale));
             }
             fence_proxy_async_smem();                       // the tensor cores read these writes
             __syncwarp();
