@@ -9,11 +9,10 @@
 // the split warps write lo = x - hi into a second buffer; W arrives already split from global memory as two stacked operands [W_hi; W_lo],
 // so one MMA of width 2*j_pad gives hi*W_hi and hi*W_lo side by side and a second one adds lo*W_hi; the
 // epilogue adds the two halves. One TMEM accumulator takes at most 8 chunks (256 buffer rows) this way; more than 256 buffer rows
-// or more than 128 output rows go to k_tc_rebuild_wide.
+// or more than 128 output rows go to k_tc_rebuild_wide, factors that fit shared memory as a whole to k_tc_rebuild_narrow. Here:
 //
 //   warp 0    TMA producer: per chunk 4 boxes of [32 rows][32 columns] of the buffer (128-byte swizzle with
-//             32-byte atoms, the only layout the tensor cores take for 32-bit MN-major operands) and one box of W; where
-//             all chunk boxes of W fit 64 KB (up to 128 buffer rows onto 64 output rows) they are loaded once and stay,
+//             32-byte atoms, the only layout the tensor cores take for 32-bit MN-major operands) and one box of W,
 //   warp 1    TMEM allocation, MMA issue into two ping-pong accumulators (one per column tile),
 //   warps 2-5 write the lo part of the buffer tile of each landed stage,
 //   warps 6-9 epilogue: TMEM -> registers -> out.
@@ -34,8 +33,8 @@ constexpr int kSpanBytes = kChunkRows * 128;         // 4 KB
 
 // The remainders of a landed chunk, by kSplitThreads threads. The tensor cores ignore the low 13 bits of an fp32 word, so the raw
 // tile is the hi operand as it stands; lo = x - hi (exact), rounded to 11 significant bits so that the same truncation cuts
-// nothing from it. Row zero_row gets remainders of zero.
-__device__ __forceinline__ void split_chunk(const uint4* hi, uint4* lo, int t, int zero_row = -1) {
+// nothing from it.
+__device__ __forceinline__ void split_chunk(const uint4* hi, uint4* lo, int t) {
 #pragma unroll
     for (int cc = 0; cc < kBufBytes / 16 / kSplitThreads; ++cc) {
         const int idx = t + cc * kSplitThreads;
@@ -45,37 +44,24 @@ __device__ __forceinline__ void split_chunk(const uint4* hi, uint4* lo, int t, i
         l.y = (__float_as_uint(__uint_as_float(v.y) - __uint_as_float(v.y & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
         l.z = (__float_as_uint(__uint_as_float(v.z) - __uint_as_float(v.z & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
         l.w = (__float_as_uint(__uint_as_float(v.w) - __uint_as_float(v.w & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
-        if (((idx >> 3) & 31) == zero_row) l = make_uint4(0u, 0u, 0u, 0u);
         lo[idx] = l;
     }
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
-k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmSrc,
-             const __grid_constant__ CUtensorMap tmSrc1, int direct_new, int r, int keep, int j_pad,
-             long long pitch, long long num_tiles, float* __restrict__ out, int stages, int w_res, int* __restrict__ err) {
+k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ CUtensorMap tmW, int r, int keep, int j_pad,
+             long long pitch, long long num_tiles, float* __restrict__ out, int stages, int* __restrict__ err) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    // stage layout: [buffer hi 16 KB][buffer lo 16 KB][W_hi ; W_lo: 2*j_pad rows of 128 bytes]; w_res: the W boxes of all
-    // chunks are loaded once and stay behind the ring (W does not depend on the column tile), the stages hold buffer data only
-    const int w_bytes = 2 * j_pad * 128;
-    // direct_new > 0 (needs w_res): the last direct_new of the r rows are bfloat16 rows in the caller's memory. Rows
-    // 0 .. r - direct_new - 1 come from the buffer as usual; r - direct_new is the last row of its chunk of 32 (cb), so that
-    // chunk gets one bfloat16 row (tmSrc1) and the chunks after it 32 each (tmSrc) into an 8 KB staging area behind the two
-    // buffer tiles; the split warps convert them into the operand layout (32-byte atoms: chunk j of k row rr sits in slot
-    // ((j >> 1) ^ (rr & 3)) * 2 + (j & 1) of its 128-byte span row). Their remainders are zero, so chunks after cb take one
-    // MMA per K step instead of two.
-    const int stage_bytes = (w_res ? 2 * kBufBytes : 2 * kBufBytes + w_bytes) + (direct_new ? 8192 : 0);
-    const int cb = direct_new ? (r - direct_new) / kChunkRows : 1 << 30;
+    // stage layout: [buffer hi 16 KB][buffer lo 16 KB][W_hi ; W_lo: 2*j_pad rows of 128 bytes]
+    const int w_bytes = 2 * j_pad * 128, stage_bytes = 2 * kBufBytes + w_bytes;
     const int nchunk = (r + kChunkRows - 1) / kChunkRows;
-    uint8_t* wres = smem + (size_t)stages * stage_bytes;
-    uint64_t* full = reinterpret_cast<uint64_t*>(wres + (w_res ? (size_t)nchunk * w_bytes : 0));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)stages * stage_bytes);
     uint64_t* split_done = full + stages;
     uint64_t* empty = split_done + stages;
     uint64_t* acc_full = empty + stages;                   // [2]
     uint64_t* acc_empty = acc_full + 2;                    // [2]
-    uint64_t* w_full = acc_empty + 2;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(w_full + 1);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
     volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -91,7 +77,6 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
             mbar_init(&split_done[s], kSplitThreads);
             mbar_init(&empty[s], 1);
         }
-        mbar_init(w_full, 1);
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], kEpiThreads);
@@ -115,31 +100,19 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
             int s = 0;
             uint32_t ph = 1;                                // parity of the empty-barrier phase to wait for
             uint8_t* st = smem;
-            const uint32_t tx_bytes = (uint32_t)(w_res ? kBufBytes : kBufBytes + w_bytes);
-            if (w_res) {
-                mbar_expect_tx(w_full, (uint32_t)(nchunk * w_bytes));
-                for (int c = 0; c < nchunk; ++c) tma_load_2d(wres + (size_t)c * w_bytes, &tmW, w_full, c * kChunkRows, 0);
-            }
             for (long long lt = 0; lt < my_tiles && alive; ++lt) {
                 const int d0 = (int)((blockIdx.x + lt * gridDim.x) * kTileD);
                 for (int c = 0; c < nchunk; ++c) {
                     if (!mbar_wait(&empty[s], ph, abort)) { alive = false; break; }
-                    if (c > cb) {                               // caller's rows only
-                        mbar_expect_tx(&full[s], 8192u);
-                        tma_load_2d(st + 2 * kBufBytes, &tmSrc, &full[s], d0, 1 + (c - cb - 1) * kChunkRows);
-                    } else {
-                        mbar_expect_tx(&full[s], c == cb ? tx_bytes + 256u : tx_bytes);
+                    mbar_expect_tx(&full[s], (uint32_t)(kBufBytes + w_bytes));
 #pragma unroll
-                        for (int sp = 0; sp < 4; ++sp) tma_load_2d(st + sp * kSpanBytes, &tmBuf, &full[s], d0 + 32 * sp, c * kChunkRows);
-                        if (c == cb) tma_load_2d(st + 2 * kBufBytes, &tmSrc1, &full[s], d0, 0);
-                        if (!w_res) tma_load_2d(st + 2 * kBufBytes, &tmW, &full[s], c * kChunkRows, 0);
-                    }
+                    for (int sp = 0; sp < 4; ++sp) tma_load_2d(st + sp * kSpanBytes, &tmBuf, &full[s], d0 + 32 * sp, c * kChunkRows);
+                    tma_load_2d(st + 2 * kBufBytes, &tmW, &full[s], c * kChunkRows, 0);
                     ++issued;
                     if (++s == stages) { s = 0; ph ^= 1u; st = smem; } else { st += stage_bytes; }
                 }
             }
             if (*abort) {
-                if (w_res) mbar_wait_quiet(w_full, 0, 20000000ll);
                 for (long long k = issued > stages ? issued - stages : 0; k < issued; ++k)
                     mbar_wait_quiet(&full[k % stages], (uint32_t)(k / stages) & 1u, 20000000ll);
             }
@@ -155,8 +128,6 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
             bool alive = true;
             int s = 0;
             uint32_t ph = 0, st = st0;
-            const uint32_t wres0 = smem_u32(wres);
-            if (w_res) alive = mbar_wait(w_full, 0, abort);
             for (long long lt = 0; lt < my_tiles && alive; ++lt) {
                 const int b = (int)(lt & 1);
                 const uint32_t par = (uint32_t)(lt >> 1);
@@ -166,12 +137,12 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
                     const uint32_t acc = tmem_base + (uint32_t)(b * n_mma);
                     if (!mbar_wait(&split_done[s], ph, abort)) { alive = false; break; }
                     tc_fence_after();
-                    const uint64_t d_w = desc_w | ((w_res ? wres0 + (uint32_t)(c * w_bytes) : st + 2 * kBufBytes) >> 4);
+                    const uint64_t d_w = desc_w | ((st + 2 * kBufBytes) >> 4);
                     const uint64_t d_hi = desc_buf | (st >> 4), d_lo = desc_buf | ((st + kBufBytes) >> 4);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {          // 8 buffer rows per MMA: one 1024-byte row group (64 descriptor units)
                         mma_tf32(acc, d_hi + 64 * k, d_w + 2 * k, idesc_fold, (c | k) != 0);   // hi*W_hi | hi*W_lo
-                        if (c <= cb) mma_tf32(acc, d_lo + 64 * k, d_w + 2 * k, idesc_half, 1);     // + lo*W_hi (zero for bfloat16 rows)
+                        mma_tf32(acc, d_lo + 64 * k, d_w + 2 * k, idesc_half, 1);     // + lo*W_hi
                     }
                     mma_commit(&empty[s]);
                     if (++s == stages) { s = 0; ph ^= 1u; st = st0; } else { st += (uint32_t)stage_bytes; }
@@ -182,32 +153,12 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
     } else if (warp < 6) {
         const int t = threadIdx.x - 64;
         const long long total = my_tiles * nchunk;
-        int s = 0, c = 0;                               // stage slot and chunk (32 buffer rows) of the current tile
+        int s = 0;
         uint32_t ph = 0;
         for (long long q = 0; q < total; ++q) {
             if (!mbar_wait(&full[s], ph, abort)) break;
             uint4* hi = reinterpret_cast<uint4*>(smem + (size_t)s * stage_bytes);
-            uint4* lo = reinterpret_cast<uint4*>(smem + (size_t)s * stage_bytes + kBufBytes);
-            if (c <= cb) {
-                // the last row of chunk cb is a placeholder for the caller's first row (a bfloat16 row: remainder zero)
-                split_chunk(hi, lo, t, c == cb ? kChunkRows - 1 : -1);
-            }
-            if (c >= cb) {
-                // bfloat16 rows from the staging area (256 bytes = 128 columns per row): 8 values -> two chunks of 4 floats
-                const uint4* src = reinterpret_cast<const uint4*>(smem + (size_t)s * stage_bytes + 2 * kBufBytes);
-                const int n_in = c == cb ? 16 : kChunkRows * 16;
-                for (int i = t; i < n_in; i += kSplitThreads) {
-                    const int rr = c == cb ? kChunkRows - 1 : i >> 4, q8 = i & 15;     // k row within the chunk, group of 8 columns
-                    const uint4 v = src[i];
-                    const uint4 a = make_uint4(v.x << 16, v.x & 0xffff0000u, v.y << 16, v.y & 0xffff0000u);
-                    const uint4 b = make_uint4(v.z << 16, v.z & 0xffff0000u, v.w << 16, v.w & 0xffff0000u);
-                    const int span = q8 >> 2, j = (q8 & 3) * 2;                          // 32-column span, 16-byte chunk within its row
-                    uint4* row = hi + span * (kSpanBytes / 16) + rr * 8;
-                    row[(((j >> 1) ^ (rr & 3)) << 1) | (j & 1)] = a;
-                    row[((((j + 1) >> 1) ^ (rr & 3)) << 1) | ((j + 1) & 1)] = b;
-                }
-            }
-            if (++c == nchunk) c = 0;
+            split_chunk(hi, hi + kBufBytes / 16, t);
             fence_proxy_async_smem();
             mbar_arrive(&split_done[s]);
             if (++s == stages) { s = 0; ph ^= 1u; }
@@ -269,6 +220,211 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
             mbar_wait_quiet(&acc_full[(my_tiles - 1) & 1], (uint32_t)((my_tiles - 1) >> 1) & 1u, kWaitLimitCycles);
         tc_fence_after();
         tmem_dealloc(tmem_base, tmem_cols);
+    }
+    if (threadIdx.x == 0 && *abort) atomicExch(err, 1);
+}
+
+// Up to 64 output rows whose factors, all chunks of them, take 64 KB (up to 128 buffer rows): they are loaded once and stay, and the
+// remainders go to TMEM, as the A operand of the second product, instead of shared memory: no store and no proxy fence for the split,
+// and a stage is the landed chunk alone, so that eight are in flight.
+// direct_new > 0: the last direct_new of the r rows are bfloat16 rows in the caller's memory. Row r - direct_new is the last row of its
+// chunk (cb), which gets one bfloat16 row (tmSrc1) in place of a placeholder; the chunks after it are 32 of them each (tmSrc). These
+// go to TMEM as they are: their remainders are zero, one product is all.
+//   warp 0 loads, warp 1 issues MMAs, warps 2-9 write remainders in two groups in turn (thread = buffer column), warps 10-13 are the epilogue.
+// Bound by DRAM. 128 rows of 11.2 M columns onto 63, half of them read in place: 1,600 -> 1,533 us against remainders in shared memory and
+// four chunks in flight (7.1 GB: 4.6 TB/s); of 262,144 columns 49 -> 47 us; short rows equal.
+constexpr int kNarrowThreads = 448;
+constexpr int kSlots = 8;                   // chunks in shared memory and, their remainders, in TMEM
+constexpr int kSlotBytes = kBufBytes + 1024;          // 16 KB of fp32 rows or 8 KB of bfloat16 rows, and the one bfloat16 row of chunk cb
+constexpr int kResidentBytes = 64 * 1024;
+constexpr uint32_t kLoCols = 256;           // TMEM: two accumulators of up to 128 columns, then the remainders, 32 columns each
+constexpr size_t kNarrowSmem = 1024 + (size_t)kSlots * kSlotBytes + kResidentBytes + (3 * kSlots + 5) * 8 + 16;
+
+__global__ void __launch_bounds__(kNarrowThreads, 1)
+k_tc_rebuild_narrow(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmSrc,
+                    const __grid_constant__ CUtensorMap tmSrc1, int direct_new, int r, int keep, int j_pad, long long pitch, long long num_tiles,
+                    float* __restrict__ out, int* __restrict__ err) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    uint8_t* wres = smem + kSlots * kSlotBytes;
+    uint64_t* full = reinterpret_cast<uint64_t*>(wres + kResidentBytes);
+    uint64_t* split_done = full + kSlots;
+    uint64_t* empty = split_done + kSlots;
+    uint64_t* acc_full = empty + kSlots;                   // [2]
+    uint64_t* acc_empty = acc_full + 2;                    // [2]
+    uint64_t* w_full = acc_empty + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(w_full + 1);
+    volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int w_bytes = 2 * j_pad * 128, n_mma = 2 * j_pad;           // n_mma <= 128
+    const int nchunk = (r + kChunkRows - 1) / kChunkRows;
+    const int cb = direct_new ? (r - direct_new) / kChunkRows : 1 << 30;
+    const long long my_tiles = num_tiles > blockIdx.x ? (num_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kSlots; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&split_done[s], 4);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(w_full, 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], kEpiThreads);
+        }
+        *abort = 0;
+        mbar_fence_init();
+        tma_prefetch_desc(&tmBuf);
+        tma_prefetch_desc(&tmW);
+    }
+    if (warp == 1) tmem_alloc(tmem_slot, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    chain_wait();
+
+    if (warp == 0) {
+        if (lane == 0) {
+            long long issued = 0;
+            bool alive = true;
+            int s = 0;
+            uint32_t ph = 1;
+            mbar_expect_tx(w_full, (uint32_t)(nchunk * w_bytes));
+            for (int c = 0; c < nchunk; ++c) tma_load_2d(wres + (size_t)c * w_bytes, &tmW, w_full, c * kChunkRows, 0);
+            for (long long lt = 0; lt < my_tiles && alive; ++lt) {
+                const int d0 = (int)((blockIdx.x + lt * gridDim.x) * kTileD);
+                for (int c = 0; c < nchunk; ++c) {
+                    if (!mbar_wait(&empty[s], ph, abort)) { alive = false; break; }
+                    uint8_t* st = smem + (size_t)s * kSlotBytes;
+                    if (c > cb) {                               // caller's rows only
+                        mbar_expect_tx(&full[s], 8192u);
+                        tma_load_2d(st, &tmSrc, &full[s], d0, 1 + (c - cb - 1) * kChunkRows);
+                    } else {
+                        mbar_expect_tx(&full[s], (uint32_t)(c == cb ? kBufBytes + 256 : kBufBytes));
+#pragma unroll
+                        for (int sp = 0; sp < 4; ++sp) tma_load_2d(st + sp * kSpanBytes, &tmBuf, &full[s], d0 + 32 * sp, c * kChunkRows);
+                        if (c == cb) tma_load_2d(st + kBufBytes, &tmSrc1, &full[s], d0, 0);
+                    }
+                    ++issued;
+                    if (++s == kSlots) { s = 0; ph ^= 1u; }
+                }
+            }
+            if (*abort) {
+                mbar_wait_quiet(w_full, 0, 20000000ll);
+                for (long long k = issued > kSlots ? issued - kSlots : 0; k < issued; ++k)
+                    mbar_wait_quiet(&full[k % kSlots], (uint32_t)(k / kSlots) & 1u, 20000000ll);
+            }
+        }
+    } else if (warp == 1) {
+        const uint32_t idesc_hi = instr_desc(2, kTileD, n_mma, 1, 0), idesc_lo = instr_desc(2, kTileD, j_pad, 0, 0);
+        const uint32_t idesc_new = instr_desc(2, kTileD, n_mma, 0, 0);
+        const uint64_t desc_w = smem_desc_k_sw128(0), desc_buf = smem_desc_mn_sw128_atom32(0, kSpanBytes);
+        const uint32_t st0 = smem_u32(smem), w0 = smem_u32(wres);
+        int s = 0;
+        uint32_t ph = 0;
+        bool alive = __all_sync(0xffffffffu, mbar_wait(w_full, 0, abort));
+        for (long long lt = 0; lt < my_tiles && alive; ++lt) {
+            const uint32_t b = (uint32_t)(lt & 1), acc = tmem_base + b * 128u;
+            alive = __all_sync(0xffffffffu, mbar_wait(&acc_empty[b], ((uint32_t)(lt >> 1) & 1u) ^ 1u, abort));
+            for (int c = 0; c < nchunk && alive; ++c) {
+                alive = __all_sync(0xffffffffu, mbar_wait(&split_done[s], ph, abort));
+                if (!alive) break;
+                tc_fence_after();
+                const uint64_t d_w = desc_w | ((w0 + (uint32_t)(c * w_bytes)) >> 4), d_hi = desc_buf | ((st0 + (uint32_t)(s * kSlotBytes)) >> 4);
+                const uint32_t lo = tmem_base + kLoCols + (uint32_t)(s * 32);
+                if (elect_one()) {
+                    if (c > cb) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) mma_tf32_ts(acc, lo + 8 * k, d_w + 2 * k, idesc_new, 1);
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {      // 8 buffer rows per MMA: one 1024-byte row group (64 descriptor units)
+                            mma_tf32(acc, d_hi + 64 * k, d_w + 2 * k, idesc_hi, (c | k) != 0);        // hi*W_hi | hi*W_lo
+                            mma_tf32_ts(acc, lo + 8 * k, d_w + 2 * k, idesc_lo, 1);                    // + lo*W_hi
+                        }
+                    }
+                    mma_commit(&empty[s]);
+                    if (c == nchunk - 1) mma_commit(&acc_full[b]);
+                }
+                __syncwarp();
+                if (++s == kSlots) { s = 0; ph ^= 1u; }
+            }
+        }
+    } else if (warp < 10) {
+        const int quarter = warp & 3, grp = (warp - 2) >> 2;
+        const uint32_t dst = tmem_base + kLoCols + (static_cast<uint32_t>(quarter * 32) << 16);
+        const int span = quarter * kSpanBytes;                              // this warp's 32 columns of a chunk of fp32 rows
+        const int piece = lane >> 3, in_piece = lane & 7;                   // 32-byte piece of a row (permuted by the row), float in it
+        const long long total = my_tiles * nchunk;
+        int c = grp % nchunk;
+        for (long long g = grp; g < total; g += 2) {                        // kSlots is even: a group sees every phase of its slots
+            const int s = (int)(g % kSlots);
+            bool ok = mbar_wait(&full[s], (uint32_t)(g / kSlots) & 1u, abort);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();                   // loaded after the MMAs of eight chunks ago: the columns of its remainders are free, too
+            uint8_t* st = smem + (size_t)s * kSlotBytes;
+            uint32_t v[32];
+            if (c > cb) {
+                const uint16_t* src = reinterpret_cast<const uint16_t*>(st) + quarter * 32 + lane;
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] = (uint32_t)src[i * kTileD] << 16;
+            } else {
+                float* hi = reinterpret_cast<float*>(st + span);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] = remainder_tf32(__float_as_uint(hi[i * 32 + ((piece ^ (i & 3)) << 3) + in_piece]));
+                if (c == cb) {                  // the caller's first row takes the placeholder's place
+                    const uint32_t x = (uint32_t)reinterpret_cast<const uint16_t*>(st + kBufBytes)[quarter * 32 + lane] << 16;
+                    hi[31 * 32 + ((piece ^ 3) << 3) + in_piece] = __uint_as_float(x);
+                    v[31] = 0u;
+                    fence_proxy_async_smem();
+                }
+            }
+            tmem_st32(dst + (uint32_t)(s * 32), v);
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&split_done[s]);
+            c += 2;
+            while (c >= nchunk) c -= nchunk;
+        }
+    } else {
+        const int quarter = warp & 3;
+        const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+        for (long long lt = 0; lt < my_tiles; ++lt) {
+            const uint32_t b = (uint32_t)(lt & 1);
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (uint32_t)(lt >> 1) & 1u, abort));
+            if (!ok) break;
+            tc_fence_after();
+            if (lt == my_tiles - 1) chain_release();
+            const long long d = (blockIdx.x + lt * gridDim.x) * kTileD + quarter * 32 + lane;
+            const uint32_t acc = lane_base + b * 128u;
+            for (int j0 = 0; j0 < j_pad; j0 += 16) {
+                uint32_t v0[16], w0[16];
+                tmem_ld16_issue(acc + (uint32_t)j0, v0);
+                tmem_ld16_issue(acc + (uint32_t)(j_pad + j0), w0);
+                tmem_ld_wait();
+                tmem_ld_use(v0);
+                tmem_ld_use(w0);
+                if (d < pitch) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (j0 + j < keep) out[(long long)(j0 + j) * pitch + d] = __uint_as_float(v0[j]) + __uint_as_float(w0[j]);
+                }
+            }
+            tc_fence_before();
+            mbar_arrive(&acc_empty[b]);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        if (my_tiles > 0 && !*abort)
+            mbar_wait_quiet(&acc_full[(my_tiles - 1) & 1], (uint32_t)((my_tiles - 1) >> 1) & 1u, kWaitLimitCycles);
+        tc_fence_after();
+        tmem_dealloc(tmem_base, 512);
     }
     if (threadIdx.x == 0 && *abort) atomicExch(err, 1);
 }
@@ -521,28 +677,30 @@ static cudaError_t launch_tc_rebuild_part(const float* Wsplit, int ldw, int j_pa
     if (kcols > ldw) return cudaErrorNotSupported;
     if (!tc::make_tmap_2d(&tmW, Wsplit, 4, (uint64_t)(2 * j_pad), (uint64_t)kcols, (uint64_t)ldw, (uint32_t)(2 * j_pad)))
         return cudaErrorNotSupported;
-    // W resident in shared memory when all its chunk boxes take at most 64 KB (up to 128 buffer rows onto 64 output rows)
-    const int nchunk = (r + tc::kChunkRows - 1) / tc::kChunkRows;
-    const size_t w_all = (size_t)nchunk * 2 * j_pad * 128;
-    const int w_res = w_all <= 64 * 1024 ? 1 : 0;
-    CUtensorMap tmSrc = tmW, tmSrc1 = tmW;
-    if (src) {
-        if (!w_res || n_new < 2 || n_new >= r || (r - n_new + 1) % tc::kChunkRows != 0 || r % tc::kChunkRows != 0) return cudaErrorNotSupported;
-        if (!tc::make_tmap_2d_plain(&tmSrc, src, 2, (uint64_t)n_new, (uint64_t)D, (uint64_t)ld_src, 128, (uint32_t)tc::kChunkRows) ||
-            !tc::make_tmap_2d_plain(&tmSrc1, src, 2, (uint64_t)n_new, (uint64_t)D, (uint64_t)ld_src, 128, 1))
-            return cudaErrorNotSupported;
-    }
-    const int stage_bytes = (w_res ? 2 * tc::kBufBytes : 2 * tc::kBufBytes + 2 * j_pad * 128) + (src ? 8192 : 0);
-    int stages = (int)((227 * 1024 - 1536 - (w_res ? w_all : 0)) / stage_bytes);
-    if (stages > 8) stages = 8;
-    if (stages < 2) return cudaErrorNotSupported;
-    const size_t smem = (size_t)stages * stage_bytes + (w_res ? w_all : 0) + 1024 + (3 * stages + 5) * 8 + 16;
     const long long num_tiles = (pitch + tc::kTileD - 1) / tc::kTileD;
     const int grid = (int)(num_tiles < 148 ? num_tiles : 148);
+    const int nchunk = kcols / tc::kChunkRows;
+    if (j_pad <= 64 && nchunk * 2 * j_pad * 128 <= tc::kResidentBytes) {
+        CUtensorMap tmSrc = tmW, tmSrc1 = tmW;
+        if (src) {
+            if (n_new < 2 || n_new >= r || (r - n_new + 1) % tc::kChunkRows != 0 || r % tc::kChunkRows != 0) return cudaErrorNotSupported;
+            if (!tc::make_tmap_2d_plain(&tmSrc, src, 2, (uint64_t)n_new, (uint64_t)D, (uint64_t)ld_src, 128, (uint32_t)tc::kChunkRows) ||
+                !tc::make_tmap_2d_plain(&tmSrc1, src, 2, (uint64_t)n_new, (uint64_t)D, (uint64_t)ld_src, 128, 1))
+                return cudaErrorNotSupported;
+        }
+        cudaError_t e = allow_smem((const void*)tc::k_tc_rebuild_narrow, 227 * 1024);
+        if (e != cudaSuccess) return e;
+        return launch_chained(tc::k_tc_rebuild_narrow, dim3(grid), dim3(tc::kNarrowThreads), tc::kNarrowSmem, st, tmBuf, tmW, tmSrc, tmSrc1,
+                              src ? n_new : 0, r, keep, j_pad, pitch, num_tiles, Bdst, err);
+    }
+    if (src) return cudaErrorNotSupported;
+    const int stage_bytes = 2 * tc::kBufBytes + 2 * j_pad * 128;
+    int stages = (227 * 1024 - 1536) / stage_bytes;
+    if (stages > 8) stages = 8;
+    const size_t smem = (size_t)stages * stage_bytes + 1024 + (3 * stages + 4) * 8 + 16;
     cudaError_t e = allow_smem((const void*)tc::k_tc_rebuild, 227 * 1024);
     if (e != cudaSuccess) return e;
-    return launch_chained(tc::k_tc_rebuild, dim3(grid), dim3(tc::kThreads), smem, st, tmBuf, tmW, tmSrc, tmSrc1, src ? n_new : 0, r, keep, j_pad, pitch,
-                          num_tiles, Bdst, stages, w_res, err);
+    return launch_chained(tc::k_tc_rebuild, dim3(grid), dim3(tc::kThreads), smem, st, tmBuf, tmW, r, keep, j_pad, pitch, num_tiles, Bdst, stages, err);
 }
 
 static cudaError_t launch_tc_rebuild_wide(const float* Wsplit, int ldw, int j_pad, const float* Bsrc, float* Bdst, int64_t pitch, int r, int keep,
