@@ -350,7 +350,7 @@ def run_workload(w, args, steps, warmup, ctx, want_e2e, want_cpu, sketches, fact
                 "algorithmic": "9*n^3 flop per n x n symmetric eigen-solve (textbook count)"}
     else:
         gbs = per_step_bytes.get(dominant, 0) / (dom_ms_per_step * 1e-3) / 1e9
-        kname = {"gram": "k_tc_gemm_nt_x3 (Gram)", "rebuild": "k_tc_rebuild", "append": "k_append",
+        kname = {"gram": "k_tc_gemm_nt_x3 (Gram)", "rebuild": "k_tc_rebuild (narrow, wide)", "append": "k_append",
                  "project": "k_tc_gemm_nt (projection)"}.get(dominant, dominant)
         traffic = NCU_TRAFFIC_PER_COLUMN.get((w.name, dominant))
         roof = {"kernel": kname, "bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
