@@ -439,8 +439,9 @@ k_tc_rebuild_narrow(const __grid_constant__ CUtensorMap tmBuf, const __grid_cons
 //   warp 0 loads buffer chunks, warp 1 issues MMAs, warp 2 loads factors, warps 4-7 write the lo parts, warps 8-15 are the
 //   epilogue (8-11: output rows 0-127, 12-15: the others).
 // 512 rows onto 255, 262,144 columns: 422 -> 282 us (two launches of the narrow kernel, each over the whole buffer, before: their
-// loads and hand-offs alone took 344 us). What bounds it is shared memory: a chunk writes 80 KB, its split moves 32 KB and its MMAs
-// read 144 KB, 2,050 cycles at 128 bytes each of the 2,400 that it takes; the MMAs themselves are 1,540.
+// loads and hand-offs alone took 344 us). A chunk loads 80 KB in its 2,400 cycles, the 34 bytes a cycle that bound the
+// loads of tc_project.cu too; shared memory is not far behind (80 KB written, 32 moved by the split, 144 read by MMAs: 2,050 cycles at 128
+// bytes); the MMAs alone are 1,540.
 constexpr int kWideThreads = 512;
 constexpr int kWideRegs = 128;              // what every thread is launched with: the sum of the shares below is 4 x 128 x 128
 constexpr int kBufStages = 3, kWSlots = 4;
