@@ -4,7 +4,7 @@
 // from the symmetric eigen-problem of K, and Sigma' V^T = diag(sigma'/sigma) U^T B.
 //
 // Method (direct, no iteration whose length depends on the data):
-//   1. K is scaled by 1 / max diagonal and reduced to a tridiagonal T = Q^T K Q by Householder reflections, fp32, the
+//   1. K is scaled by 1 / max diagonal, ordered by falling diagonal and reduced to a tridiagonal T = Q^T K Q by Householder reflections, fp32, the
 //      matrix in registers (k_tridiag). n <= 128: one thread block of 4 warps; larger: a cluster of 8 blocks works until
 //      128 rows are left, the one-block kernel does the rest.
 //   2. Every wanted eigenvalue of T (the kept ones and delta) is found by multisection on the sign changes of the
@@ -98,6 +98,7 @@ struct TriWork {
     float* trail;    // 128 x 128
     float* dmax;     // the scale K was divided by
     int* abort;      // raised by a block that gave up a wait
+    int* perm;       // G: row of K at each place of its order by falling diagonal
 };
 __host__ __device__ inline TriWork tri_work(float* w, int G) {
     TriWork t;
@@ -108,6 +109,7 @@ __host__ __device__ inline TriWork tri_work(float* w, int G) {
     t.trail = t.e + G;
     t.dmax = t.trail + 128 * 128;
     t.abort = reinterpret_cast<int*>(t.dmax + 1);
+    t.perm = t.abort + 3;
     return t;
 }
 
@@ -155,10 +157,13 @@ struct TriShared {
     float2 x[2][S::G];                       // (A v, column kk of A) by row, alternate steps (one block: two arrays, y then column)
     float rows[2][S::W][S::LR][2][S::RI];    // the same for a warp's own rows
     float g[2][S::W][S::LR];                 // a^T A a, one part per warp and lane row (one-block form)
-    float good[S::G];
+    __align__(16) unsigned key[S::G];        // the diagonal's leading bits, and the row in the others: larger key, earlier place
+    __align__(16) unsigned short col[S::G];  // row of K at each place, or the zero column of the staged rows
     float red[S::W];
     u64 bar[2];
 };
+template <typename S>
+constexpr int kOwnRows = S::G / S::CL;       // rows of the tile of a block
 
 template <typename S>
 struct TriState {
@@ -434,37 +439,56 @@ __device__ __forceinline__ bool tri_phase(TriState<S>& T, TriShared<S>& sh, int 
     return true;
 }
 
+// The rows are taken in order of falling diagonal. Reflections that start with the large rows leave the small ones' relative accuracy
+// alone; in any other order a small eigenvalue is as uncertain as 1e-7 of the largest one. Rows of a sketch are so spread by
+// construction, and gradients with heavy-tailed norms are. 64 rows, norms spread over a factor of 1,000 in no order, frozen: cosines
+// between rows of the sketch 5e-3 -> 2e-5, singular values off by 1e-2 -> 2e-7 of themselves (they are x^T K x at a freeze).
+// The diagonal and the places come before the tile, which is gathered from rows staged in shared memory: 2 to 3 us of 45 to 92 for 64
+// to 128 rows, nothing measurable of 215 and 690 us for 256 and 512.
 template <typename S>
 __global__ void __launch_bounds__(S::NT, 1)
 k_tridiag(const float* __restrict__ K, int ldk, int n, int scaled, TriWork wk, int base, int pitch, EigInfo* __restrict__ info) {
     __shared__ __align__(16) TriShared<S> sh;
+    extern __shared__ __align__(16) float staged[];         // rows of K and a zero column (not for a matrix that comes scaled)
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, lr = lane / S::LC, lc = lane % S::LC;
     const int cta = S::CL == 1 ? 0 : (int)blockIdx.x;
-    const int o = (S::G - n) & ~3;
-    float kscale = 1.f;
+    const int o = (S::G - n) & ~3, n4 = (n + 3) & ~3;
     chain_wait();
-    TriState<S> T;                                          // the loads of the tile first, all in flight together
+    TriState<S> T;
+    if (S::CL == 1 && scaled) {                             // what a cluster left: every position in use, the order is made
 #pragma unroll
-    for (int i = 0; i < S::RI; ++i) {
-        const int r = min(max(i * S::RB + (cta * S::W + w) * S::LR + lr - o, 0), n - 1);
+        for (int i = 0; i < S::RI; ++i) {
+            const int r = i * S::RB + (cta * S::W + w) * S::LR + lr;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int c = min(max(q * S::CB + 4 * lc - o, 0), (n - 1) & ~3);
-            const float4 x = *reinterpret_cast<const float4*>(K + (size_t)r * ldk + c);
-            T.A[i][2 * q] = pk(x.x, x.y);
-            T.A[i][2 * q + 1] = pk(x.z, x.w);
+            for (int q = 0; q < 4; ++q) {
+                const float4 x = *reinterpret_cast<const float4*>(K + (size_t)r * ldk + q * S::CB + 4 * lc);
+                T.A[i][2 * q] = pk(x.x, x.y);
+                T.A[i][2 * q + 1] = pk(x.z, x.w);
+            }
         }
-    }
-    if (!scaled) {
+    } else {
+        const int ps = n4 + 4;                              // pitch of a staged row; columns n4 .. n4 + 3 are zero
+        auto stage = [&](int row, int place) {              // by a warp
+            for (int c = 4 * lane; c < n4; c += 128)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s_addr(staged + (size_t)place * ps + c)), "l"(K + (size_t)row * ldk + c) : "memory");
+            if (lane == 0) *reinterpret_cast<float4*>(staged + (size_t)place * ps + n4) = make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        if (S::CL == 1)                                     // one block stages all rows while it looks at the diagonal, a cluster's blocks their own
+            for (int r = w; r < n; r += S::W) stage(r, r);
         // scale by the largest finite diagonal; rows whose norm is not finite take no part
+        constexpr int MINE = S::G / S::NT;                  // rows that a thread ranks
         float dm = 0.f;
-        bool bad = false;
-        for (int i = tid; i < n; i += S::NT) {
-            const float v = K[(size_t)i * ldk + i];
-            const bool fin = fabsf(v) <= 3.0e38f;
-            sh.good[i] = fin ? 1.f : 0.f;
-            bad |= !fin;
-            if (fin) dm = fmaxf(dm, v);
+        unsigned mine[MINE];
+        bool fin[MINE];
+#pragma unroll
+        for (int u = 0; u < MINE; ++u) {
+            const int i = tid + u * S::NT;
+            const float v = i < n ? K[(size_t)i * ldk + i] : 0.f;
+            fin[u] = fabsf(v) <= 3.0e38f;
+            dm = fin[u] ? fmaxf(dm, v) : dm;
+            mine[u] = i < n ? ((fin[u] ? __float_as_uint(fmaxf(v, 0.f)) : 0u) & ~511u) | (unsigned)(511 - i) : 0u;
+            sh.key[i] = mine[u];
+            if (!fin[u] && cta == 0) atomicOr(&info->flags, kFlagNonFinite);
         }
 #pragma unroll
         for (int x = 16; x > 0; x >>= 1) dm = fmaxf(dm, __shfl_xor_sync(0xffffffffu, dm, x));
@@ -473,14 +497,52 @@ k_tridiag(const float* __restrict__ K, int ldk, int n, int scaled, TriWork wk, i
 #pragma unroll
         for (int j = 0; j < S::W; ++j) dm = fmaxf(dm, sh.red[j]);
         if (!(dm >= 1e-30f)) dm = 0.f;                      // nothing to factor
-        kscale = dm > 0.f ? 1.f / dm : 0.f;
-        if (cta == 0) {
-            if (bad) atomicOr(&info->flags, kFlagNonFinite);
-            if (tid == 0) *wk.dmax = dm;
+        const float kscale = dm > 0.f ? 1.f / dm : 0.f;
+        if (cta == 0 && tid == 0) *wk.dmax = dm;
+        int place[MINE];                                    // of a row: how many come before it
+#pragma unroll
+        for (int u = 0; u < MINE; ++u) place[u] = 0;
+#pragma unroll 4
+        for (int j = 0; j < n4; j += 4) {
+            const uint4 k = *reinterpret_cast<const uint4*>(&sh.key[j]);
+#pragma unroll
+            for (int u = 0; u < MINE; ++u) place[u] += (k.x > mine[u]) + (k.y > mine[u]) + (k.z > mine[u]) + (k.w > mine[u]);
         }
-    } else {
-        for (int i = tid; i < n; i += S::NT) sh.good[i] = 1.f;
+#pragma unroll
+        for (int u = 0; u < MINE; ++u) {
+            const int i = tid + u * S::NT, p = i < n ? place[u] : i;
+            sh.col[p] = (unsigned short)(i < n && fin[u] ? i : n4);
+            if (cta == 0) wk.perm[p] = i;
+        }
         __syncthreads();
+        if (S::CL > 1) {
+            for (int t = w; t < kOwnRows<S>; t += S::W) {   // place t: slot t / (W LR) of the block's rows
+                const int p = (t / (S::W * S::LR)) * S::RB + cta * S::W * S::LR + t % (S::W * S::LR) - o;
+                if (p >= 0 && p < n && sh.col[p] < n4) stage(sh.col[p], t);
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = q * S::CB + 4 * lc - o;
+            const ushort4 pc = c >= 0 ? *reinterpret_cast<const ushort4*>(&sh.col[c]) : make_ushort4(n4, n4, n4, n4);
+#pragma unroll
+            for (int i = 0; i < S::RI; ++i) {
+                const int p = i * S::RB + (cta * S::W + w) * S::LR + lr - o;
+                const int row = p >= 0 ? sh.col[p] : n4;
+                float t[4] = {0.f, 0.f, 0.f, 0.f};
+                if (row < n4) {
+                    const float* src = staged + (size_t)(S::CL == 1 ? row : i * S::W * S::LR + w * S::LR + lr) * ps;
+                    t[0] = src[pc.x] * kscale;
+                    t[1] = src[pc.y] * kscale;
+                    t[2] = src[pc.z] * kscale;
+                    t[3] = src[pc.w] * kscale;
+                }
+                T.A[i][2 * q] = pk(t[0], t[1]);
+                T.A[i][2 * q + 1] = pk(t[2], t[3]);
+            }
+        }
     }
     if constexpr (S::CL > 1) {
         if (tid < 2) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_addr(&sh.bar[tid])) : "memory");
@@ -490,22 +552,7 @@ k_tridiag(const float* __restrict__ K, int ldk, int n, int scaled, TriWork wk, i
         }
     }
 #pragma unroll
-    for (int i = 0; i < S::RI; ++i) {
-        const int r = i * S::RB + (cta * S::W + w) * S::LR + lr - o;
-        const float gr = r >= 0 && r < n ? sh.good[r] : 0.f;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int c = q * S::CB + 4 * lc - o;
-            float t[4];
-            upk(T.A[i][2 * q], t[0], t[1]);
-            upk(T.A[i][2 * q + 1], t[2], t[3]);
-#pragma unroll
-            for (int s = 0; s < 4; ++s) t[s] = gr != 0.f && c >= 0 && c + s < n && sh.good[c + s] != 0.f ? t[s] * kscale : 0.f;
-            T.A[i][2 * q] = pk(t[0], t[1]);
-            T.A[i][2 * q + 1] = pk(t[2], t[3]);
-        }
-        T.vr[i] = T.y[i] = 0.f;
-    }
+    for (int i = 0; i < S::RI; ++i) T.vr[i] = T.y[i] = 0.f;
 #pragma unroll
     for (int p = 0; p < 8; ++p) T.vc[p] = 0ull;
     T.ak = T.b = T.tau = 0.f;
@@ -557,7 +604,7 @@ constexpr int kHelpWarps = 4;                      // inner products of reflecto
 constexpr int kVecThreads = 32 * (kEvWarps + kHelpWarps);
 constexpr int kChunk = 16;                         // reflectors per chunk in shared memory
 constexpr int kPoints = 32 * kEvWarps;             // places of the first cut, shared by the block's eigenvalues
-constexpr double kRankCut = 1e-7;                  // eigenvalues below this fraction of ||T|| count as zero (rounding of K and T)
+constexpr double kRankCut = 1e-7;                  // eigenvalues below this fraction of the largest diagonal count as zero (rounding of K and T)
 template <int NQ>
 constexpr int kRing = NQ == 4 ? 4 : 8;             // chunks in flight (all of them when n <= 128)
 
@@ -689,6 +736,7 @@ struct VecShared {
     int rex[kVecWarps][2][32 * NQ];                // their exponents
     float gram[32 * NQ][8];                        // inner products inside each group of four reflectors: 01 02 03 12 13 23
     float tau[128 * NQ];
+    unsigned short perm[128 * NQ];
     int first[kPoints];
     double red[2][kEvWarps + kHelpWarps];
     double delta, mid[3];
@@ -698,7 +746,7 @@ struct VecShared {
 // dependent latency: five or so passes of n / 2 fp64 steps over T, n steps of the recurrences, n / 4 groups of reflections.
 template <int NQ>                                  // quads of positions per lane: N <= 128 NQ
 __global__ void __launch_bounds__(kVecThreads, 1)
-k_tridiag_vectors(TriWork wk, int G, int n, int do_shrink, int delta_rank, int keep, float* __restrict__ Ur, int ldu,
+k_tridiag_vectors(const float* __restrict__ K, int ldk, TriWork wk, int G, int n, int do_shrink, int delta_rank, int keep, float* __restrict__ Ur, int ldu,
                   float* __restrict__ sigma_out, int n_sigma, EigInfo* __restrict__ info, float* __restrict__ Wsplit, int ldw, int j_pad) {
     constexpr int RING = kRing<NQ>;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -736,7 +784,10 @@ k_tridiag_vectors(TriWork wk, int G, int n, int do_shrink, int delta_rank, int k
         gu = fmax(gu, d + (el + er));
         gl = fmin(gl, d - (el + er));
     }
-    for (int i = tid; i < 128 * NQ; i += kVecThreads) sh.tau[i] = i < N - 2 ? wk.tau[o + i] : 0.f;
+    for (int i = tid; i < 128 * NQ; i += kVecThreads) {
+        sh.tau[i] = i < N - 2 ? wk.tau[o + i] : 0.f;
+        sh.perm[i] = (unsigned short)(i < n ? wk.perm[i] : i);
+    }
 #pragma unroll
     for (int x = 16; x > 0; x >>= 1) {
         gu = fmax(gu, __shfl_xor_sync(0xffffffffu, gu, x));
@@ -785,7 +836,7 @@ k_tridiag_vectors(TriWork wk, int G, int n, int do_shrink, int delta_rank, int k
     }
     __syncthreads();
     const bool empty = !(dmax > 0.f);
-    const double cut = (kRankCut * gm - shift) * tsc;
+    const double cut = (kRankCut - shift) * tsc;
     const int j = blockIdx.x * kVecWarps + w;      // this warp's eigenvector (w == kVecWarps: delta)
     double det;
     int dex;
@@ -1010,12 +1061,58 @@ k_tridiag_vectors(TriWork wk, int G, int n, int do_shrink, int delta_rank, int k
 
     // ---- factors ----
     if (w < kVecWarps && j < (Wsplit && j_pad > keep ? j_pad : keep)) {
+        float* px = reinterpret_cast<float*>(sh.rec[w][0]);                 // from the order of the reduction to that of K
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const int i = 4 * (lane + 32 * q) + s;
+                px[sh.perm[i]] = i < n ? x[4 * q + s] : 0.f;
+            }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const float4 t = *reinterpret_cast<const float4*>(px + 4 * (lane + 32 * q));
+            x[4 * q] = t.x;
+            x[4 * q + 1] = t.y;
+            x[4 * q + 2] = t.z;
+            x[4 * q + 3] = t.w;
+        }
         float fac = 0.f, sp = 0.f;
         if (alive) {
             const double l = fma(lam, wid, shift), kept = l - sh.delta;
             if (kept > 0.0) {
                 fac = (float)sqrt(kept / l);
                 sp = (float)sqrt(kept * (double)dmax);
+            }
+            if (!do_shrink) {
+                // a freeze that keeps the eigenvalues as they are: x^T K x in fp64, off by the square of the vector's error only
+                double dot = 0.0, nn = 0.0;
+#pragma unroll
+                for (int t = 0; t < 4 * NQ; ++t) nn = fma((double)x[t], (double)x[t], nn);
+#pragma unroll 4
+                for (int i = 0; i < n; ++i) {
+                    const float xi = px[i];
+                    double y = 0.0;
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) {
+                        const int c = 4 * (lane + 32 * q);
+                        if (c >= n) continue;
+                        const float4 k = *reinterpret_cast<const float4*>(K + (size_t)i * ldk + c);
+                        // rows that take no part are zero in x and may be anything in K
+                        y = fma(x[4 * q] != 0.f ? (double)k.x : 0.0, (double)x[4 * q], y);
+                        y = fma(x[4 * q + 1] != 0.f ? (double)k.y : 0.0, (double)x[4 * q + 1], y);
+                        y = fma(x[4 * q + 2] != 0.f ? (double)k.z : 0.0, (double)x[4 * q + 2], y);
+                        y = fma(x[4 * q + 3] != 0.f ? (double)k.w : 0.0, (double)x[4 * q + 3], y);
+                    }
+                    if (xi != 0.f) dot = fma(y, (double)xi, dot);
+                }
+#pragma unroll
+                for (int y = 16; y > 0; y >>= 1) {
+                    dot += __shfl_xor_sync(0xffffffffu, dot, y);
+                    nn += __shfl_xor_sync(0xffffffffu, nn, y);
+                }
+                if (dot > 0.0) sp = (float)sqrt(dot / nn);
             }
         }
         if (j < n_sigma && j < keep && lane == 0) sigma_out[j] = sp;
@@ -1050,32 +1147,39 @@ k_tridiag_vectors(TriWork wk, int G, int n, int do_shrink, int delta_rank, int k
     }
 }
 
+// A matrix as it comes: one block, or a cluster where the shape says so.
 template <typename S>
-cudaError_t run_cluster(const float* K, int ldk, int n, TriWork wk, EigInfo* info, cudaStream_t st) {
+cudaError_t run_tridiag(const float* K, int ldk, int n, TriWork wk, EigInfo* info, cudaStream_t st) {
+    const int n4 = (n + 3) & ~3;
+    constexpr int most = (S::CL == 1 ? S::G : kOwnRows<S>) * (S::G + 4) * 4;
+    const int smem = (S::CL == 1 ? n : kOwnRows<S>) * (n4 + 4) * 4;
+    cudaError_t e = allow_smem((const void*)k_tridiag<S>, most);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S::CL);
     cfg.blockDim = dim3(S::NT);
+    cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = st;
     cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = S::CL;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[1].val.programmaticStreamSerializationAllowed = 1;
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = S::CL;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = S::CL > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, k_tridiag<S>, K, ldk, n, 0, wk, 0, (int)S::G, info);
 }
 
 template <int NQ>
-cudaError_t run_vectors(TriWork wk, int G, int n, int do_shrink, int delta_rank, int keep, float* Ur, int ldu, float* sigma_out, int n_sigma,
+cudaError_t run_vectors(const float* K, int ldk, TriWork wk, int G, int n, int do_shrink, int delta_rank, int keep, float* Ur, int ldu, float* sigma_out, int n_sigma,
                         EigInfo* info, float* Wsplit, int ldw, int j_pad, cudaStream_t st) {
     const int rows = Wsplit && j_pad > keep ? j_pad : keep;
     const int blocks = rows > 0 ? (rows + kVecWarps - 1) / kVecWarps : 1;
     cudaError_t e = allow_smem((const void*)k_tridiag_vectors<NQ>, (int)sizeof(VecShared<NQ>));
     if (e != cudaSuccess) return e;
-    return launch_chained(k_tridiag_vectors<NQ>, dim3(blocks), dim3(kVecThreads), sizeof(VecShared<NQ>), st, wk, G, n, do_shrink, delta_rank, keep, Ur, ldu,
+    return launch_chained(k_tridiag_vectors<NQ>, dim3(blocks), dim3(kVecThreads), sizeof(VecShared<NQ>), st, K, ldk, wk, G, n, do_shrink, delta_rank, keep, Ur, ldu,
                           sigma_out, n_sigma, info, Wsplit, ldw, j_pad);
 }
 
@@ -1083,7 +1187,7 @@ cudaError_t run_vectors(TriWork wk, int G, int n, int do_shrink, int delta_rank,
 
 size_t eig_work_floats(int n) {
     const size_t G = n <= 128 ? 128 : n <= 256 ? 256 : 512;
-    const size_t direct = G * G + 3 * G + 128 * 128 + 16, iterative = (n > 256 ? (size_t)512 * 512 : (size_t)256 * 256) + 64;
+    const size_t direct = G * G + 4 * G + 128 * 128 + 16, iterative = (n > 256 ? (size_t)512 * 512 : (size_t)256 * 256) + 64;
     return direct > iterative ? direct : iterative;
 }
 
@@ -1096,16 +1200,16 @@ cudaError_t launch_eig_direct(const float* K, int ldk, int n, int do_shrink, int
     const TriWork wk = tri_work(work, G);
     cudaError_t e = cudaSuccess;
     if (G == 128) {
-        e = launch_chained(k_tridiag<Tri128>, dim3(1), dim3(Tri128::NT), 0, st, K, ldk, n, 0, wk, 0, G, info);
+        e = run_tridiag<Tri128>(K, ldk, n, wk, info, st);
     } else {
-        e = G == 256 ? run_cluster<Tri256>(K, ldk, n, wk, info, st) : run_cluster<Tri512>(K, ldk, n, wk, info, st);
+        e = G == 256 ? run_tridiag<Tri256>(K, ldk, n, wk, info, st) : run_tridiag<Tri512>(K, ldk, n, wk, info, st);
         if (e != cudaSuccess) return e;
         e = launch_chained(k_tridiag<Tri128>, dim3(1), dim3(Tri128::NT), 0, st, wk.trail, 128, 128, 1, wk, G - 128, G, info);
     }
     if (e != cudaSuccess) return e;
-    if (G == 128) return run_vectors<1>(wk, G, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out, n_sigma, info, Wsplit, ldw, j_pad, st);
-    if (G == 256) return run_vectors<2>(wk, G, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out, n_sigma, info, Wsplit, ldw, j_pad, st);
-    return run_vectors<4>(wk, G, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out, n_sigma, info, Wsplit, ldw, j_pad, st);
+    if (G == 128) return run_vectors<1>(K, ldk, wk, G, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out, n_sigma, info, Wsplit, ldw, j_pad, st);
+    if (G == 256) return run_vectors<2>(K, ldk, wk, G, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out, n_sigma, info, Wsplit, ldw, j_pad, st);
+    return run_vectors<4>(K, ldk, wk, G, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out, n_sigma, info, Wsplit, ldw, j_pad, st);
 }
 
 }  // namespace sage

@@ -56,3 +56,30 @@ def test_one_shrink_and_one_freeze(kind, ell):
         err_sigma = np.max(np.abs(sigma ** 2 - expect)) / lam[-1]
         assert st["device_flags"] == 0 and st["shrinks"] == (1 if N == 2 * ell else 0)
         assert err <= bound and err_sigma <= bound, (N, tensor_cores, err, err_sigma)
+
+
+@pytest.mark.parametrize("ell", [5, 8, 33, 64, 100, 128, 129, 200, 256])
+def test_small_rows_beside_large_ones(ell):
+    """ell rows of norms spread over three decades, in no order, frozen without a shrink: every row counts as much as in a sketch of
+    rows of one size. Scaled to unit rows the Gram matrix is that of random rows of 4,000 values, whose condition number is below 3,
+    so that an entry's rounding (fp32 sums folded every 2,048 terms: below 4e-7 of the product of the two norms) moves a singular
+    value by 6e-7 of itself; twice that is allowed. Two rows of the sketch mix as far as the reflections round small against
+    large: 1e-4 was met in this order of rows over all sizes, 1e-2 in another."""
+    D = 4000
+    r = np.random.default_rng(ell)
+    rows = r.standard_normal((ell, D)) * (10.0 ** (-3.0 * r.permutation(ell) / ell) / D ** 0.5)[:, None]
+    rows = torch.from_numpy(rows.astype(np.float32))
+    fd = sage.SageFD(D, ell, torch.float32, 0)
+    fd.set_option(4, 0)
+    fd.update(rows.cuda())
+    fd.finalize()
+    S, sigma = fd.sketch()
+    st = fd.stats()
+    fd.close()
+    expect = np.linalg.svd(rows.double().numpy(), compute_uv=False)
+    S, sigma = S.double().cpu().numpy(), sigma.double().cpu().numpy()
+    norm = np.linalg.norm(S, axis=1)
+    cosines = (S / norm[:, None]) @ (S / norm[:, None]).T - np.eye(ell)
+    assert st["device_flags"] == 0 and st["last_rank"] == ell
+    assert np.max(np.abs(sigma / expect - 1.0)) <= 1.2e-6
+    assert np.max(np.abs(norm / expect - 1.0)) <= 1.2e-6 and np.max(np.abs(cosines)) <= 2e-4
