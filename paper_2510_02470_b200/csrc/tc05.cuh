@@ -64,17 +64,64 @@ __device__ __forceinline__ void mbar_wait_quiet(uint64_t* bar, uint32_t parity, 
     while (!mbar_try_wait(bar, parity) && clock64() - t0 < limit_cycles) {}
 }
 
-// Arrival on the barrier at the same place in CTA `cta` of the cluster. What it orders is read by the
-// tensor cores, to which the arriving warp's proxy fence (or its fence behind a finished TMEM load) has shown it before; a release
-// at cluster scope, which waits for everything that its thread has in flight, made a Gram kernel's chain of hand-offs 40 % longer.
-__device__ __forceinline__ void mbar_arrive_cta(uint64_t* bar, uint32_t cta) {
+// What one CTA of a cluster hands to another: arrivals on the barrier at the same place in CTA `cta`. Behind what tensor memory
+// holds (stores that have been waited for, finished loads) a relaxed one is enough between tcgen05 fences; shared memory needs the
+// release at cluster scope (with what its thread has acquired from others of its block) and the wait that acquires there.
+__device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint64_t* bar, uint32_t cta) {
     asm volatile(
         "{\n"
         ".reg .b32 a;\n"
         "mapa.shared::cluster.u32 a, %0, %1;\n"
-        "mbarrier.arrive.shared::cluster.b64 _, [a];\n"
+        "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [a];\n"
         "}\n" ::"r"(smem_u32(bar)), "r"(cta)
         : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint64_t* bar, uint32_t cta) {
+    asm volatile(
+        "{\n"
+        ".reg .b32 a;\n"
+        "mapa.shared::cluster.u32 a, %0, %1;\n"
+        "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [a];\n"
+        "}\n" ::"r"(smem_u32(bar)), "r"(cta)
+        : "memory");
+}
+template <bool ACQUIRE>
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    if constexpr (ACQUIRE)
+        asm volatile(
+            "{\n"
+            ".reg .pred p;\n"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+            "selp.u32 %0, 1, 0, p;\n"
+            "}\n"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+    else
+        asm volatile(
+            "{\n"
+            ".reg .pred p;\n"
+            "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n"
+            "selp.u32 %0, 1, 0, p;\n"
+            "}\n"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+    return ok != 0;
+}
+template <bool ACQUIRE>
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort) {
+    if (mbar_try_wait_cluster<ACQUIRE>(bar, parity)) return true;
+    const long long t0 = clock64();
+    while (!mbar_try_wait_cluster<ACQUIRE>(bar, parity)) {
+        if (*abort) return false;
+        if (clock64() - t0 > kWaitLimitCycles) {
+            *abort = 1;
+            return false;
+        }
+    }
+    return true;
 }
 __device__ __forceinline__ void cluster_barrier() {                                    // all threads of all CTAs
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");

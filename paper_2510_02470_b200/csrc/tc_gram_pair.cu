@@ -7,14 +7,16 @@
 // A rows and half of the B rows, reads 64 bytes per cycle in all, and splits what it holds; on diagonal tiles the two halves are the
 // same rows. Per K tile and SM: 64 KB (diagonal) or 96 KB read by MMAs, 48 or 96 KB by loads and split, in the 1,020 or 1,540 cycles
 // that its 8 or 12 MMAs take at the nominal rate.
-// Measured (this kernel alone, against 128 x 128 tiles on single SMs): 512 rows of 262,144 columns 628 -> 293 us, 256 of them
-// 239 -> 100 us, 256 rows of 51,300 columns 60 -> 35 us. Loads that hit the L2 cache or no split at all leave these times as they
-// are, a quarter of the MMAs takes a fourth off: the MMAs bound it, at two thirds of their nominal rate, what cuBLAS reaches too.
+// Measured (this kernel alone, against 128 x 128 tiles on single SMs): 512 rows of 262,144 columns 628 -> 310 us, 256 of them
+// 239 -> 104 us, 256 rows of 51,300 columns 60 -> 35 us. 6 and 3 % of that are the release at cluster scope behind CTA 1's remainders
+// (two warps in turn pass them on; one warp: 12 %). Without the release, loads that hit the L2 cache or no split at all left
+// the time as it was and a quarter of the MMAs took a fourth off: the MMAs bound it, at two thirds of their nominal rate.
 // One cluster of two CTAs owns a tile and a K slice. CTA q: rows q*128 .. of the tile's row block (A, and its rows of the output) and
 // rows q*128 .. of its column block (B).
 //   warp 0     TMA loads of this CTA's rows (128-byte swizzle),
 //   warp 1     TMEM allocation; in CTA 0 the MMAs of both, into two accumulators of 256 columns in turn,
-//   warps 4-11 write the remainders of landed stages and report them to CTA 0; between stages they drain this CTA's accumulator rows
+//   warps 2, 3 of CTA 1 pass on to CTA 0 which remainders are written,
+//   warps 4-11 write the remainders of landed stages; between stages they drain this CTA's accumulator rows
 //              (4-7: columns 0-127, 8-11: the others) into 128 sums a thread, and store them at the end.
 #include "sage_internal.h"
 #include "tc05.cuh"
@@ -33,7 +35,7 @@ constexpr int kRunTiles = 8;                // as tc_gemm_x3.cu: 96 additions be
 // stage is one tile on diagonal tiles, [A][B] elsewhere: 8 and 6 stages there, 4 and 3 here. The workers take diagonal stages in two
 // groups in turn, others together: 8 pieces of 16 bytes a thread either way, all in flight at once.
 constexpr int kHiTiles = 8, kLoTiles = 6;
-constexpr size_t kPairSmem = 1024 + (size_t)(kHiTiles + kLoTiles) * kOpBytes + (2 * kHiTiles + kLoTiles + 4) * 8 + 16;
+constexpr size_t kPairSmem = 1024 + (size_t)(kHiTiles + kLoTiles) * kOpBytes + (2 * kHiTiles + 2 * kLoTiles + 4) * 8 + 16;
 
 __global__ void __launch_bounds__(kPairThreads, 1)
 k_tc_gram_pair(const __grid_constant__ CUtensorMap tm, int r, long long K, int n_diag, int n_off, float* __restrict__ C, long long ldc,
@@ -49,8 +51,9 @@ k_tc_gram_pair(const __grid_constant__ CUtensorMap tm, int r, long long K, int n
     uint8_t* lo_ring = smem + kHiTiles * kOpBytes;
     uint64_t* full = reinterpret_cast<uint64_t*>(lo_ring + kLoTiles * kOpBytes);   // [kHiTiles], local
     uint64_t* empty = full + kHiTiles;                                  // [kHiTiles], both CTAs': the MMA thread's commits go to both
-    uint64_t* split_done = empty + kHiTiles;                            // [kLoTiles], CTA 0's: arrivals from both CTAs
-    uint64_t* acc_full = split_done + kLoTiles;                         // [2], both CTAs'
+    uint64_t* split_done = empty + kHiTiles;                            // [kLoTiles], local
+    uint64_t* peer_split = split_done + kLoTiles;                       // [kLoTiles], CTA 0's: CTA 1's split_done, passed on
+    uint64_t* acc_full = peer_split + kLoTiles;                         // [2], both CTAs'
     uint64_t* acc_empty = acc_full + 2;                                 // [2], CTA 0's: arrivals from both CTAs
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
     volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -67,7 +70,8 @@ k_tc_gram_pair(const __grid_constant__ CUtensorMap tm, int r, long long K, int n
             mbar_init(&empty[s], 1);
         }
         for (int s = 0; s < kLoTiles; ++s) {
-            mbar_init(&split_done[s], 2 * kPairWorkers / groups);
+            mbar_init(&split_done[s], kPairWorkers / groups);
+            mbar_init(&peer_split[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
@@ -114,9 +118,9 @@ k_tc_gram_pair(const __grid_constant__ CUtensorMap tm, int r, long long K, int n
                 for (int kt = 0, run = 0; kt < nkt && alive; ++run) {
                     const int kt_end = kt + kRunTiles < nkt ? kt + kRunTiles : nkt;
                     const uint32_t b = (uint32_t)run & 1u, acc = tmem_base + b * 256u;
-                    alive = __all_sync(0xffffffffu, mbar_wait(&acc_empty[b], (((uint32_t)run >> 1) & 1u) ^ 1u, abort));
+                    alive = __all_sync(0xffffffffu, mbar_wait_cluster<false>(&acc_empty[b], (((uint32_t)run >> 1) & 1u) ^ 1u, abort));
                     for (int k0 = kt; kt < kt_end && alive; ++kt) {
-                        alive = __all_sync(0xffffffffu, mbar_wait(&split_done[ls], ph, abort));
+                        alive = __all_sync(0xffffffffu, mbar_wait(&split_done[ls], ph, abort) && mbar_wait_cluster<true>(&peer_split[ls], ph, abort));
                         if (!alive) break;
                         tc_fence_after();
                         const uint32_t hi = hi0 + (uint32_t)(s * stage_bytes), lo = lo0 + (uint32_t)(ls * stage_bytes);
@@ -137,6 +141,12 @@ k_tc_gram_pair(const __grid_constant__ CUtensorMap tm, int r, long long K, int n
                         if (++ls == n_lo) { ls = 0; ph ^= 1u; }
                     }
                 }
+            }
+        } else if (q == 1 && lane == 0) {                   // CTA 1's remainders are handed to the MMAs
+            for (int kt = warp - 2; kt < nkt; kt += 2) {
+                const int ls = kt % n_lo;
+                if (!mbar_wait(&split_done[ls], (uint32_t)(kt / n_lo) & 1u, abort)) break;
+                mbar_arrive_cluster(&peer_split[ls], 0);
             }
         }
     } else {
@@ -169,7 +179,7 @@ k_tc_gram_pair(const __grid_constant__ CUtensorMap tm, int r, long long K, int n
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cta(&acc_empty[b], 0);
+            if (lane == 0) mbar_arrive_cluster_relaxed(&acc_empty[b], 0);
         };
         // A group sees every phase of its slots: both rings are multiples of the number of groups.
         const int grp = diag ? half : 0, nt = 32 * kPairWorkers / groups, t = (threadIdx.x - 128) & (nt - 1);
@@ -192,7 +202,7 @@ k_tc_gram_pair(const __grid_constant__ CUtensorMap tm, int r, long long K, int n
             }
             fence_proxy_async_smem();                       // the tensor cores read these writes
             __syncwarp();
-            if (lane == 0) mbar_arrive_cta(&split_done[ls], 0);
+            if (lane == 0) mbar_arrive(&split_done[ls]);
             s += groups;
             if (s >= n_hi) { s -= n_hi; ph ^= 1u; }
             ls += groups;

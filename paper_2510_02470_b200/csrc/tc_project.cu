@@ -4,15 +4,19 @@
 // The data rows are the A operand: hi from shared memory, exactly as TMA left it, lo from TMEM, where the workers put it, so that the
 // split costs no shared-memory store and no proxy fence; the sketch, split once into [hi (64 rows) ; lo (64 rows)] when it was
 // frozen, is one 128-row B operand. Accumulator column j and 64 + j belong to output j.
-// What an SM can load bounds it, about 34 bytes a cycle: a pair of SMs works on 256 rows (cta_group::2), so that each loads half of the
-// sketch's tile, the hi rows or the lo rows, next to its 128 rows: 24 KB a K tile, 700 cycles, as long as the rows take from memory at
-// the copy rate; the MMAs take 512.
+// A pair of SMs works on 256 rows (cta_group::2), so that each loads half of the sketch's tile, the hi rows or the lo rows, next to its
+// 128 rows: 24 KB a K tile, 700 cycles at the 34 bytes a cycle that an SM was seen to load, as long as the rows take from memory at the
+// copy rate; the MMAs take 512. What bounds it is how long a slot lives: load, hand-over to CTA 0, MMAs, eight slots in all. CTA 1's
+// landed data is released at cluster scope, 2,000 cycles or so under load, beside the split; remainders and drained accumulators are
+// in tensor memory, where relaxed arrivals between tcgen05 fences do. (With default arrivals, which order nothing between two
+// CTAs: 214 and 333 us where it takes 245 and 366. The release behind the split: 263 and 392; one warp that passes all on: 503.)
 // Measured (against single SMs with 128-row tiles that loaded the whole sketch tile, remainders in shared memory, a block per tile and
-// K slice): 50,000 rows of 5,130 onto 64 365 -> 208 us (1.03 GB: 159 us at the copy rate), 20,000 of 20,000 546 -> 303 us (245), 512 of 5,130
-// 57 -> 20 us. On single SMs, the whole sketch tile loaded: 264 and 389 us, 232 and 333 without split and second products.
+// K slice): 50,000 rows of 5,130 onto 64 365 -> 245 us (1.03 GB: 159 us at the copy rate), 20,000 of 20,000 546 -> 366 us (245), 512 of 5,130
+// 57 -> 19 us. On single SMs, the whole sketch tile loaded: 264 and 389 us.
 // Pairs take equal shares of all K tiles of all row tiles, in order: a row tile may be cut, and part i of it goes to plane i. With
 // classes (structured rows) every class is a slice of its own plane and nothing is cut.
 //   warp 0     TMA loads (128-byte swizzle), warp 1 TMEM allocation and, in CTA 0, the MMAs of both,
+//   warps 12-15 of CTA 1 tell CTA 0 what has landed there,
 //   warps 4-11 remainders of landed K tiles in two groups in turn (a thread has one row), reported to CTA 0; between them they drain:
 //              thread = row, 32 outputs each.
 #include "sage_internal.h"
@@ -22,15 +26,20 @@ namespace sage {
 namespace tc {
 namespace {
 
-constexpr int kProjThreads = 384;
+constexpr int kProjThreads = 512;
+constexpr int kProjRegs = 128;               // what every thread is launched with: the sum of the shares below is 4 x 128 x 128
 constexpr int kRowBytes = 128 * 128;        // 128 rows of one K tile (32 floats)
 constexpr int kStageBytes = kRowBytes + 64 * 128;     // and half of the sketch's
 constexpr int kProjBK = 32;
 constexpr int kStages = 8;                  // K tiles in flight, in shared memory and, their remainders, in TMEM
 constexpr int kRunTiles = 3;                // K tiles, 24 additions, between drains of an accumulator
 constexpr int kGroupWarps = 4;
+// Warps that tell CTA 0 what has landed in CTA 1: a release at cluster scope takes as long as three K tiles. A forwarder has waited
+// for a slot's round before the next one itself, so that the two are never mistaken for one another.
+constexpr int kForwards = 4;
+static_assert(kStages % kForwards == 0, "");
 constexpr uint32_t kLoCol = 256;            // TMEM: two accumulators of 128 columns, then the remainders, 32 columns each
-constexpr size_t kProjSmem = 1024 + (size_t)kStages * kStageBytes + (3 * kStages + 4) * 8 + 16;
+constexpr size_t kProjSmem = 1024 + (size_t)kStages * kStageBytes + (4 * kStages + 4) * 8 + 16;
 
 struct ProjRange {                          // the K tiles of one row tile (and class) that a pair takes
     int tile, slice, part, k0, k1;
@@ -55,7 +64,8 @@ k_tc_project(const __grid_constant__ CUtensorMap tmRows, const __grid_constant__
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)kStages * kStageBytes);   // local
-    uint64_t* split_done = full + kStages;                 // CTA 0's: arrivals from both CTAs
+    uint64_t* peer_full = full + kStages;                  // CTA 0's: CTA 1's full, passed on
+    uint64_t* split_done = peer_full + kStages;            // CTA 0's: arrivals from both CTAs
     uint64_t* empty = split_done + kStages;                // both CTAs': the MMA thread's commits go to both
     uint64_t* acc_full = empty + kStages;                  // [2], likewise
     uint64_t* acc_empty = acc_full + 2;                    // [2], CTA 0's: arrivals from both CTAs
@@ -77,6 +87,7 @@ k_tc_project(const __grid_constant__ CUtensorMap tmRows, const __grid_constant__
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], 1);
+            mbar_init(&peer_full[s], 1);
             mbar_init(&split_done[s], 2 * kGroupWarps);
             mbar_init(&empty[s], 1);
         }
@@ -103,6 +114,8 @@ k_tc_project(const __grid_constant__ CUtensorMap tmRows, const __grid_constant__
         u += p.k1 - p.k0;
     }
 
+    if (warp < 4 || warp >= 12) asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
+    else asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");
     if (warp == 0) {
         if (lane == 0) {
             long long g = 0;                               // K tiles of this pair so far
@@ -137,9 +150,9 @@ k_tc_project(const __grid_constant__ CUtensorMap tmRows, const __grid_constant__
                 for (int kt = p.k0; kt < p.k1 && alive; ++run) {
                     const int kt_end = kt + kRunTiles < p.k1 ? kt + kRunTiles : p.k1;
                     const uint32_t b = run & 1u, acc = tmem_base + b * 128u;
-                    alive = __all_sync(0xffffffffu, mbar_wait(&acc_empty[b], ((run >> 1) & 1u) ^ 1u, abort));
+                    alive = __all_sync(0xffffffffu, mbar_wait_cluster<false>(&acc_empty[b], ((run >> 1) & 1u) ^ 1u, abort));
                     for (const int k0 = kt; kt < kt_end && alive; ++kt) {
-                        alive = __all_sync(0xffffffffu, mbar_wait(&split_done[s], ph, abort));
+                        alive = __all_sync(0xffffffffu, mbar_wait(&full[s], ph, abort) && mbar_wait_cluster<true>(&peer_full[s], ph, abort) && mbar_wait_cluster<false>(&split_done[s], ph, abort));
                         if (!alive) break;
                         tc_fence_after();
                         const uint32_t st = st0 + (uint32_t)(s * kStageBytes);
@@ -159,6 +172,14 @@ k_tc_project(const __grid_constant__ CUtensorMap tmRows, const __grid_constant__
                     }
                 }
                 u += p.k1 - p.k0;
+            }
+        }
+    } else if (warp >= 12) {
+        if (q == 1 && lane == 0) {                          // what has landed in CTA 1 is the MMAs' to read
+            for (long long g = warp - 12; g < u_end - u_begin; g += kForwards) {
+                const int s = (int)(g % kStages);
+                if (!mbar_wait(&full[s], (uint32_t)(g / kStages) & 1u, abort)) break;
+                mbar_arrive_cluster(&peer_full[s], 0);
             }
         }
     } else if (warp >= 4) {
@@ -186,7 +207,7 @@ k_tc_project(const __grid_constant__ CUtensorMap tmRows, const __grid_constant__
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cta(&acc_empty[b], 0);
+            if (lane == 0) mbar_arrive_cluster_relaxed(&acc_empty[b], 0);
             ++run;
         };
         long long g0 = 0;                                   // K tiles of this pair before the current range
@@ -218,7 +239,7 @@ k_tc_project(const __grid_constant__ CUtensorMap tmRows, const __grid_constant__
                 tmem_st_wait();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_cta(&split_done[s], 0);
+                if (lane == 0) mbar_arrive_cluster_relaxed(&split_done[s], 0);
                 // run d of this range is drained once K tile 3 (d + 1) + 2 has been split, when its MMAs are mostly done; the MMAs that need its
                 // accumulator again start one K tile later
                 while (ok && (int)(run - run0 + 2) * kRunTiles - 1 <= i) drain();
@@ -290,7 +311,12 @@ cudaError_t launch_tc_project(const float* rows, int64_t ld, const float* sk_spl
     const int64_t tiles = (M + 255) / 256, nkt = (cols + tc::kProjBK - 1) / tc::kProjBK;
     const int64_t pairs = slices > 1 ? std::min<int64_t>(74, tiles * slices) : project_pairs(tiles, nkt);
     const int planes = project_planes(M, K, class_F);
-    cudaError_t e = allow_smem((const void*)tc::k_tc_project, 227 * 1024);
+    // the kernel hands registers from one half of its warps to the other: only as many as the launch holds
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, tc::k_tc_project);
+    if (e != cudaSuccess) return e;
+    if (fa.numRegs != tc::kProjRegs) return cudaErrorNotSupported;
+    e = allow_smem((const void*)tc::k_tc_project, 227 * 1024);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(2 * pairs));

@@ -34,3 +34,21 @@ def test_spectrum_of_wide_buffers(n, D):
     S, sigma = S.double().cpu().numpy(), sigma.double().cpu().numpy()
     assert np.max(np.abs(sigma ** 2 - expect)) <= 9e-6 * lam[0]
     assert np.linalg.norm(S @ S.T - np.diag(sigma ** 2), 2) <= 18e-6 * lam[0]
+
+
+@pytest.mark.parametrize("n", [200, 512])
+def test_the_same_rows_give_the_same_bits(n):
+    """Two CTAs hand operands and accumulators to one another many times per launch; every order of events has one result."""
+    g = torch.Generator().manual_seed(n)
+    rows = torch.randn(n, 40004, generator=g).cuda()
+    first = None
+    for _ in range(12):
+        fd = sage.SageFD(40004, min(n, 256), torch.float32, 0)
+        fd.update(rows)
+        fd.finalize()
+        S, sigma = fd.sketch()
+        assert fd.stats()["device_flags"] == 0
+        fd.close()
+        if first is None:
+            first = S, sigma
+        assert torch.equal(S, first[0]) and torch.equal(sigma, first[1])

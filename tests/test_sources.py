@@ -1,0 +1,20 @@
+"""What no run can show: rules that the kernels' sources keep."""
+import glob
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2510_02470_b200", "csrc")
+
+
+def _instructions(name):
+    text = "".join(open(f).read() for f in sorted(glob.glob(os.path.join(CSRC, "*.cu*"))))
+    return re.findall(name + r"[\w.:]*", text)
+
+
+def test_hand_offs_between_ctas_release_at_cluster_scope():
+    """An arrival on another CTA's barrier names its scope (the default is the CTA, which orders nothing between two of them): release
+    behind shared memory, relaxed where tensor memory and its fences carry the data; and the wait that belongs to it does, too."""
+    remote = [i for i in _instructions(r"mbarrier\.arrive") if "shared::cluster" in i]
+    assert remote and all(".release.cluster." in i or ".relaxed.cluster." in i for i in remote), remote
+    waits = _instructions(r"mbarrier\.try_wait")
+    assert any(".acquire.cluster." in i for i in waits) and any(".relaxed.cluster." in i for i in waits)
