@@ -263,6 +263,7 @@ __device__ __forceinline__ bool tri_phase(TriState<S>& T, TriShared<S>& sh, int 
                 for (int t = lc & (REP - 1); t < CL; t += REP) send_pair(map_to_cta(la, t), ysum, cval, map_to_cta(lb, t));
             }
             if (!wait_bytes(s_addr(&sh.bar[b]), (sk >> 1) & 1, wk.abort)) return false;
+            __syncwarp();                                   // rows_y and rows_c, written by other lanes
         }
         // both vectors at this thread's columns (pairs) and rows
         const float2 xk = CL == 1 ? make_float2(yb[kk], cb[kk]) : xb[kk];

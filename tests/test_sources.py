@@ -18,3 +18,10 @@ def test_hand_offs_between_ctas_release_at_cluster_scope():
     assert remote and all(".release.cluster." in i or ".relaxed.cluster." in i for i in remote), remote
     waits = _instructions(r"mbarrier\.try_wait")
     assert any(".acquire.cluster." in i for i in waits) and any(".relaxed.cluster." in i for i in waits)
+
+
+def test_votes_do_not_stand_in_for_warp_barriers():
+    """A vote orders no memory: where lanes read what others wrote to shared memory before a wait that ends in one, a __syncwarp follows."""
+    text = open(os.path.join(CSRC, "eig_tridiag.cu")).read()
+    step = text[text.index("auto step = [&]"):text.index("// both vectors at this thread's columns")]
+    assert re.search(r"wait_bytes\([^;]*\)\) return [^;]*;\s*__syncwarp\(\);", step)
