@@ -439,7 +439,63 @@ sage_status_t check_handle(const sage_fd* h) {
 
 }  // namespace
 
+namespace {
+// A graph that a thread puts together launch by launch, each behind the one before it: no stream is captured, so that whatever
+// other threads do meanwhile (a synchronisation of the device ends every capture that is open in the process) does not concern it.
+struct Recorder {
+    cudaGraph_t graph = nullptr;
+    cudaGraphNode_t last = nullptr;
+    int launches = 0;
+};
+thread_local Recorder* g_recorder = nullptr;
+}  // namespace
+
 namespace sage {
+cudaError_t launch_any(const void* kernel, const LaunchShape& shape, void** args, cudaStream_t st) {
+    if (Recorder* r = g_recorder) {
+        cudaGraphNodeParams p = {};
+        p.type = cudaGraphNodeTypeKernel;
+        p.kernel.func = const_cast<void*>(kernel);
+        p.kernel.gridDim = shape.grid;
+        p.kernel.blockDim = shape.block;
+        p.kernel.sharedMemBytes = (unsigned)shape.smem;
+        p.kernel.kernelParams = args;
+        cudaGraphEdgeData edge = {};
+        if (shape.chained) {
+            edge.from_port = cudaGraphKernelNodePortProgrammatic;
+            edge.type = cudaGraphDependencyTypeProgrammatic;
+        }
+        cudaGraphNode_t node = nullptr;
+        cudaError_t e = cudaGraphAddNode_v2(&node, r->graph, r->last ? &r->last : nullptr, r->last ? &edge : nullptr, r->last ? 1 : 0, &p);
+        if (e == cudaSuccess && shape.cluster > 1) {
+            cudaLaunchAttributeValue v = {};
+            v.clusterDim.x = shape.cluster;
+            v.clusterDim.y = v.clusterDim.z = 1;
+            e = cudaGraphKernelNodeSetAttribute(node, cudaLaunchAttributeClusterDimension, &v);
+        }
+        r->last = node;
+        r->launches += 1;
+        return e;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = shape.grid;
+    cfg.blockDim = shape.block;
+    cfg.dynamicSmemBytes = shape.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    cfg.attrs = at;
+    if (shape.chained) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (shape.cluster > 1) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        at[cfg.numAttrs].val.clusterDim.x = shape.cluster;
+        at[cfg.numAttrs].val.clusterDim.y = 1;
+        at[cfg.numAttrs++].val.clusterDim.z = 1;
+    }
+    return cudaLaunchKernelExC(&cfg, kernel, args);
+}
 cudaError_t allow_smem(const void* kernel, int bytes) {
     // set once per kernel and device: which is remembered in a small list (a handful of kernels)
     struct Seen { const void* kernel; int dev, bytes; };
@@ -725,46 +781,52 @@ static sage_status_t sketch_join_appends(sage_fd* s, cudaStream_t chain) {
 }
 
 // A full buffer's cycle in the merged form. Sixteen chains share the device and one host thread enqueues for all of them, so the
-// host bounds a pass over short rows: the launches of a cycle (the same every time but for the buffer copy) are captured
-// once the sketch has run a few and replayed as a graph, one host call instead of five.
+// host bounds a pass over short rows: the launches of a cycle (the same every time but for the buffer copy) are put into a graph
+// once the sketch has run a few, one host call instead of five. A stream that the caller is capturing takes the launches themselves.
 static sage_status_t run_cycle(sage_fd* s, cudaStream_t chain) {
     const int keep = s->delta_rank - 1;
-    constexpr int kDirect = 8;                 // cycles before a capture pays
+    constexpr int kDirect = 8;                 // cycles before a graph pays
+    auto direct = [&] { return enqueue_factor(s, s->m, 1, keep, 0, chain); };
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    CU_TRY(cudaStreamIsCapturing(chain, &capturing));
+    if (capturing != cudaStreamCaptureStatusNone || !s->cycle_graphs || s->eig_variant != 0) return direct();
     sage_fd::Cycle& c = s->cycle[s->cur];
-    if (c.exec) {
-        CU_TRY(cudaGraphLaunch(c.exec, chain));
-        count(s, c.launches);
-        s->tc_launches += c.tc_launches;
-        s->cur = 1 - s->cur;
-        s->fill = keep;
-        return SAGE_OK;
-    }
-    if (!s->cycle_graphs || s->cycles_run < kDirect) {
-        ++s->cycles_run;
-        return enqueue_factor(s, s->m, 1, keep, 0, chain);
-    }
-    const int cur = s->cur, fill = s->fill;
-    const int64_t l0 = s->launches, t0 = s->tc_launches;
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(chain, cudaStreamCaptureModeThreadLocal);
-    sage_status_t rc = SAGE_ERR_CUDA;
-    if (e == cudaSuccess) {
-        rc = enqueue_factor(s, s->m, 1, keep, 0, chain);
-        e = cudaStreamEndCapture(chain, &g);
-        if (e == cudaSuccess && rc == SAGE_OK) e = cudaGraphInstantiate(&c.exec, g, 0);
-        if (g) cudaGraphDestroy(g);
-    }
-    if (e != cudaSuccess || rc != SAGE_OK) {   // not captured: nothing has run yet
-        (void)cudaGetLastError();
-        c = sage_fd::Cycle();
-        s->cycle_graphs = false;
-        s->cur = cur;
+    if (!c.exec) {
+        if (s->cycles_run < kDirect) {
+            ++s->cycles_run;
+            return direct();
+        }
+        const int cur = s->cur, fill = s->fill;
+        const int64_t l0 = s->launches, t0 = s->tc_launches;
+        Recorder rec;
+        cudaError_t e = cudaGraphCreate(&rec.graph, 0);
+        sage_status_t rc = SAGE_ERR_CUDA;
+        if (e == cudaSuccess) {
+            g_recorder = &rec;
+            rc = direct();
+            g_recorder = nullptr;
+            if (rc == SAGE_OK) e = cudaGraphInstantiate(&c.exec, rec.graph, 0);
+            cudaGraphDestroy(rec.graph);
+        }
+        c.launches = rec.launches;
+        c.tc_launches = (int)(s->tc_launches - t0);
+        g_launches.fetch_sub(s->launches - l0, std::memory_order_relaxed);
+        s->cur = cur;                          // nothing has run yet
         s->fill = fill;
-        return enqueue_factor(s, s->m, 1, keep, 0, chain);
+        s->launches = l0;
+        s->tc_launches = t0;
+        if (e != cudaSuccess || rc != SAGE_OK) {
+            (void)cudaGetLastError();
+            c = sage_fd::Cycle();
+            s->cycle_graphs = false;
+            return direct();
+        }
     }
-    c.launches = (int)(s->launches - l0);
-    c.tc_launches = (int)(s->tc_launches - t0);
     CU_TRY(cudaGraphLaunch(c.exec, chain));
+    count(s, c.launches);
+    s->tc_launches += c.tc_launches;
+    s->cur = 1 - s->cur;
+    s->fill = keep;
     return SAGE_OK;
 }
 

@@ -1156,21 +1156,7 @@ cudaError_t run_tridiag(const float* K, int ldk, int n, TriWork wk, EigInfo* inf
     const int smem = (S::CL == 1 ? n : kOwnRows<S>) * (n4 + 4) * 4;
     cudaError_t e = allow_smem((const void*)k_tridiag<S>, most);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(S::CL);
-    cfg.blockDim = dim3(S::NT);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = S::CL;
-    at[1].val.clusterDim.y = 1;
-    at[1].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = S::CL > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, k_tridiag<S>, K, ldk, n, 0, wk, 0, (int)S::G, info);
+    return launch(k_tridiag<S>, LaunchShape{dim3(S::CL), dim3(S::NT), (size_t)smem, (unsigned)S::CL}, st, K, ldk, n, 0, wk, 0, (int)S::G, info);
 }
 
 template <int NQ>

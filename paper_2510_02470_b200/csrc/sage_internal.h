@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <algorithm>
+#include <tuple>
 
 #include "sage.h"
 
@@ -16,19 +17,28 @@ namespace sage {
 // chain_wait() in it returns when every kernel before it on the stream has finished and its results are visible (each kernel
 // of the chain waits, so this holds for all of them), and nothing of theirs is touched before. chain_release() lets the next
 // one start; kernels that run long call it near their end, so that the next does not sit on an SM for nothing.
+// Every launch of a shrink cycle goes through launch(): it enqueues, or adds the launch to the graph that the calling thread is
+// putting together (see run_cycle in api.cu).
+struct LaunchShape {
+    dim3 grid, block;
+    size_t smem = 0;
+    unsigned cluster = 1;
+    bool chained = true;
+};
+cudaError_t launch_any(const void* kernel, const LaunchShape& shape, void** args, cudaStream_t st);
 template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+cudaError_t launch(void (*kernel)(P...), const LaunchShape& shape, cudaStream_t st, A... a) {
+    std::tuple<P...> values(static_cast<P>(a)...);
+    return std::apply(
+        [&](auto&... v) {
+            void* args[] = {&v...};
+            return launch_any(reinterpret_cast<const void*>(kernel), shape, args, st);
+        },
+        values);
+}
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... a) {
+    return launch(kernel, LaunchShape{grid, block, smem}, st, a...);
 }
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -212,8 +222,5 @@ cudaError_t launch_select(const float* scores, int64_t N, int64_t k, int64_t* id
 // Hooks into the C ABI's bookkeeping for entry points defined outside api.cu.
 void set_error_message(const char* msg);   // becomes the calling thread's sage_last_error()
 void count_launches(int k);                // adds to sage_launch_count()
-
-int launches_append();
-int launches_gemm_nt(int splits);
 
 }  // namespace sage

@@ -269,21 +269,8 @@ cudaError_t run_cluster_sort(const SortArgs& a, u64* b0, u64* b1, int64_t k, dou
                              long long* kc_out, cudaStream_t st) {
     cudaError_t e = allow_smem((const void*)k_sort_cluster<MODE>, (int)sizeof(ClusterShared));
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kClSize);
-    cfg.blockDim = dim3(kClThreads);
-    cfg.dynamicSmemBytes = sizeof(ClusterShared);
-    cfg.stream = st;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kClSize;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, k_sort_cluster<MODE>, a, b0, b1, k, keep_rate, idx, order, starts, kc_out);
+    return launch(k_sort_cluster<MODE>, LaunchShape{dim3(kClSize), dim3(kClThreads), sizeof(ClusterShared), (unsigned)kClSize}, st, a, b0, b1, k, keep_rate, idx,
+                  order, starts, kc_out);
 }
 
 // ---- few picks: the k-th key first, then only the k best are put in order --------------------------------------------
@@ -459,21 +446,7 @@ cudaError_t run_rank(const u64* keys, const float* scores, int n, int64_t k, int
 cudaError_t run_top_keys(const float* scores, int64_t N, int64_t k, u64* out, cudaStream_t st) {
     cudaError_t e = allow_smem((const void*)k_top_keys, (int)sizeof(FilterShared));
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kClSize);
-    cfg.blockDim = dim3(kClThreads);
-    cfg.dynamicSmemBytes = sizeof(FilterShared);
-    cfg.stream = st;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kClSize;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, k_top_keys, scores, N, k, out);
+    return launch(k_top_keys, LaunchShape{dim3(kClSize), dim3(kClThreads), sizeof(FilterShared), (unsigned)kClSize}, st, scores, N, k, out);
 }
 
 // ---- three launches per pass, any N ------------------------------------------------------------------------------

@@ -374,13 +374,10 @@ cudaError_t launch_gemm_nt(const void* A, sage_dtype_t dt, int64_t lda, const fl
     kps = ((kps + BK - 1) / BK) * BK;
     if (class_F > 0) kps = class_F;
     const int a_shared = class_F > 0 ? 1 : 0;
-    dim3 grid((M + BM - 1) / BM, (N + BN - 1) / BN, splits);
+    const LaunchShape shape{dim3((M + BM - 1) / BM, (N + BN - 1) / BN, splits), dim3(256), 0, 1, false};
     if (dt == SAGE_F32)
-        k_gemm_nt<float><<<grid, 256, 0, st>>>(static_cast<const float*>(A), lda, Bm, ldb, M, N, K, kps, a_shared, C, ldc, split_stride);
-    else
-        k_gemm_nt<__nv_bfloat16><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(A), lda, Bm, ldb, M, N, K, kps, a_shared, C,
-                                                       ldc, split_stride);
-    return cudaGetLastError();
+        return launch(k_gemm_nt<float>, shape, st, static_cast<const float*>(A), lda, Bm, ldb, M, N, K, kps, a_shared, C, ldc, split_stride);
+    return launch(k_gemm_nt<__nv_bfloat16>, shape, st, static_cast<const __nv_bfloat16*>(A), lda, Bm, ldb, M, N, K, kps, a_shared, C, ldc, split_stride);
 }
 
 cudaError_t launch_to_bf16(const float* src, int64_t lds, int rows, int64_t cols, __nv_bfloat16* hi, __nv_bfloat16* lo, int64_t ldd,
@@ -418,9 +415,8 @@ cudaError_t launch_gram_sym_reduce(const float* parts, int splits, int64_t strid
 cudaError_t launch_rebuild(const float* Ur, int ldu, const float* Bsrc, float* Bdst, int64_t pitch, int64_t D, int r, int keep,
                            int m_total, cudaStream_t st) {
     (void)D;
-    dim3 grid((unsigned)((pitch + RN - 1) / RN), (unsigned)((m_total + RM - 1) / RM));
-    k_rebuild<<<grid, 256, 0, st>>>(Ur, ldu, Bsrc, Bdst, pitch, r, keep, m_total);
-    return cudaGetLastError();
+    const LaunchShape shape{dim3((unsigned)((pitch + RN - 1) / RN), (unsigned)((m_total + RM - 1) / RM)), dim3(256), 0, 1, false};
+    return launch(k_rebuild, shape, st, Ur, ldu, Bsrc, Bdst, pitch, r, keep, m_total);
 }
 
 }  // namespace sage

@@ -251,21 +251,8 @@ cudaError_t launch_tc_gram_pair(const float* B, int64_t ldb, int r, int64_t K, i
     if (e != cudaSuccess) return e;
     if (fa.numRegs != tc::kPairRegs) return cudaErrorNotSupported;
     if ((e = allow_smem((const void*)tc::k_tc_gram_pair, 227 * 1024)) != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2u * (unsigned)(n_off ? n_off + 2 * n_diag : n_diag));
-    cfg.blockDim = dim3(tc::kPairThreads);
-    cfg.dynamicSmemBytes = tc::kPairSmem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, tc::k_tc_gram_pair, tm, r, (long long)K, n_diag, n_off, C, (long long)ldc, (long long)split_stride, err);
+    const unsigned pairs = (unsigned)(n_off ? n_off + 2 * n_diag : n_diag);
+    return launch(tc::k_tc_gram_pair, LaunchShape{dim3(2 * pairs), dim3(tc::kPairThreads), tc::kPairSmem, 2}, st, tm, r, K, n_diag, n_off, C, ldc, split_stride, err);
 }
 
 }  // namespace sage

@@ -318,22 +318,8 @@ cudaError_t launch_tc_project(const float* rows, int64_t ld, const float* sk_spl
     if (fa.numRegs != tc::kProjRegs) return cudaErrorNotSupported;
     e = allow_smem((const void*)tc::k_tc_project, 227 * 1024);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * pairs));
-    cfg.blockDim = dim3(tc::kProjThreads);
-    cfg.dynamicSmemBytes = tc::kProjSmem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, tc::k_tc_project, tmRows, tmSk, (int)M, ell, (int)nkt, slices, (long long)class_F,
-                              (long long)(tiles * slices * nkt), planes, out, (long long)plane_stride, err);
+    return launch(tc::k_tc_project, LaunchShape{dim3((unsigned)(2 * pairs)), dim3(tc::kProjThreads), tc::kProjSmem, 2}, st, tmRows, tmSk, (int)M, ell, (int)nkt, slices,
+                  class_F, tiles * slices * nkt, planes, out, plane_stride, err);
 }
 
 }  // namespace sage

@@ -1,0 +1,93 @@
+"""The host code behind the C ABI (csrc/api.cu) against a runtime that keeps books (fake_cuda.cpp): what it enqueues, and what it
+leaves behind where a call of the runtime fails. Runs on the CPU."""
+import ctypes as C
+import os
+import subprocess
+
+import pytest
+
+import paper_2510_02470_b200 as sage
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("host") / "libhost.so")
+    csrc = os.path.join(ROOT, "paper_2510_02470_b200", "csrc")
+    cmd = ["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", csrc, "-I", os.path.join(CUDA, "include"),
+           "-x", "c++", os.path.join(csrc, "api.cu"), os.path.join(HERE, "fake_cuda.cpp"), "-o", out, "-Wl,-z,defs", "-Wl,-Bsymbolic", "-lpthread"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
+    L = C.CDLL(out)
+    for name, (res, args) in sage.SIGNATURES.items():
+        if hasattr(L, name):
+            getattr(L, name).restype, getattr(L, name).argtypes = res, args
+    return L
+
+
+def _handle(L, D=64, ell=4, P=1, dtype=0):
+    h = C.c_void_p()
+    assert L.sage_fd_create(C.byref(h), D, ell, dtype, 0) == 0
+    if P > 1:
+        assert L.sage_fd_set_option(h, 6, P) == 0
+    return h
+
+
+def _appends(L):
+    buf = (C.c_longlong * 5000)()
+    n = L.fake_appends(buf, 1000)
+    return [tuple(buf[5 * i:5 * i + 5]) for i in range(n)]
+
+
+def _calls(L, name):
+    return L.fake_calls(name.encode())
+
+
+def test_cycles_become_graphs_without_a_capture(lib):
+    """The merged form replays its cycles as graphs. A captured stream would be every other thread's business: a synchronisation of
+    the device anywhere in the process ends the capture and fails itself."""
+    h = _handle(lib, P=2)
+    b0, g0 = _calls(lib, "cudaStreamBeginCapture"), _calls(lib, "cudaGraphLaunch")
+    assert lib.sage_fd_update(h, 0x1000, 2 * 5 * 40, 64, None) == 0
+    assert _calls(lib, "cudaStreamBeginCapture") == b0 and _calls(lib, "cudaGraphLaunch") > g0
+    st = sage.SageStats()
+    assert lib.sage_fd_stats(h, C.byref(st)) == 0
+    launches = st.kernel_launches
+    lib.sage_fd_destroy(h)
+    # the same rows with direct launches (per-kernel timing on): as many kernels
+    h = _handle(lib, P=2)
+    lib.sage_fd_set_option(h, 3, 1)
+    assert lib.sage_fd_update(h, 0x1000, 2 * 5 * 40, 64, None) == 0
+    assert lib.sage_fd_stats(h, C.byref(st)) == 0 and st.kernel_launches == launches
+    lib.sage_fd_destroy(h)
+
+
+def test_a_captured_stream_takes_no_graphs(lib):
+    """Updates that the caller captures run launch by launch, also when the sketch has graphs of its cycles by then: a graph cannot be
+    launched into a capture."""
+    h = _handle(lib, P=2)
+    assert lib.sage_fd_update(h, 0x1000, 2 * 5 * 40, 64, None) == 0
+    g0, i0 = _calls(lib, "cudaGraphLaunch"), _calls(lib, "cudaGraphInstantiate")
+    lib.fake_capturing(1)
+    assert lib.sage_fd_update(h, 0x1000, 2 * 5 * 40, 64, None) == 0
+    lib.fake_capturing(0)
+    assert _calls(lib, "cudaGraphLaunch") == g0 and _calls(lib, "cudaGraphInstantiate") == i0
+    lib.sage_fd_destroy(h)
+
+
+@pytest.mark.parametrize("what", ["cudaGraphCreate", "cudaGraphAddNode_v2", "cudaGraphInstantiate"])
+def test_a_cycle_that_cannot_become_a_graph_runs_directly(lib, what):
+    h = _handle(lib, P=2)
+    lib.fake_fail(what.encode(), 1)
+    assert lib.sage_fd_update(h, 0x1000, 2 * 5 * 40, 64, None) == 0
+    st = sage.SageStats()
+    assert lib.sage_fd_stats(h, C.byref(st)) == 0
+    launches = st.kernel_launches
+    lib.sage_fd_destroy(h)
+    h = _handle(lib, P=2)
+    assert lib.sage_fd_update(h, 0x1000, 2 * 5 * 40, 64, None) == 0
+    assert lib.sage_fd_stats(h, C.byref(st)) == 0 and st.kernel_launches == launches
+    lib.sage_fd_destroy(h)
