@@ -686,6 +686,9 @@ sage_status_t sage_fd_reset(sage_fd_t* h) {
     h->rows_in_place = 0;
     h->app_pending = false;
     h->in_epoch = -1;
+    h->pend = RowSrc();
+    h->pend_n = 0;
+    h->used = nullptr;
     for (sage_fd* k : h->kids) ST_TRY(sage_fd_reset(k));
     return SAGE_OK;
 }
@@ -1029,10 +1032,15 @@ static sage_status_t update_from(sage_fd* h, RowSrc src, int64_t n, cudaStream_t
         if (s->used) {
             const sage_status_t fl = flush_pending(s, s->used);
             if (rc == SAGE_OK) rc = fl;
-            cudaError_t e = cudaEventRecord(s->ev_rows, s->used);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, s->ev_rows, 0);
+            // every sketch is flushed and joined, whatever failed before: nothing of this call may read its rows later
+            auto join = [&]() -> sage_status_t {
+                CU_TRY(cudaEventRecord(s->ev_rows, s->used));
+                CU_TRY(cudaStreamWaitEvent(st, s->ev_rows, 0));
+                return SAGE_OK;
+            };
+            const sage_status_t jn = join();
+            if (rc == SAGE_OK) rc = jn;
             s->used = nullptr;
-            if (rc == SAGE_OK) CU_TRY(e);
         }
     }
     return rc;

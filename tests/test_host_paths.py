@@ -91,3 +91,25 @@ def test_a_cycle_that_cannot_become_a_graph_runs_directly(lib, what):
     assert lib.sage_fd_update(h, 0x1000, 2 * 5 * 40, 64, None) == 0
     assert lib.sage_fd_stats(h, C.byref(st)) == 0 and st.kernel_launches == launches
     lib.sage_fd_destroy(h)
+
+
+@pytest.mark.parametrize("what", ["cudaEventRecord", "cudaStreamWaitEvent", "cudaLaunchKernelExC"])
+@pytest.mark.parametrize("nth", range(1, 9))
+def test_no_row_of_a_failed_update_is_read_later(lib, what, nth):
+    """Whichever call of the runtime fails during an update of the merged form, the rows that it held back for a joint append are
+    either appended by that call or forgotten: after a reset, an update appends its own rows only."""
+    h = _handle(lib, P=4)
+    assert lib.sage_fd_update(h, 0x1000, 7, 64, None) == 0
+    _appends(lib)
+    lib.fake_fail(what.encode(), nth)
+    rc = lib.sage_fd_update(h, 0x100000, 18, 64, None)
+    lib.fake_fail(what.encode(), 1 << 30)
+    first = _appends(lib)
+    lib.sage_fd_join(h, None)
+    assert lib.sage_fd_reset(h) == 0
+    assert lib.sage_fd_update(h, 0x900000, 40, 64, None) == 0
+    later = _appends(lib)
+    assert later and all(0x900000 <= a[0] < 0x900000 + 40 * 256 and (a[3] == 0 or 0x900000 <= a[2] < 0x900000 + 40 * 256) for a in later), later
+    assert sum(a[1] + a[3] for a in later) == 40
+    assert rc in (0, 4) and all(0x100000 <= a[0] < 0x100000 + 18 * 256 for a in first)
+    lib.sage_fd_destroy(h)
