@@ -543,7 +543,8 @@ int64_t sage_select_count(int64_t N, double keep_rate) {
     return (int64_t)k;
 }
 
-// Forgets the captured cycles (their launches hold what the options said); waits for the device if there are any.
+// Forgets the graphs of the cycles, where an option changes that their launches hold (which kernels, delta's rank; the iterative
+// solve is not in graphs); waits for the device if there are any.
 static void drop_cycles(sage_fd* s) {
     if (s->cycle[0].exec || s->cycle[1].exec) cudaDeviceSynchronize();
     for (sage_fd::Cycle& c : s->cycle) {
@@ -700,11 +701,9 @@ sage_status_t sage_fd_set_option(sage_fd_t* h, int key, double value) {
         for (sage_fd* k : h->kids) k->prof.mask = h->prof.mask;
         return SAGE_OK;
     }
-    {
-        DeviceGuard g(h->device);
-        drop_cycles(h);
-    }
     if (key == 4) {                          // 0: CUDA-core kernels only, 1: tensor-core kernels where possible
+        DeviceGuard g(h->device);
+        if (h->use_tc != (value != 0.0)) drop_cycles(h);
         h->use_tc = value != 0.0;
         for (sage_fd* k : h->kids) k->use_tc = h->use_tc;
         return SAGE_OK;
@@ -733,6 +732,8 @@ sage_status_t sage_fd_set_option(sage_fd_t* h, int key, double value) {
     }
     const int v = (int)value;
     if (key == 1 && v >= 2 && v <= h->m - 1) {
+        DeviceGuard g(h->device);
+        if (h->delta_rank != v) drop_cycles(h);
         h->delta_rank = v;
         for (sage_fd* k : h->kids) k->delta_rank = v;
         return SAGE_OK;
@@ -1827,7 +1828,8 @@ sage_status_t sage_fd_import(sage_fd_t* h, const void* src_host, size_t bytes, v
     ST_TRY(sage_fd_reset(h));
     ST_TRY(sage_fd_set_option(h, 6, (double)hd.P));
     h->block = hd.block;
-    h->delta_rank = hd.delta_rank;                           // (the call above dropped the captured cycles)
+    if (h->delta_rank != hd.delta_rank) drop_cycles(h);
+    h->delta_rank = hd.delta_rank;
     for (sage_fd* k : h->kids) k->delta_rank = hd.delta_rank;
     if (hd.nsk > 1) ST_TRY(ensure_sketches(h));
     const char* q = static_cast<const char*>(src_host) + sizeof hd;

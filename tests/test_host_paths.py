@@ -113,3 +113,37 @@ def test_no_row_of_a_failed_update_is_read_later(lib, what, nth):
     assert sum(a[1] + a[3] for a in later) == 40
     assert rc in (0, 4) and all(0x100000 <= a[0] < 0x100000 + 18 * 256 for a in first)
     lib.sage_fd_destroy(h)
+
+
+def test_options_that_no_cycle_holds_leave_its_graphs_alone(lib):
+    """Only an option that changes a cycle's launches costs the graphs and the wait for the device that goes with it; a call that is
+    refused changes nothing."""
+    h = _handle(lib, P=2)
+    assert lib.sage_fd_update(h, 0x1000, 400, 64, None) == 0
+    for key, value, status in ((3, 0, 0), (5, 1, 0), (5, 0, 0), (9, 0, 0), (8, 1, 0), (8, 0, 0), (4, 1, 0), (1, 3, 2), (6, 3, 2), (77, 1, 2)):
+        n0, i0 = _calls(lib, "cudaDeviceSynchronize"), _calls(lib, "cudaGraphInstantiate")
+        assert lib.sage_fd_set_option(h, key, value) == status
+        assert lib.sage_fd_update(h, 0x1000, 100, 64, None) == 0
+        assert _calls(lib, "cudaDeviceSynchronize") == n0 and _calls(lib, "cudaGraphInstantiate") == i0, key
+    for key, value in ((4, 0), (4, 1)):
+        d0 = _calls(lib, "cudaGraphExecDestroy")
+        assert lib.sage_fd_set_option(h, key, value) == 0 and _calls(lib, "cudaGraphExecDestroy") > d0
+        assert lib.sage_fd_update(h, 0x1000, 400, 64, None) == 0
+    assert lib.sage_fd_reset(h) == 0
+    d0 = _calls(lib, "cudaGraphExecDestroy")
+    assert lib.sage_fd_set_option(h, 1, 3) == 0 and _calls(lib, "cudaGraphExecDestroy") > d0
+    lib.sage_fd_destroy(h)
+
+
+def test_a_checkpoint_with_another_rank_costs_the_graphs(lib):
+    a, b = _handle(lib, P=2), _handle(lib, P=2)
+    lib.sage_fd_set_option(a, 1, 3)
+    assert lib.sage_fd_update(a, 0x1000, 10, 64, None) == 0 and lib.sage_fd_update(b, 0x1000, 400, 64, None) == 0
+    need = C.c_size_t()
+    lib.sage_fd_export_size(a, C.byref(need))
+    blob = C.create_string_buffer(need.value)
+    assert lib.sage_fd_export(a, blob, need.value, None) == 0
+    d0 = _calls(lib, "cudaGraphExecDestroy")
+    assert lib.sage_fd_import(b, blob, need.value, None) == 0 and _calls(lib, "cudaGraphExecDestroy") > d0
+    lib.sage_fd_destroy(a)
+    lib.sage_fd_destroy(b)
