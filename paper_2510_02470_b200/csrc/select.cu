@@ -192,7 +192,7 @@ k_sort_cluster(SortArgs a, u64* __restrict__ b0, u64* __restrict__ b1, int64_t k
         if (MODE == EMIT_PICK && last) {
             // quotas: k_c = floor(k n_c / n), the k - sum largest remainders (ties: smaller class) get one more
             const long long n_valid = (long long)sh.excl[a.C];
-            double kd = floor(keep_rate * (double)n_valid + 0.5);
+            double kd = floor(__dadd_rn(__dmul_rn(keep_rate, (double)n_valid), 0.5));     // rounded twice, as sage_select_count does
             kd = kd < 0.0 ? 0.0 : kd > (double)n_valid ? (double)n_valid : kd;
             const long long kk = n_valid > 0 ? (long long)kd : 0;
             if (tid < a.C) {

@@ -32,6 +32,15 @@ def test_selection_by_class_at_the_edges(N, C):
     assert kc == kc_ref.tolist() and np.array_equal(idx.cpu().numpy(), idx_ref)
 
 
+@pytest.mark.parametrize("n,rate", [(11, 0.04545454545454545), (25, 0.019999999999999997), (35, 0.014285714285714284), (44, 0.011363636363636362)])
+def test_quota_of_the_classes_is_the_count_of_a_selection(n, rate):
+    """floor(rate n + 0.5) with the product rounded first: a fused multiply-add gives one less here."""
+    a = np.linspace(-1.0, 1.0, n).astype(np.float32)
+    labels = np.zeros(n, dtype=np.int32)
+    idx, kc = sage.sage_select_classes(torch.from_numpy(a).to(DEV), torch.from_numpy(labels).to(DEV), 3, rate)
+    assert sage.sage_select_count(n, rate) == 1 and kc == [1, 0, 0] and idx.cpu().tolist() == [n - 1]
+
+
 @pytest.mark.parametrize("N,C,ell", [(1, 1, 4), (9000, 255, 33), (9000, 256, 16), (132000, 12, 8), (2000, 20000, 5)])
 def test_class_centroids_at_the_edges(N, C, ell):
     """The centroid is a sum in fp64 of the library's own fp32 projections, rounded once: 2^-24, and 1e-6 for the fp32 dot
