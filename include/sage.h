@@ -211,8 +211,8 @@ sage_status_t sage_select_classes(const float* scores, const int32_t* labels, in
  * (about 4.07 MiB, held by every device that loads the library until the process exits), so
  *   N <= 262,144 scores; larger N returns SAGE_ERR_UNSUPPORTED with a message naming the limit.
  * Arguments, ordering, tie rule and k_out are those of sage_select; it runs on the CURRENT device.
- * The first call on each device looks up the array's device address (a synchronous query, no
- * allocation); make that first call before starting any stream capture. All calls on a device share the
+ * The first call on each device looks up the array's device address and loads the kernels of every size (synchronous queries; the
+ * driver may take device memory for their code); make that first call before starting any stream capture. All calls on a device share the
  * one array: nothing in it needs clearing between calls (every word is written before it is read), but
  * two calls whose kernels can overlap on the GPU (different streams, no ordering) race on it and give
  * undefined results. Calls neither allocate nor free: no cudaMalloc, cudaFree or stream-ordered pool. */

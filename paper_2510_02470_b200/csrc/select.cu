@@ -670,6 +670,20 @@ cudaError_t launch_select(const float* scores, int64_t N, int64_t k, int64_t* id
     return sort_launches(a, scratch, k, idx, nullptr, st);
 }
 
+// Brings every kernel that launch_select can take, whatever its sizes, onto the current device: with lazy loading the first launch of
+// a kernel loads it, and its code takes device memory.
+static cudaError_t load_selection() {
+    cudaError_t e = allow_smem((const void*)k_rank, kRankMax * 8);
+    if (e == cudaSuccess) e = allow_smem((const void*)k_top_keys, (int)sizeof(FilterShared));
+    if (e == cudaSuccess) e = allow_smem((const void*)k_sort_cluster<EMIT_TOPK>, (int)sizeof(ClusterShared));
+    for (const void* kernel : {(const void*)k_rank, (const void*)k_top_keys, (const void*)k_sort_cluster<EMIT_TOPK>, (const void*)k_make_keys, (const void*)k_histogram,
+                               (const void*)k_scan, (const void*)k_scatter}) {
+        cudaFuncAttributes fa;
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+    }
+    return e;
+}
+
 cudaError_t launch_class_order(const int* labels, int64_t N, int C, void* scratch, unsigned* order, unsigned* starts, cudaStream_t st) {
     const SortArgs a = {nullptr, labels, N, C, 0, label_passes_of(C)};
     cudaError_t e = cudaSuccess;
@@ -784,6 +798,13 @@ extern "C" sage_status_t sage_select_static(const float* scores, int64_t N, doub
                     char msg[200];
                     snprintf(msg, sizeof msg, "sage_select_static: cudaGetSymbolAddress failed on device %d: %s", dev,
                              cudaGetErrorString(e));
+                    sage::set_error_message(msg);
+                    return SAGE_ERR_CUDA;
+                }
+                e = sage::load_selection();   // other sizes run other kernels
+                if (e != cudaSuccess) {
+                    char msg[200];
+                    snprintf(msg, sizeof msg, "sage_select_static: loading its kernels failed on device %d: %s", dev, cudaGetErrorString(e));
                     sage::set_error_message(msg);
                     return SAGE_ERR_CUDA;
                 }

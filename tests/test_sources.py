@@ -25,3 +25,18 @@ def test_votes_do_not_stand_in_for_warp_barriers():
     text = open(os.path.join(CSRC, "eig_tridiag.cu")).read()
     step = text[text.index("auto step = [&]"):text.index("// both vectors at this thread's columns")]
     assert re.search(r"wait_bytes\([^;]*\)\) return [^;]*;\s*__syncwarp\(\);", step)
+
+
+def test_the_first_static_selection_loads_every_kernel_of_the_others():
+    """sage_select_static promises that no call but the first on a device loads anything, whatever the sizes: every kernel that the
+    launchers behind it name is in the list that the first call goes through."""
+    text = open(os.path.join(CSRC, "select.cu")).read()
+
+    def body(name):
+        at = re.search(r"\n[^\n]*\b" + name + r"\([^;{]*\{", text)
+        return text[at.start():text.index("\n}\n", at.end())]
+
+    used = set()
+    for f in ("run_rank", "run_top_keys", "run_cluster_sort", "sort_launches"):
+        used |= set(re.findall(r"launch(?:_chained)?\((k_\w+)", body(f))) | set(re.findall(r"\b(k_\w+)<<<", body(f)))
+    assert used == set(re.findall(r"\(const void\*\)(k_\w+)", body("load_selection"))) and len(used) >= 7
