@@ -1597,12 +1597,13 @@ sage_status_t sage_score_classes(sage_fd_t* h, const int32_t* labels, int32_t nu
     }
     h->class_num = num_classes;
     void* scratch = nullptr;
-    CU_TRY(scratch_alloc(&scratch, class_scratch_bytes(h->N_total, h->ell, num_classes), st));
+    const size_t bytes = class_scratch_bytes(h->N_total, h->ell, num_classes);
+    if (bytes > 0) CU_TRY(scratch_alloc(&scratch, bytes, st));
     const cudaError_t e = launch_class_scores(h->zhat, labels, h->N_total, h->ell, num_classes, h->class_U, h->class_counts, scores, scratch, st);
-    const cudaError_t e2 = cudaFreeAsync(scratch, st);
+    const cudaError_t e2 = scratch ? cudaFreeAsync(scratch, st) : cudaSuccess;
     CU_TRY(e);
     CU_TRY(e2);
-    count(h, h->N_total > 0 ? 4 : 2);
+    count(h, class_score_launches(h->N_total, h->ell, num_classes));
     return SAGE_OK;
 }
 

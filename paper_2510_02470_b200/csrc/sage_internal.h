@@ -197,13 +197,15 @@ cudaError_t launch_consensus_score(const double* zsum, const float* zhat, int64_
                                    cudaStream_t st);
 
 // Class-balanced variant. U (C x ell) receives the unit centroids, counts (C) the class sizes, scores (N) the
-// per-class agreement scores; labels outside [0, C) score 0. scratch: class_scratch_bytes.
+// per-class agreement scores; labels outside [0, C) score 0. scratch: class_scratch_bytes (may be none).
 size_t class_scratch_bytes(int64_t N, int ell, int C);
+int class_score_launches(int64_t N, int ell, int C);
 cudaError_t launch_class_scores(const float* zhat, const int* labels, int64_t N, int ell, int C, float* U, int* counts, float* scores,
                                 void* scratch, cudaStream_t st);
 // Rows grouped by class, ascending index inside a class, rows without a class last: order (N); starts (C + 1): first place of
 // each class. scratch: select_scratch_bytes.
 cudaError_t launch_class_order(const int* labels, int64_t N, int C, void* scratch, unsigned* order, unsigned* starts, cudaStream_t st);
+int class_order_launches(int64_t N, int C);
 // starts as above; counts (C, may be null): class sizes.
 cudaError_t launch_class_starts(const int* labels, int64_t N, int C, unsigned* starts, unsigned* counts, cudaStream_t st);
 // Per-class top-k_c. One launch, quotas included, where class_select_in_one says so: kc receives the C quotas and their sum.

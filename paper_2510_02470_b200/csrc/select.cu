@@ -703,6 +703,10 @@ cudaError_t launch_class_order(const int* labels, int64_t N, int C, void* scratc
     return cudaGetLastError();
 }
 
+int class_order_launches(int64_t N, int C) {
+    return N > kClusterMax ? 2 + 1 + 3 * label_passes_of(C) + 1 : C > 255 ? 3 : 1;
+}
+
 cudaError_t launch_class_starts(const int* labels, int64_t N, int C, unsigned* starts, unsigned* counts, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(starts, 0, (size_t)(C + 1) * sizeof(unsigned), st);
     if (e != cudaSuccess) return e;

@@ -59,3 +59,27 @@ def test_class_centroids_at_the_edges(N, C, ell):
     assert np.array_equal(cnt.cpu().numpy(), cnt_ref)
     assert np.max(np.abs(U.double().cpu().numpy() - U_ref)) <= 6.1e-8
     assert np.max(np.abs(a.double().cpu().numpy() - a_ref)) <= 1e-6
+
+
+@pytest.mark.parametrize("N,C,ell", [(2, 1, 4), (100, 1000, 64), (255, 3, 32), (256, 2, 33), (257, 300, 65), (511, 7, 256), (512, 1, 64), (512, 1, 65), (512, 700, 130), (2048, 40, 64), (2049, 40, 64), (2048, 9765, 8), (2048, 9766, 8)])
+def test_class_centroids_of_few_rows(N, C, ell):
+    """Around the size from which rows are grouped by class first; bounds as above. The launch counter follows the path."""
+    D = 20
+    r = np.random.default_rng(N * 7 + C)
+    labels = r.integers(-1, C + 1, size=N).astype(np.int32)
+    labels[N // 2:] = C - 1                                          # one large class
+    fd = sage.SageFD(D, ell, torch.float32, 0)
+    fd.load_sketch(torch.from_numpy(r.standard_normal((ell, D)).astype(np.float32)).to(DEV))
+    fd.score(torch.from_numpy((r.standard_normal((N, D)) + 0.3).astype(np.float32)).to(DEV))
+    zhat = fd.intermediates(N)[0].double().cpu().numpy()
+    n0 = fd.stats()["kernel_launches"]
+    a = fd.score_classes(torch.from_numpy(labels).to(DEV), C)
+    launches = fd.stats()["kernel_launches"] - n0
+    U, cnt = fd.class_centroids()
+    fd.close()
+    a_ref, U_ref, cnt_ref = cb.class_scores(zhat, labels, C)
+    assert np.array_equal(cnt.cpu().numpy(), cnt_ref)
+    assert np.max(np.abs(U.double().cpu().numpy() - U_ref)) <= 6.1e-8
+    assert np.max(np.abs(a.double().cpu().numpy() - a_ref)) <= 1e-6
+    few = N <= 2048 and N * max(32, 1 << (ell - 1).bit_length()) <= 32768 * C and N * C <= 20000000
+    assert launches == (2 if few else (3 if C > 255 else 1) + (3 if C <= 8192 else 2))
