@@ -1686,7 +1686,7 @@ sage_status_t sage_select_classes(const float* scores, const int32_t* labels, in
                 CU_TRY(cudaMemcpyAsync(d_offs, offs.data(), (size_t)C * 8, cudaMemcpyHostToDevice, st));
                 CU_TRY(launch_class_pick(scores, labels, N, C, scratch, d_starts, d_kc, d_offs, idx, st));
                 CU_TRY(cudaStreamSynchronize(st));        // kc / offs are host vectors of this call
-                count(nullptr, 4 + 3 * (4 + (C <= 255 ? 1 : 2)));
+                count(nullptr, class_pick_launches(N, C));
             }
             return SAGE_OK;
         };

@@ -212,7 +212,8 @@ cudaError_t launch_class_starts(const int* labels, int64_t N, int C, unsigned* s
 bool class_select_in_one(int64_t N, int C);
 cudaError_t launch_class_select(const float* scores, const int* labels, int64_t N, int C, double keep_rate, void* scratch, int64_t* idx,
                                 long long* kc, cudaStream_t st);
-// Otherwise with given quotas: idx[offs[c] + r] = the r-th best example of class c, r < kc[c].
+// Otherwise with given quotas: idx[offs[c] + r] = the r-th best example of class c, r < kc[c]. class_pick_launches: with launch_class_starts.
+int class_pick_launches(int64_t N, int C);
 cudaError_t launch_class_pick(const float* scores, const int* labels, int64_t N, int C, void* scratch, const unsigned* starts, const long long* kc,
                               const long long* offs, int64_t* idx, cudaStream_t st);
 

@@ -137,6 +137,7 @@ cudaError_t launch_select(const float*, int64_t, int64_t, int64_t*, void*, cudaS
 cudaError_t select_scratch_bytes(int64_t N, size_t* bytes) { *bytes = (size_t)N * 32 + 4096; return cudaSuccess; }
 size_t class_scratch_bytes(int64_t, int, int) { return 4096; }
 int class_score_launches(int64_t, int, int) { return 1; }
+int class_pick_launches(int64_t, int) { return 1; }
 size_t eig_work_floats(int n) { return (size_t)n * n; }
 int eig_launches(int, int) { return 1; }
 int project_planes(int64_t, int64_t, int64_t) { return 1; }

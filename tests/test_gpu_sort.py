@@ -21,7 +21,7 @@ def test_selection_at_the_edges(N):
         assert np.array_equal(sage.sage_select(s, rate).cpu().numpy(), oracle.select(a.astype(np.float64), rate)), rate
 
 
-@pytest.mark.parametrize("N,C", [(8193, 255), (8192, 256), (131072, 255), (131073, 10), (140000, 300), (3000, 65535)])
+@pytest.mark.parametrize("N,C", [(8193, 255), (8192, 256), (131072, 255), (131073, 10), (140000, 300), (3000, 65535), (1, 256), (98304, 300), (98305, 300)])
 def test_selection_by_class_at_the_edges(N, C):
     r = np.random.default_rng(N + C)
     a = (r.integers(-50, 51, size=N) / 50.0).astype(np.float32)
