@@ -497,18 +497,19 @@ cudaError_t launch_any(const void* kernel, const LaunchShape& shape, void** args
     return cudaLaunchKernelExC(&cfg, kernel, args);
 }
 cudaError_t allow_smem(const void* kernel, int bytes) {
-    // set once per kernel and device: which is remembered in a small list (a handful of kernels)
+    // set once per kernel and device, which is remembered: an array, as this runs below entry points that must not throw
     struct Seen { const void* kernel; int dev, bytes; };
     static std::mutex mu;
-    static std::vector<Seen> seen;
+    static Seen seen[256];
+    static int n_seen = 0;
     int dev = 0;
     const cudaError_t e0 = cudaGetDevice(&dev);
     if (e0 != cudaSuccess) return e0;
     std::lock_guard<std::mutex> lock(mu);
-    for (Seen& x : seen)
-        if (x.kernel == kernel && x.dev == dev && x.bytes >= bytes) return cudaSuccess;
+    for (int i = 0; i < n_seen; ++i)
+        if (seen[i].kernel == kernel && seen[i].dev == dev && seen[i].bytes >= bytes) return cudaSuccess;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) seen.push_back({kernel, dev, bytes});
+    if (e == cudaSuccess && n_seen < 256) seen[n_seen++] = {kernel, dev, bytes};
     return e;
 }
 void set_error_message(const char* msg) { set_err("%s", msg); }

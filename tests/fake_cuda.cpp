@@ -4,6 +4,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -18,6 +19,7 @@ struct Append {
 };
 std::vector<Append> appends;
 int capturing = 0;
+thread_local bool no_memory = false;
 cudaError_t last = cudaSuccess;
 
 cudaError_t book(const char* name) {
@@ -36,7 +38,22 @@ T handle() {
 void kernel(int) {}
 }  // namespace
 
+void* operator new(size_t n) {
+    if (no_memory) throw std::bad_alloc();
+    if (void* p = std::malloc(n ? n : 1)) return p;
+    throw std::bad_alloc();
+}
+void operator delete(void* p) noexcept { std::free(p); }
+void operator delete(void* p, size_t) noexcept { std::free(p); }
+
 extern "C" {
+int fake_allow_smem_without_memory() {                // what the launchers call before a kernel of much shared memory
+    static char kernel;
+    no_memory = true;
+    const cudaError_t e = sage::allow_smem(&kernel, 1024);
+    no_memory = false;
+    return (int)e;
+}
 int fake_calls(const char* name) { return calls[name]; }
 void fake_fail(const char* name, int nth_from_now) { fail_at[name] = calls[name] + nth_from_now; }
 void fake_capturing(int on) { capturing = on; }
@@ -70,7 +87,7 @@ cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t cudaGetLastError() { const cudaError_t e = last; last = cudaSuccess; return e; }
 const char* cudaGetErrorString(cudaError_t) { return "fake"; }
 cudaError_t cudaDeviceSynchronize() { BOOK; return cudaSuccess; }
-cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { BOOK; return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { BOOK; *e = handle<cudaEvent_t>(); return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { BOOK; *e = handle<cudaEvent_t>(); return cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t) { BOOK; return cudaSuccess; }

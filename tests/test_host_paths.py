@@ -3,6 +3,7 @@ leaves behind where a call of the runtime fails. Runs on the CPU."""
 import ctypes as C
 import os
 import subprocess
+import sys
 
 import pytest
 
@@ -147,3 +148,11 @@ def test_a_checkpoint_with_another_rank_costs_the_graphs(lib):
     assert lib.sage_fd_import(b, blob, need.value, None) == 0 and _calls(lib, "cudaGraphExecDestroy") > d0
     lib.sage_fd_destroy(a)
     lib.sage_fd_destroy(b)
+
+
+def test_launchers_do_not_throw(lib):
+    """Below the entry points of the C ABI nothing that the launchers keep books with may throw where host memory is short. In a
+    process of its own, which an exception out of the library would end."""
+    code = f"import ctypes; L = ctypes.CDLL({lib._name!r}); print('status', L.fake_allow_smem_without_memory())"
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0 and r.stdout.strip() == "status 0", r.stderr[-500:]
