@@ -496,7 +496,7 @@ cudaError_t launch_any(const void* kernel, const LaunchShape& shape, void** args
     }
     return cudaLaunchKernelExC(&cfg, kernel, args);
 }
-cudaError_t allow_smem(const void* kernel, int bytes) {
+cudaError_t allow_smem(const void* kernel, int bytes, int regs) {
     // set once per kernel and device, which is remembered: an array, as this runs below entry points that must not throw
     struct Seen { const void* kernel; int dev, bytes; };
     static std::mutex mu;
@@ -508,7 +508,14 @@ cudaError_t allow_smem(const void* kernel, int bytes) {
     std::lock_guard<std::mutex> lock(mu);
     for (int i = 0; i < n_seen; ++i)
         if (seen[i].kernel == kernel && seen[i].dev == dev && seen[i].bytes >= bytes) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = cudaSuccess;
+    if (regs > 0) {
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, kernel);
+        if (e != cudaSuccess) return e;
+        if (fa.numRegs != regs) return cudaErrorInvalidKernelImage;
+    }
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess && n_seen < 256) seen[n_seen++] = {kernel, dev, bytes};
     return e;
 }

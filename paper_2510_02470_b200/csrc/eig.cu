@@ -1041,8 +1041,9 @@ cudaError_t launch_eig_shrink(const float* K, int ldk, int n, int do_shrink, int
     if (n <= 0 || n > 512) return cudaErrorInvalidValue;
     if (variant == 0) {
         const cudaError_t e = launch_eig_direct(K, ldk, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out, n_sigma, work, info, Wsplit, ldw, j_pad, st);
-        if (e == cudaSuccess) return e;
-        (void)cudaGetLastError();          // no cluster launch on this device: the kernels below serve every n <= 512
+        // where a cluster of eight blocks cannot be launched (its first launch), the kernels below serve every n <= 512
+        if (n <= 128 || (e != cudaErrorInvalidClusterSize && e != cudaErrorLaunchOutOfResources)) return e;
+        (void)cudaGetLastError();
     }
     if (n <= kMaxFast) {
         const int T = (n + 63) / 64;
@@ -1052,32 +1053,20 @@ cudaError_t launch_eig_shrink(const float* K, int ldk, int n, int do_shrink, int
 #define SAGE_EIG_FAST(TT)                                                                                              \
     e = cudaFuncSetAttribute(k_eig_shrink_fast<TT, 1024, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); \
     if (e != cudaSuccess) return e;                                                                                    \
-    k_eig_shrink_fast<TT, 1024, false><<<1, 1024, bytes, st>>>(K, ldk, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out,  \
-                                                               n_sigma, max_sweeps, info, Wsplit, ldw, j_pad, work);
+    return launch(k_eig_shrink_fast<TT, 1024, false>, LaunchShape{dim3(1), dim3(1024), bytes, 1, false}, st, K, ldk, n, do_shrink, delta_rank, keep, \
+                  Ur, ldu, sigma_out, n_sigma, max_sweeps, info, Wsplit, ldw, j_pad, work);
         if (T == 1) { SAGE_EIG_FAST(1) } else if (T == 2) { SAGE_EIG_FAST(2) } else { SAGE_EIG_FAST(3) }
 #undef SAGE_EIG_FAST
-        return cudaGetLastError();
     }
     {   // thread-block cluster, matrix in `work` (>= 512*512 + 64 floats when n > 256, else >= 256*256 + 64)
         const size_t bytes = 3 * 512 * sizeof(float) + 3 * 512 * sizeof(int) + 32;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(8);
-        cfg.blockDim = dim3(256);
-        cfg.dynamicSmemBytes = bytes;
-        cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 8;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        cudaError_t e = n <= 256 ? cudaLaunchKernelEx(&cfg, k_eig_shrink_cluster<4>, K, ldk, n, do_shrink, delta_rank, keep, Ur, ldu,
-                                                      sigma_out, n_sigma, max_sweeps, info, Wsplit, ldw, j_pad, work)
-                                 : cudaLaunchKernelEx(&cfg, k_eig_shrink_cluster<8>, K, ldk, n, do_shrink, delta_rank, keep, Ur, ldu,
-                                                      sigma_out, n_sigma, max_sweeps, info, Wsplit, ldw, j_pad, work);
-        if (e == cudaSuccess) return cudaGetLastError();
-        (void)cudaGetLastError();          // no cluster launch on this device: the one-CTA kernel below serves n <= 512
+        const LaunchShape shape{dim3(8), dim3(256), bytes, 8, false};
+        const cudaError_t e = n <= 256 ? launch(k_eig_shrink_cluster<4>, shape, st, K, ldk, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out, n_sigma, max_sweeps,
+                                                info, Wsplit, ldw, j_pad, work)
+                                       : launch(k_eig_shrink_cluster<8>, shape, st, K, ldk, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out, n_sigma, max_sweeps,
+                                                info, Wsplit, ldw, j_pad, work);
+        if (e != cudaErrorInvalidClusterSize && e != cudaErrorLaunchOutOfResources) return e;
+        (void)cudaGetLastError();          // the one-CTA kernel below serves n <= 512
     }
     const size_t aux = (4 * 512 + 2 * kWarps + 8) * sizeof(float);
     const size_t xbytes = (size_t)n * n * sizeof(float);
@@ -1091,9 +1080,8 @@ cudaError_t launch_eig_shrink(const float* K, int ldk, int n, int do_shrink, int
     const size_t smem = aux + (use_smem ? xbytes : 0) + 64;
     cudaError_t e = cudaFuncSetAttribute(k_eig_shrink, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_eig_shrink<<<1, kThreads, smem, st>>>(K, ldk, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out, n_sigma, work, use_smem,
-                                            max_sweeps, info, Wsplit, ldw, j_pad);
-    return cudaGetLastError();
+    return launch(k_eig_shrink, LaunchShape{dim3(1), dim3(kThreads), smem, 1, false}, st, K, ldk, n, do_shrink, delta_rank, keep, Ur, ldu, sigma_out, n_sigma, work,
+                  use_smem, max_sweeps, info, Wsplit, ldw, j_pad);
 }
 
 }  // namespace sage

@@ -45,8 +45,10 @@ __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 #endif
 
-// Lets a kernel use up to `bytes` of dynamic shared memory; the driver is asked once per kernel and device.
-cudaError_t allow_smem(const void* kernel, int bytes);
+// Lets a kernel use up to `bytes` of dynamic shared memory; the driver is asked once per kernel and device. regs > 0: the kernel hands
+// registers from some of its warps to others and has to be compiled with exactly that many a thread; cudaErrorInvalidKernelImage
+// otherwise, which callers report: the launchers' cudaErrorNotSupported, for which they take other kernels, is about operands only.
+cudaError_t allow_smem(const void* kernel, int bytes, int regs = 0);
 
 // Device-side flags accumulated in the handle's status word.
 constexpr uint32_t kFlagNotConverged = 1u;

@@ -245,12 +245,8 @@ cudaError_t launch_tc_gram_pair(const float* B, int64_t ldb, int r, int64_t K, i
     if (ldc % 4 || ldc < r || split_stride % 4 || (reinterpret_cast<uintptr_t>(C) & 15u)) return cudaErrorNotSupported;
     CUtensorMap tm;
     if (!tc::make_tmap_2d(&tm, B, 4, (uint64_t)r, (uint64_t)K, (uint64_t)ldb, 128)) return cudaErrorNotSupported;
-    // the kernel hands registers from one half of its warps to the other: only as many as the launch holds
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, tc::k_tc_gram_pair);
+    const cudaError_t e = allow_smem((const void*)tc::k_tc_gram_pair, 227 * 1024, tc::kPairRegs);
     if (e != cudaSuccess) return e;
-    if (fa.numRegs != tc::kPairRegs) return cudaErrorNotSupported;
-    if ((e = allow_smem((const void*)tc::k_tc_gram_pair, 227 * 1024)) != cudaSuccess) return e;
     const unsigned pairs = (unsigned)(n_off ? n_off + 2 * n_diag : n_diag);
     return launch(tc::k_tc_gram_pair, LaunchShape{dim3(2 * pairs), dim3(tc::kPairThreads), tc::kPairSmem, 2}, st, tm, r, K, n_diag, n_off, C, ldc, split_stride, err);
 }

@@ -311,12 +311,7 @@ cudaError_t launch_tc_project(const float* rows, int64_t ld, const float* sk_spl
     const int64_t tiles = (M + 255) / 256, nkt = (cols + tc::kProjBK - 1) / tc::kProjBK;
     const int64_t pairs = slices > 1 ? std::min<int64_t>(74, tiles * slices) : project_pairs(tiles, nkt);
     const int planes = project_planes(M, K, class_F);
-    // the kernel hands registers from one half of its warps to the other: only as many as the launch holds
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, tc::k_tc_project);
-    if (e != cudaSuccess) return e;
-    if (fa.numRegs != tc::kProjRegs) return cudaErrorNotSupported;
-    e = allow_smem((const void*)tc::k_tc_project, 227 * 1024);
+    const cudaError_t e = allow_smem((const void*)tc::k_tc_project, 227 * 1024, tc::kProjRegs);
     if (e != cudaSuccess) return e;
     return launch(tc::k_tc_project, LaunchShape{dim3((unsigned)(2 * pairs)), dim3(tc::kProjThreads), tc::kProjSmem, 2}, st, tmRows, tmSk, (int)M, ell, (int)nkt, slices,
                   class_F, tiles * slices * nkt, planes, out, plane_stride, err);

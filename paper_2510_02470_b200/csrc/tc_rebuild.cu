@@ -713,12 +713,8 @@ static cudaError_t launch_tc_rebuild_wide(const float* Wsplit, int ldw, int j_pa
     if (!tc::make_tmap_2d(&tmBuf, Bsrc, 4, (uint64_t)r, (uint64_t)pitch, (uint64_t)pitch, tc::kChunkRows, 1) ||
         !tc::make_tmap_2d(&tmW, Wsplit, 4, (uint64_t)rows, (uint64_t)kcols, (uint64_t)ldw, 128))
         return cudaErrorNotSupported;
-    // the kernel hands registers from one half of its warps to the other: only as many as the launch holds
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, tc::k_tc_rebuild_wide);
+    const cudaError_t e = allow_smem((const void*)tc::k_tc_rebuild_wide, 227 * 1024, tc::kWideRegs);
     if (e != cudaSuccess) return e;
-    if (fa.numRegs != tc::kWideRegs) return cudaErrorNotSupported;
-    if ((e = allow_smem((const void*)tc::k_tc_rebuild_wide, 227 * 1024)) != cudaSuccess) return e;
     const long long num_tiles = (pitch + tc::kTileD - 1) / tc::kTileD;
     return launch_chained(tc::k_tc_rebuild_wide, dim3((int)(num_tiles < 148 ? num_tiles : 148)), dim3(tc::kWideThreads), tc::kWideSmem, st, tmBuf, tmW,
                           r, keep, j_pad, j_pad > 128 ? 128 : j_pad, pitch, num_tiles, Bdst, err);

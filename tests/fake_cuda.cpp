@@ -54,6 +54,10 @@ int fake_allow_smem_without_memory() {                // what the launchers call
     no_memory = false;
     return (int)e;
 }
+int fake_allow_smem(int regs) {                       // a kernel that was compiled with 64 registers a thread
+    static char kernels[256];
+    return (int)sage::allow_smem(&kernels[regs], 1024, regs);
+}
 int fake_calls(const char* name) { return calls[name]; }
 void fake_fail(const char* name, int nth_from_now) { fail_at[name] = calls[name] + nth_from_now; }
 void fake_capturing(int on) { capturing = on; }
@@ -88,6 +92,11 @@ cudaError_t cudaGetLastError() { const cudaError_t e = last; last = cudaSuccess;
 const char* cudaGetErrorString(cudaError_t) { return "fake"; }
 cudaError_t cudaDeviceSynchronize() { BOOK; return cudaSuccess; }
 cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaFuncGetAttributes(cudaFuncAttributes* fa, const void*) {
+    *fa = cudaFuncAttributes();
+    fa->numRegs = 64;
+    return cudaSuccess;
+}
 cudaError_t cudaEventCreate(cudaEvent_t* e) { BOOK; *e = handle<cudaEvent_t>(); return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { BOOK; *e = handle<cudaEvent_t>(); return cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t) { BOOK; return cudaSuccess; }

@@ -55,6 +55,8 @@ def test_one_shrink_and_one_freeze(kind, ell):
         err = np.linalg.norm(S.T @ S - (V * kept) @ V.T, 2) / lam[-1]
         err_sigma = np.max(np.abs(sigma ** 2 - expect)) / lam[-1]
         assert st["device_flags"] == 0 and st["shrinks"] == (1 if N == 2 * ell else 0)
+        # each factorisation (a full buffer shrinks, what is left is frozen) takes two tensor-core kernels, or none, and the direct solve
+        assert st["tensor_core_launches"] == tensor_cores * 2 * (2 if N == 2 * ell else 1) and st["last_sweeps"] == 0
         assert err <= bound and err_sigma <= bound, (N, tensor_cores, err, err_sigma)
 
 

@@ -26,7 +26,9 @@ def test_spectrum_of_wide_buffers(n, D):
     S, sigma = fd.sketch()
     st = fd.stats()
     fd.close()
+    # a factorisation takes its Gram matrix and its rebuild on tensor cores, the direct solve between them; 512 rows shrink, then freeze
     assert st["device_flags"] == 0 and st["shrinks"] == (1 if n > 256 else 0)
+    assert st["tensor_core_launches"] == (4 if n == 512 else 2) and st["last_sweeps"] == 0
     lam = np.zeros(n)
     sv = np.linalg.svd(rows.double().numpy(), compute_uv=False) ** 2
     lam[:len(sv)] = sv

@@ -156,3 +156,10 @@ def test_launchers_do_not_throw(lib):
     code = f"import ctypes; L = ctypes.CDLL({lib._name!r}); print('status', L.fake_allow_smem_without_memory())"
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0 and r.stdout.strip() == "status 0", r.stderr[-500:]
+
+
+def test_a_kernel_compiled_with_other_registers_is_an_error(lib):
+    """Kernels that move registers between warps run with the count they were written for only. Another count is an error of its own,
+    not the "not supported" for which callers quietly take the CUDA-core kernels."""
+    assert lib.fake_allow_smem(64) == 0 and lib.fake_allow_smem(0) == 0
+    assert lib.fake_allow_smem(63) == 200            # cudaErrorInvalidKernelImage; cudaErrorNotSupported is 801
