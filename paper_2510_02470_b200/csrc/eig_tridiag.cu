@@ -564,7 +564,7 @@ k_tridiag(const float* __restrict__ K, int ldk, int n, int scaled, TriWork wk, i
     bool ok = tri_phase<S, 0>(T, sh, o, wk, base, pitch, cta, w, lr, lc);
     ok = ok && tri_phase<S, 1>(T, sh, o, wk, base, pitch, cta, w, lr, lc);
     ok = ok && tri_phase<S, 2>(T, sh, o, wk, base, pitch, cta, w, lr, lc);
-    if (S::CL > 1 || S::G == 128) chain_release();
+    chain_release();
     if constexpr (S::G != 256) ok = ok && tri_phase<S, 3>(T, sh, o, wk, base, pitch, cta, w, lr, lc);
     if constexpr (S::CL == 1) {
         if (tid == S::NT - 1) {                             // the last diagonal element; two positions have no reflector
@@ -608,13 +608,6 @@ constexpr int kPoints = 32 * kEvWarps;             // places of the first cut, s
 constexpr double kRankCut = 1e-7;                  // eigenvalues below this fraction of the largest diagonal count as zero (rounding of K and T)
 template <int NQ>
 constexpr int kRing = NQ == 4 ? 4 : 8;             // chunks in flight (all of them when n <= 128)
-
-// Row of the split rebuild factors [W_hi ; W_lo] that holds output row j: stacked as two blocks of j_pad rows, or, when
-// more than 128 output rows are kept, as one such pair per 128 output rows (the rebuild kernel takes 128 at a time).
-__device__ __forceinline__ size_t split_row(int j, int j_pad, bool lo) {
-    if (j_pad <= 128) return (size_t)(lo ? j_pad + j : j);
-    return (size_t)(j >> 7) * 256 + (size_t)(j & 127) + (lo ? 128 : 0);
-}
 
 __device__ __forceinline__ double pow2(int ex) {   // 2^ex, 0 below the normal range
     return ex < -1022 ? 0.0 : __hiloint2double((1023 + (ex > 1023 ? 1023 : ex)) << 20, 0);

@@ -43,6 +43,13 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Row of the split rebuild factors [W_hi ; W_lo] that holds output row j: stacked as two blocks of j_pad rows, or, when
+// more than 128 output rows are kept, as one such pair per 128 output rows, as k_tc_rebuild_wide reads them.
+__device__ __forceinline__ size_t split_row(int j, int j_pad, bool lo) {
+    if (j_pad <= 128) return (size_t)(lo ? j_pad + j : j);
+    return (size_t)(j >> 7) * 256 + (size_t)(j & 127) + (lo ? 128 : 0);
+}
 #endif
 
 // Lets a kernel use up to `bytes` of dynamic shared memory; the driver is asked once per kernel and device. regs > 0: the kernel hands

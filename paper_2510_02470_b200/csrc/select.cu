@@ -284,7 +284,6 @@ constexpr int64_t kFilterMax = 1 << 18;                     // 500,000 scores, a
 constexpr int kBins = 2048;
 struct FilterShared {
     unsigned hist[kBins];
-    unsigned sum[kBins];
     unsigned wsum[kClWarps];
     unsigned nless[kClWarps], neq[kClWarps];
     unsigned cta_less, cta_eq;                               // read by the other blocks

@@ -150,11 +150,16 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* tmap) {
 // Makes shared-memory writes of ordinary threads visible to the async proxy (tensor cores, TMA).
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// What the tensor cores do not read of an fp32 word (kind::tf32 ignores its low 13 bits): exact, then rounded to 11 significant
-// bits, so that the same truncation cuts nothing from it.
+// What the tensor cores do not read of an fp32 word (kind::tf32 ignores its low 13 bits, so that the raw word is the hi operand): exact,
+// then rounded to 11 significant bits, so that the same truncation cuts nothing from it (a truncated remainder would bias sums of
+// like-signed products).
 __device__ __forceinline__ uint32_t remainder_tf32(uint32_t x, float scale = 1.f) {
     const float l = scale * (__uint_as_float(x) - __uint_as_float(x & 0xffffe000u));
     return (__float_as_uint(l) + 0x1000u) & 0xffffe000u;
+}
+
+__device__ __forceinline__ uint4 remainder_tf32(const uint4 v) {
+    return make_uint4(remainder_tf32(v.x), remainder_tf32(v.y), remainder_tf32(v.z), remainder_tf32(v.w));
 }
 
 // True in one lane of a converged warp, the same one each time.

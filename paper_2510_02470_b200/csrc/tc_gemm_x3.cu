@@ -46,16 +46,6 @@ constexpr int BK = 32;                      // fp32 elements per 128-byte K tile
 constexpr int kChunkTiles = 8;              // K tiles accumulated in TMEM between drains (32 MMA steps: bias below 1e-6; 4 -> 8 gave 8 %, 16 no more)
 constexpr int kAccs = 4;                    // accumulators in TMEM (4 x 128 columns)
 
-// The tensor cores read an fp32 word as tf32 by ignoring its low 13 bits, so the raw tile already is the hi operand
-// (hi = x with those bits cleared) and only the remainder has to be written: lo = x - hi, exact, then rounded to 11
-// significant bits so that the hardware's truncation of lo finds nothing to cut (a truncated lo would bias sums of
-// like-signed products).
-__device__ __forceinline__ uint32_t lo_of(uint32_t x) {
-    const float l = __uint_as_float(x) - __uint_as_float(x & 0xffffe000u);
-    return (__float_as_uint(l) + 0x1000u) & 0xffffe000u;
-}
-__device__ __forceinline__ uint4 lo4(const uint4 v) { return make_uint4(lo_of(v.x), lo_of(v.y), lo_of(v.z), lo_of(v.w)); }
-
 __global__ void __launch_bounds__(kThreads, 1)
 k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M, int N,
                 int b_box_rows, int sym, long long K, long long k_per_split, int a_shared, float* __restrict__ C, long long ldc,
@@ -268,7 +258,7 @@ k_tc_gemm_nt_x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     if (c + u * kGroup < chunks16) v[u] = hi[c + u * kGroup];
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
-                    if (c + u * kGroup < chunks16) lo[c + u * kGroup] = lo4(v[u]);
+                    if (c + u * kGroup < chunks16) lo[c + u * kGroup] = remainder_tf32(v[u]);
             }
             if (direct_new) {
                 // the caller's bfloat16 rows: 4 x 16 bytes (32 values) per row and K tile -> 8 chunks of 4 floats in the operand tile

@@ -31,21 +31,10 @@ constexpr int kChunkRows = 32;              // buffer rows per stage (MMA K = 4 
 constexpr int kBufBytes = kChunkRows * kTileD * 4;   // 16 KB: 4 spans of [32 rows][128 bytes]
 constexpr int kSpanBytes = kChunkRows * 128;         // 4 KB
 
-// The remainders of a landed chunk, by kSplitThreads threads. The tensor cores ignore the low 13 bits of an fp32 word, so the raw
-// tile is the hi operand as it stands; lo = x - hi (exact), rounded to 11 significant bits so that the same truncation cuts
-// nothing from it.
+// The remainders of a landed chunk, by kSplitThreads threads.
 __device__ __forceinline__ void split_chunk(const uint4* hi, uint4* lo, int t) {
 #pragma unroll
-    for (int cc = 0; cc < kBufBytes / 16 / kSplitThreads; ++cc) {
-        const int idx = t + cc * kSplitThreads;
-        const uint4 v = hi[idx];
-        uint4 l;
-        l.x = (__float_as_uint(__uint_as_float(v.x) - __uint_as_float(v.x & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
-        l.y = (__float_as_uint(__uint_as_float(v.y) - __uint_as_float(v.y & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
-        l.z = (__float_as_uint(__uint_as_float(v.z) - __uint_as_float(v.z & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
-        l.w = (__float_as_uint(__uint_as_float(v.w) - __uint_as_float(v.w & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
-        lo[idx] = l;
-    }
+    for (int cc = 0; cc < kBufBytes / 16 / kSplitThreads; ++cc) lo[t + cc * kSplitThreads] = remainder_tf32(hi[t + cc * kSplitThreads]);
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
