@@ -3,24 +3,29 @@
 // value is reduced by delta and clamped at zero). With K = B B^T = U Sigma^2 U^T the left factor U and sigma^2 come
 // from the symmetric eigen-problem of K, and Sigma' V^T = diag(sigma'/sigma) U^T B.
 //
-// Method (direct, no iteration whose length depends on the data):
-//   1. K is scaled by 1 / max diagonal, ordered by falling diagonal and reduced to a tridiagonal T = Q^T K Q by Householder reflections, fp32, the
-//      matrix in registers (k_tridiag). n <= 128: one thread block of 4 warps; larger: a cluster of 8 blocks works until
-//      128 rows are left, the one-block kernel does the rest.
+// Method (direct; only the number of passes in step 2 depends on the data):
+//   1. K is scaled by 1 / max diagonal, ordered by falling diagonal and reduced to a tridiagonal T = Q^T K Q by Householder
+//      reflections, fp32, the matrix in registers (k_tridiag). n <= 128: one thread block of 4 warps; larger: a cluster of 8
+//      blocks works until 128 rows are left, the one-block kernel does the rest.
 //   2. Every wanted eigenvalue of T (the kept ones and delta) is found by multisection on the sign changes of the
-//      leading principal minors, in fp64, one warp per eigenvalue, 32 places per pass over T, with secants at the end.
+//      leading principal minors, in fp64, one warp per eigenvalue, 32 places per pass over T, with secants at the end: four
+//      passes where eigenvalues are apart, up to twenty in a cluster.
 //   3. Its eigenvector is read off the forward and the backward three-term recurrence, joined where their product (the
 //      diagonal of the resolvent) is largest, in fp64.
 //   4. The reflections are applied to it in reverse (fp32, groups of four), it is scaled and written.
 //   2-4 are one kernel (k_tridiag_vectors), three vectors per thread block, no communication between blocks.
 // T is perturbed by less than half an ulp of fp32 (T's own rounding is larger) so that repeated eigenvalues of K come
-// apart: the gaps of 1e-10 that this leaves are wide for fp64 eigenvalues, and vectors computed independently of each other
-// are orthogonal to about 1e-6 at worst (projections, repeated blocks), 1e-12 typically.
+// apart and vectors can be computed independently of each other. Gaps may be as small as 1e-11 of the largest eigenvalue, but the
+// vectors across such a gap live at different places of T: rows of sketches were orthogonal to 1e-7 to 7e-7 of the largest squared
+// row norm, 32 to 512 rows, over clusters of two, three and five values, eightfold eigenvalues, glued Wilkinson matrices and
+// repeated Laplacians (the iterative solve: 7e-7 to 5e-4 on the same).
 //
 // Why: the solve is a chain of dependent steps, and this one is shorter than the iterative solve's (sweeps x (n - 1) rounds):
 // n - 2 steps of about 1,050 cycles for the reduction, then 30 to 75 thousand cycles, all eigenvectors side by side. Measured, one
-// solve in a row of solves, iterative -> direct: 64 rows 156 -> 44 us, 128 rows 389 -> 89 us (random matrices; 254 -> 95 us
-// in a run on last-layer rows), 256 rows 1,422 -> 213 us, 512 rows 7,093 -> 705 us. Error of the shrunk sketch, relative to the
+// solve in a row of solves, iterative -> direct: 64 rows 156 -> 46 us, 128 rows 377 -> 92 us, 256 rows 1,378 -> 214 us, 512 rows
+// 6,479 -> 692 us (random matrices). Rows of low rank are the other way round: the iterative solve stops at the rank (rank 8 of 64,
+// 128, 256, 512 rows: 25, 32, 55, 134 us) and this one does not: looking for the end of the rank cost its loop over the columns 3 to
+// 12 % wherever it was put. Error of the shrunk sketch, relative to the
 // largest eigenvalue: 3 to 5e-7 at every size (iterative: 1e-6 at 64 rows to 6e-6 at 512).
 #include "sage_internal.h"
 

@@ -5,10 +5,10 @@
 // split costs no shared-memory store and no proxy fence; the sketch, split once into [hi (64 rows) ; lo (64 rows)] when it was
 // frozen, is one 128-row B operand. Accumulator column j and 64 + j belong to output j.
 // A pair of SMs works on 256 rows (cta_group::2), so that each loads half of the sketch's tile, the hi rows or the lo rows, next to its
-// 128 rows: 24 KB a K tile, 700 cycles at the 34 bytes a cycle that an SM was seen to load, as long as the rows take from memory at the
-// copy rate; the MMAs take 512. What bounds it is how long a slot lives: load, hand-over to CTA 0, MMAs, eight slots in all. CTA 1's
-// landed data is released at cluster scope, 2,000 cycles or so under load, beside the split; remainders and drained accumulators are
-// in tensor memory, where relaxed arrivals between tcgen05 fences do. (With default arrivals, which order nothing between two
+// 128 rows: 24 KB a K tile, 700 cycles, as long as the rows take from memory at the copy rate; the MMAs take 512. What bounds it is how
+// long a slot lives: load, hand-over to CTA 0, MMAs, eight slots in all (tensor pipe 56 %, DRAM 49 % of nominal, shared memory 31 %
+// busy). CTA 1's landed data is released at cluster scope, 2,000 cycles or so under load, beside the split; remainders and drained
+// accumulators are in tensor memory, where relaxed arrivals between tcgen05 fences do. (With default arrivals, which order nothing between two
 // CTAs: 214 and 333 us where it takes 245 and 366. The release behind the split: 263 and 392; one warp that passes all on: 503.)
 // Measured (against single SMs with 128-row tiles that loaded the whole sketch tile, remainders in shared memory, a block per tile and
 // K slice): 50,000 rows of 5,130 onto 64 365 -> 245 us (1.03 GB: 159 us at the copy rate), 20,000 of 20,000 546 -> 366 us (245), 512 of 5,130

@@ -220,8 +220,9 @@ k_tc_rebuild(const __grid_constant__ CUtensorMap tmBuf, const __grid_constant__ 
 // chunk (cb), which gets one bfloat16 row (tmSrc1) in place of a placeholder; the chunks after it are 32 of them each (tmSrc). These
 // go to TMEM as they are: their remainders are zero, one product is all.
 //   warp 0 loads, warp 1 issues MMAs, warps 2-9 write remainders in two groups in turn (thread = buffer column), warps 10-13 are the epilogue.
-// Bound by DRAM. 128 rows of 11.2 M columns onto 63, half of them read in place: 1,600 -> 1,533 us against remainders in shared memory and
-// four chunks in flight (7.1 GB: 4.6 TB/s); of 262,144 columns 49 -> 47 us; short rows equal.
+// 128 rows of 11.2 M columns onto 63, half of them read in place: 1,600 -> 1,533 us against remainders in shared memory and four chunks in
+// flight; of 262,144 columns 49 -> 47 us; short rows equal. That is 7.1 GB at 4.6 TB/s, 0.70 of the copy rate, and nothing on the
+// chip is near its limit (tensor pipe 28 %, shared memory 31 %, DRAM 50 % of nominal): what holds it there is not known.
 constexpr int kNarrowThreads = 448;
 constexpr int kSlots = 8;                   // chunks in shared memory and, their remainders, in TMEM
 constexpr int kSlotBytes = kBufBytes + 1024;          // 16 KB of fp32 rows or 8 KB of bfloat16 rows, and the one bfloat16 row of chunk cb
@@ -428,9 +429,8 @@ k_tc_rebuild_narrow(const __grid_constant__ CUtensorMap tmBuf, const __grid_cons
 //   warp 0 loads buffer chunks, warp 1 issues MMAs, warp 2 loads factors, warps 4-7 write the lo parts, warps 8-15 are the
 //   epilogue (8-11: output rows 0-127, 12-15: the others).
 // 512 rows onto 255, 262,144 columns: 422 -> 282 us (two launches of the narrow kernel, each over the whole buffer, before: their
-// loads and hand-offs alone took 344 us). A chunk loads 80 KB in its 2,400 cycles, the 34 bytes a cycle that bound the
-// loads of tc_project.cu too; shared memory is not far behind (80 KB written, 32 moved by the split, 144 read by MMAs: 2,050 cycles at 128
-// bytes); the MMAs alone are 1,540.
+// loads and hand-offs alone took 344 us). The tensor pipe is busy 80 % of that; loads (80 KB a chunk, 34 bytes a cycle) and shared
+// memory (60 %) are not far behind.
 constexpr int kWideThreads = 512;
 constexpr int kWideRegs = 128;              // what every thread is launched with: the sum of the shares below is 4 x 128 x 128
 constexpr int kBufStages = 3, kWSlots = 4;
