@@ -45,8 +45,17 @@ ALL = ("c1", "c2", "c3", "c4", "c5")
 # DRAM bytes per launch of the dominant streaming kernels from one ncu capture each (profiles/): the capture ran on a
 # scaled-down D and the traffic grows in proportion to D, so the figure is stored per buffer column.
 # (Gram and rebuild: launches of cycles that read their 65 new rows in place, as 7 of 8 cycles of c5 do.)
-NCU_TRAFFIC_PER_COLUMN = {("c5", "rebuild"): (431.471e6 + 246.243e6) / 1117396, ("c5", "gram"): (433.734e6 + 3.507e6) / 1117396,
+NCU_TRAFFIC_PER_COLUMN = {("c5", "rebuild"): (431.463e6 + 243.809e6) / 1117396, ("c5", "gram"): (433.728e6 + 4.061e6) / 1117396,
                           ("c5", "project"): (1294.674e6 + 3.727e6) / 1117396}
+
+
+def rounded(x):
+    """Figures with six digits."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: rounded(v) for k, v in x.items()}
+    return [rounded(v) for v in x] if isinstance(x, list) else x
 
 
 def measured_peaks():
@@ -350,8 +359,10 @@ def run_workload(w, args, steps, warmup, ctx, want_e2e, want_cpu, sketches, fact
                 "algorithmic": "9*n^3 flop per n x n symmetric eigen-solve (textbook count)"}
     else:
         gbs = per_step_bytes.get(dominant, 0) / (dom_ms_per_step * 1e-3) / 1e9
-        kname = {"gram": "k_tc_gemm_nt_x3 (Gram)", "rebuild": "k_tc_rebuild (narrow, wide)", "append": "k_append",
-                 "project": "k_tc_gemm_nt (projection)"}.get(dominant, dominant)
+        rebuild = "k_tc_rebuild_narrow" if ell <= 64 else "k_tc_rebuild" if ell <= 128 else "k_tc_rebuild_wide"
+        project = "k_tc_gemm_nt" if e == 2 else "k_tc_project" if ell <= 64 else "k_tc_gemm_nt_x3"
+        kname = {"gram": "k_tc_gemm_nt_x3 (Gram)" if ell <= 64 else "k_tc_gram_pair", "rebuild": rebuild, "append": "k_append",
+                 "project": f"{project} (projection)"}.get(dominant, dominant)
         traffic = NCU_TRAFFIC_PER_COLUMN.get((w.name, dominant))
         roof = {"kernel": kname, "bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": gbs / peaks["hbm_gbs"], "traffic": traffic * D if traffic else None,
@@ -539,8 +550,11 @@ def main():
         for k in ("config", "passes", "roofline", "kernels_profiled_step", "class_balanced", "cpu_baseline", "e2e",
                   "gpu_launches", "clocks", "fd_stats"):
             line[k] = head[k]
-        line["workloads"] = {n: r for n, r in results.items() if n != headline}
-        print(json.dumps(line))
+        # one line, short enough to be kept whole: the other workloads with their main figures; all of them in full on stderr
+        line["workloads"] = {n: {k: r[k] for k in ("value", "ms_per_step", "steps", "warmup")} | {"e2e": r["e2e"]["value"] if r["e2e"] else None}
+                             for n, r in results.items() if n != headline}
+        print(json.dumps(results), file=sys.stderr)
+        print(json.dumps(rounded(line)))
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
