@@ -141,7 +141,10 @@ k_tc_gram_pair(const __grid_constant__ CUtensorMap tm, int r, long long K, int n
                     }
                 }
             }
-        } else if (q == 1 && lane == 0) {                   // CTA 1's remainders are handed to the MMAs
+        } else if (q == 1 && lane == 0) {
+            // CTA 1's remainders are handed to the MMAs. On the diagonal a warp passes on every round of its slots (a ring of 6). Off it
+            // (a ring of 3) the two take a slot's rounds in turn, and a round is not mistaken for the one two before: all workers
+            // split every K tile there, so that K tile kt - 2, which this warp has seen done, was done after kt - 3.
             for (int kt = warp - 2; kt < nkt; kt += 2) {
                 const int ls = kt % n_lo;
                 if (!mbar_wait(&split_done[ls], (uint32_t)(kt / n_lo) & 1u, abort)) break;
