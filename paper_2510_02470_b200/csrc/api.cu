@@ -238,6 +238,22 @@ struct sage_fd {
     int cycles_run = 0;
     bool cycle_graphs = true;
     cudaStream_t used = nullptr;   // the stream that reads rows of the current update call
+    bool sketching_in_blocks = false;  // pass 1 works on `blk`; the buffers B hold the frozen sketch only
+    size_t buffer_rows = 0;        // rows that the buffers B are allocated for: m, or ell in B[0] alone
+    struct Block {                 // shrink cycles in blocks: see block_kernels.cu
+        bool able = false;         // the shapes allow it and the memory is there
+        int L = 0, M = 0;          // cycles of a block, logical rows of a full one: m + (L - 1)(ell + 1)
+        int ldP = 0, ldu = 0, j_pad = 0, slices = 0;
+        int64_t pitch = 0, ldT = 0;
+        __nv_bfloat16 *S[2] = {nullptr, nullptr}, *R = nullptr, *T = nullptr;
+        int R_planes = 0;          // planes a row that R and parts are allocated for
+        float *P = nullptr, *C = nullptr, *U = nullptr, *K = nullptr, *parts = nullptr;
+        int cur = 0;               // S[cur]: the sketch that the block began with
+        int s_rows = 0, n_raw = 0; // its rows, and the rows given since
+        int n_gram = 0;            // logical rows whose inner products are in P
+        int cycles = 0;            // cycles done
+        int np = 0;                // planes a row of R
+    } blk;
 };
 
 namespace {
@@ -266,6 +282,8 @@ cudaError_t timed(sage_fd* h, int cls, int nlaunch, cudaStream_t st, F&& f) {
     count(h, nlaunch);
     return e;
 }
+
+constexpr size_t kBlockBytes = (size_t)40 << 30;              // sketches that would take more work cycle by cycle
 
 constexpr size_t kGramPartFloats = (size_t)148 * 128 * 128;   // >= 296 tiles of 64 x 64
 
@@ -563,6 +581,12 @@ static void drop_cycles(sage_fd* s) {
     for (sage_fd* k : s->kids) drop_cycles(k);
 }
 
+static bool block_setup(sage_fd* h);
+static void block_free(sage_fd* h);
+static cudaError_t alloc_buffers(sage_fd* h, size_t rows);
+enum Form { BY_OPTIONS, BY_CYCLES, IN_BLOCKS };
+static sage_status_t settle_form(sage_fd* h, Form form = BY_OPTIONS);
+
 static sage_status_t create_handle(sage_fd_t** out, int64_t D, int32_t ell, sage_dtype_t row_dtype, int device, bool sketch_only,
                                    bool pooled = false, cudaStream_t pool_stream = nullptr) {
     if (!out || D < 1 || (row_dtype != SAGE_F32 && row_dtype != SAGE_BF16) || device < 0) {
@@ -591,7 +615,6 @@ static sage_status_t create_handle(sage_fd_t** out, int64_t D, int32_t ell, sage
     h->sketch_only = sketch_only;
     h->block = ell + 1;
     h->pitch = ((D + 31) / 32) * 32;
-    const size_t bbytes = (size_t)h->m * h->pitch * sizeof(float);
     h->ldk = (h->m + 3) & ~3;
     const size_t mm = (size_t)h->m * h->ldk * sizeof(float);
     auto fail = [&](cudaError_t e, const char* what) {
@@ -600,8 +623,8 @@ static sage_status_t create_handle(sage_fd_t** out, int64_t D, int32_t ell, sage
         return e == cudaErrorMemoryAllocation ? SAGE_ERR_ALLOC : SAGE_ERR_CUDA;
     };
     cudaError_t e;
-    for (int i = 0; i < 2; ++i)
-        if ((e = dev_malloc(h, (void**)&h->B[i], bbytes)) != cudaSuccess) return fail(e, "cudaMalloc(buffer)");
+    h->sketching_in_blocks = block_setup(h);
+    if ((e = alloc_buffers(h, h->sketching_in_blocks ? ell : h->m)) != cudaSuccess) return fail(e, "cudaMalloc(buffer)");
     h->gram_part_floats = kGramPartFloats;
     const size_t slices = h->m > 256 ? kOffSlices : h->m > 128 ? 74 : 0;
     if (slices * h->m * ((h->m + 3) / 4 * 4) > h->gram_part_floats) h->gram_part_floats = slices * h->m * ((h->m + 3) / 4 * 4);
@@ -665,6 +688,7 @@ void sage_fd_destroy(sage_fd_t* h) {
     void* memory[] = {h->B[0], h->B[1], h->gram_parts, h->Wsplit, h->Kmat, h->Ur, h->eig_work, h->sigma, h->info, h->zhat, h->znorm, h->zwork,
                       h->partials, h->zred, h->bias_t, h->zsum, h->u, h->class_U, h->class_counts, h->P16, h->S32split, h->tc_err};
     for (void* p : memory) dev_free(h, p);
+    block_free(h);
     if (h->side) cudaStreamDestroy(h->side);
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
@@ -698,8 +722,10 @@ sage_status_t sage_fd_reset(sage_fd_t* h) {
     h->pend = RowSrc();
     h->pend_n = 0;
     h->used = nullptr;
+    h->blk.s_rows = h->blk.n_raw = h->blk.n_gram = h->blk.cycles = 0;
+    h->blk.np = h->dtype == SAGE_F32 ? 3 : 1;
     for (sage_fd* k : h->kids) ST_TRY(sage_fd_reset(k));
-    return SAGE_OK;
+    return settle_form(h);
 }
 
 sage_status_t sage_fd_set_option(sage_fd_t* h, int key, double value) {
@@ -714,7 +740,7 @@ sage_status_t sage_fd_set_option(sage_fd_t* h, int key, double value) {
         if (h->use_tc != (value != 0.0)) drop_cycles(h);
         h->use_tc = value != 0.0;
         for (sage_fd* k : h->kids) k->use_tc = h->use_tc;
-        return SAGE_OK;
+        return h->state == SKETCHING ? settle_form(h) : SAGE_OK;
     }
     if (key == 9) {                          // 1: whole shrink cycles read their new rows in place (no append), 0: always append
         h->direct_rows = value != 0.0;
@@ -744,7 +770,7 @@ sage_status_t sage_fd_set_option(sage_fd_t* h, int key, double value) {
         if (h->delta_rank != v) drop_cycles(h);
         h->delta_rank = v;
         for (sage_fd* k : h->kids) k->delta_rank = v;
-        return SAGE_OK;
+        return settle_form(h);
     }
     if (key == 2 && v >= 1 && v <= 1000) {
         h->max_sweeps = v;
@@ -763,7 +789,7 @@ sage_status_t sage_fd_set_option(sage_fd_t* h, int key, double value) {
             }
         }
         h->P = v;
-        return SAGE_OK;
+        return settle_form(h);
     }
     if (key == 7 && v >= 1 && v <= (1 << 20) && (double)v == value) { // rows per dealt block of the merged form
         h->block = v;
@@ -771,6 +797,334 @@ sage_status_t sage_fd_set_option(sage_fd_t* h, int key, double value) {
     }
     set_err("sage_fd_set_option: unknown key %d or value %g out of range", key, value);
     return SAGE_ERR_INVALID_ARG;
+}
+
+// ---- shrink cycles in blocks (block_kernels.cu) ----------------------------------------------------------------
+//
+// A block's rows are read twice, for their inner products and when the kept rows are formed at its end; the solves in between run on
+// small matrices. Where a block ends depends on the number of rows given since the reset only, and every product is formed in the same
+// order whenever its rows came: the sketch does not depend on how the rows are cut into calls, to the bit. Rows of a block that is not
+// complete when an update returns stay in the store (as rows of an incomplete cycle stay in the buffer otherwise).
+
+// Cycles of a block: as many as make 352 new rows, at least 4. Per cycle the kernels that read the rows cost 1 / L of a launch that takes
+// little longer for more rows; beyond that the inner products among a block's rows, which grow with the square, take over. The first
+// block ends with the first shrink.
+static int block_cycles(int ell) { return std::max(4, 352 / (ell + 1)); }
+static int block_cycles_now(const sage_fd* h) { return h->blk.s_rows < h->ell - 1 ? 1 : h->blk.L; }
+
+static BlockMap block_full_map(const sage_fd* h, int np, bool first) {
+    const int s_rows = first ? 0 : h->ell - 1;
+    BlockMap m = block_map(s_rows, np, (first ? h->m : h->blk.M) - s_rows, 0);
+    m.P += 64;                                     // a part of the rows in place: two places' surplus more
+    return m;
+}
+static int block_most_tiles(const sage_fd* h, int np) {
+    return std::max(block_tiles(block_full_map(h, np, false), 0), block_tiles(block_full_map(h, np, true), 0));
+}
+// K slices of a block's inner products: fixed for a handle, as the sums must not depend on how many rows a launch has. The number with
+// which a full block's tiles end soonest on 74 pairs of SMs, a slice costing 6 K tiles besides its own.
+static int block_slices(int64_t D, int tiles) {
+    const int nkt = (int)((D + 63) / 64);
+    int best = 1;
+    double best_cost = 1e300;
+    for (int s = 1; s <= std::min(nkt, 74); ++s) {
+        const double cost = (double)((tiles * s + 73) / 74) * ((double)((nkt + s - 1) / s) + 6.0) + 0.02 * tiles * s;
+        if (cost < best_cost) { best_cost = cost; best = s; }
+    }
+    return best;
+}
+
+static void block_free(sage_fd* h) {
+    auto& k = h->blk;
+    void* memory[] = {k.S[0], k.S[1], k.R, k.T, k.P, k.C, k.U, k.K, k.parts};
+    for (void* p : memory) dev_free(h, p);
+    k = sage_fd::Block();
+}
+
+// Memory of the rows' planes and of their partial inner products for np planes a row.
+static cudaError_t block_alloc_rows(sage_fd* h, int np) {
+    auto& k = h->blk;
+    cudaError_t e = dev_malloc(h, (void**)&k.R, (size_t)np * k.M * k.pitch * sizeof(__nv_bfloat16));
+    const int64_t ldT = (std::max(block_full_map(h, np, false).P, block_full_map(h, np, true).P) + 63) / 64 * 64;
+    if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.T, (size_t)3 * k.j_pad * ldT * sizeof(__nv_bfloat16));
+    if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.parts, (size_t)block_most_tiles(h, np) * k.slices * 65536 * sizeof(float));
+    k.ldT = ldT;
+    k.R_planes = np;
+    return e;
+}
+
+static sage_fd::Block block_shape(const sage_fd* h) {
+    sage_fd::Block k;
+    k.L = block_cycles(h->ell);
+    k.M = h->m + (k.L - 1) * (h->ell + 1);
+    k.ldP = (k.M + 3) & ~3;
+    k.ldu = (h->m + 3) & ~3;
+    k.j_pad = (h->ell + 31) / 32 * 32;
+    k.pitch = (h->D + 63) / 64 * 64;
+    k.np = h->dtype == SAGE_F32 ? 3 : 1;
+    return k;
+}
+
+// Sets blk up; false where blocks do not apply (then nothing is allocated).
+static bool block_setup(sage_fd* h) {
+    if (!launch_block_gram || h->sketch_only) return false;
+    auto& k = h->blk;
+    k = block_shape(h);
+    const int np = k.np;
+    k.slices = block_slices(h->D, block_tiles(block_full_map(h, np, false), 0));
+    const size_t s_bytes = (size_t)3 * (h->ell - 1) * k.pitch * sizeof(__nv_bfloat16);
+    const size_t bytes = 2 * s_bytes + (size_t)np * k.M * k.pitch * sizeof(__nv_bfloat16) + (size_t)block_most_tiles(h, np) * k.slices * 65536 * sizeof(float);
+    cudaError_t e = bytes <= kBlockBytes ? cudaSuccess : cudaErrorMemoryAllocation;
+    for (int i = 0; i < 2; ++i)
+        if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.S[i], s_bytes);
+    if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.P, (size_t)k.M * k.ldP * sizeof(float));
+    if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.C, (size_t)h->ell * k.ldP * sizeof(float));
+    if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.U, (size_t)(k.L + 1) * h->m * k.ldu * sizeof(float));
+    if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.K, (size_t)2 * h->m * h->ldk * sizeof(float));
+    // (rows of bfloat16 handles may be products of two factors: room for two planes at once, unless they are very long)
+    if (e == cudaSuccess) e = block_alloc_rows(h, bytes <= kBlockBytes / 64 ? std::max(np, 2) : np);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        block_free(h);
+        return false;
+    }
+    k.able = true;
+    return true;
+}
+
+static BlockSmall block_small(const sage_fd* h) {
+    const auto& k = h->blk;
+    return {h->m, h->ell - 1, h->ell + 1, k.P, k.ldP, k.C, k.U, k.ldu, (int64_t)h->m * k.ldu, k.K, (int64_t)h->m * h->ldk, h->ldk};
+}
+static BlockSource block_source(const sage_fd* h, const void* in_place, int64_t ld) {
+    return {h->blk.S[h->blk.cur], h->blk.R, h->blk.pitch, in_place, ld};
+}
+
+// The rows of R with np planes each from here on (structured rows of a bfloat16 handle are products: two planes).
+static sage_status_t block_widen(sage_fd* h, int np, cudaStream_t st) {
+    auto& k = h->blk;
+    if (k.np >= np) return SAGE_OK;
+    if (k.R_planes < np || k.n_raw > 0) {                  // new memory, as rows that are there move apart
+        __nv_bfloat16* old = k.R;
+        const int have = k.np;
+        CU_TRY(cudaStreamSynchronize(st));
+        CU_TRY(dev_free(h, k.T));
+        CU_TRY(dev_free(h, k.parts));
+        k.T = nullptr;
+        k.parts = nullptr;
+        k.R = nullptr;
+        const cudaError_t e = block_alloc_rows(h, np);
+        if (e == cudaSuccess && k.n_raw > 0) {
+            CU_TRY(cudaMemsetAsync(k.R, 0, (size_t)np * k.n_raw * k.pitch * 2, st));
+            for (int i = 0; i < k.n_raw; ++i)
+                CU_TRY(cudaMemcpyAsync(k.R + (size_t)i * np * k.pitch, old + (size_t)i * have * k.pitch, (size_t)have * k.pitch * 2, cudaMemcpyDeviceToDevice, st));
+        }
+        CU_TRY(cudaStreamSynchronize(st));
+        CU_TRY(dev_free(h, old));
+        CU_TRY(e);
+    }
+    k.np = np;
+    return SAGE_OK;
+}
+
+static sage_status_t block_gram(sage_fd* h, const BlockMap& map, const BlockSource& src, cudaStream_t st) {
+    auto& k = h->blk;
+    const int first = k.n_gram, nl = block_rows(map);
+    if (first >= nl) return SAGE_OK;
+    CU_TRY(timed(h, K_GRAM, 1, st, [&] { return launch_block_gram(src, map, first, h->D, k.slices, k.parts, h->tc_err, st); }));
+    h->tc_launches += 1;
+    CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_block_gram_reduce(k.parts, map, first, k.slices, k.P, k.ldP, st); }));
+    k.n_gram = nl;
+    return SAGE_OK;
+}
+
+static sage_status_t block_solve(sage_fd* h, int r, int do_shrink, int keep, cudaStream_t st) {
+    auto& k = h->blk;
+    const int c = k.cycles;
+    const float* K = c == 0 ? k.P : k.K + (size_t)(c & 1) * h->m * h->ldk;
+    CU_TRY(timed(h, K_EIG, eig_launches(r, h->eig_variant), st, [&] {
+        return launch_eig_shrink(K, c == 0 ? k.ldP : h->ldk, r, do_shrink, h->delta_rank, keep, k.U + (size_t)c * h->m * k.ldu, k.ldu, h->sigma, h->ell, h->eig_work,
+                                 h->max_sweeps, h->info, nullptr, 0, 0, h->eig_variant, st);
+    }));
+    return SAGE_OK;
+}
+
+// The kept rows after ncyc cycles: into the other sketch copy, or in fp32 to rows 0 .. keep - 1 of `rows`.
+static sage_status_t block_rebuild(sage_fd* h, const BlockMap& map, const BlockSource& src, int carried, int ncyc, int r_last, int keep, float* rows, cudaStream_t st) {
+    auto& k = h->blk;
+    CU_TRY(timed(h, K_REBUILD, 2, st, [&] {
+        const cudaError_t e = launch_block_factors(block_small(h), map, carried, ncyc, r_last, keep, k.T, k.j_pad, k.ldT, st);
+        if (e != cudaSuccess) return e;
+        return launch_block_rebuild(src, map, h->D, k.T, k.j_pad, k.ldT, keep, rows ? nullptr : k.S[1 - k.cur], rows, rows ? h->pitch : k.pitch, h->tc_err, st);
+    }));
+    h->tc_launches += 1;
+    return SAGE_OK;
+}
+
+// Products of the rows that have come since the last cycle, and what they give of the open window.
+static sage_status_t block_catch_up(sage_fd* h, const BlockMap& map, const BlockSource& src, cudaStream_t st) {
+    auto& k = h->blk;
+    const int before = k.n_gram;
+    ST_TRY(block_gram(h, map, src, st));
+    if (k.cycles > 0 && k.n_gram > before)
+        CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_block_step(block_small(h), 0, k.cycles, before, k.n_gram, false, st); }));
+    return SAGE_OK;
+}
+
+// Ends an open block at its last cycle: the kept rows are formed, the rows behind them (fewer than a cycle's) begin the next block.
+static sage_status_t block_end_early(sage_fd* h, cudaStream_t st) {
+    auto& k = h->blk;
+    if (k.cycles == 0) return SAGE_OK;
+    const int keep = h->ell - 1, raw = h->m + (k.cycles - 1) * (h->ell + 1) - k.s_rows, rest = k.n_raw - raw;
+    const BlockMap map = block_map(k.s_rows, k.np, raw, 0);
+    ST_TRY(block_rebuild(h, map, block_source(h, nullptr, 0), k.cycles, k.cycles, h->m, keep, nullptr, st));
+    const size_t row = (size_t)k.np * k.pitch;             // (raw >= ell + 1 > rest: the two ranges lie apart)
+    if (rest > 0) CU_TRY(cudaMemcpyAsync(k.R, k.R + raw * row, rest * row * sizeof(__nv_bfloat16), cudaMemcpyDeviceToDevice, st));
+    k.cur = 1 - k.cur;
+    k.s_rows = keep;
+    k.n_raw = rest;
+    k.n_gram = k.cycles = 0;
+    return SAGE_OK;
+}
+
+static sage_status_t block_feed(sage_fd* h, RowSrc src, int64_t n, cudaStream_t st) {
+    auto& k = h->blk;
+    const int keep = h->ell - 1, step = h->ell + 1, m = h->m;
+    if (src.outer() && h->dtype == SAGE_BF16) ST_TRY(block_widen(h, 2, st));
+    while (n > 0) {
+        const int L = block_cycles_now(h), M = m + (L - 1) * step;
+        const int nl = k.s_rows + k.n_raw, take = (int)std::min<int64_t>(n, M - nl);
+        // Rows that complete a block stay where the caller holds them, from one on whose plane has the place it would have in the store:
+        // sums over planes are formed 16 at a time.
+        int at = M;                                // the first logical row in place
+        if (take == M - nl && h->direct_rows && k.np == 1 && !src.outer() && (reinterpret_cast<uintptr_t>(src.rows) & 15u) == 0 && ((src.ld * 2) & 15) == 0) {
+            at = std::min(M, k.s_rows + (k.n_raw + 31) / 32 * 32);
+            if (L > 1) h->rows_in_place += (M - at) / step * step;       // whole cycles
+        }
+        const int copied = std::min(take, at - nl);
+        if (copied > 0)
+            CU_TRY(timed(h, K_APPEND, 1, st, [&] {
+                if (src.outer()) return launch_block_append_outer(src.q, src.ldq, src.feat, src.ldf, src.dt, copied, src.C, src.F, k.R, k.pitch, k.np, k.n_raw, st);
+                return launch_block_append(src.rows, src.dt, copied, src.ld, h->D, k.R, k.pitch, k.np, k.n_raw, st);
+            }));
+        const RowSrc rest = src.advanced(copied);
+        const BlockMap map = block_map(k.s_rows, k.np, k.n_raw + copied, take - copied);
+        const BlockSource from = block_source(h, rest.rows, rest.ld);
+        k.n_raw += take;
+        h->rows_seen += take;
+        src = src.advanced(take);
+        n -= take;
+        if (nl + take >= m + k.cycles * step) ST_TRY(block_catch_up(h, map, from, st));
+        while (k.cycles < L && nl + take >= m + k.cycles * step) {
+            ST_TRY(block_solve(h, m, 1, keep, st));
+            const int c = ++k.cycles;
+            if (c < L) CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_block_step(block_small(h), c - 1, c, keep + c * step, k.n_gram, true, st); }));
+        }
+        if (k.cycles == L) {
+            ST_TRY(block_rebuild(h, map, from, L - 1, L, m, keep, nullptr, st));
+            k.cur = 1 - k.cur;
+            k.s_rows = keep;
+            k.n_raw = k.n_gram = k.cycles = 0;
+        }
+    }
+    h->fill = k.s_rows + k.n_raw - k.cycles * step;
+    return SAGE_OK;
+}
+
+// An update that the caller captures has to leave the handle as it found it where its rows are a number of whole cycles, so that it can
+// be replayed: it begins and ends between blocks, with the sketch in the same copy. What is open before it is ended at once, on a
+// stream of the library's own, and not by the graph.
+static sage_status_t block_feed_captured(sage_fd* h, RowSrc src, int64_t n, cudaStream_t st) {
+    auto& k = h->blk;
+    if (k.cycles > 0) {
+        allow_work_beside_capture(true);
+        auto now = [&]() -> sage_status_t {
+            CU_TRY(cudaStreamWaitEvent(h->side, h->ev_rows, 0));
+            ST_TRY(block_end_early(h, h->side));
+            CU_TRY(cudaStreamSynchronize(h->side));
+            return SAGE_OK;
+        };
+        const sage_status_t rc = now();
+        allow_work_beside_capture(false);
+        ST_TRY(rc);
+    }
+    const int cur = k.cur;
+    ST_TRY(block_feed(h, src, n, st));
+    ST_TRY(block_end_early(h, st));
+    if (k.cur != cur) {
+        CU_TRY(cudaMemcpyAsync(k.S[cur], k.S[k.cur], (size_t)3 * k.s_rows * k.pitch * sizeof(__nv_bfloat16), cudaMemcpyDeviceToDevice, st));
+        k.cur = cur;
+    }
+    return SAGE_OK;
+}
+
+// The freeze: one more solve on the open window, its rows straight to the frozen sketch.
+static sage_status_t block_freeze(sage_fd* h, cudaStream_t st) {
+    auto& k = h->blk;
+    const int r = h->fill, ell = h->ell, do_shrink = r > ell ? 1 : 0, keep = do_shrink ? ell - 1 : std::min(r, ell);
+    if (r > 0) {
+        const BlockMap map = block_map(k.s_rows, k.np, k.n_raw, 0);
+        const BlockSource src = block_source(h, nullptr, 0);
+        ST_TRY(block_catch_up(h, map, src, st));
+        ST_TRY(block_solve(h, r, do_shrink, keep, st));
+        ST_TRY(block_rebuild(h, map, src, k.cycles, k.cycles + 1, r, keep, h->B[0], st));
+    } else {
+        CU_TRY(cudaMemsetAsync(h->sigma, 0, ell * sizeof(float), st));
+    }
+    if (keep < ell) CU_TRY(cudaMemsetAsync(h->B[0] + (size_t)keep * h->pitch, 0, (size_t)(ell - keep) * h->pitch * sizeof(float), st));
+    h->cur = 0;
+    h->fill = keep;
+    return SAGE_OK;
+}
+
+// Buffers of `rows` rows: two of m rows for cycle-by-cycle sketching, or one of ell rows for the frozen sketch.
+static cudaError_t alloc_buffers(sage_fd* h, size_t rows) {
+    const size_t bytes = rows * h->pitch * sizeof(float);
+    cudaError_t e = dev_malloc(h, (void**)&h->B[0], bytes);
+    if (e == cudaSuccess && rows == (size_t)h->m) e = dev_malloc(h, (void**)&h->B[1], bytes);
+    h->buffer_rows = rows;
+    return e;
+}
+
+// Rows that B holds become a block's first rows, or the other way round, when an option changes the form of pass 1. Sketching only.
+static sage_status_t settle_form(sage_fd* h, Form form) {
+    bool want = !h->sketch_only && h->P == 1 && h->use_tc && h->delta_rank == h->ell && launch_block_gram != nullptr;
+    if (form != BY_OPTIONS) want = form == IN_BLOCKS;
+    if (want == h->sketching_in_blocks) return SAGE_OK;
+    DeviceGuard g(h->device);
+    CU_TRY(cudaDeviceSynchronize());
+    auto& k = h->blk;
+    const int keep = h->ell - 1;
+    if (want) {
+        if (!block_setup(h)) return SAGE_OK;       // cycle by cycle, as before
+        k.s_rows = std::min(h->fill, keep);
+        const int rest = h->fill - k.s_rows;
+        if (rest > 0 && h->dtype == SAGE_BF16) ST_TRY(block_widen(h, 2, nullptr));       // rows of either kind
+        CU_TRY(launch_block_append(h->B[h->cur], SAGE_F32, k.s_rows, h->pitch, h->D, k.S[0], k.pitch, 3, 0, nullptr));
+        CU_TRY(launch_block_append(h->B[h->cur] + (size_t)k.s_rows * h->pitch, SAGE_F32, rest, h->pitch, h->D, k.R, k.pitch, k.np, 0, nullptr));
+        k.n_raw = rest;
+        h->sketching_in_blocks = true;
+    } else {
+        if (h->buffer_rows != (size_t)h->m) {
+            for (float*& b : h->B) {
+                CU_TRY(dev_free(h, b));
+                b = nullptr;
+            }
+            if (h->fill == 0) block_free(h);       // first, where memory is short
+            CU_TRY(alloc_buffers(h, h->m));
+        }
+        h->cur = 0;
+        if (h->fill > 0) {
+            ST_TRY(block_end_early(h, nullptr));
+            CU_TRY(launch_block_unpack(k.S[k.cur], k.pitch, 3, k.s_rows, h->D, h->B[0], h->pitch, nullptr));
+            CU_TRY(launch_block_unpack(k.R, k.pitch, k.np, k.n_raw, h->D, h->B[0] + (size_t)k.s_rows * h->pitch, h->pitch, nullptr));
+            CU_TRY(cudaDeviceSynchronize());
+        }
+        block_free(h);
+        h->sketching_in_blocks = false;
+    }
+    CU_TRY(cudaDeviceSynchronize());
+    return SAGE_OK;
 }
 
 // ---- one sketch: feed rows, factor, freeze ------------------------------------------------------------------
@@ -1017,8 +1371,17 @@ static sage_status_t update_from(sage_fd* h, RowSrc src, int64_t n, cudaStream_t
     ST_TRY(ensure_sketches(h));
     static std::atomic<long long> epochs{0};
     const int64_t epoch = epochs.fetch_add(1) + 1;
-    CU_TRY(cudaEventRecord(h->ev_in, st));
     sage_status_t rc = SAGE_OK;
+    if (h->sketching_in_blocks) {
+        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+        CU_TRY(cudaStreamIsCapturing(st, &capturing));
+        h->dealt += n;
+        if (capturing != cudaStreamCaptureStatusNone) return block_feed_captured(h, src, n, st);
+        ST_TRY(block_feed(h, src, n, st));
+        CU_TRY(cudaEventRecord(h->ev_rows, st));
+        return SAGE_OK;
+    }
+    CU_TRY(cudaEventRecord(h->ev_in, st));
     if (h->P == 1) {
         rc = sketch_feed(h, src, n, st, h->ev_in, epoch, false);
         h->dealt += n;
@@ -1133,7 +1496,9 @@ sage_status_t sage_fd_finalize(sage_fd_t* h, void* cuda_stream) {
     DeviceGuard g(h->device);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int nsk = (int)h->kids.size() + 1;            // sketches that exist (1 unless the merged form has been fed)
-    if (nsk == 1) {
+    if (h->sketching_in_blocks) {
+        ST_TRY(block_freeze(h, st));
+    } else if (nsk == 1) {
         ST_TRY(sketch_freeze(h, (h->P > 1 && h->chain) ? h->chain : st));
     } else {
         // every sketch is frozen on its own, then sketch a absorbs sketch a + s for s = 1, 2, 4, ...: the rows the
@@ -1721,7 +2086,38 @@ struct ExportSketch {
     int32_t rows, pad;
     EigInfo info;
 };
-const char kExportMagic[8] = {'S', 'A', 'G', 'E', 'F', 'D', '1', 0};
+// A sketch in the middle of a block: its planes, D values a row, and its small matrices follow.
+struct ExportBlock {
+    int32_t s_rows, n_raw, n_gram, cycles, np, cycles_of_block;
+};
+const char kExportMagic[8] = {'S', 'A', 'G', 'E', 'F', 'D', '1', 0}, kExportMagicBlock[8] = {'S', 'A', 'G', 'E', 'F', 'D', '2', 0};
+
+// The device arrays of an open block, one call of f(array, pitch, width, rows), in bytes, for each.
+extern "C++" template <typename F>
+sage_status_t each_block_array(const sage_fd* h, const sage_fd::Block& k, const ExportBlock& eb, F&& f) {
+    const size_t row = (size_t)h->D * 2, pitch = (size_t)k.pitch * 2, ldP = (size_t)k.ldP * 4, ldu = (size_t)k.ldu * 4, ldk = (size_t)h->ldk * 4;
+    ST_TRY(f((void*)k.S[k.cur], pitch, row, (size_t)3 * eb.s_rows));
+    ST_TRY(f((void*)k.R, pitch, row, (size_t)eb.np * eb.n_raw));
+    ST_TRY(f((void*)k.P, ldP, ldP, (size_t)eb.n_gram));
+    if (eb.cycles > 0) {
+        ST_TRY(f((void*)k.C, ldP, ldP, (size_t)h->ell - 1));
+        ST_TRY(f((void*)k.U, ldu, ldu, (size_t)eb.cycles * h->m));
+        ST_TRY(f((void*)(k.K + (size_t)(eb.cycles & 1) * h->m * h->ldk), ldk, ldk, (size_t)h->m));
+    }
+    return SAGE_OK;
+}
+ExportBlock export_block(const sage_fd* h) {
+    const auto& k = h->blk;
+    return {k.s_rows, k.n_raw, k.n_gram, k.cycles, k.np, k.L};
+}
+size_t export_block_bytes(const sage_fd* h, const ExportBlock& eb) {
+    size_t total = 0;
+    each_block_array(h, block_shape(h), eb, [&](void*, size_t, size_t width, size_t rows) {
+        total += width * rows;
+        return SAGE_OK;
+    });
+    return total;
+}
 
 int export_rows(const sage_fd* s, bool frozen) { return frozen ? s->ell : s->fill; }
 }  // namespace
@@ -1738,6 +2134,10 @@ sage_status_t sage_fd_export_size(const sage_fd_t* h, size_t* bytes) {
     }
     const bool frozen = h->state == FROZEN;
     size_t total = sizeof(ExportHeader);
+    if (!frozen && h->sketching_in_blocks) {
+        *bytes = total + sizeof(ExportSketch) + sizeof(ExportBlock) + export_block_bytes(h, export_block(h));
+        return SAGE_OK;
+    }
     const int nsk = frozen ? 1 : (int)h->kids.size() + 1;
     for (int p = 0; p < nsk; ++p) {
         const sage_fd* s = p == 0 ? h : h->kids[(size_t)p - 1];
@@ -1770,8 +2170,27 @@ sage_status_t sage_fd_export(sage_fd_t* h, void* dst_host, size_t capacity, size
     hd.dealt = h->dealt;
     hd.nsk = frozen ? 1 : (int)h->kids.size() + 1;
     hd.delta_rank = h->delta_rank;
+    const bool in_block = !frozen && h->sketching_in_blocks;
+    if (in_block) std::memcpy(hd.magic, kExportMagicBlock, 8);
     std::memcpy(out, &hd, sizeof hd);
     out += sizeof hd;
+    if (in_block) {
+        ExportSketch es = {};
+        es.rows = h->fill;
+        CU_TRY(cudaMemcpy(&es.info, h->info, sizeof(EigInfo), cudaMemcpyDeviceToHost));
+        std::memcpy(out, &es, sizeof es);
+        out += sizeof es;
+        const ExportBlock eb = export_block(h);
+        std::memcpy(out, &eb, sizeof eb);
+        out += sizeof eb;
+        ST_TRY(each_block_array(h, h->blk, eb, [&](void* p, size_t pitch, size_t width, size_t rows) -> sage_status_t {
+            if (rows > 0) CU_TRY(cudaMemcpy2D(out, width, p, pitch, width, rows, cudaMemcpyDeviceToHost));
+            out += width * rows;
+            return SAGE_OK;
+        }));
+        if (written) *written = (size_t)(out - static_cast<char*>(dst_host));
+        return SAGE_OK;
+    }
     for (int p = 0; p < hd.nsk; ++p) {
         sage_fd* s = sketch_at(h, p);
         ExportSketch es = {};
@@ -1801,6 +2220,55 @@ sage_status_t sage_fd_export(sage_fd_t* h, void* dst_host, size_t capacity, size
     return SAGE_OK;
 }
 
+// A checkpoint from the middle of a block: q, left: what follows its header.
+static sage_status_t import_block(sage_fd* h, const ExportHeader& hd, const char* q, size_t left) {
+    ExportSketch es;
+    ExportBlock eb;
+    const sage_fd::Block shape = block_shape(h);
+    auto refuse = [] {
+        set_err("sage_fd_import: truncated or inconsistent checkpoint");
+        return SAGE_ERR_INVALID_ARG;
+    };
+    if (left < sizeof es + sizeof eb) return refuse();
+    std::memcpy(&es, q, sizeof es);
+    std::memcpy(&eb, q + sizeof es, sizeof eb);
+    q += sizeof es + sizeof eb;
+    left -= sizeof es + sizeof eb;
+    if (hd.frozen || hd.P != 1 || hd.nsk != 1 || hd.delta_rank != h->ell || h->sketch_only || eb.cycles_of_block != shape.L || eb.s_rows < 0 || eb.s_rows >= h->ell ||
+        eb.n_raw < 0 || eb.n_raw >= shape.M - eb.s_rows || eb.n_gram < 0 || eb.n_gram > eb.s_rows + eb.n_raw || eb.cycles < 0 || eb.cycles >= (eb.s_rows < h->ell - 1 ? 1 : shape.L) ||
+        eb.np < shape.np || eb.np > (h->dtype == SAGE_F32 ? 3 : 2) || es.rows != eb.s_rows + eb.n_raw - eb.cycles * (h->ell + 1) || es.rows < 0 || es.rows >= h->m ||
+        (eb.cycles > 0 && eb.n_gram < h->m + (eb.cycles - 1) * (h->ell + 1)) || left < export_block_bytes(h, eb))
+        return refuse();
+    DeviceGuard g(h->device);
+    ST_TRY(sage_fd_reset(h));
+    ST_TRY(sage_fd_set_option(h, 6, 1.0));
+    h->block = hd.block;
+    h->delta_rank = hd.delta_rank;
+    ST_TRY(settle_form(h, IN_BLOCKS));
+    if (!h->sketching_in_blocks) {
+        set_err("sage_fd_import: no memory for the rows of a block");
+        return SAGE_ERR_ALLOC;
+    }
+    auto& k = h->blk;
+    ST_TRY(block_widen(h, eb.np, nullptr));
+    CU_TRY(cudaMemcpy(h->info, &es.info, sizeof(EigInfo), cudaMemcpyHostToDevice));
+    k.cur = 0;
+    ST_TRY(each_block_array(h, k, eb, [&](void* p, size_t pitch, size_t width, size_t rows) -> sage_status_t {
+        if (rows > 0) CU_TRY(cudaMemcpy2D(p, pitch, q, width, width, rows, cudaMemcpyHostToDevice));
+        q += width * rows;
+        return SAGE_OK;
+    }));
+    k.s_rows = eb.s_rows;
+    k.n_raw = eb.n_raw;
+    k.n_gram = eb.n_gram;
+    k.cycles = eb.cycles;
+    h->fill = es.rows;
+    h->dealt = hd.dealt;
+    h->rows_seen = hd.dealt;
+    CU_TRY(cudaDeviceSynchronize());
+    return settle_form(h);
+}
+
 sage_status_t sage_fd_import(sage_fd_t* h, const void* src_host, size_t bytes, void* cuda_stream) {
     ST_TRY(check_handle(h));
     ExportHeader hd;
@@ -1809,12 +2277,14 @@ sage_status_t sage_fd_import(sage_fd_t* h, const void* src_host, size_t bytes, v
         return SAGE_ERR_INVALID_ARG;
     }
     std::memcpy(&hd, src_host, sizeof hd);
-    if (std::memcmp(hd.magic, kExportMagic, 8) != 0 || hd.D != h->D || hd.ell != h->ell || hd.dtype != (int32_t)h->dtype || hd.P < 1 ||
+    const bool in_block = std::memcmp(hd.magic, kExportMagicBlock, 8) == 0;
+    if ((!in_block && std::memcmp(hd.magic, kExportMagic, 8) != 0) || hd.D != h->D || hd.ell != h->ell || hd.dtype != (int32_t)h->dtype || hd.P < 1 ||
         hd.P > 64 || hd.nsk < 1 || hd.nsk > hd.P || hd.block < 1 || hd.dealt < 0 || hd.delta_rank < 2 || hd.delta_rank > h->m - 1) {
         set_err("sage_fd_import: not a checkpoint of a sketch with D=%lld ell=%d and this row type", (long long)h->D, h->ell);
         return SAGE_ERR_INVALID_ARG;
     }
     // sizes first: nothing of the handle changes unless the whole checkpoint is consistent
+    if (in_block) return import_block(h, hd, static_cast<const char*>(src_host) + sizeof hd, bytes - sizeof hd);
     {
         const char* q = static_cast<const char*>(src_host) + sizeof hd;
         size_t left = bytes - sizeof hd;
@@ -1841,6 +2311,7 @@ sage_status_t sage_fd_import(sage_fd_t* h, const void* src_host, size_t bytes, v
     h->delta_rank = hd.delta_rank;
     for (sage_fd* k : h->kids) k->delta_rank = hd.delta_rank;
     if (hd.nsk > 1) ST_TRY(ensure_sketches(h));
+    ST_TRY(settle_form(h, BY_CYCLES));                  // the rows go to the buffers first
     const char* q = static_cast<const char*>(src_host) + sizeof hd;
     for (int p = 0; p < hd.nsk; ++p) {
         sage_fd* s = sketch_at(h, p);
@@ -1860,6 +2331,7 @@ sage_status_t sage_fd_import(sage_fd_t* h, const void* src_host, size_t bytes, v
     }
     h->dealt = hd.dealt;
     h->rows_seen = hd.dealt;
+    if (!hd.frozen) ST_TRY(settle_form(h));
     if (hd.frozen) {
         CU_TRY(cudaMemcpy(h->sigma, q, (size_t)h->ell * sizeof(float), cudaMemcpyHostToDevice));
         CU_TRY(cudaDeviceSynchronize());

@@ -231,6 +231,87 @@ cudaError_t select_scratch_bytes(int64_t N, size_t* bytes);
 int select_launches(int64_t N, int64_t k);
 cudaError_t launch_select(const float* scores, int64_t N, int64_t k, int64_t* idx, void* scratch, cudaStream_t st);
 
+// ---- blocks of shrink cycles (block_kernels.cu, tc_gram_block.cu, tc_rebuild_block.cu) -------------------------------------------
+// A block holds the rows of several shrink cycles: logical rows 0 .. s_rows - 1 are the sketch as it stood when the block began, the
+// rows given since follow. Each is kept as planes of bfloat16 that add up to it exactly, one plane after the other: 3 for rows of the
+// sketch, np for rows in the store, 1 for bfloat16 rows that stay where the caller holds them. The planes of the three places lie
+// behind one another in the order of the logical rows, each place rounded up to 32 planes (the surplus reads as zero).
+struct BlockMap {
+    int s_rows, np, n_store, n_in;
+    int oR, oI, P;                 // where the planes of the store begin, those in place, and the end
+};
+struct BlockSource {
+    const __nv_bfloat16 *S, *R;
+    int64_t pitch;                 // of S and R: values, a multiple of 64
+    const void* in_place;
+    int64_t ld_in;
+};
+#ifdef __CUDACC__
+#define SAGE_HD __host__ __device__
+#else
+#define SAGE_HD
+#endif
+SAGE_HD inline int block_rows(const BlockMap& m) { return m.s_rows + m.n_store + m.n_in; }
+SAGE_HD inline int block_phys(const BlockMap& m, int i) {         // the first plane of logical row i
+    const int r = i - m.s_rows;
+    return r < 0 ? 3 * i : r < m.n_store ? m.oR + m.np * r : m.oI + (r - m.n_store);
+}
+SAGE_HD inline int block_planes(const BlockMap& m, int i) { return i < m.s_rows ? 3 : i < m.s_rows + m.n_store ? m.np : 1; }
+inline BlockMap block_map(int s_rows, int np, int n_store, int n_in) {
+    auto up = [](int x) { return (x + 31) & ~31; };
+    const int oR = up(3 * s_rows), oI = oR + up(np * n_store);
+    return {s_rows, np, n_store, n_in, oR, oI, oI + up(n_in)};
+}
+// Tiles of 256 x 256 planes on and above the diagonal whose column block is `first` or later.
+inline int block_tiles(const BlockMap& m, int first) {
+    const int nb = (m.P + 255) / 256;
+    return nb * (nb + 1) / 2 - first * (first + 1) / 2;
+}
+#ifndef SAGE_OPTIONAL
+#define SAGE_OPTIONAL __attribute__((weak))      // a library linked without the block kernels does without blocks
+#endif
+// Between the two calls this thread may wait for streams while a stream is being captured somewhere.
+void allow_work_beside_capture(bool on) SAGE_OPTIONAL;
+// Planes of n rows (dense: rows, pitch ld; or factors) to rows row0 .. of the store: np planes a row, zero beyond D.
+cudaError_t launch_block_append(const void* rows, sage_dtype_t dt, int64_t n, int64_t ld, int64_t D, __nv_bfloat16* R, int64_t pitch, int np,
+                                int64_t row0, cudaStream_t st) SAGE_OPTIONAL;
+cudaError_t launch_block_append_outer(const void* q, int64_t ldq, const void* feat, int64_t ldf, sage_dtype_t dt, int64_t n, int C, int F,
+                                      __nv_bfloat16* R, int64_t pitch, int np, int64_t row0, cudaStream_t st) SAGE_OPTIONAL;
+// out[i] = the sum of the np planes of row i, i < n (fp32, pitch ldo, zero beyond D up to ldo).
+cudaError_t launch_block_unpack(const __nv_bfloat16* R, int64_t pitch, int np, int n, int64_t D, float* out, int64_t ldo, cudaStream_t st) SAGE_OPTIONAL;
+// Inner products of planes, as partial tiles: see tc_gram_block.cu. Tiles that hold a row from logical row first_new on;
+// block_tiles(map, block_phys(map, first_new) / 256) * slices of 65,536 floats at parts.
+cudaError_t launch_block_gram(const BlockSource& src, const BlockMap& map, int first_new, int64_t D, int slices, float* parts, int* err,
+                              cudaStream_t st) SAGE_OPTIONAL;
+// P[i][j] and P[j][i] (pitch ldP) for j >= first_new, i <= j: the sums over planes and slices, fp64.
+cudaError_t launch_block_gram_reduce(const float* parts, const BlockMap& map, int first_new, int slices, float* P, int ldP, cudaStream_t st) SAGE_OPTIONAL;
+// The inner products of a block seen from its cycle c: the kept rows of cycle c are combinations of logical rows before
+// b_c = keep + c step, its window is them and logical rows b_c .. b_c + step - 1. U[k] (m x keep, pitch ldu, U_stride floats apart): the
+// factors that cycle k's solve left. C (keep x columns, pitch ldP): inner products of the kept rows with logical rows b_c on.
+struct BlockSmall {
+    int m, keep, step;
+    const float* P;
+    int ldP;
+    float* C;
+    const float* U;
+    int ldu;
+    int64_t U_stride;
+    float* K;                      // the window's matrix of a cycle c > 0 (that of cycle 0 is P): K + (c & 1) * K_stride, pitch ldk
+    int64_t K_stride;
+    int ldk;
+};
+// Columns [col0, col1) of C from cycle c0's to cycle c1's (c0 = 0: from P), and what they give of window c1; inner: also the inner
+// products of the kept rows with each other, from window c1 - 1.
+cudaError_t launch_block_step(const BlockSmall& b, int c0, int c1, int col0, int col1, bool inner, cudaStream_t st) SAGE_OPTIONAL;
+// The kept rows after ncyc cycles as combinations of planes: T[t][j][p], t < 3, j < j_pad (the planes of the coefficients, pitch ldT), for
+// p < P rounded up to 64; carried: the cycles behind which launch_block_step has been. The last cycle's factors have keep_last columns and its window r_last rows.
+cudaError_t launch_block_factors(const BlockSmall& b, const BlockMap& map, int carried, int ncyc, int r_last, int keep_last, __nv_bfloat16* T, int j_pad, int64_t ldT,
+                                 cudaStream_t st) SAGE_OPTIONAL;
+// out[j] = sum_p (T[0] + T[1] + T[2])[j][p] plane_p for j < keep: as three planes a row (planes, pitch of the source) or in fp32
+// (rows, pitch ldo, d < ldo).
+cudaError_t launch_block_rebuild(const BlockSource& src, const BlockMap& map, int64_t D, const __nv_bfloat16* T, int j_pad, int64_t ldT, int keep,
+                                 __nv_bfloat16* planes, float* rows, int64_t ldo, int* err, cudaStream_t st) SAGE_OPTIONAL;
+
 // Hooks into the C ABI's bookkeeping for entry points defined outside api.cu.
 void set_error_message(const char* msg);   // becomes the calling thread's sage_last_error()
 void count_launches(int k);                // adds to sage_launch_count()

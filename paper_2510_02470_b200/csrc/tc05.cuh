@@ -137,6 +137,17 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* t
                  "l"(reinterpret_cast<uint64_t>(tmap)), "r"(smem_u32(bar)), "r"(x), "r"(y)
                  : "memory");
 }
+// The same for a CTA of a pair: the bytes are reported to the barrier at this place in CTA 0 of the cluster.
+__device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const CUtensorMap* tmap, uint64_t* bar, int x, int y) {
+    asm volatile(
+        "{\n"
+        ".reg .b32 a;\n"
+        "mapa.shared::cluster.u32 a, %2, 0;\n"
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [a];\n"
+        "}\n" ::"r"(smem_u32(smem_dst)),
+        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(smem_u32(bar)), "r"(x), "r"(y)
+        : "memory");
+}
 // 4-D tile load (coordinates innermost first; c0 must make c0 * element size a multiple of 16 bytes).
 __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* tmap, uint64_t* bar, int c0, int c1, int c2, int c3) {
     asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(
@@ -243,6 +254,16 @@ __device__ __forceinline__ void mma_tf32_pair(uint32_t d_tmem, uint64_t adesc, u
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+__device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "setp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n"
+        "}\n" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
 // A from TMEM: lane = row, one 32-bit column per element of the contraction index.
 __device__ __forceinline__ void mma_tf32_ts_pair(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
@@ -329,6 +350,17 @@ __device__ __forceinline__ uint64_t smem_desc_mn_sw128_atom32(uint32_t smem_addr
     d |= static_cast<uint64_t>(512 >> 4) << 32;
     d |= static_cast<uint64_t>(1) << 46;
     d |= static_cast<uint64_t>(1) << 61;                              // 128-byte swizzle, 32-byte atoms
+    return d;
+}
+// The same for 16-bit values in the 128-byte swizzle: boxes of [k rows][128 bytes], 8 k rows to a group of 1024 bytes, consecutive
+// spans of 64 values `span_bytes` apart. One MMA (16 k rows) covers two groups.
+__device__ __forceinline__ uint64_t smem_desc_mn_sw128(uint32_t smem_addr_bytes, uint32_t span_bytes) {
+    uint64_t d = 0;
+    d |= static_cast<uint64_t>((smem_addr_bytes & 0x3ffffu) >> 4);
+    d |= static_cast<uint64_t>((span_bytes >> 4) & 0x3fffu) << 16;
+    d |= static_cast<uint64_t>(1024 >> 4) << 32;
+    d |= static_cast<uint64_t>(1) << 46;
+    d |= static_cast<uint64_t>(2) << 61;
     return d;
 }
 // Instruction descriptor: fp32 accumulate, A and B of one format (1 = bf16, 2 = tf32), M x N tile.
