@@ -1,8 +1,10 @@
 // The kept rows at the end of a block from its planes: out[j][d] = sum_p T[j][p] plane_p[d] (see block_kernels.cu for T). The planes are
 // the MMA's M side, 128 values d of a row on the lanes of TMEM, contiguous in memory (MN-major); T, itself as three bfloat16 planes
 // that add up to it exactly, is the N side. Three MMAs (T's planes) per 16 planes of the block add into one accumulator.
-// One CTA per tile of 128 DS values; the tile's planes are read once, T (out of L2) once per tile.
-//   warp 0 loads, warp 1 issues MMAs, warps 4-11 are the epilogue and drains (two accumulators in turn).
+// One pair of SMs per tile of 256 DS values, each with half of the values and half of T's rows: the tile's planes are read once, T (out of
+// L2) once per tile.
+//   warp 0 loads, warp 1 of CTA 0 issues the MMAs of both, warps 4-11 are the epilogue and drain (two accumulators in turn).
+// Both CTAs' loads report to CTA 0's barriers.
 // The result is written as three planes a row again, or in fp32 at the freeze.
 #include "block.cuh"
 
@@ -14,7 +16,7 @@ constexpr int kThreads = 384;
 constexpr int kChunk = 64;                  // planes per stage
 constexpr int kSpanBytes = kChunk * 128;    // 64 planes x 64 values
 
-__host__ __device__ constexpr int stage_bytes(int ds, int j_pad) { return 2 * ds * kSpanBytes + 3 * j_pad * 128; }
+__host__ __device__ constexpr int stage_bytes(int ds, int j_pad) { return 2 * ds * kSpanBytes + 3 * (j_pad / 2) * 128; }   // of one CTA
 __host__ __device__ constexpr int stage_count(int ds, int j_pad) {
     const int n = (227 * 1024 - 2048) / stage_bytes(ds, j_pad);
     return n > 8 ? 8 : n;
@@ -42,7 +44,8 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nchunk = (map.P + kChunk - 1) / kChunk;
     const int nruns = (nchunk + kRunChunks - 1) / kRunChunks;
-    const long long my_tiles = num_tiles > blockIdx.x ? (num_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    const int q = blockIdx.x & 1;
+    const long long pair = blockIdx.x >> 1, pairs = gridDim.x >> 1, my_tiles = num_tiles > pair ? (num_tiles - pair + pairs - 1) / pairs : 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) {
@@ -51,7 +54,7 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], 256);
+            mbar_init(&acc_empty[b], 16);
         }
         *abort = 0;
         mbar_fence_init();
@@ -60,9 +63,9 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
         tma_prefetch_desc(&tmI);
         tma_prefetch_desc(&tmT);
     }
-    if (warp == 1) tmem_alloc(tmem_slot, 512);
+    if (warp == 1) tmem_alloc_pair(tmem_slot, 512);
     tc_fence_before();
-    __syncthreads();
+    cluster_barrier();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     chain_wait();
@@ -74,32 +77,32 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
             int s = 0;
             uint32_t ph = 1;
             for (long long lt = 0; lt < my_tiles && alive; ++lt) {
-                const int d0 = (int)((blockIdx.x + lt * gridDim.x) * (128 * DS));
+                const int d0 = (int)((2 * (pair + lt * pairs) + q) * (128 * DS));
                 for (int c = 0; c < nchunk; ++c) {
                     if (!mbar_wait(&empty[s], ph, abort)) { alive = false; break; }
                     uint8_t* st = smem + (size_t)s * sbytes;
-                    mbar_expect_tx(&full[s], (uint32_t)sbytes);
+                    if (q == 0) mbar_expect_tx(&full[s], 2 * (uint32_t)sbytes);
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const BlockBox box = block_box(map, c * kChunk + 32 * h);
                         const CUtensorMap* tm = box.place == 0 ? &tmS : box.place == 1 ? &tmR : &tmI;
 #pragma unroll
-                        for (int sp = 0; sp < 2 * DS; ++sp) tma_load_2d(st + sp * kSpanBytes + h * 4096, tm, &full[s], d0 + 64 * sp, box.row);
+                        for (int sp = 0; sp < 2 * DS; ++sp) tma_load_2d_pair(st + sp * kSpanBytes + h * 4096, tm, &full[s], d0 + 64 * sp, box.row);
                     }
                     for (int t = 0; t < 3; ++t)
-                        tma_load_2d(st + 2 * DS * kSpanBytes + t * j_pad * 128, &tmT, &full[s], c * kChunk, t * j_pad);
+                        tma_load_2d_pair(st + 2 * DS * kSpanBytes + t * j_pad * 64, &tmT, &full[s], c * kChunk, t * j_pad + q * (j_pad / 2));
                     ++issued;
                     if (++s == stages) { s = 0; ph ^= 1u; }
                 }
             }
-            if (*abort)
+            if (q == 0 && *abort)
                 for (long long k = issued > stages ? issued - stages : 0; k < issued; ++k)
                     mbar_wait_quiet(&full[k % stages], (uint32_t)(k / stages) & 1u, 20000000ll);
         }
-    } else if (warp == 1) {
-        const uint32_t idesc = instr_desc(1, 128, j_pad, 1, 0);             // A (planes) MN-major, B (T) K-major
+    } else if (warp == 1 && q == 0) {
+        const uint32_t idesc = instr_desc(1, 256, j_pad, 1, 0);             // A (planes) MN-major, B (T) K-major
         const uint64_t desc_a = smem_desc_mn_sw128(0, kSpanBytes), desc_t = smem_desc_k_sw128(0);
-        const uint32_t st0 = smem_u32(smem), t_bytes = (uint32_t)j_pad * 128u;
+        const uint32_t st0 = smem_u32(smem), t_bytes = (uint32_t)j_pad * 64u;
         bool alive = true;
         int s = 0;
         uint32_t ph = 0;
@@ -108,9 +111,9 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
             for (int c0 = 0; c0 < nchunk && alive; c0 += kRunChunks, ++run) {
                 const int c1 = c0 + kRunChunks < nchunk ? c0 + kRunChunks : nchunk;
                 const uint32_t b = run & 1u, acc = tmem_base + b * 256u;
-                alive = __all_sync(0xffffffffu, mbar_wait(&acc_empty[b], ((run >> 1) & 1u) ^ 1u, abort));
+                alive = __all_sync(0xffffffffu, mbar_wait_cluster<false>(&acc_empty[b], ((run >> 1) & 1u) ^ 1u, abort));
                 for (int c = c0; c < c1 && alive; ++c) {
-                    alive = __all_sync(0xffffffffu, mbar_wait(&full[s], ph, abort));
+                    alive = __all_sync(0xffffffffu, mbar_wait_cluster<true>(&full[s], ph, abort));
                     if (!alive) break;
                     tc_fence_after();
                     const uint32_t st = st0 + (uint32_t)(s * sbytes), tt = st + 2 * DS * kSpanBytes;
@@ -122,10 +125,10 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
                                 const uint64_t da = desc_a | ((st + (uint32_t)(2 * x * kSpanBytes + k * 2048)) >> 4);
 #pragma unroll
                                 for (int t = 0; t < 3; ++t)
-                                    mma_bf16(acc + (uint32_t)(x * j_pad), da, (desc_t | ((tt + (uint32_t)t * t_bytes) >> 4)) + 2 * k, idesc, c != c0 || k != 0 || t != 0);
+                                    mma_bf16_pair(acc + (uint32_t)(x * j_pad), da, (desc_t | ((tt + (uint32_t)t * t_bytes) >> 4)) + 2 * k, idesc, c != c0 || k != 0 || t != 0);
                             }
-                        mma_commit(&empty[s]);
-                        if (c == c1 - 1) mma_commit(&acc_full[b]);
+                        mma_commit_pair(&empty[s]);
+                        if (c == c1 - 1) mma_commit_pair(&acc_full[b]);
                     }
                     __syncwarp();
                     if (++s == stages) { s = 0; ph ^= 1u; }
@@ -160,9 +163,10 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
                         for (int j = 0; j < 16; ++j) sum[j0 + j] += __uint_as_float(v[j]);
                     }
                 tc_fence_before();
-                mbar_arrive(&acc_empty[b]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster_relaxed(&acc_empty[b], 0);
             }
-            const long long d = (blockIdx.x + lt * gridDim.x) * (128 * DS) + x * 128 + quarter * 32 + lane;
+            const long long d = (2 * (pair + lt * pairs) + q) * (128 * DS) + x * 128 + quarter * 32 + lane;
             if (!ok) break;
             if (rows) {
                 if (d < ldo)
@@ -191,13 +195,15 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
             }
         }
     }
+    // no MMA may be in flight when TMEM is freed, and no barrier of a CTA may go while the other still arrives on it
+    const long long last = my_tiles * nruns - 1;
+    if (warp == 1 && last >= 0 && !*abort) mbar_wait_quiet(&acc_full[last & 1], (uint32_t)(last >> 1) & 1u, kWaitLimitCycles);
     tc_fence_before();
     __syncthreads();
+    cluster_barrier();
     if (warp == 1) {
-        const long long last = my_tiles * nruns - 1;
-        if (last >= 0 && !*abort) mbar_wait_quiet(&acc_full[last & 1], (uint32_t)(last >> 1) & 1u, kWaitLimitCycles);
         tc_fence_after();
-        tmem_dealloc(tmem_base, 512);
+        tmem_dealloc_pair(tmem_base, 512);
     }
     if (threadIdx.x == 0 && *abort) atomicExch(err, 1);
 }
@@ -208,16 +214,16 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
 // See sage_internal.h.
 cudaError_t launch_block_rebuild(const BlockSource& src, const BlockMap& map, int64_t D, const __nv_bfloat16* T, int j_pad, int64_t ldT, int keep,
                                  __nv_bfloat16* planes, float* rows, int64_t ldo, int* err, cudaStream_t st) {
-    if (j_pad < 16 || j_pad > 256 || (j_pad & 15) || keep > j_pad || map.P < 1) return cudaErrorInvalidValue;
+    if (j_pad < 32 || j_pad > 256 || (j_pad & 31) || keep > j_pad || map.P < 1) return cudaErrorInvalidValue;
     CUtensorMap tmS, tmR, tmI, tmT;
     const int64_t k64 = (map.P + 63) / 64 * 64;
     if (k64 > ldT || !tc::block_tmaps(src, map, D, &tmS, &tmR, &tmI) ||
-        !tc::make_tmap_2d(&tmT, T, 2, (uint64_t)(3 * j_pad), (uint64_t)k64, (uint64_t)ldT, (uint32_t)j_pad))
+        !tc::make_tmap_2d(&tmT, T, 2, (uint64_t)(3 * j_pad), (uint64_t)k64, (uint64_t)ldT, (uint32_t)(j_pad / 2)))
         return cudaErrorInvalidValue;
     // two tiles of 128 values share a stage's factors where the rows are long enough to fill the SMs twice that way
     const bool two = j_pad <= 64 && ldo >= (int64_t)148 * 512;
-    const long long tiles = (ldo + (two ? 255 : 127)) / (two ? 256 : 128);
-    const int grid = (int)(tiles < 148 ? tiles : 148);
+    const long long tiles = (ldo + (two ? 511 : 255)) / (two ? 512 : 256);
+    const int pairs = (int)(tiles < 74 ? tiles : 74);
     const int ds = two ? 2 : 1;
     const size_t smem = (size_t)tc::stage_count(ds, j_pad) * tc::stage_bytes(ds, j_pad) + 1024 + 20 * 8 + 16;
     auto kernel = two            ? tc::k_tc_rebuild_block<2, 64>
@@ -226,7 +232,7 @@ cudaError_t launch_block_rebuild(const BlockSource& src, const BlockMap& map, in
                                  : tc::k_tc_rebuild_block<1, 128>;
     const cudaError_t e = allow_smem((const void*)kernel, 227 * 1024);
     if (e != cudaSuccess) return e;
-    return launch_chained(kernel, dim3(grid), dim3(tc::kThreads), smem, st, tmS, tmR, tmI, tmT, map, j_pad, keep, tiles,
+    return launch(kernel, LaunchShape{dim3(2 * pairs), dim3(tc::kThreads), smem, 2}, st, tmS, tmR, tmI, tmT, map, j_pad, keep, tiles,
                           reinterpret_cast<unsigned short*>(planes), rows, ldo, err);
 }
 
