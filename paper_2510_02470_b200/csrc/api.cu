@@ -807,9 +807,10 @@ sage_status_t sage_fd_set_option(sage_fd_t* h, int key, double value) {
 // complete when an update returns stay in the store (as rows of an incomplete cycle stay in the buffer otherwise).
 
 // Cycles of a block: as many as make 352 new rows, at least 4. Per cycle the kernels that read the rows cost 1 / L of a launch that takes
-// little longer for more rows; beyond that the inner products among a block's rows, which grow with the square, take over. The first
-// block ends with the first shrink.
-static int block_cycles(int ell) { return std::max(4, 352 / (ell + 1)); }
+// little longer for more rows; beyond that the inner products among a block's rows, which grow with the square, take over: 4 cycles where
+// rows are long (64 rows, 11.2 M values: 5 cycles are 544 planes and a third block of 256 of them, 2.3 ms a cycle instead of 1.7). The
+// first block ends with the first shrink.
+static int block_cycles(int64_t D, int ell) { return D >= ((int64_t)1 << 18) ? 4 : std::max(4, 352 / (ell + 1)); }
 static int block_cycles_now(const sage_fd* h) { return h->blk.s_rows < h->ell - 1 ? 1 : h->blk.L; }
 
 static BlockMap block_full_map(const sage_fd* h, int np, bool first) {
@@ -822,13 +823,18 @@ static int block_most_tiles(const sage_fd* h, int np) {
     return std::max(block_tiles(block_full_map(h, np, false), 0), block_tiles(block_full_map(h, np, true), 0));
 }
 // K slices of a block's inner products: fixed for a handle, as the sums must not depend on how many rows a launch has. The number with
-// which a full block's tiles end soonest on 74 pairs of SMs, a slice costing 6 K tiles besides its own.
+// which the tiles of a full block end soonest on 74 pairs of SMs, and to a quarter those of a launch with an eighth of them (the first block,
+// the freeze, rows of short calls); a slice costs 6 K tiles besides its own, and a partial tile 0.35 in the reduction. Measured, Gram +
+// reduction of a full block and of the first one, us: 262,144 values, ell 256: 2 slices 919 + 200, 875; 8 (taken) 939 + 227, 238;
+// 20: 961 + 317, 109. 51,300 values, ell 128: 2: 195 + 80, 187; 6: 83 + 83, 76 (7 taken); 20: 83 + 106, 37. 5,130 fp32 values, ell 64:
+// 1: 52 + 59, 50; 4 (taken): 27 + 61, 25; 12: 38 + 75, 24.
 static int block_slices(int64_t D, int tiles) {
     const int nkt = (int)((D + 63) / 64);
     int best = 1;
     double best_cost = 1e300;
     for (int s = 1; s <= std::min(nkt, 74); ++s) {
-        const double cost = (double)((tiles * s + 73) / 74) * ((double)((nkt + s - 1) / s) + 6.0) + 0.02 * tiles * s;
+        const double each = (double)((nkt + s - 1) / s) + 6.0;
+        const double cost = ((tiles * s + 73) / 74 + 0.25 * ((std::max(1, tiles / 8) * s + 73) / 74)) * each + 0.35 * tiles * s;
         if (cost < best_cost) { best_cost = cost; best = s; }
     }
     return best;
@@ -855,7 +861,7 @@ static cudaError_t block_alloc_rows(sage_fd* h, int np) {
 
 static sage_fd::Block block_shape(const sage_fd* h) {
     sage_fd::Block k;
-    k.L = block_cycles(h->ell);
+    k.L = block_cycles(h->D, h->ell);
     k.M = h->m + (k.L - 1) * (h->ell + 1);
     k.ldP = (k.M + 3) & ~3;
     k.ldu = (h->m + 3) & ~3;

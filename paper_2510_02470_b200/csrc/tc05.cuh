@@ -148,6 +148,16 @@ __device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const CUtensorM
         "l"(reinterpret_cast<uint64_t>(tmap)), "r"(smem_u32(bar)), "r"(x), "r"(y)
         : "memory");
 }
+__device__ __forceinline__ void tma_load_4d_pair(void* smem_dst, const CUtensorMap* tmap, uint64_t* bar, int c0, int c1, int c2, int c3) {
+    asm volatile(
+        "{\n"
+        ".reg .b32 a;\n"
+        "mapa.shared::cluster.u32 a, %2, 0;\n"
+        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [a];\n"
+        "}\n" ::"r"(smem_u32(smem_dst)),
+        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+        : "memory");
+}
 // 4-D tile load (coordinates innermost first; c0 must make c0 * element size a multiple of 16 bytes).
 __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* tmap, uint64_t* bar, int c0, int c1, int c2, int c3) {
     asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(
@@ -352,13 +362,13 @@ __device__ __forceinline__ uint64_t smem_desc_mn_sw128_atom32(uint32_t smem_addr
     d |= static_cast<uint64_t>(1) << 61;                              // 128-byte swizzle, 32-byte atoms
     return d;
 }
-// The same for 16-bit values in the 128-byte swizzle: boxes of [k rows][128 bytes], 8 k rows to a group of 1024 bytes, consecutive
-// spans of 64 values `span_bytes` apart. One MMA (16 k rows) covers two groups.
-__device__ __forceinline__ uint64_t smem_desc_mn_sw128(uint32_t smem_addr_bytes, uint32_t span_bytes) {
+// The same for 16-bit values in the 128-byte swizzle: groups of 8 k rows x 128 bytes, `group_bytes` apart; consecutive spans of 64 values
+// `span_bytes` apart. One MMA (16 k rows) covers two groups.
+__device__ __forceinline__ uint64_t smem_desc_mn_sw128(uint32_t smem_addr_bytes, uint32_t span_bytes, uint32_t group_bytes) {
     uint64_t d = 0;
     d |= static_cast<uint64_t>((smem_addr_bytes & 0x3ffffu) >> 4);
     d |= static_cast<uint64_t>((span_bytes >> 4) & 0x3fffu) << 16;
-    d |= static_cast<uint64_t>(1024 >> 4) << 32;
+    d |= static_cast<uint64_t>(group_bytes >> 4) << 32;
     d |= static_cast<uint64_t>(1) << 46;
     d |= static_cast<uint64_t>(2) << 61;
     return d;

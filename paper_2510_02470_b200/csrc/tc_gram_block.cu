@@ -11,6 +11,9 @@
 //   warp 1     TMEM; in CTA 0 the MMAs of both, into two accumulators of 256 columns in turn,
 //   warps 4-11 drain this CTA's accumulator rows (4-7: columns 0-127, 8-11: the others).
 // Both CTAs' loads report to CTA 0's barriers.
+// What bounds it: bytes in flight. A K tile's 512 cycles of MMAs need 32 KB of each SM, and a load takes 2.6 us (4.6 us on rows 22 MB
+// apart) when all SMs load: seven stages of 32 KB, of which six are on their way. 1,793 planes of 262,144 values: 920 us, with six stages 940.
+// Boxes of two K tiles (256 bytes a row, as k_tc_rebuild_block loads them) make three stages of 64 KB: 1,410 us.
 #include "block.cuh"
 
 namespace sage {
@@ -22,13 +25,15 @@ constexpr int kRegs = 168;                  // what every thread is launched wit
 constexpr int kOpBytes = 128 * 128;         // 128 rows of one K tile (64 values)
 constexpr int kBK = 64;
 constexpr int kRunTiles = 8;
-constexpr int kStages = 6;
+constexpr int kStages = 7;
+struct PlaceTmaps {
+    CUtensorMap place[3];
+};
 constexpr int kDrainWarps = 8;
 constexpr size_t kSmem = 1024 + (size_t)kStages * 2 * kOpBytes + (2 * kStages + 4) * 8 + 16;
 
 __global__ void __launch_bounds__(kThreads, 1)
-k_tc_gram_block(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmI,
-                BlockMap map, int first_blk, int tiles, int slices, int nkt_all, float* __restrict__ parts, int* __restrict__ err) {
+k_tc_gram_block(const __grid_constant__ PlaceTmaps tm, BlockMap map, int first_blk, int tiles, int slices, int nkt_all, float* __restrict__ parts, int* __restrict__ err) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * 2 * kOpBytes);   // [kStages], CTA 0's: bytes of both CTAs
@@ -67,9 +72,7 @@ k_tc_gram_block(const __grid_constant__ CUtensorMap tmS, const __grid_constant__
         }
         *abort = 0;
         mbar_fence_init();
-        tma_prefetch_desc(&tmS);
-        tma_prefetch_desc(&tmR);
-        tma_prefetch_desc(&tmI);
+        for (int i = 0; i < 3; ++i) tma_prefetch_desc(&tm.place[i]);
     }
     if (warp == 1) tmem_alloc_pair(tmem_slot, 512);
     tc_fence_before();
@@ -92,13 +95,13 @@ k_tc_gram_block(const __grid_constant__ CUtensorMap tmS, const __grid_constant__
                     const int n = cols_of(b);
                     const bool diag = a == b && n == 256;
                     const uint32_t bytes = diag ? kOpBytes : kOpBytes + n * 64;
-                    const CUtensorMap* tm[8];
+                    const CUtensorMap* from[8];
                     int y[8];
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
-                        const BlockBox box = block_box(map, (i < 4 ? a * 256 + q * 128 : b * 256 + q * (n / 2)) + (i & 3) * 32);
-                        tm[i] = box.place == 0 ? &tmS : box.place == 1 ? &tmR : &tmI;
-                        y[i] = box.row;
+                        const int p = (i < 4 ? a * 256 + q * 128 : b * 256 + q * (n / 2)) + (i & 3) * 32, place = block_place(map, p);
+                        from[i] = &tm.place[place];
+                        y[i] = block_place_row(map, p, place);
                     }
                     for (int kt = k0; kt < k1; ++kt) {
                         if (!mbar_wait(&empty[s], ph, abort)) { alive = false; break; }
@@ -106,7 +109,7 @@ k_tc_gram_block(const __grid_constant__ CUtensorMap tmS, const __grid_constant__
                         if (q == 0) mbar_expect_tx(&full[s], 2 * bytes);
 #pragma unroll
                         for (int i = 0; i < 8; ++i)
-                            if (i < 4 || (!diag && (i - 4) * 64 < n)) tma_load_2d_pair(st + i * 4096, tm[i], &full[s], kt * kBK, y[i]);
+                            if (i < 4 || (!diag && (i - 4) * 64 < n)) tma_load_2d_pair(st + i * 4096, from[i], &full[s], kt * kBK, y[i]);
                         ++issued;
                         if (++s == kStages) { s = 0; ph ^= 1u; }
                     }
@@ -213,30 +216,22 @@ k_tc_gram_block(const __grid_constant__ CUtensorMap tmS, const __grid_constant__
 }
 
 }  // namespace
-
-// See block.cuh.
-bool block_tmaps(const BlockSource& src, const BlockMap& map, int64_t D, CUtensorMap* tmS, CUtensorMap* tmR, CUtensorMap* tmI) {
-    auto make = [&](CUtensorMap* out, const void* base, int rows, int64_t ld) {
-        return make_tmap_2d(out, base, 2, (uint64_t)(rows > 0 ? rows : 1), (uint64_t)D, (uint64_t)ld, 32);
-    };
-    return make(tmS, src.S, 3 * map.s_rows, src.pitch) && make(tmR, src.R, map.np * map.n_store, src.pitch) &&
-           make(tmI, map.n_in > 0 ? src.in_place : src.R, map.n_in > 0 ? map.n_in : 1, map.n_in > 0 ? src.ld_in : src.pitch);
-}
-
 }  // namespace tc
 
 // See sage_internal.h.
 cudaError_t launch_block_gram(const BlockSource& src, const BlockMap& map, int first_new, int64_t D, int slices, float* parts, int* err,
                               cudaStream_t st) {
-    CUtensorMap tmS, tmR, tmI;
-    if (!tc::block_tmaps(src, map, D, &tmS, &tmR, &tmI)) return cudaErrorInvalidValue;
+    tc::PlaceTmaps tm;
+    const tc::Place places[3] = {tc::place_of(src, map, 0), tc::place_of(src, map, 1), tc::place_of(src, map, 2)};
+    for (int i = 0; i < 3; ++i)
+        if (!tc::make_tmap_2d(&tm.place[i], places[i].base, 2, (uint64_t)std::max(places[i].rows, 1), (uint64_t)D, (uint64_t)places[i].ld, 32)) return cudaErrorInvalidValue;
     const int nkt = (int)((D + tc::kBK - 1) / tc::kBK);
     if (slices < 1 || slices > nkt || map.P < 1) return cudaErrorInvalidValue;
     const int first = block_phys(map, first_new) >> 8, tiles = block_tiles(map, first);
     const cudaError_t e = allow_smem((const void*)tc::k_tc_gram_block, 227 * 1024, tc::kRegs);
     if (e != cudaSuccess) return e;
     const int pairs = std::min(74, tiles * slices);
-    return launch(tc::k_tc_gram_block, LaunchShape{dim3(2 * pairs), dim3(tc::kThreads), tc::kSmem, 2}, st, tmS, tmR, tmI, map, first, tiles, slices, nkt,
+    return launch(tc::k_tc_gram_block, LaunchShape{dim3(2 * pairs), dim3(tc::kThreads), tc::kSmem, 2}, st, tm, map, first, tiles, slices, nkt,
                   parts, err);
 }
 

@@ -12,11 +12,51 @@ namespace sage {
 namespace tc {
 namespace {
 
+// Planes are loaded 32 at a time, 128 values of each: 256 consecutive bytes at every visit of a row. On rows megabytes apart each visit is
+// another page, and what a stream of loads reaches depends on the bytes per visit (see make_tmap_4d_ktiles): 544 planes of 11.2 M values
+// 3.74 ms with boxes of 128 bytes a row, 3.06 ms so. In shared memory: [group of 8 planes][128-byte half][8 planes][128 bytes], each half of a
+// group in the 128-byte swizzle.
+constexpr int kBoxPlanes = 32, kBoxCols = 128, kBoxBytes = kBoxPlanes * kBoxCols * 2, kGroupBytes = 2048;
+
+// The three places: whole boxes, and boxes of 8 planes x 64 values for what is not whole (a place's last planes, a row's end).
+struct BlockTmaps {
+    CUtensorMap box[3], piece[3];
+    int rows[3];                   // planes of each place
+    int whole_cols;                // values of a row that whole boxes reach
+};
+bool block_tmaps(const BlockSource& src, const BlockMap& map, int64_t D, BlockTmaps* out) {
+    out->whole_cols = (int)(D / 64 * 64);
+    for (int i = 0; i < 3; ++i) {
+        const auto [base, ld, rows] = place_of(src, map, i);
+        out->rows[i] = rows;
+        if (!make_tmap_2d(&out->piece[i], base, 2, (uint64_t)std::max(rows, 1), (uint64_t)D, (uint64_t)ld, 8)) return false;
+        out->box[i] = out->piece[i];               // stays so, unused, where no box is whole
+        if (D < 64) continue;
+        // (a place without 8 planes has no whole box either: its map only answers "past the end")
+        if (!make_tmap_4d_ktiles(&out->box[i], base, 2, (uint64_t)std::max(rows / 8 * 8, 8), (uint64_t)out->whole_cols, (uint64_t)ld, kBoxPlanes, 2)) return false;
+    }
+    return true;
+}
+
+// One box: planes p .. p + 31 of the block (p a multiple of 32; zeros past its end), values x .. x + 127 (zeros past the row's end). Reports
+// kBoxBytes to the barrier of CTA 0.
+__device__ __forceinline__ void load_block_box(uint8_t* dst, const BlockTmaps& tm, const BlockMap& m, uint64_t* bar, int p, int x) {
+    const int place = block_place(m, p), row = block_place_row(m, p, place), rows = tm.rows[place];
+    if (x + kBoxCols <= tm.whole_cols && (row + kBoxPlanes <= rows || row >= rows)) {
+        tma_load_4d_pair(dst, &tm.box[place], bar, 0, 0, x >> 6, row >= rows ? 1 << 20 : row >> 3);
+    } else {
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) tma_load_2d_pair(dst + g * kGroupBytes + h * 1024, &tm.piece[place], bar, x + 64 * h, row + 8 * g);
+    }
+}
+
 constexpr int kThreads = 384;
 constexpr int kChunk = 64;                  // planes per stage
-constexpr int kSpanBytes = kChunk * 128;    // 64 planes x 64 values
+constexpr int kTileBytes = kChunk * 256;    // 64 planes x 128 values
 
-__host__ __device__ constexpr int stage_bytes(int ds, int j_pad) { return 2 * ds * kSpanBytes + 3 * (j_pad / 2) * 128; }   // of one CTA
+__host__ __device__ constexpr int stage_bytes(int ds, int j_pad) { return ds * kTileBytes + 3 * (j_pad / 2) * 128; }   // of one CTA
 __host__ __device__ constexpr int stage_count(int ds, int j_pad) {
     const int n = (227 * 1024 - 2048) / stage_bytes(ds, j_pad);
     return n > 8 ? 8 : n;
@@ -28,8 +68,7 @@ constexpr int kRunChunks = 5;               // 60 additions to an accumulator, w
 
 template <int DS, int JW>                   // tiles of 128 values; output rows per epilogue warp
 __global__ void __launch_bounds__(kThreads, 1)
-k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmI,
-                   const __grid_constant__ CUtensorMap tmT, BlockMap map, int j_pad, int keep, long long num_tiles,
+k_tc_rebuild_block(const __grid_constant__ BlockTmaps tm, const __grid_constant__ CUtensorMap tmT, BlockMap map, int j_pad, int keep, long long num_tiles,
                    unsigned short* __restrict__ planes, float* __restrict__ rows, long long ldo, int* __restrict__ err) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -58,9 +97,7 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
         }
         *abort = 0;
         mbar_fence_init();
-        tma_prefetch_desc(&tmS);
-        tma_prefetch_desc(&tmR);
-        tma_prefetch_desc(&tmI);
+        for (int i = 0; i < 3; ++i) tma_prefetch_desc(&tm.box[i]);
         tma_prefetch_desc(&tmT);
     }
     if (warp == 1) tmem_alloc_pair(tmem_slot, 512);
@@ -82,15 +119,11 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
                     if (!mbar_wait(&empty[s], ph, abort)) { alive = false; break; }
                     uint8_t* st = smem + (size_t)s * sbytes;
                     if (q == 0) mbar_expect_tx(&full[s], 2 * (uint32_t)sbytes);
+                    for (int h = 0; h < 2; ++h)
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const BlockBox box = block_box(map, c * kChunk + 32 * h);
-                        const CUtensorMap* tm = box.place == 0 ? &tmS : box.place == 1 ? &tmR : &tmI;
-#pragma unroll
-                        for (int sp = 0; sp < 2 * DS; ++sp) tma_load_2d_pair(st + sp * kSpanBytes + h * 4096, tm, &full[s], d0 + 64 * sp, box.row);
-                    }
+                        for (int x = 0; x < DS; ++x) load_block_box(st + x * kTileBytes + h * kBoxBytes, tm, map, &full[s], c * kChunk + 32 * h, d0 + 128 * x);
                     for (int t = 0; t < 3; ++t)
-                        tma_load_2d_pair(st + 2 * DS * kSpanBytes + t * j_pad * 64, &tmT, &full[s], c * kChunk, t * j_pad + q * (j_pad / 2));
+                        tma_load_2d_pair(st + DS * kTileBytes + t * j_pad * 64, &tmT, &full[s], c * kChunk, t * j_pad + q * (j_pad / 2));
                     ++issued;
                     if (++s == stages) { s = 0; ph ^= 1u; }
                 }
@@ -101,7 +134,7 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
         }
     } else if (warp == 1 && q == 0) {
         const uint32_t idesc = instr_desc(1, 256, j_pad, 1, 0);             // A (planes) MN-major, B (T) K-major
-        const uint64_t desc_a = smem_desc_mn_sw128(0, kSpanBytes), desc_t = smem_desc_k_sw128(0);
+        const uint64_t desc_a = smem_desc_mn_sw128(0, 1024, kGroupBytes), desc_t = smem_desc_k_sw128(0);
         const uint32_t st0 = smem_u32(smem), t_bytes = (uint32_t)j_pad * 64u;
         bool alive = true;
         int s = 0;
@@ -116,13 +149,13 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
                     alive = __all_sync(0xffffffffu, mbar_wait_cluster<true>(&full[s], ph, abort));
                     if (!alive) break;
                     tc_fence_after();
-                    const uint32_t st = st0 + (uint32_t)(s * sbytes), tt = st + 2 * DS * kSpanBytes;
+                    const uint32_t st = st0 + (uint32_t)(s * sbytes), tt = st + DS * kTileBytes;
                     if (elect_one()) {
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
 #pragma unroll
                             for (int x = 0; x < DS; ++x) {
-                                const uint64_t da = desc_a | ((st + (uint32_t)(2 * x * kSpanBytes + k * 2048)) >> 4);
+                                const uint64_t da = desc_a | ((st + (uint32_t)(x * kTileBytes + k * 2 * kGroupBytes)) >> 4);
 #pragma unroll
                                 for (int t = 0; t < 3; ++t)
                                     mma_bf16_pair(acc + (uint32_t)(x * j_pad), da, (desc_t | ((tt + (uint32_t)t * t_bytes) >> 4)) + 2 * k, idesc, c != c0 || k != 0 || t != 0);
@@ -215,9 +248,10 @@ k_tc_rebuild_block(const __grid_constant__ CUtensorMap tmS, const __grid_constan
 cudaError_t launch_block_rebuild(const BlockSource& src, const BlockMap& map, int64_t D, const __nv_bfloat16* T, int j_pad, int64_t ldT, int keep,
                                  __nv_bfloat16* planes, float* rows, int64_t ldo, int* err, cudaStream_t st) {
     if (j_pad < 32 || j_pad > 256 || (j_pad & 31) || keep > j_pad || map.P < 1) return cudaErrorInvalidValue;
-    CUtensorMap tmS, tmR, tmI, tmT;
+    tc::BlockTmaps tm;
+    CUtensorMap tmT;
     const int64_t k64 = (map.P + 63) / 64 * 64;
-    if (k64 > ldT || !tc::block_tmaps(src, map, D, &tmS, &tmR, &tmI) ||
+    if (k64 > ldT || !tc::block_tmaps(src, map, D, &tm) ||
         !tc::make_tmap_2d(&tmT, T, 2, (uint64_t)(3 * j_pad), (uint64_t)k64, (uint64_t)ldT, (uint32_t)(j_pad / 2)))
         return cudaErrorInvalidValue;
     // two tiles of 128 values share a stage's factors where the rows are long enough to fill the SMs twice that way
@@ -232,7 +266,7 @@ cudaError_t launch_block_rebuild(const BlockSource& src, const BlockMap& map, in
                                  : tc::k_tc_rebuild_block<1, 128>;
     const cudaError_t e = allow_smem((const void*)kernel, 227 * 1024);
     if (e != cudaSuccess) return e;
-    return launch(kernel, LaunchShape{dim3(2 * pairs), dim3(tc::kThreads), smem, 2}, st, tmS, tmR, tmI, tmT, map, j_pad, keep, tiles,
+    return launch(kernel, LaunchShape{dim3(2 * pairs), dim3(tc::kThreads), smem, 2}, st, tm, tmT, map, j_pad, keep, tiles,
                           reinterpret_cast<unsigned short*>(planes), rows, ldo, err);
 }
 
