@@ -245,6 +245,7 @@ struct sage_fd {
         int L = 0, M = 0;          // cycles of a block, logical rows of a full one: m + (L - 1)(ell + 1)
         int ldP = 0, ldu = 0, j_pad = 0, slices = 0;
         int64_t pitch = 0, ldT = 0;
+        void *memory = nullptr, *row_memory = nullptr;       // what the arrays below lie in: R, T and parts in the second
         __nv_bfloat16 *S[2] = {nullptr, nullptr}, *R = nullptr, *T = nullptr;
         int R_planes = 0;          // planes a row that R and parts are allocated for
         float *P = nullptr, *C = nullptr, *U = nullptr, *K = nullptr, *parts = nullptr;
@@ -842,21 +843,40 @@ static int block_slices(int64_t D, int tiles) {
 
 static void block_free(sage_fd* h) {
     auto& k = h->blk;
-    void* memory[] = {k.S[0], k.S[1], k.R, k.T, k.P, k.C, k.U, k.K, k.parts};
-    for (void* p : memory) dev_free(h, p);
+    dev_free(h, k.memory);
+    dev_free(h, k.row_memory);
     k = sage_fd::Block();
 }
 
-// Memory of the rows' planes and of their partial inner products for np planes a row.
+// One allocation for several arrays, each on a 1,024-byte boundary.
+struct Arena {
+    struct Part {
+        void** at;
+        size_t begin;
+    } part[8];
+    int n = 0;
+    size_t bytes = 0;
+    void add(void* at, size_t size) {              // at: the address of the array's pointer
+        part[n++] = {static_cast<void**>(at), bytes};
+        bytes += (size + 1023) & ~(size_t)1023;
+    }
+    cudaError_t allocate(sage_fd* h, void** memory) {
+        const cudaError_t e = dev_malloc(h, memory, bytes);
+        for (int i = 0; i < n && e == cudaSuccess; ++i) *part[i].at = static_cast<char*>(*memory) + part[i].begin;
+        return e;
+    }
+};
+
+// Memory of the rows' planes, of what multiplies them and of their partial inner products, for np planes a row.
 static cudaError_t block_alloc_rows(sage_fd* h, int np) {
     auto& k = h->blk;
-    cudaError_t e = dev_malloc(h, (void**)&k.R, (size_t)np * k.M * k.pitch * sizeof(__nv_bfloat16));
-    const int64_t ldT = (std::max(block_full_map(h, np, false).P, block_full_map(h, np, true).P) + 63) / 64 * 64;
-    if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.T, (size_t)3 * k.j_pad * ldT * sizeof(__nv_bfloat16));
-    if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.parts, (size_t)block_most_tiles(h, np) * k.slices * 65536 * sizeof(float));
-    k.ldT = ldT;
+    k.ldT = (std::max(block_full_map(h, np, false).P, block_full_map(h, np, true).P) + 63) / 64 * 64;
     k.R_planes = np;
-    return e;
+    Arena a;
+    a.add(&k.R, (size_t)np * k.M * k.pitch * sizeof(__nv_bfloat16));
+    a.add(&k.T, (size_t)3 * k.j_pad * k.ldT * sizeof(__nv_bfloat16));
+    a.add(&k.parts, (size_t)block_most_tiles(h, np) * k.slices * 65536 * sizeof(float));
+    return a.allocate(h, &k.row_memory);
 }
 
 static sage_fd::Block block_shape(const sage_fd* h) {
@@ -881,12 +901,14 @@ static bool block_setup(sage_fd* h) {
     const size_t s_bytes = (size_t)3 * (h->ell - 1) * k.pitch * sizeof(__nv_bfloat16);
     const size_t bytes = 2 * s_bytes + (size_t)np * k.M * k.pitch * sizeof(__nv_bfloat16) + (size_t)block_most_tiles(h, np) * k.slices * 65536 * sizeof(float);
     cudaError_t e = bytes <= kBlockBytes ? cudaSuccess : cudaErrorMemoryAllocation;
-    for (int i = 0; i < 2; ++i)
-        if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.S[i], s_bytes);
-    if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.P, (size_t)k.M * k.ldP * sizeof(float));
-    if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.C, (size_t)h->ell * k.ldP * sizeof(float));
-    if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.U, (size_t)(k.L + 1) * h->m * k.ldu * sizeof(float));
-    if (e == cudaSuccess) e = dev_malloc(h, (void**)&k.K, (size_t)2 * h->m * h->ldk * sizeof(float));
+    Arena a;
+    a.add(&k.S[0], s_bytes);
+    a.add(&k.S[1], s_bytes);
+    a.add(&k.P, (size_t)k.M * k.ldP * sizeof(float));
+    a.add(&k.C, (size_t)h->ell * k.ldP * sizeof(float));
+    a.add(&k.U, (size_t)(k.L + 1) * h->m * k.ldu * sizeof(float));
+    a.add(&k.K, (size_t)2 * h->m * h->ldk * sizeof(float));
+    if (e == cudaSuccess) e = a.allocate(h, &k.memory);
     // (rows of bfloat16 handles may be products of two factors: room for two planes at once, unless they are very long)
     if (e == cudaSuccess) e = block_alloc_rows(h, bytes <= kBlockBytes / 64 ? std::max(np, 2) : np);
     if (e != cudaSuccess) {
@@ -900,7 +922,7 @@ static bool block_setup(sage_fd* h) {
 
 static BlockSmall block_small(const sage_fd* h) {
     const auto& k = h->blk;
-    return {h->m, h->ell - 1, h->ell + 1, k.P, k.ldP, k.C, k.U, k.ldu, (int64_t)h->m * k.ldu, k.K, (int64_t)h->m * h->ldk, h->ldk};
+    return {h->m, h->ell - 1, h->ell + 1, k.P, k.ldP, k.C, k.U, k.ldu, (int64_t)h->m * k.ldu, k.K, (int64_t)h->m * h->ldk, h->ldk, k.U + (size_t)k.L * h->m * k.ldu};
 }
 static BlockSource block_source(const sage_fd* h, const void* in_place, int64_t ld) {
     return {h->blk.S[h->blk.cur], h->blk.R, h->blk.pitch, in_place, ld};
@@ -912,13 +934,12 @@ static sage_status_t block_widen(sage_fd* h, int np, cudaStream_t st) {
     if (k.np >= np) return SAGE_OK;
     if (k.R_planes < np || k.n_raw > 0) {                  // new memory, as rows that are there move apart
         __nv_bfloat16* old = k.R;
+        void* old_memory = k.row_memory;
         const int have = k.np;
-        CU_TRY(cudaStreamSynchronize(st));
-        CU_TRY(dev_free(h, k.T));
-        CU_TRY(dev_free(h, k.parts));
-        k.T = nullptr;
+        k.row_memory = nullptr;
+        k.R = k.T = nullptr;
         k.parts = nullptr;
-        k.R = nullptr;
+        CU_TRY(cudaStreamSynchronize(st));
         const cudaError_t e = block_alloc_rows(h, np);
         if (e == cudaSuccess && k.n_raw > 0) {
             CU_TRY(cudaMemsetAsync(k.R, 0, (size_t)np * k.n_raw * k.pitch * 2, st));
@@ -926,7 +947,7 @@ static sage_status_t block_widen(sage_fd* h, int np, cudaStream_t st) {
                 CU_TRY(cudaMemcpyAsync(k.R + (size_t)i * np * k.pitch, old + (size_t)i * have * k.pitch, (size_t)have * k.pitch * 2, cudaMemcpyDeviceToDevice, st));
         }
         CU_TRY(cudaStreamSynchronize(st));
-        CU_TRY(dev_free(h, old));
+        CU_TRY(dev_free(h, old_memory));
         CU_TRY(e);
     }
     k.np = np;
@@ -1024,7 +1045,7 @@ static sage_status_t block_feed(sage_fd* h, RowSrc src, int64_t n, cudaStream_t 
         while (k.cycles < L && nl + take >= m + k.cycles * step) {
             ST_TRY(block_solve(h, m, 1, keep, st));
             const int c = ++k.cycles;
-            if (c < L) CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_block_step(block_small(h), c - 1, c, keep + c * step, k.n_gram, true, st); }));
+            if (c < L) CU_TRY(timed(h, K_GRAM_REDUCE, block_step_launches(m, true), st, [&] { return launch_block_step(block_small(h), c - 1, c, keep + c * step, k.n_gram, true, st); }));
         }
         if (k.cycles == L) {
             ST_TRY(block_rebuild(h, map, from, L - 1, L, m, keep, nullptr, st));

@@ -13,7 +13,6 @@
 namespace sage {
 namespace {
 
-constexpr int kCols = 8;                    // columns per thread block
 constexpr int kThreads = 256;
 
 __device__ __forceinline__ float to_f32(float v) { return v; }
@@ -161,20 +160,24 @@ __global__ void __launch_bounds__(256) k_block_gram_reduce(const float* __restri
 }
 
 // ---- products with W ---------------------------------------------------------------------------------------------------
-// out[r][0 .. 7] = sum_{i < n} A[i][r] x[i][0 .. 7] for r < rows, in fp32. A thread has 4 values of r and 2 columns of one of KS parts of the
-// sum over i, which are added in order: A's elements come out of L2 (or shared memory) as they are needed, AHEAD loads in flight a thread,
-// x out of shared memory. A's rows hold at least rows rounded up to 4 values. clean: sums that are not finite count as zero. Ends with a
-// barrier behind the last read of x and the last write of out.
+// out[r][c] = sum_{i < n} A[i][r] x[i][c] for r < rows, c < COLS, in fp32. A thread has 4 values of r and a quarter of the columns of one of KS
+// parts of the sum over i, which are added in order: A's elements come out of L2 (or shared memory) as they are needed, AHEAD loads in
+// flight a thread, x out of shared memory. A's rows hold at least rows rounded up to 4 values. clean: sums that are not finite count as
+// zero. Ends with a barrier behind the last read of x and the last write of out. (16 columns, half the reads of A in all: steps of windows of
+// 256 and 512 rows 30 and 25 % longer, as what each block reads is what it waits for.)
 template <int JG>                            // groups of 4 r
 struct Apply {
-    static constexpr int NT = JG == 16 ? 512 : 1024, KS = NT / (4 * JG), AHEAD = JG == 16 ? 16 : 8;
-    float red[KS][kCols][4 * JG];
+    static constexpr int NT = JG == 16 ? 512 : 1024, KS = NT / (4 * JG), AHEAD = JG == 16 ? 16 : 8, COLS = 8, OWN = COLS / 4;
+    typedef float Row[COLS];
+    float red[KS][COLS][4 * JG];
 
-    __device__ __forceinline__ void run(const float* A, int64_t lda, int n, int rows, const float (*x)[kCols], float (*out)[kCols], bool clean) {
+    __device__ __forceinline__ void run(const float* A, int64_t lda, int n, int rows, const Row* x, Row* out, bool clean) {
         const int jg = threadIdx.x % JG, cp = threadIdx.x / JG % 4, ks = threadIdx.x / (4 * JG);
         for (int r0 = 0; r0 < rows; r0 += 4 * JG) {
             const int r = r0 + 4 * jg;
-            float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+            float4 acc[OWN];
+#pragma unroll
+            for (int u = 0; u < OWN; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (r < rows) {
                 const int i0 = n * ks / KS, i1 = n * (ks + 1) / KS;
                 const float* a = A + (int64_t)i0 * lda + r;
@@ -184,15 +187,15 @@ struct Apply {
 #pragma unroll
                     for (int u = 0; u < AHEAD; ++u) v[u] = *reinterpret_cast<const float4*>(a + u * lda);
 #pragma unroll
-                    for (int u = 0; u < AHEAD; ++u) add(acc, v[u], x[i + u], cp);
+                    for (int u = 0; u < AHEAD; ++u) add(acc, v[u], x[i + u] + OWN * cp);
                 }
 #pragma unroll 4
-                for (; i < i1; ++i, a += lda) add(acc, *reinterpret_cast<const float4*>(a), x[i], cp);
+                for (; i < i1; ++i, a += lda) add(acc, *reinterpret_cast<const float4*>(a), x[i] + OWN * cp);
             }
-            *reinterpret_cast<float4*>(&red[ks][2 * cp][4 * jg]) = acc[0];
-            *reinterpret_cast<float4*>(&red[ks][2 * cp + 1][4 * jg]) = acc[1];
+#pragma unroll
+            for (int u = 0; u < OWN; ++u) *reinterpret_cast<float4*>(&red[ks][OWN * cp + u][4 * jg]) = acc[u];
             __syncthreads();
-            for (int t = threadIdx.x; t < 4 * JG * kCols; t += NT) {
+            for (int t = threadIdx.x; t < 4 * JG * COLS; t += NT) {
                 const int c = t / (4 * JG), rr = t % (4 * JG);
                 float s = red[0][c][rr];
 #pragma unroll
@@ -202,74 +205,96 @@ struct Apply {
             __syncthreads();
         }
     }
-    static __device__ __forceinline__ void add(float4 (&acc)[2], float4 v, const float (&row)[kCols], int cp) {
-        const float2 x = *reinterpret_cast<const float2*>(&row[2 * cp]);
+    static __device__ __forceinline__ void add(float4 (&acc)[OWN], float4 v, const float* row) {
+        const float2 x = *reinterpret_cast<const float2*>(row);
         acc[0] = make_float4(fmaf(v.x, x.x, acc[0].x), fmaf(v.y, x.x, acc[0].y), fmaf(v.z, x.x, acc[0].z), fmaf(v.w, x.x, acc[0].w));
         acc[1] = make_float4(fmaf(v.x, x.y, acc[1].x), fmaf(v.y, x.y, acc[1].y), fmaf(v.z, x.y, acc[1].z), fmaf(v.w, x.y, acc[1].w));
     }
 };
 
-// Between two solves: see launch_block_step. Blocks 0 .. n_inner - 1 take 8 columns of W K W^T each (K W^T first), the others 8 columns of
+// K W^T for windows of more than 128 rows: Y (m x keep, pitch ldu), 4 JG rows and 8 columns a block. In k_block_step a block would read all
+// of K by itself.
+template <int JG>
+__global__ void __launch_bounds__(Apply<JG>::NT, 1) k_block_inner(BlockSmall b, int c1) {
+    constexpr int NT = Apply<JG>::NT, cols = Apply<JG>::COLS;
+    extern __shared__ __align__(16) float smem[];
+    auto x = reinterpret_cast<typename Apply<JG>::Row*>(smem), y = x + b.m;
+    Apply<JG>& apply = *reinterpret_cast<Apply<JG>*>(y + 4 * JG);
+    const float* U = b.U + (int64_t)(c1 - 1) * b.U_stride;
+    const float* K = c1 == 1 ? b.P : b.K + ((c1 - 1) & 1) * b.K_stride;
+    const int j0 = blockIdx.x * cols, r0 = blockIdx.y * 4 * JG, rows = min(4 * JG, b.m - r0);
+    chain_wait();
+    chain_release();
+    for (int t = threadIdx.x; t < b.m * cols; t += NT) x[t / cols][t % cols] = j0 + t % cols < b.keep ? __ldcg(U + (int64_t)(t / cols) * b.ldu + j0 + t % cols) : 0.f;
+    __syncthreads();
+    apply.run(K + r0, c1 == 1 ? b.ldP : b.ldk, b.m, rows, x, y, true);       // (a row whose norm is not finite: its coefficients are zero)
+    for (int t = threadIdx.x; t < rows * cols; t += NT)
+        if (j0 + t % cols < b.keep) b.Y[(int64_t)(r0 + t / cols) * b.ldu + j0 + t % cols] = y[t / cols][t % cols];
+}
+
+// Between two solves: see launch_block_step. Blocks 0 .. n_inner - 1 take 8 columns of W K W^T each (K W^T first, see also k_block_inner), the others 8 of
 // the products with rows still to come. Bound by latency: every round trip to L2 counts. ahead: the launch follows a solve, so that
 // everything but W was there before that solve began; it is fetched before the wait for it (K into shared memory where it fits).
 template <int JG>
 __global__ void __launch_bounds__(Apply<JG>::NT, 1) k_block_step(BlockSmall b, int c0, int c1, int col0, int col1, int n_inner, int ahead) {
-    constexpr int NT = Apply<JG>::NT;
+    constexpr int NT = Apply<JG>::NT, cols = Apply<JG>::COLS;
     extern __shared__ __align__(16) float smem[];
-    float(*x)[kCols] = reinterpret_cast<float(*)[kCols]>(smem);              // [m]
-    float(*y)[kCols] = x + b.m;                                              // [m]
+    auto x = reinterpret_cast<typename Apply<JG>::Row*>(smem), y = x + b.m;  // [m] each
     Apply<JG>& apply = *reinterpret_cast<Apply<JG>*>(y + b.m);
     const int m = b.m, keep = b.keep, step = b.step, tid = threadIdx.x;
     if (!ahead) chain_wait();
     float* Kn = b.K + (c1 & 1) * b.K_stride;
     if ((int)blockIdx.x < n_inner) {
-        const int j0 = blockIdx.x * kCols;
+        const int j0 = blockIdx.x * cols;
         const float* U = b.U + (int64_t)(c1 - 1) * b.U_stride;
-        const float* K = c1 == 1 ? b.P : b.K + ((c1 - 1) & 1) * b.K_stride;
-        int64_t ldk = c1 == 1 ? b.ldP : b.ldk;
         if constexpr (JG == 16) {
+            const float* K = c1 == 1 ? b.P : b.K + ((c1 - 1) & 1) * b.K_stride;
+            const int64_t ldk = c1 == 1 ? b.ldP : b.ldk;
             float* Ks = reinterpret_cast<float*>(&apply + 1);
             const int m4 = (m + 3) & ~3;
             for (int t = tid; t < m * (m4 / 4); t += NT) {
                 const int i = t / (m4 / 4), c = 4 * (t % (m4 / 4));
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(Ks + i * m4 + c)), "l"(K + i * ldk + c) : "memory");
             }
-            K = Ks;
-            ldk = m4;
+            if (ahead) chain_wait();
+            chain_release();
+            for (int t = tid; t < m * cols; t += NT) {
+                const int i = t / cols, c = t % cols;
+                x[i][c] = j0 + c < keep ? __ldcg(U + (int64_t)i * b.ldu + j0 + c) : 0.f;
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncthreads();
+            apply.run(Ks, m4, m, m, x, y, true);                             // (a row whose norm is not finite: its coefficients are zero)
+        } else {
+            if (ahead) chain_wait();
+            chain_release();
+            for (int t = tid; t < m * cols; t += NT) y[t / cols][t % cols] = j0 + t % cols < keep ? __ldcg(b.Y + (int64_t)(t / cols) * b.ldu + j0 + t % cols) : 0.f;
+            __syncthreads();
         }
-        if (ahead) chain_wait();
-        chain_release();
-        for (int t = tid; t < m * kCols; t += NT) {
-            const int i = t / kCols, c = t % kCols;
-            x[i][c] = j0 + c < keep ? __ldcg(U + (int64_t)i * b.ldu + j0 + c) : 0.f;
-        }
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        __syncthreads();
-        apply.run(K, ldk, m, m, x, y, true);                                // (a row whose norm is not finite: its coefficients are zero)
         apply.run(U, b.ldu, m, keep, y, x, false);
-        for (int t = tid; t < keep * kCols; t += NT) {                       // one triangle, and its mirror image
-            const int i = t / kCols, j = j0 + t % kCols;
+        for (int t = tid; t < keep * cols; t += NT) {                       // one triangle, and its mirror image
+            const int i = t / cols, j = j0 + t % cols;
             if (j < keep && i <= j) {
-                const float v = x[i][t % kCols];
+                const float v = x[i][t % cols];
                 Kn[(int64_t)i * b.ldk + j] = v;
                 Kn[(int64_t)j * b.ldk + i] = v;
             }
         }
         return;
     }
-    const int g0 = col0 + ((int)blockIdx.x - n_inner) * kCols;
+    const int g0 = col0 + ((int)blockIdx.x - n_inner) * cols;
     const float* top = c0 == 0 ? b.P : b.C;
     const int e0 = keep + c0 * step, w0 = keep + c1 * step;                  // the first rows behind the kept ones of windows c0 and c1
-    for (int t = tid; t < keep * kCols; t += NT) {
-        const int i = t / kCols, g = g0 + t % kCols;
+    for (int t = tid; t < keep * cols; t += NT) {
+        const int i = t / cols, g = g0 + t % cols;
         float v = 0.f;
         if (g < e0 && c0 == 0) v = g == i ? 1.f : 0.f;                       // coefficients: rows of window c0 enter as themselves
         else if (g < col1 && (g < e0 || g >= e0 + step || c1 > c0 + 1)) v = __ldcg(top + (int64_t)i * b.ldP + g);
-        x[i][t % kCols] = v;
+        x[i][t % cols] = v;
     }
-    if (g0 + kCols > w0 && g0 < w0 + step)                                   // products of the window's rows with each other, as far as they are there
-        for (int t = tid; t < step * kCols; t += NT) {
-            const int i = t / kCols, g = g0 + t % kCols;
+    if (g0 + cols > w0 && g0 < w0 + step)                                   // products of the window's rows with each other, as far as they are there
+        for (int t = tid; t < step * cols; t += NT) {
+            const int i = t / cols, g = g0 + t % cols;
             if (g < w0 || g >= col1 || g >= w0 + step || w0 + i >= col1) continue;
             const float v = __ldcg(b.P + (int64_t)(w0 + i) * b.ldP + g);
             Kn[(int64_t)(keep + i) * b.ldk + keep + g - w0] = v;
@@ -277,24 +302,24 @@ __global__ void __launch_bounds__(Apply<JG>::NT, 1) k_block_step(BlockSmall b, i
         }
     for (int c = c0; c < c1; ++c) {
         const int e = keep + c * step;
-        for (int t = tid; t < step * kCols; t += NT) {
-            const int i = t / kCols, g = g0 + t % kCols;
+        for (int t = tid; t < step * cols; t += NT) {
+            const int i = t / cols, g = g0 + t % cols;
             float v = 0.f;
             if (g >= e + step) v = g < col1 ? __ldcg(b.P + (int64_t)(e + i) * b.ldP + g) : 0.f;
             else if (g >= e) v = g - e == i ? 1.f : 0.f;
-            x[keep + i][t % kCols] = v;
+            x[keep + i][t % cols] = v;
         }
         if (ahead) chain_wait();                                             // (one cycle: c1 == c0 + 1)
         __syncthreads();
         apply.run(b.U + (int64_t)c * b.U_stride, b.ldu, m, keep, x, y, false);
-        for (int t = tid; t < keep * kCols; t += NT) x[t / kCols][t % kCols] = y[t / kCols][t % kCols];
+        for (int t = tid; t < keep * cols; t += NT) x[t / cols][t % cols] = y[t / cols][t % cols];
     }
     chain_release();
     __syncthreads();
-    for (int t = tid; t < keep * kCols; t += NT) {
-        const int i = t / kCols, g = g0 + t % kCols;
+    for (int t = tid; t < keep * cols; t += NT) {
+        const int i = t / cols, g = g0 + t % cols;
         if (g >= col1) continue;
-        const float v = x[i][t % kCols];
+        const float v = x[i][t % cols];
         b.C[(int64_t)i * b.ldP + g] = v;
         if (g >= w0 && g < w0 + step) {
             Kn[(int64_t)i * b.ldk + keep + g - w0] = v;
@@ -303,16 +328,15 @@ __global__ void __launch_bounds__(Apply<JG>::NT, 1) k_block_step(BlockSmall b, i
     }
 }
 
-// The product of the W of a block's cycles, 8 logical rows (columns of the product) a block: a row enters with its cycle's W and is
+// The product of the W of a block's cycles, a few logical rows (columns of the product) to a thread block: a row enters with its cycle's W and is
 // multiplied by the later ones. c_from: the cycles before it have been multiplied by k_block_step already (C). The last block fills the
 // surplus planes of the three places with zeros.
 template <int JG>
 __global__ void __launch_bounds__(Apply<JG>::NT, 1) k_block_factors(BlockSmall b, BlockMap map, int c_from, int ncyc, int r_last, int keep_last, unsigned short* __restrict__ T, int j_pad,
                                                             int64_t ldT) {
-    constexpr int NT = Apply<JG>::NT;
+    constexpr int NT = Apply<JG>::NT, cols = Apply<JG>::COLS;
     extern __shared__ __align__(16) float smem[];
-    float(*x)[kCols] = reinterpret_cast<float(*)[kCols]>(smem);
-    float(*y)[kCols] = x + b.m;
+    auto x = reinterpret_cast<typename Apply<JG>::Row*>(smem), y = x + b.m;
     Apply<JG>& apply = *reinterpret_cast<Apply<JG>*>(y + b.m);
     const int tid = threadIdx.x, keep = b.keep;
     chain_wait();
@@ -324,30 +348,30 @@ __global__ void __launch_bounds__(Apply<JG>::NT, 1) k_block_factors(BlockSmall b
             for (int t = tid; t < (to[s] - from[s]) * 3 * j_pad; t += NT) T[(int64_t)(t / (to[s] - from[s])) * ldT + from[s] + t % (to[s] - from[s])] = 0;
         return;
     }
-    const int nl = block_rows(map), g0 = blockIdx.x * kCols;
+    const int nl = block_rows(map), g0 = blockIdx.x * cols;
     auto enters = [&](int g) { return g < b.m ? 0 : (g - b.m) / b.step + 1; };
-    for (int t = tid; t < b.m * kCols; t += NT) {
-        const int i = t / kCols, g = g0 + t % kCols;
-        x[i][t % kCols] = i < keep && g < nl && enters(g) < c_from ? __ldcg(b.C + (int64_t)i * b.ldP + g) : 0.f;
+    for (int t = tid; t < b.m * cols; t += NT) {
+        const int i = t / cols, g = g0 + t % cols;
+        x[i][t % cols] = i < keep && g < nl && enters(g) < c_from ? __ldcg(b.C + (int64_t)i * b.ldP + g) : 0.f;
     }
     __syncthreads();
     for (int c = max(enters(g0), c_from); c < ncyc; ++c) {
         const bool last = c == ncyc - 1;
         const float* U = b.U + (int64_t)c * b.U_stride;
-        const int cols = last ? keep_last : keep;
-        apply.run(U, b.ldu, last ? min(keep, r_last) : keep, cols, x, y, false);
-        for (int t = tid; t < cols * kCols; t += NT) {
-            const int j = t / kCols, g = g0 + t % kCols;
-            float v = y[j][t % kCols];
+        const int wide = last ? keep_last : keep;
+        apply.run(U, b.ldu, last ? min(keep, r_last) : keep, wide, x, y, false);
+        for (int t = tid; t < wide * cols; t += NT) {
+            const int j = t / cols, g = g0 + t % cols;
+            float v = y[j][t % cols];
             if (g < nl && enters(g) == c) v = U[(int64_t)(g - c * b.step) * b.ldu + j];      // its place in window c
-            x[j][t % kCols] = v;
+            x[j][t % cols] = v;
         }
         __syncthreads();
     }
-    for (int t = tid; t < j_pad * kCols; t += NT) {
-        const int j = t / kCols, g = g0 + t % kCols;
+    for (int t = tid; t < j_pad * cols; t += NT) {
+        const int j = t / cols, g = g0 + t % cols;
         if (g >= nl) continue;
-        float v = j < keep_last ? x[j][t % kCols] : 0.f;
+        float v = j < keep_last ? x[j][t % cols] : 0.f;
         const int p0 = block_phys(map, g), np = block_planes(map, g);
         for (int s = 0; s < 3; ++s) {
             const unsigned hi = __float_as_uint(v) & 0xffff0000u;
@@ -358,7 +382,7 @@ __global__ void __launch_bounds__(Apply<JG>::NT, 1) k_block_factors(BlockSmall b
 }
 
 template <int JG>
-size_t small_smem(int m) { return (size_t)2 * m * kCols * sizeof(float) + sizeof(Apply<JG>); }
+size_t small_smem(int m) { return (size_t)2 * m * sizeof(typename Apply<JG>::Row) + sizeof(Apply<JG>); }
 constexpr int kSmallSmem = 160 * 1024;
 // Windows of up to this many rows: the product of the W is carried along from step to step, beside the inner products (columns before
 // the window of C). Larger ones have more columns than there are SMs as it is, and form it at the end of the block.
@@ -412,13 +436,23 @@ cudaError_t launch_block_gram_reduce(const float* parts, const BlockMap& map, in
 
 cudaError_t launch_block_step(const BlockSmall& b, int c0, int c1, int col0, int col1, bool inner, cudaStream_t st) {
     if (inner && b.m <= kCarryRows) col0 = 0;
-    const int n_inner = inner ? (b.keep + kCols - 1) / kCols : 0, n_cols = col1 > col0 ? (col1 - col0 + kCols - 1) / kCols : 0;
+    constexpr int cols = Apply<16>::COLS;
+    const int n_inner = inner ? (b.keep + cols - 1) / cols : 0, n_cols = col1 > col0 ? (col1 - col0 + cols - 1) / cols : 0;
     if (n_inner + n_cols == 0) return cudaSuccess;
     auto go = [&](auto kernel, int threads, size_t smem) -> cudaError_t {
         const cudaError_t e = allow_smem((const void*)kernel, kSmallSmem);
         if (e != cudaSuccess) return e;
         return launch_chained(kernel, dim3(n_inner + n_cols), dim3(threads), smem, st, b, c0, c1, col0, col1, n_inner, inner && c1 == c0 + 1 ? 1 : 0);
     };
+    if (inner && b.m > 128) {
+        auto first = [&](auto kernel, int threads, int rows, size_t apply) -> cudaError_t {
+            const cudaError_t e = allow_smem((const void*)kernel, kSmallSmem);
+            if (e != cudaSuccess) return e;
+            return launch_chained(kernel, dim3(n_inner, (b.m + rows - 1) / rows), dim3(threads), (size_t)(b.m + rows) * cols * sizeof(float) + apply, st, b, c1);
+        };
+        const cudaError_t e = b.m <= 256 ? first(k_block_inner<16>, Apply<16>::NT, 64, sizeof(Apply<16>)) : first(k_block_inner<32>, Apply<32>::NT, 128, sizeof(Apply<32>));
+        if (e != cudaSuccess) return e;
+    }
     if (b.m <= 128) return go(k_block_step<16>, Apply<16>::NT, small_smem<16>(b.m) + (inner ? (size_t)b.m * ((b.m + 3) & ~3) * sizeof(float) : 0));
     if (b.m <= 256) return go(k_block_step<32>, Apply<32>::NT, small_smem<32>(b.m));
     return go(k_block_step<64>, Apply<64>::NT, small_smem<64>(b.m));
@@ -429,7 +463,7 @@ cudaError_t launch_block_factors(const BlockSmall& b, const BlockMap& map, int c
     auto go = [&](auto kernel, int threads, size_t smem) -> cudaError_t {
         const cudaError_t e = allow_smem((const void*)kernel, kSmallSmem);
         if (e != cudaSuccess) return e;
-        return launch_chained(kernel, dim3((block_rows(map) + kCols - 1) / kCols + 1), dim3(threads), smem, st, b, map, b.m <= kCarryRows ? carried : 0, ncyc, r_last, keep_last,
+        return launch_chained(kernel, dim3((block_rows(map) + Apply<16>::COLS - 1) / Apply<16>::COLS + 1), dim3(threads), smem, st, b, map, b.m <= kCarryRows ? carried : 0, ncyc, r_last, keep_last,
                               reinterpret_cast<unsigned short*>(T), j_pad, ldT);
     };
     if (b.m <= 128) return go(k_block_factors<16>, Apply<16>::NT, small_smem<16>(b.m));

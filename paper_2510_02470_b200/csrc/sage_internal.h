@@ -299,7 +299,9 @@ struct BlockSmall {
     float* K;                      // the window's matrix of a cycle c > 0 (that of cycle 0 is P): K + (c & 1) * K_stride, pitch ldk
     int64_t K_stride;
     int ldk;
+    float* Y;                      // scratch, m x keep, pitch ldu
 };
+inline int block_step_launches(int m, bool inner) { return inner && m > 128 ? 2 : 1; }
 // Columns [col0, col1) of C from cycle c0's to cycle c1's (c0 = 0: from P), and what they give of window c1; inner: also the inner
 // products of the kept rows with each other, from window c1 - 1.
 cudaError_t launch_block_step(const BlockSmall& b, int c0, int c1, int col0, int col1, bool inner, cudaStream_t st) SAGE_OPTIONAL;
