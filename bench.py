@@ -44,9 +44,7 @@ FP32_ALU_PEAK_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12     # SMs x FMA lanes x 2 
 ALL = ("c1", "c2", "c3", "c4", "c5")
 # DRAM bytes per launch of the dominant streaming kernels from one ncu capture each (profiles/): the capture ran on a
 # scaled-down D and the traffic grows in proportion to D, so the figure is stored per buffer column.
-# (Gram and rebuild: launches of cycles that read their 65 new rows in place, as 7 of 8 cycles of c5 do.)
-NCU_TRAFFIC_PER_COLUMN = {("c5", "rebuild"): (431.463e6 + 243.809e6) / 1117396, ("c5", "gram"): (433.728e6 + 4.061e6) / 1117396,
-                          ("c5", "project"): (1294.674e6 + 3.727e6) / 1117396}
+NCU_TRAFFIC_PER_COLUMN = {("c5", "project"): (1294.674e6 + 3.727e6) / 1117396}
 
 
 def rounded(x):
@@ -340,10 +338,17 @@ def run_workload(w, args, steps, warmup, ctx, want_e2e, want_cpu, sketches, fact
     # rows that whole shrink cycles read in place (never appended; bf16, 2 bytes instead of the buffer's 4): counted by the
     # library since the reset at the start of the last step
     in_place = stats.get("rows_in_place", 0)
+    # single sketches shrink in blocks of several cycles: a row is np planes of bfloat16, a row of the sketch three; a block's planes are
+    # read for their inner products and for the rebuild, which writes the kept rows' planes (fp32 at the freeze)
+    blocks = sketches == 1
+    np_planes = 3 if e == 4 else 2 if factored else 1
+    n_blocks = -(-max(full - 1, 0) // (4 if D >= 1 << 18 else max(4, 352 // (ell + 1)))) + 1
+    planes_read = (N * np_planes + n_blocks * 3 * keep) * 2 * D
     per_step_bytes = {
-        "append": (N - in_place) * D * (e + 4),
-        "gram": (full * m + r_final) * D * 4 - in_place * D * (4 - e),
-        "rebuild": (full * (m + keep) + (r_final + max(keep_final, ell))) * D * 4 - in_place * D * (4 - e),
+        **({} if blocks else {"append": (N - in_place) * D * (e + 4)}),
+        "gram": planes_read if blocks else (full * m + r_final) * D * 4 - in_place * D * (4 - e),
+        "rebuild": planes_read + (n_blocks * 3 * keep * 2 + ell * 4) * D if blocks else
+        (full * (m + keep) + (r_final + max(keep_final, ell))) * D * 4 - in_place * D * (4 - e),
         "project": N * D * e,
         "normalise": N * ell * 8,
         "score": N * ell * 4 + N * 4,
@@ -359,9 +364,9 @@ def run_workload(w, args, steps, warmup, ctx, want_e2e, want_cpu, sketches, fact
                 "algorithmic": "9*n^3 flop per n x n symmetric eigen-solve (textbook count)"}
     else:
         gbs = per_step_bytes.get(dominant, 0) / (dom_ms_per_step * 1e-3) / 1e9
-        rebuild = "k_tc_rebuild_narrow" if ell <= 64 else "k_tc_rebuild" if ell <= 128 else "k_tc_rebuild_wide"
+        rebuild = "k_block_factors + k_tc_rebuild_block" if blocks else "k_tc_rebuild_narrow" if ell <= 64 else "k_tc_rebuild" if ell <= 128 else "k_tc_rebuild_wide"
         project = "k_tc_gemm_nt" if e == 2 else "k_tc_project" if ell <= 64 else "k_tc_gemm_nt_x3"
-        kname = {"gram": "k_tc_gemm_nt_x3 (Gram)" if ell <= 64 else "k_tc_gram_pair", "rebuild": rebuild, "append": "k_append",
+        kname = {"gram": "k_tc_gram_block" if blocks else "k_tc_gemm_nt_x3 (Gram)" if ell <= 64 else "k_tc_gram_pair", "rebuild": rebuild, "append": "k_block_append" if blocks else "k_append",
                  "project": f"{project} (projection)"}.get(dominant, dominant)
         traffic = NCU_TRAFFIC_PER_COLUMN.get((w.name, dominant))
         roof = {"kernel": kname, "bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
@@ -385,7 +390,7 @@ def run_workload(w, args, steps, warmup, ctx, want_e2e, want_cpu, sketches, fact
         kernels[name] = entry
     roof_pass2_s = max(N * D * e / (peaks["hbm_gbs"] * 1e9), 2.0 * N * ell * D / (peaks["bf16_tflops_sustained"] * 1e12))
     # pass-1 roofline: the bytes of the method with every row appended to an fp32 buffer (append read + write, Gram read,
-    # rebuild read + write); cycles that read their rows in place move fewer, so the fraction compares TIME with that model
+    # rebuild read + write, every cycle); blocks of cycles move fewer, so the fraction compares TIME with that model
     p1_bytes = N * D * (e + 4) + (full * m + r_final) * D * 4 + (full * (m + keep) + (r_final + max(keep_final, ell))) * D * 4
     roof_pass1_s = p1_bytes / (peaks["hbm_gbs"] * 1e9)
     stream_ms = sum(prof_all[k]["ms"] for k in ("append", "gram", "gram_reduce", "rebuild"))

@@ -64,7 +64,11 @@ typedef enum { SAGE_F32 = 0, SAGE_BF16 = 1 } sage_dtype_t;
  *   ell        sketch size, 2 <= ell <= 256.
  *   row_dtype  element type of every rows pointer later given to this handle.
  *   device     CUDA device ordinal; all later calls must be made with pointers of this device.
- * Allocates about 2 * (2*ell) * D * 4 bytes of device memory. Synchronous. */
+ * Device memory, in bytes per column: 4 ell for the frozen sketch and, while sketching in blocks of L = max(4, 352 / (ell + 1)) shrink
+ * cycles (4 for D >= 2^18), 12 (ell - 1) for two copies of its planes and 2 (bfloat16) or 6 (float32) for each of the up to
+ * ell - 1 + L (ell + 1) rows of a block (bfloat16 handles: 4 where that is below 640 MB in all, for structured rows). Where that would be
+ * more than 40 GiB, or is not there, and in the forms of pass 1 that options 1, 4 and 6 choose: 2 * (2*ell) * D * 4 bytes, a buffer
+ * that shrinks cycle by cycle. Synchronous. */
 sage_status_t sage_fd_create(sage_fd_t** out, int64_t D, int32_t ell, sage_dtype_t row_dtype, int device);
 
 /* Releases everything the handle owns (synchronises the device first). NULL is allowed. */
@@ -287,11 +291,10 @@ sage_status_t sage_fd_stats(sage_fd_t* h, sage_stats_t* out);
  * is initialised; streams that share a queue do not overlap, so with P > 8 set it to 32 before the process touches CUDA.)
  * Outside a scoring pass: key 8 = 1 for the strict-memory form of Phase II (see sage_score_apply), 0 (default) to keep the
  * N x ell normalised projections.
- * At any time: key 9 = 1 (default) lets a shrink cycle whose ell + 1 new rows all lie in one sage_fd_update call read them
- * where the caller holds them instead of appending them to the buffer first (bfloat16 rows, ell = 32 or 64, tensor-core
- * kernels, the paper's single sketch: the Gram and rebuild kernels take rows 0 .. ell - 2 from the buffer and convert the
- * caller's rows on the way into the operand tiles; same arithmetic and the same results as the appended form); rows that do
- * not fill a cycle are appended as before. 0: always append. Either way `rows` must stay unchanged until the work enqueued by
+ * At any time: key 9 = 1 (default) lets shrink cycles read their rows where the caller holds them instead of copying them first:
+ * bfloat16 rows on 16-byte boundaries (base and pitch), tensor-core kernels, the paper's single sketch, rows that complete a block within
+ * one sage_fd_update call; same arithmetic and the same bits as the copied form; rows that do
+ * not are copied. 0: always copy. Either way `rows` must stay unchanged until the work enqueued by
  * the call has run (stream order on cuda_stream takes care of that for work enqueued there afterwards). */
 sage_status_t sage_fd_set_option(sage_fd_t* h, int key, double value);
 

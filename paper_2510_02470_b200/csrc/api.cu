@@ -253,6 +253,7 @@ struct sage_fd {
         int s_rows = 0, n_raw = 0; // its rows, and the rows given since
         int n_gram = 0;            // logical rows whose inner products are in P
         int cycles = 0;            // cycles done
+        bool step_due = false;     // window `cycles` has not been begun: that waits for its rows
         int np = 0;                // planes a row of R
     } blk;
 };
@@ -724,6 +725,7 @@ sage_status_t sage_fd_reset(sage_fd_t* h) {
     h->pend_n = 0;
     h->used = nullptr;
     h->blk.s_rows = h->blk.n_raw = h->blk.n_gram = h->blk.cycles = 0;
+    h->blk.step_due = false;
     h->blk.np = h->dtype == SAGE_F32 ? 3 : 1;
     for (sage_fd* k : h->kids) ST_TRY(sage_fd_reset(k));
     return settle_form(h);
@@ -809,7 +811,7 @@ sage_status_t sage_fd_set_option(sage_fd_t* h, int key, double value) {
 
 // Cycles of a block: as many as make 352 new rows, at least 4. Per cycle the kernels that read the rows cost 1 / L of a launch that takes
 // little longer for more rows; beyond that the inner products among a block's rows, which grow with the square, take over: 4 cycles where
-// rows are long (64 rows, 11.2 M values: 5 cycles are 544 planes and a third block of 256 of them, 2.3 ms a cycle instead of 1.7). The
+// rows are long (ell 64, 11.2 M values: 5 cycles are 544 planes and a third block of 256 of them, 2.3 ms of Gram and rebuild a cycle; 4: 2.0). The
 // first block ends with the first shrink.
 static int block_cycles(int64_t D, int ell) { return D >= ((int64_t)1 << 18) ? 4 : std::max(4, 352 / (ell + 1)); }
 static int block_cycles_now(const sage_fd* h) { return h->blk.s_rows < h->ell - 1 ? 1 : h->blk.L; }
@@ -988,14 +990,25 @@ static sage_status_t block_rebuild(sage_fd* h, const BlockMap& map, const BlockS
     return SAGE_OK;
 }
 
-// Products of the rows that have come since the last cycle, and what they give of the open window.
-static sage_status_t block_catch_up(sage_fd* h, const BlockMap& map, const BlockSource& src, cudaStream_t st) {
+// The step into window `cycles`, if it is due; columns from `before` on are new and have all cycles before them.
+static sage_status_t block_step(sage_fd* h, int before, cudaStream_t st) {
     auto& k = h->blk;
-    const int before = k.n_gram;
-    ST_TRY(block_gram(h, map, src, st));
-    if (k.cycles > 0 && k.n_gram > before)
-        CU_TRY(timed(h, K_GRAM_REDUCE, 1, st, [&] { return launch_block_step(block_small(h), 0, k.cycles, before, k.n_gram, false, st); }));
+    const int c = k.cycles;
+    if (!k.step_due && (c == 0 || k.n_gram == before)) return SAGE_OK;
+    const bool due = k.step_due;
+    k.step_due = false;
+    CU_TRY(timed(h, K_GRAM_REDUCE, block_step_launches(h->m, due), st, [&] {
+        return launch_block_step(block_small(h), due ? c - 1 : 0, c, due ? h->ell - 1 + c * (h->ell + 1) : before, before, k.n_gram, due, st);
+    }));
     return SAGE_OK;
+}
+
+// Products of the rows that have come since the last cycle, and what they give of the open window. (In one launch with a step that waited
+// for them: 6,000 rows of 5,130, ell 64, in calls of 64 rows 12.2 ms with a launch each, 11.8 so.)
+static sage_status_t block_catch_up(sage_fd* h, const BlockMap& map, const BlockSource& src, cudaStream_t st) {
+    const int before = h->blk.n_gram;
+    ST_TRY(block_gram(h, map, src, st));
+    return block_step(h, before, st);
 }
 
 // Ends an open block at its last cycle: the kept rows are formed, the rows behind them (fewer than a cycle's) begin the next block.
@@ -1004,6 +1017,7 @@ static sage_status_t block_end_early(sage_fd* h, cudaStream_t st) {
     if (k.cycles == 0) return SAGE_OK;
     const int keep = h->ell - 1, raw = h->m + (k.cycles - 1) * (h->ell + 1) - k.s_rows, rest = k.n_raw - raw;
     const BlockMap map = block_map(k.s_rows, k.np, raw, 0);
+    ST_TRY(block_step(h, k.n_gram, st));
     ST_TRY(block_rebuild(h, map, block_source(h, nullptr, 0), k.cycles, k.cycles, h->m, keep, nullptr, st));
     const size_t row = (size_t)k.np * k.pitch;             // (raw >= ell + 1 > rest: the two ranges lie apart)
     if (rest > 0) CU_TRY(cudaMemcpyAsync(k.R, k.R + raw * row, rest * row * sizeof(__nv_bfloat16), cudaMemcpyDeviceToDevice, st));
@@ -1045,13 +1059,15 @@ static sage_status_t block_feed(sage_fd* h, RowSrc src, int64_t n, cudaStream_t 
         while (k.cycles < L && nl + take >= m + k.cycles * step) {
             ST_TRY(block_solve(h, m, 1, keep, st));
             const int c = ++k.cycles;
-            if (c < L) CU_TRY(timed(h, K_GRAM_REDUCE, block_step_launches(m, true), st, [&] { return launch_block_step(block_small(h), c - 1, c, keep + c * step, k.n_gram, true, st); }));
+            k.step_due = c < L;
+            if (c < L && nl + take >= m + c * step) ST_TRY(block_step(h, k.n_gram, st));
         }
         if (k.cycles == L) {
             ST_TRY(block_rebuild(h, map, from, L - 1, L, m, keep, nullptr, st));
             k.cur = 1 - k.cur;
             k.s_rows = keep;
             k.n_raw = k.n_gram = k.cycles = 0;
+            k.step_due = false;
         }
     }
     h->fill = k.s_rows + k.n_raw - k.cycles * step;
@@ -2207,6 +2223,8 @@ sage_status_t sage_fd_export(sage_fd_t* h, void* dst_host, size_t capacity, size
         CU_TRY(cudaMemcpy(&es.info, h->info, sizeof(EigInfo), cudaMemcpyDeviceToHost));
         std::memcpy(out, &es, sizeof es);
         out += sizeof es;
+        ST_TRY(block_step(h, h->blk.n_gram, nullptr));         // a step that waits for rows: the same bits now as with them
+        CU_TRY(cudaDeviceSynchronize());
         const ExportBlock eb = export_block(h);
         std::memcpy(out, &eb, sizeof eb);
         out += sizeof eb;

@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(Apply<JG>::NT, 1) k_block_inner(BlockSmall b, 
 // the products with rows still to come. Bound by latency: every round trip to L2 counts. ahead: the launch follows a solve, so that
 // everything but W was there before that solve began; it is fetched before the wait for it (K into shared memory where it fits).
 template <int JG>
-__global__ void __launch_bounds__(Apply<JG>::NT, 1) k_block_step(BlockSmall b, int c0, int c1, int col0, int col1, int n_inner, int ahead) {
+__global__ void __launch_bounds__(Apply<JG>::NT, 1) k_block_step(BlockSmall b, int c0, int c1, int col0, int col1, int n_inner, int n_cols, int late1, int ahead) {
     constexpr int NT = Apply<JG>::NT, cols = Apply<JG>::COLS;
     extern __shared__ __align__(16) float smem[];
     auto x = reinterpret_cast<typename Apply<JG>::Row*>(smem), y = x + b.m;  // [m] each
@@ -282,7 +282,12 @@ __global__ void __launch_bounds__(Apply<JG>::NT, 1) k_block_step(BlockSmall b, i
         }
         return;
     }
-    const int g0 = col0 + ((int)blockIdx.x - n_inner) * cols;
+    int g0 = col0 + ((int)blockIdx.x - n_inner) * cols;
+    if ((int)blockIdx.x >= n_inner + n_cols) {                               // columns that come late, from cycle 0 on
+        g0 = col1 + ((int)blockIdx.x - n_inner - n_cols) * cols;
+        c0 = 0;
+        col1 = late1;
+    }
     const float* top = c0 == 0 ? b.P : b.C;
     const int e0 = keep + c0 * step, w0 = keep + c1 * step;                  // the first rows behind the kept ones of windows c0 and c1
     for (int t = tid; t < keep * cols; t += NT) {
@@ -309,7 +314,7 @@ __global__ void __launch_bounds__(Apply<JG>::NT, 1) k_block_step(BlockSmall b, i
             else if (g >= e) v = g - e == i ? 1.f : 0.f;
             x[keep + i][t % cols] = v;
         }
-        if (ahead) chain_wait();                                             // (one cycle: c1 == c0 + 1)
+        if (ahead) chain_wait();                                             // (one cycle then)
         __syncthreads();
         apply.run(b.U + (int64_t)c * b.U_stride, b.ldu, m, keep, x, y, false);
         for (int t = tid; t < keep * cols; t += NT) x[t / cols][t % cols] = y[t / cols][t % cols];
@@ -434,15 +439,16 @@ cudaError_t launch_block_gram_reduce(const float* parts, const BlockMap& map, in
     return launch_chained(kernel, dim3((nl + 3) / 4, (nl - first_new + 31) / 32), dim3(256), 0, st, parts, map, first_new, slices, P, ldP);
 }
 
-cudaError_t launch_block_step(const BlockSmall& b, int c0, int c1, int col0, int col1, bool inner, cudaStream_t st) {
+cudaError_t launch_block_step(const BlockSmall& b, int c0, int c1, int col0, int col1, int late1, bool inner, cudaStream_t st) {
     if (inner && b.m <= kCarryRows) col0 = 0;
     constexpr int cols = Apply<16>::COLS;
     const int n_inner = inner ? (b.keep + cols - 1) / cols : 0, n_cols = col1 > col0 ? (col1 - col0 + cols - 1) / cols : 0;
-    if (n_inner + n_cols == 0) return cudaSuccess;
+    const int n_late = late1 > col1 ? (late1 - col1 + cols - 1) / cols : 0;
+    if (n_inner + n_cols + n_late == 0) return cudaSuccess;
     auto go = [&](auto kernel, int threads, size_t smem) -> cudaError_t {
         const cudaError_t e = allow_smem((const void*)kernel, kSmallSmem);
         if (e != cudaSuccess) return e;
-        return launch_chained(kernel, dim3(n_inner + n_cols), dim3(threads), smem, st, b, c0, c1, col0, col1, n_inner, inner && c1 == c0 + 1 ? 1 : 0);
+        return launch_chained(kernel, dim3(n_inner + n_cols + n_late), dim3(threads), smem, st, b, c0, c1, col0, col1, n_inner, n_cols, late1, inner && n_late == 0 ? 1 : 0);
     };
     if (inner && b.m > 128) {
         auto first = [&](auto kernel, int threads, int rows, size_t apply) -> cudaError_t {

@@ -302,9 +302,10 @@ struct BlockSmall {
     float* Y;                      // scratch, m x keep, pitch ldu
 };
 inline int block_step_launches(int m, bool inner) { return inner && m > 128 ? 2 : 1; }
-// Columns [col0, col1) of C from cycle c0's to cycle c1's (c0 = 0: from P), and what they give of window c1; inner: also the inner
-// products of the kept rows with each other, from window c1 - 1.
-cudaError_t launch_block_step(const BlockSmall& b, int c0, int c1, int col0, int col1, bool inner, cudaStream_t st) SAGE_OPTIONAL;
+// Columns [col0, col1) of C from cycle c0's to cycle c1's (c0 = 0: from P), those of [col1, late1) from cycle 0's, and what they give of
+// window c1; inner: c1 = c0 + 1, also the inner products of the kept rows with each other, from window c0 (and, without late columns,
+// the launch follows window c0's solve).
+cudaError_t launch_block_step(const BlockSmall& b, int c0, int c1, int col0, int col1, int late1, bool inner, cudaStream_t st) SAGE_OPTIONAL;
 // The kept rows after ncyc cycles as combinations of planes: T[t][j][p], t < 3, j < j_pad (the planes of the coefficients, pitch ldT), for
 // p < P rounded up to 64; carried: the cycles behind which launch_block_step has been. The last cycle's factors have keep_last columns and its window r_last rows.
 cudaError_t launch_block_factors(const BlockSmall& b, const BlockMap& map, int carried, int ncyc, int r_last, int keep_last, __nv_bfloat16* T, int j_pad, int64_t ldT,
